@@ -115,8 +115,6 @@ typedef struct {
  *                           256-row-tile kernel would run (several activation tiles)
  *   LSTM_B200_PROJ_SMEM_KB = 48..200  shared-memory budget of the 128-row-tile projection kernel (ring depth)
  *   LSTM_B200_CTAS  = <n>   at most n CTAs per direction in the recurrent kernels (measurement)
- *   LSTM_B200_TC_ISSUE = 1|2  fewer issuing threads (and accumulators) in the batched tensor-core recurrence than the
- *                           three it uses where the K extent allows
  *   LSTM_B200_COMPACT = 0   keep row/column-pruned units as explicit zeros, = 1 always run on the surviving units
  *                           (unset: handles with max_B >= 5 compact, smaller ones keep the zeros; see below)
  * Row/column-pruned stacks (Section 4.2, Algorithm 1: whole rows and columns of the gate matrices are zero).

@@ -34,8 +34,7 @@ struct Layer {
     uint4 *wfrag[2] = {nullptr, nullptr};  // register-resident kernel: operand-A fragments
     uint4 *xfrag[2] = {nullptr, nullptr};  //   and Wx in the same layout (projection fused into the kernel's prologue)
     int nkw_x = 0;
-    __nv_bfloat16 *wtc = nullptr;          // batched tensor-core kernel: [D * ncta * RA][ld64] rows 4*unit+gate per CTA
-    alignas(64) unsigned char tmap_wtc[128];
+    uint4 *wtc[2] = {nullptr, nullptr};    // batched tensor-core kernel: [cta][8-column piece][row 4 * unit + gate]
     uint4 *frag2[2] = {nullptr, nullptr};  // H-LSTM: fragments of the gate output matrices W
     float *bias_out = nullptr;             // H-LSTM: [D][H][4] bias of the gate pre-activations
     int csr_max_slice_entries = 0;     // largest per-CTA slice (entries, padded)
@@ -65,13 +64,11 @@ struct lstm_handle {
     int csr_nw = 0, csr_kspan = 0, csr_mt = 0, csr_slots = 0;
     long long csr_conflicts = 0;       // shared-memory wavefronts per step and CTA lost to bank conflicts (worst CTA, worst matrix)
     int mma_mt = 0, mma_nkr = 0, mma_nks = 0, mma_nw = 0;
-    // batched tensor-core recurrence (more than four batch rows): weight-tile rows, K blocks, planes, stamps
     bool seq_dirs = false;             // bidirectional layers run one direction after the other, each on all SMs
+    // batched tensor-core recurrence: partition and exchange words (two sets: a launch clears the other one)
     bool use_tcb = false;
-    bool tcb_pair = false;             // the batched recurrence splits K over clusters of two CTAs
-    int tcb_RA = 0, tcb_nkb = 0, tcb_ld = 0, tcb_ldh = 0, tcb_mapN = 0;
-    __nv_bfloat16 *hplanes = nullptr; unsigned *tcb_flags = nullptr;
-    alignas(64) unsigned char tmap_planes[128];
+    RecurTcPlan tcb = {0, 0, 0, 0, 0};
+    unsigned *tcb_xch = nullptr; int tcb_set = 0, tcb_dirty = 0;
     // H-LSTM cell: width of the hidden layer inside each gate (0: plain LSTM), pass-2 column tiles per warp
     int Hh = 0, hl_nkw2 = 0;
     unsigned long long *rxch = nullptr; size_t rxch_words = 0;
@@ -402,6 +399,28 @@ std::vector<uint32_t> pack_fragments(const float *m, int U, int K, int ncta, int
     return f;
 }
 
+// Rows of a [4H x H] recurrent matrix (row q*H + j) as the batched tensor-core kernel wants them: per CTA [8-column
+// piece of its K range][row 4 * unit + gate of its units, in pair mode of both CTAs' units] 8 bf16.
+std::vector<uint16_t> pack_tc_rows(const float *m, int H, const RecurTcPlan &p)
+{
+    const int units = p.pair ? 2 * p.upc : p.upc, rows = 4 * units, pieces = p.KH / 8;
+    std::vector<uint16_t> out((size_t)p.ncta * pieces * rows * 8, 0);
+    for (int c = 0; c < p.ncta; ++c) {
+        const int k0 = p.pair ? (c & 1) * p.KH : 0, k1 = std::min(H, k0 + p.KH), u0 = (p.pair ? c / 2 : c) * units;
+        uint16_t *dst = out.data() + (size_t)c * pieces * rows * 8;
+        const int nu = std::max(0, std::min(units, H - u0));
+        for (int k = k0; k < k1; k += 8) {                      // reads run down the rows, writes are contiguous
+            const int n = std::min(8, k1 - k);
+            uint16_t *d8 = dst + (size_t)((k - k0) >> 3) * rows * 8;
+            for (int r = 0; r < 4 * nu; ++r) {
+                const float *src = m + (size_t)((r & 3) * H + u0 + (r >> 2)) * H + k;
+                for (int e = 0; e < n; ++e) d8[r * 8 + e] = f32_to_bf16_rne(src[e]);
+            }
+        }
+    }
+    return out;
+}
+
 // Tiling of the layer-wavefront kernel, or use_wave = false when the stack does not qualify: one direction, two
 // to four layers, bf16 dense, at most 16 units per CTA with the SMs split evenly between the layers, and the
 // widest layer's slice (4 * units rows by 2H columns) inside registers + shared memory.
@@ -434,10 +453,10 @@ void free_all(lstm_handle *h)
     for (auto &ly : h->layers) {
         cudaFree(ly.wx); cudaFree(ly.bias); cudaFree(ly.wx_rowptr); cudaFree(ly.wx_ent);
         for (int d = 0; d < 2; ++d) { cudaFree(ly.wh[d]); cudaFree(ly.wh_ptr[d]); cudaFree(ly.wh_ent[d]); cudaFree(ly.wfrag[d]); cudaFree(ly.xfrag[d]); cudaFree(ly.frag2[d]); cudaFree(ly.csr_reg_ent[d]); cudaFree(ly.csr_reg_rows[d]); }
-        cudaFree(ly.bias_out); cudaFree(ly.wtc);
+        cudaFree(ly.bias_out); cudaFree(ly.wtc[0]); cudaFree(ly.wtc[1]);
     }
     cudaFree(h->G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
-    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); cudaFree(h->hplanes); cudaFree(h->tcb_flags); cudaFree(h->status_dev);
+    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); cudaFree(h->tcb_xch); cudaFree(h->status_dev);
     for (int l = 0; l < kMaxWaveLayers; ++l) cudaFree(h->wave_frag[l]);
     cudaFree(h->wave_xch);
     cudaFree(h->cmap); cudaFree(h->rem_idx); cudaFree(h->rem_bias);
@@ -561,16 +580,20 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                              recur_csr_reg_fuse_smem_bytes(nw, kspan, mt, h->upc) <= (size_t)h->smem_optin - 64;
         }
     }
-    // does the batched tensor-core recurrence fit with the current split of the SMs?
-    auto tcb_fits = [&](int *kbs, int *stages) -> bool {
+    // Batched tensor-core recurrence (handles made for more than four sequences), with the current split of the SMs: as
+    // clusters of two where the device can co-schedule them, else every CTA alone.  bf16 CSR handles use it too, with the
+    // zeros multiplied.
+    auto plan_tcb = [&](int ncta, int dirs_side_by_side) -> bool {
         const char *env = getenv("LSTM_B200_RECUR");
-        const int RA = round_up(4 * h->upc, 8), nkb = (H + 63) / 64;
-        if (!(bf16 && !csr && max_B > 4 && RA <= 128) || (env && (strcmp(env, "mma") == 0 || strcmp(env, "simt") == 0))) return false;
-        const int B = std::min(max_B, 32), N = round_up(2 * B, 16);
-        return h->ncta_dir <= 160 && recur_tc_plan(RA, nkb, N, h->upc, B, (size_t)h->smem_optin - kTcStaticSmem, 0, kbs, stages);
+        if (!bf16 || (csr && !h->csr_dense_proj) || max_B <= 4 || (env && (strcmp(env, "mma") == 0 || strcmp(env, "simt") == 0))) return false;
+        const size_t smem = (size_t)h->smem_optin - kTcStaticSmem;
+        if (recur_tc_prepare((int)smem) != cudaSuccess) { cudaGetLastError(); return false; }
+        if (!(env && strcmp(env, "tc1") == 0) && recur_tc_plan(H, ncta, max_B, 1, smem, &h->tcb) &&
+            recur_tc_pair_supported(h->tcb.ncta * dirs_side_by_side, h->tcb.rows, recur_tc_smem_bytes(h->tcb.KH, h->tcb.upc, h->tcb.rows, 1))) return true;
+        return recur_tc_plan(H, ncta, max_B, 0, smem, &h->tcb);
     };
-    int kbs_tmp = 0, stages_tmp = 0;
-    if (D == 2 && bf16 && !csr && !h->use_mma && !tcb_fits(&kbs_tmp, &stages_tmp)) {
+    h->use_tcb = plan_tcb(h->ncta_dir, D);
+    if (D == 2 && bf16 && !csr && !h->use_mma && !h->use_tcb) {
         // Side by side, each direction has half the SMs and a slice twice as tall; when that slice fits
         // neither the register-resident kernel nor (for handles made for batches) the tensor-core one, run
         // the directions one after the other on all SMs instead: twice the steps, but every step on-chip.
@@ -579,28 +602,8 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         h->upc = (H + h->ncta_dir - 1) / h->ncta_dir;
         h->threads = std::max(128, 32 * std::min(h->upc, 16));
         plan_mma(h);
-        if (h->use_mma) h->seq_dirs = true;
+        if (h->use_mma) { h->seq_dirs = true; h->use_tcb = plan_tcb(h->ncta_dir, 1); }
         else { h->ncta_dir = nc; h->upc = up; h->threads = th; }
-    }
-    if (tcb_fits(&kbs_tmp, &stages_tmp)) {   // batched tensor-core recurrence, beside the kernels for up to four sequences
-        h->use_tcb = true; h->tcb_RA = round_up(4 * h->upc, 8); h->tcb_nkb = (H + 63) / 64; h->tcb_ld = h->tcb_nkb * 64;
-        h->tcb_ldh = round_up(H, 64);      // rows of the planes start on 128-byte lines: a TMA box row is one line, not two
-        // pair mode: two CTAs of a cluster split K (half the tensor instructions per step) when the pairs do
-        // not straddle directions, the doubled tile fits, and the device can co-schedule the clusters
-        const char *env = getenv("LSTM_B200_RECUR");
-        const int Bp = std::min(max_B, 32), Np = round_up(2 * Bp, 16);
-        int kp = 0, sp = 0;
-        // a pair's tile holds both CTAs' rows back to back: 2 x 4 x units is already a multiple of the 8-row swizzle
-        // group, so the rows are not padded (at 11 units per CTA the 8 rows saved per K block let the ring hold a
-        // whole step's operand)
-        const int RAp = 4 * h->upc;
-        if (!(env && strcmp(env, "tc1") == 0) && (h->ncta_dir % 2) == 0 &&
-            recur_tc_plan(RAp, h->tcb_nkb, Np, h->upc, Bp, (size_t)h->smem_optin - kTcStaticSmem, 1, &kp, &sp) &&
-            recur_tc_prepare(h->smem_optin - kTcStaticSmem) == cudaSuccess &&
-            recur_tc_pair_supported(h->ncta_dir * (h->seq_dirs ? 1 : D), recur_tc_smem_bytes(RAp, h->tcb_nkb, Np, sp, kp, h->upc, Bp, 1))) {
-            h->tcb_pair = true;
-            h->tcb_RA = RAp;
-        }
     }
     h->layers.resize(layers);
     if (const char *env = getenv("LSTM_B200_SPIN_LIMIT")) { long long v = atoll(env); if (v > 0) h->spin_limit = v; }
@@ -619,7 +622,6 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         std::vector<float> bias_p((size_t)N, 0.0f);
         std::vector<uint16_t> wx16; std::vector<float> wx32;
         std::vector<int> px_rowptr; std::vector<CsrEntry> px_ent;
-        std::vector<uint16_t> tcb_rows;
         if (!csr) { if (bf16) wx16.assign((size_t)N * ly.ldk, 0); else wx32.assign((size_t)N * ly.ldk, 0.0f); }
         else { px_rowptr.assign(N + 1, 0); if (h->csr_dense_proj) wx16.assign((size_t)N * ly.ldk, 0); }
 
@@ -704,18 +706,9 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                     if (rc == LSTM_OK) cudaStreamSynchronize(st);
                 }
                 if (rc == LSTM_OK && h->use_tcb) {
-                    // the same slices as plain K-major rows for the tensor-core kernel's TMA tiles
-                    const size_t rows_dir = (size_t)h->ncta_dir * h->tcb_RA;
-                    if (d == 0) tcb_rows.assign((size_t)D * rows_dir * h->tcb_ld, 0);
-                    for (int c = 0; c < h->ncta_dir; ++c) {
-                        int u0, nu; unit_range_host(H, h->ncta_dir, c, u0, nu);
-                        for (int u = 0; u < nu; ++u)
-                            for (int q = 0; q < 4; ++q) {
-                                const float *srow = m.data() + (size_t)(q * H + u0 + u) * H;
-                                uint16_t *drow = tcb_rows.data() + ((size_t)d * rows_dir + (size_t)c * h->tcb_RA + 4 * u + q) * h->tcb_ld;
-                                for (int k = 0; k < H; ++k) drow[k] = f32_to_bf16_rne(srow[k]);
-                            }
-                    }
+                    const std::vector<uint16_t> p = pack_tc_rows(m.data(), H, h->tcb);
+                    rc = upload(h, (uint16_t **)&ly.wtc[d], p.data(), p.size() * 2, st, "recurrent weight rows");
+                    if (rc == LSTM_OK) cudaStreamSynchronize(st);
                 }
             } else {
                 HostCsr cx, ch;
@@ -749,6 +742,15 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                 snprintf(name, sizeof name, "wh[layer %d, dir %d]", l, d);
                 rc = matrix_to_csr(h, 4 * H, H, src.wh, src.mask_h, src.wh_rowptr, src.wh_col, src.wh_val, ch, name);
                 if (rc) break;
+                if (h->use_tcb) {
+                    std::vector<float> m((size_t)4 * H * H, 0.0f);
+                    for (int r = 0; r < 4 * H; ++r)
+                        for (int e = ch.rowptr[r]; e < ch.rowptr[r + 1]; ++e) m[(size_t)r * H + ch.col[e]] = ch.val[e];
+                    const std::vector<uint16_t> p = pack_tc_rows(m.data(), H, h->tcb);
+                    rc = upload(h, (uint16_t **)&ly.wtc[d], p.data(), p.size() * 2, st, "recurrent weight rows");
+                    if (rc == LSTM_OK) cudaStreamSynchronize(st);
+                    if (rc) break;
+                }
                 if (h->use_csr_reg) {
                     csr_lane_lists(ch.rowptr.data(), ch.col.data(), ch.val.data(), H, h->ncta_dir, h->csr_nw, h->csr_kspan, ly.csr_lists[d]);
                     h->csr_slots = std::max(h->csr_slots, ly.csr_lists[d].longest);
@@ -780,11 +782,6 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         }
         if (rc) break;
         rc = upload(h, &ly.bias, bias_p.data(), bias_p.size() * 4, st, "bias");
-        if (rc == LSTM_OK && h->use_tcb && !tcb_rows.empty()) {
-            rc = upload(h, (uint16_t **)&ly.wtc, tcb_rows.data(), tcb_rows.size() * 2, st, "recurrent weight tiles");
-            if (rc == LSTM_OK && !recur_tc_encode_weights(ly.tmap_wtc, ly.wtc, (long long)D * h->ncta_dir * h->tcb_RA, h->tcb_ld, h->tcb_pair ? 2 * h->tcb_RA : h->tcb_RA))
-                rc = fail(h, LSTM_ERR_CUDA, "tensor map of the recurrent weight tiles could not be encoded");
-        }
         if (rc == LSTM_OK && !csr)
             rc = bf16 ? upload(h, (uint16_t **)&ly.wx, wx16.data(), wx16.size() * 2, st, "input weights")
                       : upload(h, (float **)&ly.wx, wx32.data(), wx32.size() * 4, st, "input weights");
@@ -841,8 +838,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     h->xch_words = (size_t)D * 2 * max_B * H;
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->xch, h->xch_words * 8, true, st, "exchange buffer");
     if (rc == LSTM_OK && h->use_tcb) {
-        rc = dev_alloc(h, &h->hplanes, (size_t)D * 2 * kTcPlaneRows * h->tcb_ldh * 2, true, st, "h planes");
-        if (rc == LSTM_OK) rc = dev_alloc(h, &h->tcb_flags, (size_t)D * h->ncta_dir * sizeof(unsigned), true, st, "stamps");
+        rc = dev_alloc(h, &h->tcb_xch, (size_t)2 * D * 2 * round_up(H, 16) * h->tcb.rows * sizeof(unsigned), true, st, "exchange words");
     }
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->status_dev, sizeof(int), true, st, "status word");
     if (rc == LSTM_OK && h->use_wave) {
@@ -858,7 +854,6 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                                          : recur_dense_prepare(h->smem_optin - 64);
         if (e == cudaSuccess && h->use_tc) e = proj_tc_prepare();
         if (e == cudaSuccess && csr) e = proj_csr_prepare(h->smem_optin - 64);
-        if (e == cudaSuccess && h->use_tcb) e = recur_tc_prepare(h->smem_optin - kTcStaticSmem);
         if (e != cudaSuccess) rc = fail(h, LSTM_ERR_CUDA, "kernel set-up failed: %s", cudaGetErrorString(e));
     }
     if (rc == LSTM_OK && cudaStreamSynchronize(st) != cudaSuccess)
@@ -1279,7 +1274,6 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
     if ((unsigned long long)h->stamp_next + (unsigned long long)L * D * ((unsigned long long)T + 1ull) + 2ull >= 0xffffffffull) {
         if (cudaMemsetAsync(h->xch, 0, h->xch_words * 8, st) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
         if (h->rxch && cudaMemsetAsync(h->rxch, 0, h->rxch_words * 8, st) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
-        if (h->tcb_flags && cudaMemsetAsync(h->tcb_flags, 0, (size_t)D * h->ncta_dir * sizeof(unsigned), st) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
         if (h->wave_xch && cudaMemsetAsync(h->wave_xch, 0, h->wave_xch_words * 8, st) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
         h->stamp_next = 1;
     }
@@ -1356,58 +1350,37 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             continue;
         }
-        int tc_kbs = 0, tc_stages = 0;
-        // the batched kernel serves this call if the operand ring for this batch fits beside the resident slice
-        // (the plan made at create time covers up to 32 sequences; larger batches may not fit and then run as
-        // passes of four on the kernels below)
-        if (h->use_tcb && B > 4 && B <= kTcMaxBatch &&
-            recur_tc_plan(h->tcb_RA, h->tcb_nkb, round_up(2 * B, 16), h->upc, B, (size_t)h->smem_optin - kTcStaticSmem, h->tcb_pair ? 1 : 0, &tc_kbs, &tc_stages)) {
-            RecurTcArgs m;
-            memset(&m, 0, sizeof m);
-            m.dir0 = h->seq_dirs ? pass : 0; m.ndirs = h->seq_dirs ? 1 : D;
-            m.H = H; m.B = B; m.T = T; m.D = D; m.ncta_dir = h->ncta_dir; m.nsplit = nsplit;
-            m.RA = h->tcb_RA; m.nkb = h->tcb_nkb; m.N = round_up(2 * B, 16);
-            m.pair = h->tcb_pair ? 1 : 0;
-            m.kbs = tc_kbs; m.stages = tc_stages;
-            {
-                // issuing threads: as many as the smaller K share of a CTA allows, at most three
-                const int nkb_min = m.pair ? m.nkb / 2 : m.nkb;
-                int ni = nkb_min >= 3 ? 3 : nkb_min >= 2 ? 2 : 1;
-                if (const char *e = getenv("LSTM_B200_TC_ISSUE")) {
-                    const int want = atoi(e);
-                    if (want >= 1 && want <= ni) ni = want;
-                }
-                m.nissue = ni;
-                const int cols = ni * m.N;
-                m.tmem_cols = cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
+        if (h->use_tcb && B > 4) {
+            // passes of at most tcb.rows batch rows, as equal as possible
+            const int passes = (B + h->tcb.rows - 1) / h->tcb.rows, dirs = h->seq_dirs ? 1 : D;
+            for (int p = 0; p < passes; ++p) {
+                RecurTcArgs m;
+                memset(&m, 0, sizeof m);
+                m.dir0 = h->seq_dirs ? pass : 0; m.ndirs = dirs;
+                m.Bs = B; m.b0 = (int)((long long)B * p / passes); m.B = (int)((long long)B * (p + 1) / passes) - m.b0;
+                m.H = H; m.T = T; m.D = D; m.nsplit = nsplit;
+                m.ncta_dir = h->tcb.ncta; m.upc = h->tcb.upc; m.KH = h->tcb.KH; m.pair = h->tcb.pair;
+                m.spin_limit = h->spin_limit;
+                m.withhold_cta = h->withhold_cta < 0 ? -1 : h->withhold_cta % (h->tcb.ncta * dirs);
+                m.wpack[0] = ly.wtc[0]; m.wpack[1] = ly.wtc[1];
+                m.G = h->G;
+                m.g_split_stride = (long long)M * N;
+                const size_t so = (size_t)l * D * B * H;
+                m.h0 = h0 ? h0 + so : nullptr; m.c0 = c0 ? c0 + so : nullptr;
+                m.hT = hT ? hT + so : nullptr; m.cT = cT ? cT + so : nullptr;
+                m.xb_next = (l < L - 1 && h->use_tc) ? h->xbn[l & 1] : nullptr;
+                m.y = l == L - 1 ? y : m.xb_next ? nullptr : h->ybuf[l & 1];
+                m.xb_ld = h->ldn;
+                m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
+                m.xch = h->tcb_xch; m.set = h->tcb_set; m.xch_rows = h->tcb.rows; m.clear_rows = h->tcb_dirty;
+                m.status = h->status_dev;
+                if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+                e = launch_recur_tc(m, st);
+                ++h->last_launches;
+                if (e == cudaSuccess) { h->tcb_set ^= 1; h->tcb_dirty = m.B; }
+                if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+                if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             }
-            m.ldh = h->tcb_ldh;
-            m.stamp_base = h->stamp_next;
-            h->stamp_next += (unsigned)T + 1u;
-            m.spin_limit = h->spin_limit;
-            m.withhold_cta = h->withhold_cta;
-            m.G = h->G;
-            m.g_split_stride = (long long)M * N;
-            const size_t so = (size_t)l * D * B * H;
-            m.h0 = h0 ? h0 + so : nullptr; m.c0 = c0 ? c0 + so : nullptr;
-            m.hT = hT ? hT + so : nullptr; m.cT = cT ? cT + so : nullptr;
-            m.y = l == L - 1 ? y : h->ybuf[l & 1];
-            m.xb_next = (l < L - 1 && h->use_tc) ? h->xbn[l & 1] : nullptr;
-            m.xb_ld = h->ldn;
-            m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
-            m.hbuf = h->hplanes; m.flags = h->tcb_flags;
-            m.status = h->status_dev;
-            if (h->tcb_mapN != B) {
-                if (!recur_tc_encode_planes(h->tmap_planes, h->hplanes, D, H, h->tcb_ldh, B))
-                    return fail(h, LSTM_ERR_CUDA, "tensor map of the h planes could not be encoded");
-                h->tcb_mapN = B;
-            }
-            const size_t smem = recur_tc_smem_bytes(m.RA, m.nkb, m.N, m.stages, m.kbs, h->upc, B, m.pair);
-            if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
-            e = launch_recur_tc(ly.tmap_wtc, h->tmap_planes, m, smem, st);
-            ++h->last_launches;
-            if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
-            if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             continue;
         }
         if (h->use_csr_reg) {
@@ -1679,10 +1652,7 @@ int lstm_info(const lstm_handle *h, int64_t *out, int n)
     }
     const Layer &l0 = h->layers[0];
     const int launches = h->last_launches > 0 ? h->last_launches : h->L * 2 + (h->use_tc ? 1 : 0);
-    int ik = 0, is = 0;
-    const int tcb_at_max = (h->use_tcb && !h->Hh && h->max_B > 4 && h->max_B <= kTcMaxBatch &&
-                            recur_tc_plan(h->tcb_RA, h->tcb_nkb, round_up(2 * h->max_B, 16), h->upc, h->max_B, (size_t)h->smem_optin - kTcStaticSmem,
-                                          h->tcb_pair ? 1 : 0, &ik, &is)) ? (h->tcb_pair ? 2 : 1) : 0;
+    const int tcb_at_max = h->use_tcb && h->max_B > 4 ? (h->tcb.pair ? 2 : 1) : 0;
     if (h->use_csr_reg) shp.smem = recur_csr_reg_smem_bytes(h->csr_nw, h->csr_kspan, h->csr_mt, h->upc, h->max_B);
     const int64_t vals[19] = {h->sm_count, h->ncta_dir, h->use_mma ? h->mma_nw * 32 : h->use_csr_reg ? h->csr_nw * 32 : h->threads, (int64_t)shp.smem,
                               rows_res, rows_str, (l0.plan_M >= 0) ? l0.plan.nsplit : 1, h->use_tc ? 1 : 0, launches,

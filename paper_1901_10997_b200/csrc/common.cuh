@@ -186,49 +186,45 @@ cudaError_t recur_csr_reg_prepare(int slots, int nw, int max_smem);
 cudaError_t launch_recur_csr_reg(const RecurCsrArgs &a, int slots, int nw, size_t smem, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------
-// Batched recurrent kernel on tcgen05 (bf16 weights, dense, more than four batch rows).  The CTA's slice of
-// Wh sits in shared memory as K-major 128-byte-swizzled tiles of RA rows (4 * units per CTA rounded up to 8)
-// per 64 columns; h travels through global memory as bf16 planes [D][2 parities][64 rows][ldh] (row 2b = hi,
-// 2b+1 = lo part of batch row b) and one stamp per producer CTA.
+// Batched recurrent kernel on tcgen05 (bf16 weights, several batch rows).  A CTA owns upc units; clusters of two split
+// the K range (KH columns each).  The weights go to tensor memory, h travels as phase-bit words in 16-byte chunks.
 // ---------------------------------------------------------------------------------------------------
-constexpr int kTcMaxBatch = 64;       // sequences per call the batched tensor-core recurrence serves
-constexpr int kTcStaticSmem = 1024;   // bytes kept free for the kernel's static shared memory (barriers, flags: under 600)
-constexpr int kTcPlaneRows = 128;     // rows of one parity of the h planes: hi and lo row of every sequence
+constexpr int kTcMaxRows = 64;        // batch rows of one pass; larger calls run several passes
+constexpr int kTcStaticSmem = 1024;   // bytes kept free for the kernel's static shared memory (barriers, flags: under 100)
+// Accumulators (one issuing warp each) and the tensor-memory columns set aside for them with rg groups of eight batch
+// rows: an issuing warp needs about 370 cycles for a group of twelve instructions up to N = 32, 470 at N = 48, most of
+// it between the instructions, so two of them share the work; from N = 80 on the tensor cores are the limit.
+__host__ __device__ constexpr int tc_accumulators(int rg) { return rg <= 4 ? 2 : 1; }
+__host__ __device__ constexpr int tc_acc_columns(int rg) { return rg <= 4 ? 32 * rg : 128; }
+struct RecurTcPlan { int upc, ncta, KH, pair, rows; };   // units per CTA, CTAs per direction, K columns per CTA, clusters of two, rows per pass
 struct RecurTcArgs {
     int dir0, ndirs;            // directions this launch runs: dir0 .. dir0 + ndirs - 1 (ndirs = 0 means all D)
-    int H, B, T, D;
-    int ncta_dir;
+    int H, B, T, D;             // B: batch rows of this pass ...
+    int Bs, b0;                 // ... of the call's Bs, starting at row b0
+    int ncta_dir, upc, KH, pair;
     int nsplit;
-    int RA, nkb;                // rows of a weight tile; 64-column K blocks
-    int N;                      // MMA N: 2 * B rounded up to 16
-    int stages;                 // depth of the operand ring
-    int kbs;                    // K blocks per ring stage
-    int pair;                   // 1: clusters of two CTAs split K (launched with cluster dimension 2)
-    int nissue;                 // threads issuing tensor instructions, each with its own accumulator: 1 to 3, <= K blocks of any CTA
-    int tmem_cols;              // power of two >= max(32, nissue * N)
-    int ldh;                    // row stride of the planes (elements, multiple of 8)
-    unsigned stamp_base;
     long long spin_limit;
     int withhold_cta;
+    const uint4 *wpack[2];      // per direction [cta][KH / 8 pieces][rows] 8 bf16: row 4 * unit + gate of the CTA's (pair's) units,
+                                //   the CTA's K range
     const float *G;
     long long g_split_stride;
     const float *h0, *c0;
     float *hT, *cT;
-    float *y;
+    float *y;                   // or nullptr when only the bf16 planes are wanted
     __nv_bfloat16 *xb_next;
     long long xb_plane;
     int xb_ld;
-    __nv_bfloat16 *hbuf;
-    unsigned *flags;            // [D][ncta_dir]
+    unsigned *xch;              // exchange words [2 sets][D][2 slots][16 columns][8 rows of xch_rows] blocks of 128
+    int set;                    // the set this launch uses; it clears the other one for the next launch
+    int xch_rows, clear_rows;   // rows allocated; rows the previous launch may have written
     int *status;
 };
-size_t recur_tc_smem_bytes(int RA, int nkb, int N, int stages, int kbs, int upc, int B, int pair);
-bool recur_tc_plan(int RA, int nkb, int N, int upc, int B, size_t max_smem, int pair, int *kbs_out, int *stages_out);
-bool recur_tc_pair_supported(int grid, size_t smem);
-bool recur_tc_encode_weights(void *map128, const void *w, long long rows, int ld, int RA);
-bool recur_tc_encode_planes(void *map128, const void *hbuf, int D, int H, int ldh, int B);
+size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair);
+bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, size_t max_smem, RecurTcPlan *p);
+bool recur_tc_pair_supported(int grid, int rows, size_t smem);
 cudaError_t recur_tc_prepare(int max_smem);
-cudaError_t launch_recur_tc(const void *tmap_w, const void *tmap_h, const RecurTcArgs &a, size_t smem, cudaStream_t st);
+cudaError_t launch_recur_tc(const RecurTcArgs &a, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------
 // H-LSTM recurrent kernel (one ReLU hidden layer of width Hh inside each gate; bf16 weights, dense).

@@ -68,6 +68,39 @@ __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v)
 {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
+// ---------------------------------------------------------------------------------------------------
+// Exchange words: one hidden value in 32 bits, {bf16 hi : 16 | bf16 lo : 16} with hi = bf16(h), lo = bf16(h - hi), the
+// two terms the tensor cores multiply.  |h| = |o tanh(c)| <= 1, so bit 30 (the top exponent bit of hi) is always 0 in a
+// value and carries a PHASE instead: step s writes slot s & 1 with phase bit 1 ^ (s >> 1 & 1), so a slot's phase flips
+// every time it is rewritten and a consumer that polls the word itself can tell new from old.  A slot is reused two
+// steps later, when its writer has seen every other CTA's words of the step between, i.e. when all have read it.  A NaN
+// keeps its lo term (a NaN), so it still reaches every product.
+// ---------------------------------------------------------------------------------------------------
+constexpr unsigned kPhaseBit = 0x40000000u;
+__device__ __forceinline__ unsigned word_phase(int s) { return ((s >> 1) & 1) ? 0u : kPhaseBit; }
+__device__ __forceinline__ unsigned split_word(float h)
+{
+    const __nv_bfloat16 hi = __float2bfloat16_rn(h), lo = __float2bfloat16_rn(h - __bfloat162float(hi));
+    return ((unsigned)__bfloat16_as_ushort(hi) << 16) | (unsigned)__bfloat16_as_ushort(lo);
+}
+__device__ __forceinline__ unsigned pack_word(float h, unsigned phase) { return (split_word(h) & ~kPhaseBit) | phase; }
+__device__ __forceinline__ bool words_ready(const uint4 &w, unsigned phase)
+{
+    return (((w.x ^ phase) | (w.y ^ phase) | (w.z ^ phase) | (w.w ^ phase)) & kPhaseBit) == 0;
+}
+__device__ __forceinline__ uint4 ld_relaxed_v4(const unsigned *p)
+{
+    uint4 v;
+    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 ld_nc_u4(const uint4 *p)
+{
+    uint4 v;
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 __device__ __forceinline__ int ld_volatile_s32(const int *p)
 {
     int v;

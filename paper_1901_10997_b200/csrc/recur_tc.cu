@@ -2,59 +2,68 @@
 // forward pass (paper, Section 4, cell equations with zero hidden layers per gate)
 //     z = G[t] + Wh h_{t-1};  i,f,o = sigmoid(z_i,z_f,z_o), g = tanh(z_g);  c_t = f c_{t-1} + i g;
 //     h_t = o tanh(c_t)
-// for batches of five to kTcMaxBatch sequences, where the per-step product Wh_slice [4u x H] . h_{t-1} [H x B]
-// is a real (if skinny) matrix product and one tcgen05.mma chain per step replaces the ceil(B/4) passes of
-// the register-resident kernel.
+// for several sequences at once, up to kTcMaxRows per pass, where the per-step product
+// Wh_slice [4u x H] . h_{t-1} [H x B] is a real (if skinny) matrix product.
 //
-// One cooperative launch runs all T steps of one layer (both directions on disjoint CTA groups).  A CTA
-// owns a contiguous range of hidden units; its slice of Wh (rows 4*unit + gate) is loaded ONCE by TMA into
-// shared memory as 128-byte-swizzled K-major tiles (one per 64 columns) and stays there.  h travels
-// between CTAs through global memory as the tensor cores want it: two bf16 planes per batch row (row 2b =
-// hi, row 2b+1 = lo, so products keep about 16 mantissa bits), K-major.  Per step:
-//   warp 0   waits until its own CTA has published the previous step, polls one stamp per producer CTA
-//            (relaxed loads, all in flight together, one fence after the last; bounded), then streams the
-//            [2B x H] operand into a ring of shared-memory stages with TMA (up to four 64-column blocks per
-//            stage, one issuing lane per block, zero fill at the tail).  Every CTA (pair) reads the whole
-//            operand from L2, 148 SMs at once: this fetch, about 20 bytes per clock and SM, is the longest
-//            single part of a step;
-//   warps 1-3 issue M = 128, N = 2B (rounded up to 16), K = 16 tcgen05.mma instructions.  One thread issues
-//            such an instruction every 70 cycles or so whatever its shape, while the tensor cores finish it
-//            in far less at these N, so the K blocks are dealt round-robin to up to three issuing threads in
-//            three warps, each with a TMEM accumulator of its own (measured for 48 instructions: 3400
-//            cycles from one thread, 2340 from two, 1410 from four).  The weight tile has only 4*units
-//            (<= 128) real rows: the rows beyond read whatever follows in shared memory and produce
-//            accumulator rows nobody reads;
-//   warps 4-7 request their projection terms, then read the accumulator rows of the CTA's units back
-//            (tcgen05.ld), add the issuers' accumulators and the hi and lo columns, and finish the (unit,
-//            batch row) pairs: gates, c/h update, outputs, and the new h as bf16 planes; then one thread
-//            fences and raises the CTA's stamp.
-// Pair mode (chosen at create time when the CTA count per direction is even, the doubled tile fits and the
-// device can co-schedule the clusters): CTAs 2p and 2p+1 are launched as a cluster of two; each keeps the
-// weight rows of BOTH CTAs' units but only half of the K blocks, so each issues half the tensor
-// instructions per step; the partial sums of the partner's units are collected in shared memory and
-// sent to the partner's with one bulk copy (cp.async.bulk shared::cta -> shared::cluster) that completes on the
-// partner's mbarrier, and every CTA finishes its own units from its own and the received partial sums.  The wait for the partner is bounded like the rest,
-// and a cluster barrier at the common exit keeps a CTA resident while its partner may still write into it.
-// Every wait (stamps, mbarriers) is bounded; on expiry the CTA records a timeout status and all roles fall
-// through to the common exit where tensor memory is released.  No TMA multicast is used.
+// One cooperative launch runs all T steps of one layer (both directions on disjoint CTA groups).  A CTA owns upc
+// consecutive hidden units (upc a multiple of four, all four gate rows of a unit).  Two CTAs form a cluster: each
+// keeps the weight rows of BOTH CTAs' units (2 x 4 x upc <= 128 rows) but only its half of the K range, so each
+// fetches and multiplies half of h, and the partial sums of the partner's units travel through distributed shared
+// memory.  What a step does, and why it is laid out like this:
+//
+//   * The weights sit in TENSOR MEMORY as the A operand (row = lane, two bf16 per column) for the whole sequence:
+//     128 rows by up to 896 columns.  Shared memory is then free for the B operand of a whole step, and an
+//     instruction reads only its small B tile from it.  The issuing thread must be elected from a converged warp and
+//     take its operands from warp-uniform values: measured for 48 instructions of N = 16 / 48, 970 / 1370 cycles; the
+//     same loop entered by "lane == 0" with per-thread operands took 8260.
+//   * h travels between the CTAs as 32-bit words with a phase bit (device_util.cuh), in 16-byte chunks of four units
+//     of one batch row; the consumers poll the words themselves, twelve warps with all their chunks in
+//     flight, split them into the bf16 hi and lo planes and store those as the swizzled B operand (rows 0 .. Bp-1 hi,
+//     Bp .. 2 Bp - 1 lo).  A step has no stamps, no release or acquire fence and no second trip for the data.
+//     LDG.128 reads a row range that all SMs share at 55 - 60 bytes per clock and SM (24 when a quarter warp's 128 bytes
+//     straddle two lines), a tensor copy at about 20.
+//   * The K range is handed to the issuing warps in groups as they arrive (a named barrier each: an issuing thread's
+//     mbarrier wait queues behind its own instructions), so the products overlap the fetch.
+//   * Accumulator row = 4 x unit + gate = TMEM lane: a thread reads its row's hi and lo columns for a few batch
+//     rows, sends them to the partner (st.async, completes on the partner's mbarrier) or adds what the partner sent,
+//     applies its gate's function, and a 4 x 4 transpose inside the quad gives every thread all four gates of a (unit,
+//     batch row) of its own; c stays in registers.
+//   * A step is bound by the instructions on this chain (16 warps on four schedulers), so every address is a fixed
+//     offset from a pointer that advances by one step.
+//
+// Per step (launch time / T, one layer), against the previous kernel (weights in shared memory as the A operand, h planes by
+// tensor copies behind one stamp per CTA, three "lane == 0" issuing threads): H = 1500, 20 rows 5.8 -> 4.5 us; two directions of
+// 800, 16 rows 4.7 -> 2.9 us; 50 rows in a pass 8.0 us (batches above 64 ran as passes of four rows before).
+//
+// Pair mode needs K for both halves and clusters of two; otherwise (narrow layers, or LSTM_B200_RECUR=tc1) a CTA works
+// alone on its own rows and all of K.  Every wait on another CTA is bounded; on expiry the CTA records a timeout status,
+// stops waiting for the rest of the launch and runs to the common exit, where tensor memory is released.
 #include "common.cuh"
 #include "device_util.cuh"
 
-#include <cuda.h>
 #include <cstdio>
 #include <cstring>
 
 namespace lstm {
 namespace {
 
-constexpr int kThreads = 256;                  // producer warp, three issuing warps, four finishing warps
-constexpr int kFinishTid0 = 128;                // first thread of the finishing warps
-constexpr int kMaxStages = 8;
-constexpr int kFlagLoads = 5;                   // stamps one lane polls: up to 160 CTAs per direction
-constexpr int kPre = 2;                         // (unit, batch row) items per thread whose projection terms are prefetched
-constexpr int kMaxSplit = 4;                    // split-K partial sums of the projection
+constexpr int kWarps = 16, kThreads = kWarps * 32;     // 128 registers a thread
+constexpr int kPollers = 12;                    // warps that fetch the operand (a multiple of 4 keeps their addresses linear)
+constexpr int kIssuer = 12;                     // first of the warps that issue the products; all warps finish
+constexpr int kMaxGroups = 5;                   // operand groups of 16 * kPollers columns
+constexpr int kGroupBar = 2;                    // named barrier of group 0: polling warps arrive, an issuing warp waits
 
-// ---- two-CTA cluster helpers (pair mode): the partner's shared memory and barriers
+// batch rows a worker thread finishes per accumulator row
+__host__ __device__ constexpr int tc_rows_per_thread(int rg) { return rg <= 2 ? 4 : rg <= 4 ? 8 : 16; }
+// operand groups a lane has in flight: 16-byte chunks of rg batch rows each, at most twelve (registers)
+__host__ __device__ constexpr int tc_groups_in_flight(int rg) { return 12 / rg < kMaxGroups ? 12 / rg : kMaxGroups; }
+// floats between the rows of received partial sums: a multiple of 4 off the bank period
+__host__ __device__ constexpr int tc_partial_pitch(int rg)
+{
+    return (8 * rg + tc_rows_per_thread(rg) - 1) / tc_rows_per_thread(rg) * tc_rows_per_thread(rg) + 4;
+}
+
+// ---- two-CTA cluster helpers: the partner's shared memory and barriers
 __device__ __forceinline__ uint32_t cluster_ctarank()
 {
     uint32_t r;
@@ -67,538 +76,514 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t local_smem_addr, uint32_
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_smem_addr), "r"(rank));
     return r;
 }
-// shared memory of this CTA -> shared memory of another CTA of the cluster (addresses and size multiples of 16
-// bytes); the bytes are counted on the destination CTA's barrier
-__device__ __forceinline__ void bulk_copy_to_cta(uint32_t remote_dst, uint32_t local_src, uint32_t bytes, uint32_t remote_bar)
+// 16 bytes into another CTA's shared memory; the bytes are counted on that CTA's barrier
+__device__ __forceinline__ void st_async_v4(uint32_t remote_dst, float a, float b, float c, float d, uint32_t remote_bar)
 {
-    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(remote_dst), "r"(local_src), "r"(bytes), "r"(remote_bar) : "memory");
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(remote_dst), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(__float_as_uint(c)), "r"(__float_as_uint(d)), "r"(remote_bar) : "memory");
 }
 __device__ __forceinline__ void cluster_sync_all()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-
-
-__global__ void __launch_bounds__(kThreads, 1)
-recur_tc_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_h, const RecurTcArgs a)
+__device__ __forceinline__ bool elect_one()
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long full_bar[kMaxStages], empty_bar[kMaxStages], accum_bar, w_bar, partial_bar;
-    __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s, pub_s;
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p)::"memory");
+    return p != 0;
+}
+// D[tmem] += A[tmem] . B[smem]
+__device__ __forceinline__ void umma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint4 &v)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+// N columns of this warp's lane quadrant (no wait)
+template <int N> __device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[N])
+{
+    if constexpr (N == 4)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(taddr));
+    else if constexpr (N == 8)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "r"(taddr));
+    else
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+                       "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]) : "r"(taddr));
+}
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int H = a.H, B = a.B, T = a.T, D = a.D, N = a.N, S = a.stages, RA = a.RA, nkb = a.nkb, kbs = a.kbs;
-    const int NB = (2 * B + 7) & ~7;             // rows of a fetched operand block: the copy leaves out the rows that only pad N
+// 4 x 4 transpose inside a quad: lane j of the quad enters with its row v[0..3] and leaves with column j
+__device__ __forceinline__ void quad_transpose(float &v0, float &v1, float &v2, float &v3, int j)
+{
+    const bool o1 = j & 1, o2 = j & 2;
+    const float s0 = o1 ? v0 : v1, s1 = o1 ? v2 : v3;
+    const float r0 = __shfl_xor_sync(0xffffffffu, s0, 1), r1 = __shfl_xor_sync(0xffffffffu, s1, 1);
+    if (o1) { v0 = r0; v2 = r1; } else { v1 = r0; v3 = r1; }
+    // now (v0, v1) = rows (j & ~1, j | 1) of column (j & 1), (v2, v3) the same of column 2 + (j & 1)
+    const float s2 = o2 ? v0 : v2, s3 = o2 ? v1 : v3;
+    const float r2 = __shfl_xor_sync(0xffffffffu, s2, 2), r3 = __shfl_xor_sync(0xffffffffu, s3, 2);
+    if (o2) { v0 = r2; v1 = r3; } else { v2 = r2; v3 = r3; }
+}
+
+// RG: groups of eight batch rows of a pass
+template <int RG>
+__global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs a)
+{
+    constexpr int Bp = 8 * RG, N = 2 * Bp, RS = tc_rows_per_thread(RG), NSUB = (Bp + RS - 1) / RS, PZ = tc_partial_pitch(RG);
+    constexpr int KI = tc_groups_in_flight(RG), NACC = tc_accumulators(RG);
+    constexpr uint32_t tmem = 0;                                            // all 512 columns are ours: they start at address 0
+    constexpr uint32_t acc_col = 512u - tc_acc_columns(RG);                 // accumulators behind the weights
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ __align__(8) unsigned long long accum_bar, partial_bar[2];
+    __shared__ uint32_t tmem_base_s;
+    __shared__ int abort_s;
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int H = a.H, B = a.B, T = a.T, D = a.D, upc = a.upc;
     const int d = a.dir0 + blockIdx.x / a.ncta_dir;
     const int cta = blockIdx.x % a.ncta_dir;
-    int u0, nu;
-    unit_range(H, a.ncta_dir, cta, u0, nu);
-    const int upc = (H + a.ncta_dir - 1) / a.ncta_dir;
-    // Pair mode: CTAs 2p and 2p+1 form a cluster; each keeps the rows of BOTH CTAs' units (RT = 2 RA rows) but
-    // only half of the K blocks, multiplies its half, and hands the partner the partial sums of the partner's
-    // units through distributed shared memory: half the tensor instructions per step and CTA.
     const int pair = a.pair;
     const int rank = pair ? (int)cluster_ctarank() : 0;
-    const int RT = pair ? 2 * RA : RA;                                      // rows of a weight tile
-    const int nkb_half = (nkb + 1) / 2;
-    const int kb_lo = (pair && rank) ? nkb_half : 0;                        // first K block of this CTA
-    const int nkb_my = pair ? (rank ? nkb - nkb_half : nkb_half) : nkb;     // K blocks of this CTA
-    const int nkb_alloc = pair ? nkb_half : nkb;                            // same layout in both CTAs of a pair
-    const int groups = (nkb_my + kbs - 1) / kbs;                            // ring stages one step's operand takes
-    const bool whole = groups <= S && nkb_my <= 32;                         // the ring holds it all: every step starts at stage 0
+    const int RA = 4 * upc, RT = pair ? 2 * RA : RA;                        // accumulator rows of one CTA's units; of the tile
+    const int k_lo = rank * a.KH, k_n = min(a.KH, H - k_lo);                // this CTA's K range
+    const int nk16 = (k_n + 15) >> 4;
+    const int ngroups = (nk16 + kPollers - 1) / kPollers;                   // warp w fetches piece w of every group
+    const int nissue = min(NACC, ngroups);                                  // issuing warps, each with an accumulator
 
-    // shared-memory carve-up (tiles need 1024-byte alignment): weight tiles, operand ring, then scratch
+    // shared memory: operand tiles of 64 columns [N rows][128 bytes, swizzled], then the partner's partial sums [2][RA][PZ]
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t a_tiles = base;                                          // [nkb_alloc][RT rows][128 B]
-    const uint32_t ring = a_tiles + (uint32_t)nkb_alloc * RT * 128;         // [S][kbs][N rows][128 B]
-    unsigned char *gen = smem_raw + (ring + (uint32_t)(S * kbs * N) * 128 - smem_u32(smem_raw));
-    float *zs = reinterpret_cast<float *>(gen);                             // [B][4*upc] gate pre-activations (h part)
-    const int zld = 4 * upc;
-    float *c_s = zs + zld * B;                                              // [B][units of this CTA]
-    float *zs2 = c_s + ((upc * B + 3) & ~3);                                // [B][4*upc] partial sums received from the partner (pair mode)
-    float *zsp = zs2 + (pair ? zld * B : 0);                                // [B][4*upc] partial sums of the partner's units, before they are sent
-    // checked build: the carve-up ends inside the launch's shared memory, and so does the 128-row read of the last weight tile
-    LSTM_CHECK_SMEM_END((size_t)(reinterpret_cast<unsigned char *>(zsp + (pair ? zld * B : 0)) - smem_raw), a.status);
-    LSTM_CHECK_SMEM_END((size_t)(a_tiles - smem_u32(smem_raw)) + (size_t)(nkb_alloc - 1) * RT * 128 + (size_t)128 * 128, a.status);
+    unsigned char *op = smem_raw + (base - smem_u32(smem_raw));
+    const int tiles = (a.KH + 63) >> 6;
+    float *zs2 = reinterpret_cast<float *>(op + (size_t)tiles * N * 128);
+    LSTM_CHECK_SMEM_END(reinterpret_cast<unsigned char *>(zs2 + (pair ? 2 * RA * PZ : 0)) - smem_raw, a.status);
 
     if (tid == 0) {
         abort_s = 0;
-        pub_s = 0;
-        for (int s = 0; s < S; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), (uint32_t)a.nissue); }
-        mbar_init(smem_u32(&accum_bar), (uint32_t)a.nissue);
-        mbar_init(smem_u32(&w_bar), 1);
-        mbar_init(smem_u32(&partial_bar), 1);
+        mbar_init(smem_u32(&accum_bar), (uint32_t)nissue);
+        mbar_init(smem_u32(&partial_bar[0]), 1);
+        mbar_init(smem_u32(&partial_bar[1]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(&tmem_base_s)), "r"((uint32_t)a.tmem_cols) : "memory");
+    if (warp == kIssuer) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&tmem_base_s)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    for (int i = tid; i < nu * B; i += kThreads) {
-        const int b = i / nu, u = i - b * nu;
-        c_s[i] = a.c0 ? a.c0[((size_t)d * B + b) * H + u0 + u] : 0.0f;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (pair) cluster_sync_all();               // the partner's barriers are initialised before anything reaches them
-    const uint32_t tmem_base = tmem_base_s;
-    volatile int *abort_flag = &abort_s;
-    volatile int *pub = &pub_s;                 // steps this CTA has published (h0 counts as one)
+    if (tid == 0 && tmem_base_s != 0) atomicExch(a.status, kStatusInternal);
+    volatile int *abort_v = &abort_s;
 
-    __nv_bfloat16 *hbuf_d = a.hbuf + (size_t)d * 2 * kTcPlaneRows * a.ldh;  // [parity][kTcPlaneRows rows][ldh]
-    unsigned *flags_d = a.flags + (size_t)d * a.ncta_dir;
-
-    if (warp == 0) {
-        // ================= stamps and TMA =================
-        // the CTA's weight tiles, once (one lane per tile)
-        if (lane == 0) mbar_expect_tx(smem_u32(&w_bar), (uint32_t)nkb_my * RT * 128);
-        __syncwarp();
-        for (int kb = lane; kb < nkb_my; kb += 32)
-            tma_load_2d(a_tiles + (uint32_t)kb * RT * 128, &tmap_w, smem_u32(&w_bar), (kb_lo + kb) * 64,
-                        (d * a.ncta_dir + (pair ? (cta & ~1) : cta)) * RA);
-        // ring position as a stage index and a phase bit (a 64-bit divide per stage would cost the issuing
-        // thread more than the copies it issues)
-        int st = 0;
-        uint32_t ph = 0;
-        bool live = true;
-        for (int s = 0; s < T && live; ++s) {
-            // Do not poll before this CTA has published its own part of the previous step: loads that spin
-            // ahead of the data queue up in front of the SM's own stores and delay every consumer.
-            if (lane == 0) {
-                long long t_start = 0;
-                for (int it = 0; *pub < s + 1; ++it) {
-                    if ((it & 63) == 63) {
-                        const long long now = clock64();
-                        if (t_start == 0) t_start = now;
-                        if (now - t_start > a.spin_limit || *abort_flag) { *abort_flag = 1; break; }
-                    }
-                }
-            }
-            __syncwarp();
-            // every producer's stamp of the previous step (the prologue publishes h0 with stamp_base): relaxed
-            // loads, all in flight together, and one fence once they all show the stamp (acquire loads in the
-            // polling loop were measured far slower)
-            const unsigned want = a.stamp_base + (unsigned)s;
-            long long t_start = 0;
-            int rounds = 0;
-            bool aborted = false;
-            bool seen[kFlagLoads];
-#pragma unroll
-            for (int k = 0; k < kFlagLoads; ++k) seen[k] = lane + 32 * k >= a.ncta_dir;
-            while (true) {
-                // only the stamps not yet seen are asked for again: most producers are early, and the lines
-                // that hold the stamps are the busiest in the L2 (every CTA reads and writes them)
-                unsigned v[kFlagLoads];
-#pragma unroll
-                for (int k = 0; k < kFlagLoads; ++k)
-                    if (!seen[k]) v[k] = ld_relaxed_u32(flags_d + lane + 32 * k);
-                bool ok = true;
-#pragma unroll
-                for (int k = 0; k < kFlagLoads; ++k) {
-                    if (!seen[k]) seen[k] = (int)(v[k] - want) >= 0;
-                    ok &= seen[k];
-                }
-                // both votes are taken by all lanes every round, so the warp leaves the loop as one
-                if (__any_sync(0xffffffffu, *abort_flag != 0)) { aborted = true; break; }
-                if (__all_sync(0xffffffffu, ok)) break;
-                if ((++rounds & 15) == 0) {
-                    const long long now = clock64();
-                    if (t_start == 0) t_start = now;
-                    if (now - t_start > a.spin_limit || ld_volatile_s32(a.status) != kStatusOk) *abort_flag = 1;
-                }
-            }
-            if (aborted) break;
-            fence_acq_rel_gpu();                                    // acquire: the planes behind the stamps
-            asm volatile("fence.proxy.async.global;" ::: "memory");    // they were written with ordinary stores
-            const int row0 = (d * 2 + ((s + 1) & 1)) * kTcPlaneRows;   // planes of step s-1 live in parity (s-1)&1
-            if (whole) {
-                // the ring holds the whole operand (every step starts at stage 0 with the same phase): lane i < groups
-                // opens stage i, then one lane per K block issues its copy, all in the same instruction
-                int ok = 1;
-                if (lane < groups) {
-                    const int nblk = min(kbs, nkb_my - lane * kbs);
-                    ok = mbar_wait(smem_u32(&empty_bar[lane]), ((uint32_t)s & 1u) ^ 1u, abort_flag) ? 1 : 0;
-                    if (ok) mbar_expect_tx(smem_u32(&full_bar[lane]), (uint32_t)(nblk * NB) * 128);
-                }
-                if (!__all_sync(0xffffffffu, ok)) break;
-                if (lane < nkb_my)
-                    tma_load_2d(ring + (uint32_t)(lane * N) * 128, &tmap_h, smem_u32(&full_bar[lane / kbs]), (kb_lo + lane) * 64, row0);
-                continue;
-            }
-            for (int g0 = 0; g0 < nkb_my; g0 += kbs) {
-                const int nblk = min(kbs, nkb_my - g0);
-                int ok = 1;
-                if (lane == 0) {
-                    ok = mbar_wait(smem_u32(&empty_bar[st]), ph ^ 1u, abort_flag) ? 1 : 0;
-                    if (ok) mbar_expect_tx(smem_u32(&full_bar[st]), (uint32_t)(nblk * NB) * 128);
-                }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok) { live = false; break; }
-                // one lane per K block of the stage: issuing a tensor copy occupies a thread for a while
-                if (lane < nblk)
-                    tma_load_2d(ring + (uint32_t)((st * kbs + lane) * N) * 128, &tmap_h, smem_u32(&full_bar[st]), (kb_lo + g0 + lane) * 64, row0);
-                if (++st == S) { st = 0; ph ^= 1u; }
-            }
-        }
-    } else if (warp <= 3) {
-        // ================= MMA issue =================
-        // issuer w = warp - 1 < nissue takes the K blocks whose index is w modulo nissue (no CTA has fewer K blocks
-        // than issuers) into the accumulator at TMEM column w * N; every issuer passes every stage and commits to
-        // its barriers, blocks or not
-        const int w = warp - 1;
-        if (lane == 0 && w < a.nissue) {
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-            bool ok = mbar_wait(smem_u32(&w_bar), 0u, abort_flag);
-            // descriptors differ only in their start-address field (units of 16 bytes): build one of each and add
-            const uint64_t adesc0 = umma_desc_sw128(a_tiles), bdesc0 = umma_desc_sw128(ring);
-            const uint32_t a_step = (uint32_t)(RT * 128) >> 4, b_step = (uint32_t)(N * 128) >> 4;
-            const uint32_t acc = tmem_base + (uint32_t)(w * N);
-            int st = 0;
-            uint32_t ph = 0;
-            for (int s = 0; s < T && ok; ++s) {
-                uint32_t accumulate = 0u;
-                int next = w;                                   // this issuer's next K block
-                if (whole) { st = 0; ph = (uint32_t)s & 1u; }
-                for (int g0 = 0; g0 < nkb_my; g0 += kbs) {
-                    const int nblk = min(kbs, nkb_my - g0);
-                    ok = mbar_wait(smem_u32(&full_bar[st]), ph, abort_flag);
-                    if (!ok) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    for (; next < g0 + nblk; next += a.nissue) {
-                        const int l = next - g0;
-                        const uint64_t adesc = adesc0 + (uint64_t)((uint32_t)(g0 + l) * a_step);
-                        const uint64_t bdesc = bdesc0 + (uint64_t)((uint32_t)(st * kbs + l) * b_step);
-                        umma_bf16(acc, adesc, bdesc, idesc, accumulate);
-                        umma_bf16(acc, adesc + 2, bdesc + 2, idesc, 1u);
-                        umma_bf16(acc, adesc + 4, bdesc + 4, idesc, 1u);
-                        umma_bf16(acc, adesc + 6, bdesc + 6, idesc, 1u);
-                        accumulate = 1u;
-                    }
-                    umma_commit(smem_u32(&empty_bar[st]));
-                    if (++st == S) { st = 0; ph ^= 1u; }
-                }
-                if (ok) umma_commit(smem_u32(&accum_bar));
-            }
-        }
-    } else {
-        // ================= accumulator read-back and the cell =================
-        const int ftid = tid - kFinishTid0;              // 0..127
-        const int lq = warp & 3;                         // TMEM lane quadrant this warp may read
-        const int nuB = nu * B;
-        int u0_partner = 0, nu_partner = 0;
-        uint32_t zs2_remote = 0, partial_bar_remote = 0;
-        if (pair) {
-            unit_range(H, a.ncta_dir, cta ^ 1, u0_partner, nu_partner);
-            zs2_remote = map_to_cta(smem_u32(zs2), (uint32_t)(rank ^ 1));
-            partial_bar_remote = map_to_cta(smem_u32(&partial_bar), (uint32_t)(rank ^ 1));
-        }
-        // the planes of h0 (stamp_base): this CTA's units
-        for (int p = ftid; p < nuB; p += 128) {
-            const int b = p / nu, u = p - b * nu;
-            const float v = a.h0 ? a.h0[((size_t)d * B + b) * H + u0 + u] : 0.0f;
-            const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-            __nv_bfloat16 *row = hbuf_d + ((size_t)1 * kTcPlaneRows + 2 * b) * a.ldh + u0 + u;     // step -1 -> parity 1
-            row[0] = hi;
-            row[a.ldh] = __float2bfloat16_rn(v - __bfloat162float(hi));
-        }
-        bar_sync(1, 128);
-        if (ftid == 0) {
-            if ((int)blockIdx.x != a.withhold_cta) {
-                fence_acq_rel_gpu();
-                st_relaxed_u32(flags_d + cta, a.stamp_base);
-            }
-            *pub = 1;
-        }
-        const size_t gs4 = (size_t)(a.g_split_stride / 4);
-        // the first kPre items of this thread: batch row and unit, fixed for the whole sequence
-        int pb[kPre], pu[kPre];
-#pragma unroll
-        for (int i = 0; i < kPre; ++i) {
-            const int p = ftid + 128 * i;
-            pb[i] = p < nuB ? p / nu : 0;
-            pu[i] = p < nuB ? p - pb[i] * nu : 0;
-        }
-        for (int s = 0; s < T; ++s) {
-            const int t = d ? (T - 1 - s) : s;
-            // projection terms of the first items: requested before the wait, they do not depend on h
-            float4 gpre[kPre][kMaxSplit];
-#pragma unroll
-            for (int i = 0; i < kPre; ++i) {
-                const int p = ftid + 128 * i;
-                if (p < nuB) {
-                    const int b = pb[i], j = u0 + pu[i];
-                    const float4 *gp = reinterpret_cast<const float4 *>(a.G + (((size_t)t * B + b) * D + d) * 4 * H + (size_t)j * 4);
-#pragma unroll
-                    for (int sp = 0; sp < kMaxSplit; ++sp)
-                        if (sp < a.nsplit) gpre[i][sp] = ld_nc_f4(gp + (size_t)sp * gs4);
-                }
-            }
-            if (!mbar_wait(smem_u32(&accum_bar), (uint32_t)s & 1u, abort_flag)) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            // accumulator row = 4 * unit + gate; in pair mode rows [0, RA) belong to the even CTA's units and
-            // rows [RA, 2 RA) to the odd CTA's: the partner's rows go to the partner's shared memory
-            const int row = lq * 32 + lane;
-            const int half = (pair && row >= RA) ? 1 : 0;
-            const int lr = row - half * RA;
-            const bool mine = !pair || half == rank;
-            const bool row_ok = row < RT && lr < 4 * (mine ? nu : nu_partner);
-            if (lq * 32 < (pair ? RT : 4 * nu)) {
-                // the first four column chunks of 16 (all there are up to 32 sequences) are requested before
-                // one wait; batches above 32 read their remaining chunks one at a time (registers)
-                const int nchunk = (2 * B + 15) >> 4;
-                {
-                    float z[4][8];
-                    // one issuer's accumulator after the other; hi and lo columns are added on the way
-                    for (int wi = 0; wi < a.nissue; ++wi) {
-                        uint32_t x[4][16];
-#pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            if (c < nchunk) tmem_ld16(tmem_base + ((uint32_t)(lq * 32) << 16) + (uint32_t)(wi * N + c * 16), x[c]);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            if (c < nchunk) {
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) {
-                                    const float zz = __uint_as_float(x[c][2 * i]) + __uint_as_float(x[c][2 * i + 1]);
-                                    z[c][i] = wi ? z[c][i] + zz : zz;
-                                }
-                            }
-                    }
-                    if (row_ok) {
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            if (c < nchunk) {
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) {
-                                    const int b = c * 8 + i;
-                                    if (b < B) {
-                                        (mine ? zs : zsp)[b * zld + lr] = z[c][i];
-                                    }
-                                }
-                            }
-                        }
-                    }
-                }
-#pragma unroll 1
-                for (int c = 4; c < nchunk; ++c) {
-                    uint32_t w[16];
-                    tmem_ld16(tmem_base + ((uint32_t)(lq * 32) << 16) + (uint32_t)(c * 16), w);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    for (int wi = 1; wi < a.nissue; ++wi) {
-                        uint32_t x[16];
-                        tmem_ld16(tmem_base + ((uint32_t)(lq * 32) << 16) + (uint32_t)(wi * N + c * 16), x);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) w[i] = __float_as_uint(__uint_as_float(w[i]) + __uint_as_float(x[i]));
-                    }
-                    if (row_ok) {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int b = c * 8 + i;
-                            const float z = __uint_as_float(w[2 * i]) + __uint_as_float(w[2 * i + 1]);
-                            if (b < B) {
-                                (mine ? zs : zsp)[b * zld + lr] = z;
-                            }
-                        }
-                    }
-                }
-            }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            bar_sync(1, 128);
-            if (pair) {
-                // one bulk copy carries the partner's partial sums into its shared memory and completes on its
-                // barrier; ours arrive the same way (bounded wait)
-                if (ftid == 0) {
-                    const uint32_t bytes = (uint32_t)(zld * B) * 4u;
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    mbar_expect_tx(smem_u32(&partial_bar), bytes);
-                    bulk_copy_to_cta(zs2_remote, smem_u32(zsp), bytes, partial_bar_remote);
-                }
-                if (!mbar_wait(smem_u32(&partial_bar), (uint32_t)s & 1u, abort_flag)) break;
-            }
-            __nv_bfloat16 *hp = hbuf_d + (size_t)(s & 1) * kTcPlaneRows * a.ldh;
-            // one (unit, batch row) item: gates, c/h update, the new h as planes, outputs
-            auto finish_item = [&](int p, int b, int u, const float4 &gsum) {
-                const int j = u0 + u;
-                float4 z4 = *reinterpret_cast<const float4 *>(zs + b * zld + 4 * u);
-                if (pair) {
-                    const float4 y4 = *reinterpret_cast<const float4 *>(zs2 + b * zld + 4 * u);
-                    z4.x += y4.x; z4.y += y4.y; z4.z += y4.z; z4.w += y4.w;
-                }
-                const float gi = sigmoid_fast(z4.x + gsum.x);
-                const float gf = sigmoid_fast(z4.y + gsum.y);
-                const float gg = tanh_fast(z4.z + gsum.z);
-                const float go = sigmoid_fast(z4.w + gsum.w);
-                const float cn = fmaf(gf, c_s[p], gi * gg);
-                const float hn = go * tanh_fast(cn);
-                c_s[p] = cn;
-                const __nv_bfloat16 hi = __float2bfloat16_rn(hn);
-                const __nv_bfloat16 lo = __float2bfloat16_rn(hn - __bfloat162float(hi));
-                hp[(size_t)(2 * b) * a.ldh + j] = hi;
-                hp[(size_t)(2 * b + 1) * a.ldh + j] = lo;
-                a.y[((size_t)t * B + b) * D * H + (size_t)d * H + j] = hn;
-                if (a.xb_next) {
-                    const size_t xi = ((size_t)t * B + b) * a.xb_ld + (size_t)d * H + j;
-                    a.xb_next[xi] = hi;
-                    a.xb_next[a.xb_plane + xi] = lo;
-                }
-                if (s == T - 1) {
-                    if (a.hT) a.hT[((size_t)d * B + b) * H + j] = hn;
-                    if (a.cT) a.cT[((size_t)d * B + b) * H + j] = cn;
-                }
-            };
-            // consecutive threads, consecutive units; the first kPre items have their projection terms in registers
-#pragma unroll
-            for (int i = 0; i < kPre; ++i) {
-                const int p = ftid + 128 * i;
-                if (p < nuB) {
-                    float4 gsum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll
-                    for (int sp = 0; sp < kMaxSplit; ++sp)
-                        if (sp < a.nsplit) { gsum.x += gpre[i][sp].x; gsum.y += gpre[i][sp].y; gsum.z += gpre[i][sp].z; gsum.w += gpre[i][sp].w; }
-                    finish_item(p, pb[i], pu[i], gsum);
-                }
-            }
-            for (int p = ftid + 128 * kPre; p < nuB; p += 128) {
-                const int b = p / nu, u = p - b * nu;
-                const float4 *gp = reinterpret_cast<const float4 *>(a.G + (((size_t)t * B + b) * D + d) * 4 * H + (size_t)(u0 + u) * 4);
-                float4 gsum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                for (int sp = 0; sp < a.nsplit; ++sp) {
-                    const float4 g4 = __ldg(gp + (size_t)sp * gs4);
-                    gsum.x += g4.x; gsum.y += g4.y; gsum.z += g4.z; gsum.w += g4.w;
-                }
-                finish_item(p, b, u, gsum);
-            }
-            bar_sync(1, 128);
-            if (ftid == 0) {
-                if ((int)blockIdx.x != a.withhold_cta) {
-                    st_release_u32(flags_d + cta, a.stamp_base + (unsigned)s + 1u);
-                }
-                *pub = s + 2;
-            }
+    // Exchange words: this launch's set starts with every phase bit at 0, the first words carry 1; the other set, which
+    // the next launch will use, is cleared here, every CTA its own words.
+    // Block (16 columns, 8 batch rows) = 512 contiguous bytes, [column / 4][row][4 words]: a warp's load of a block is four
+    // full lines, each by eight consecutive lanes.
+    const int Hq = (H + 3) & ~3, nq = Hq >> 2, rgx = a.xch_rows >> 3;       // chunks of four units; row groups allocated
+    const unsigned slot_words = (unsigned)((H + 15) >> 4) * rgx * 128u;
+    const size_t set_words = (size_t)2 * D * slot_words;
+    auto chunk_word = [&](int q, int b) -> unsigned { return (((unsigned)(q >> 2) * rgx + (b >> 3)) * 32u + (q & 3) * 8u + (b & 7)) * 4u; };
+    unsigned *xch_d = a.xch + (size_t)a.set * set_words + (size_t)d * 2 * slot_words;
+    {
+        unsigned *other = a.xch + (size_t)(a.set ^ 1) * set_words + (size_t)d * 2 * slot_words;
+        const int cq = cta * (upc >> 2), qn = max(0, min(upc >> 2, nq - cq));
+        for (int i = tid; i < 2 * qn * a.clear_rows; i += kThreads) {
+            const int sl = i / (qn * a.clear_rows), r = i - sl * qn * a.clear_rows, q = r / a.clear_rows, b = r - q * a.clear_rows;
+            *reinterpret_cast<uint4 *>(other + (size_t)sl * slot_words + chunk_word(cq + q, b)) = make_uint4(0, 0, 0, 0);
         }
     }
+    // weights into tensor memory: warp w writes lane quadrant w % 4, every fourth 8-column piece
+    {
+        const int row = (warp & 3) * 32 + lane, pieces = a.KH >> 3;
+        const uint4 *src = a.wpack[d] + (size_t)cta * pieces * RT + row;
+        const uint32_t dst = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        for (int p0 = warp >> 2; p0 < pieces; p0 += 32) {
+            uint4 v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = p0 + 4 * i < pieces && row < RT ? ld_nc_u4(src + (size_t)(p0 + 4 * i) * RT) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (p0 + 4 * i < pieces) tmem_st4(dst + (uint32_t)(p0 + 4 * i) * 4u, v[i]);
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    }
+    for (int i = tid; i < tiles * N * 8; i += kThreads) reinterpret_cast<uint4 *>(op)[i] = make_uint4(0, 0, 0, 0);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 1) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)a.tmem_cols) : "memory");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (pair) cluster_sync_all();               // the partner's barriers are initialised before anything reaches them
+
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+    const uint64_t bdesc0 = umma_desc_sw128(base);
+    // Polling: of a block a lane takes chunk qq (four columns) of batch row rr; half a warp stores eight rows by 16 bytes,
+    // which the swizzle spreads over all banks.
+    const int qq = lane >> 3, rr = lane & 7;
+    const int q0 = (k_lo >> 2) + warp * 4 + qq;
+    const unsigned *src0 = xch_d + ((size_t)((k_lo >> 4) + warp) * rgx * 32 + lane) * 4;
+    const unsigned src_group = 128u * kPollers * (unsigned)rgx;             // words from group to group
+    unsigned char *dst0 = op + (warp >> 2) * (N * 128) + rr * 128 + ((((warp & 3) * 32) + qq * 8) ^ (rr << 4));
+    constexpr int kDstGroup = kPollers / 4 * N * 128;
+    int n_lane = 0;                                                         // groups this lane has a chunk in
+    for (int i = 0; i < ngroups; ++i)
+        if (warp < kPollers && i * kPollers + warp < nk16 && q0 + i * 4 * kPollers < nq) n_lane = i + 1;
+    const unsigned rg_mask = (1u << max(0, min(RG, (B - rr + 7) >> 3))) - 1u;
+    // finishing: TMEM lane quadrant, accumulator row, batch rows [sub * RS, + RS)
+    const int row = (warp & 3) * 32 + lane, sub = warp >> 2, fq = lane & 3;
+    const int side = pair && row >= RA ? 1 : 0, lr = row - side * RA;
+    const bool fin = sub < NSUB && (warp & 3) * 32 < RT;                    // this warp reads accumulators
+    const bool mine = row < RT && side == rank;
+    const int u = lr >> 2, j = cta * upc + u;                               // unit of this row, if it is ours
+    const bool own = mine && fin && j < Hq, real = own && j < H;
+    const int fb0 = sub * RS;
+    const float act_k = (fq == 2 ? -2.0f : -1.0f) * 1.4426950408889634f, act_sc = fq == 2 ? 2.0f : 1.0f, act_of = fq == 2 ? -1.0f : 0.0f;
+    const uint32_t zs2_remote = pair ? map_to_cta(smem_u32(zs2), (uint32_t)(rank ^ 1)) + (uint32_t)(lr * PZ + fb0) * 4u : 0u;
+    const uint32_t partial_remote = pair ? map_to_cta(smem_u32(partial_bar), (uint32_t)(rank ^ 1)) : 0u;
+    const uint32_t abort_remote = pair ? map_to_cta(smem_u32(&abort_s), (uint32_t)(rank ^ 1)) : 0u;
+    const float *zs2_mine = zs2 + lr * PZ + fb0;
+    const size_t state0 = ((size_t)d * a.Bs + a.b0) * H + j;                // element of (pass row 0, unit j) in the state arrays
+    // projection terms, outputs: pointers that advance by one timestep per step
+    const long long gstep = (long long)D * 4 * H, dir = d ? -1 : 1;
+    const long long m0 = (long long)(d ? T - 1 : 0) * a.Bs + a.b0 + fb0;    // row of G of this thread's first batch row
+    const float *gp = a.G + m0 * gstep + (long long)d * 4 * H + 4 * (long long)j + fq;
+    const int nrow = real ? max(0, min(RS, B - fb0)) : 0;
+    const float *gpre = a.G + (m0 + 2 * dir * a.Bs + lane) * gstep + (long long)d * 4 * H + 4 * (long long)(j - (lane >> 2));
+    const bool pre = lane < RS && fb0 + lane < B && fin && mine && j - (lane >> 2) < H;
+    float *yp = a.y ? a.y + (m0 + fq) * D * H + (long long)d * H + j : nullptr;
+    __nv_bfloat16 *xp = a.xb_next ? a.xb_next + (m0 + fq) * a.xb_ld + (long long)d * H + j : nullptr;
+    const long long gadv = dir * a.Bs * gstep, yadv = dir * a.Bs * D * H, xadv = dir * a.Bs * a.xb_ld;
+    const int ystep = 4 * D * H, xstep = 4 * a.xb_ld;
+    unsigned *const out0 = xch_d + chunk_word(j >> 2, fb0 + fq) + (j & 3);
+    const int nitem = own ? max(0, min(RS / 4, (B - fb0 - fq + 3) >> 2)) : 0;       // (unit, batch row) items of this thread
+    const int npub = (int)blockIdx.x != a.withhold_cta ? nitem : 0, nout = real ? nitem : 0;
+
+    // c of (unit, batch row fb0 + 4 m + fq)
+    float c[RS / 4], hn[RS / 4];
+#pragma unroll
+    for (int m = 0; m < RS / 4; ++m) {
+        c[m] = a.c0 && m < nout ? a.c0[state0 + (size_t)(fb0 + 4 * m + fq) * H] : 0.0f;
+        hn[m] = 0.0f;
     }
-    if (tid == 0 && abort_s) atomicExch(a.status, kStatusTimeout);
+
+#pragma unroll 1
+    for (int s = 0; s < T; ++s) {
+        // ---- projection terms of this thread's row; the lines of a later step are requested into L2
+        float g[RS];
+#pragma unroll
+        for (int i = 0; i < RS; ++i) g[i] = i < nrow ? ld_nc_early(gp + i * gstep) : 0.0f;
+        if (a.nsplit > 1)
+            for (int sp = 1; sp < a.nsplit; ++sp)
+#pragma unroll
+                for (int i = 0; i < RS; ++i)
+                    if (i < nrow) g[i] += ld_nc_early(gp + sp * a.g_split_stride + i * gstep);
+        if (pre && s + 2 < T) asm volatile("prefetch.global.L2 [%0];" ::"l"(gpre));
+        gp += gadv;
+        gpre += gadv;
+        // (an aborted CTA opens no further phase: the open one never completes, and a second arrival would exceed its count)
+        if (pair && tid == 0 && !*abort_v) mbar_expect_tx(smem_u32(&partial_bar[s & 1]), (uint32_t)(RA * NSUB * RS * 4));
+
+        if (warp >= kIssuer && warp < kIssuer + nissue) {
+            // ---- products: issuing warp w takes every nissue-th group, one elected thread, an accumulator of its own
+            const int w = warp - kIssuer;
+            for (int gi = w; gi < ngroups; gi += nissue) {
+                bar_sync(kGroupBar + gi, (kPollers + 1) * 32);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const int n = min(kPollers, nk16 - gi * kPollers);
+                if (elect_one()) {
+                    const uint64_t bd = bdesc0 + (uint64_t)(gi * (kDstGroup / 16));
+                    const uint32_t ad = tmem + (uint32_t)(gi * kPollers * 8), acc = acc_col + (uint32_t)(w * N);
+                    if (n == kPollers) {
+#pragma unroll
+                        for (int t4 = 0; t4 < kPollers / 4; ++t4)
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk)
+                                umma_bf16_ta(acc, ad + (t4 * 4 + kk) * 8, bd + (uint64_t)(t4 * (N * 128 / 16) + kk * 2), idesc, gi >= nissue || t4 + kk ? 1u : 0u);
+                    } else {
+#pragma unroll 1
+                        for (int k = 0; k < n; ++k)
+                            umma_bf16_ta(acc, ad + k * 8, bd + (uint64_t)((k >> 2) * (N * 128 / 16) + (k & 3) * 2), idesc, gi >= nissue || k ? 1u : 0u);
+                    }
+                    if (gi + nissue >= ngroups) umma_commit(smem_u32(&accum_bar));
+                }
+                __syncwarp();
+            }
+        } else if (warp < kPollers) {
+            // ---- operand: h_{s-1} of this CTA's K range, KI groups at a time
+            auto store_piece = [&](unsigned char *dst, const uint4 &w, unsigned keep) {
+                if (LSTM_CHECK_INDEX(dst - op + Bp * 128 + 7, tiles * N * 128, a.status)) {
+                    *reinterpret_cast<uint2 *>(dst) = make_uint2(__byte_perm(w.x, w.y, 0x7632u) & keep, __byte_perm(w.z, w.w, 0x7632u) & keep);
+                    *reinterpret_cast<uint2 *>(dst + Bp * 128) = make_uint2(__byte_perm(w.x, w.y, 0x5410u), __byte_perm(w.z, w.w, 0x5410u));
+                }
+            };
+            const unsigned phase = word_phase(s - 1);
+            const unsigned *src = src0 + (size_t)((s - 1) & 1) * slot_words;
+            if (s == 0 && a.h0) {
+                for (int i = 0; i < n_lane; ++i)
+                    for (int rg = 0; rg < RG; ++rg)
+                        if (rg_mask & (1u << rg)) {
+                            const int k = 4 * (q0 + i * 4 * kPollers);
+                            const float *hp = a.h0 + ((size_t)d * a.Bs + a.b0 + rg * 8 + rr) * H + k;
+                            uint4 v = make_uint4(split_word(hp[0]), 0, 0, 0);
+                            if (k + 1 < H) v.y = split_word(hp[1]);
+                            if (k + 2 < H) v.z = split_word(hp[2]);
+                            if (k + 3 < H) v.w = split_word(hp[3]);
+                            store_piece(dst0 + i * kDstGroup + rg * 1024, v, 0xffffffffu);
+                        }
+            }
+#pragma unroll 1
+            for (int i0 = 0; i0 < ngroups; i0 += KI, src += KI * src_group) {
+                unsigned pending = 0;                       // bit i * RG + rg: chunk not here yet
+                uint4 w[KI][RG];
+                if (s > 0 && !*abort_v) {
+#pragma unroll
+                    for (int i = 0; i < KI; ++i)
+                        if (i0 + i < n_lane) pending |= rg_mask << (i * RG);
+                }
+                auto request = [&]() {
+#pragma unroll
+                    for (int i = 0; i < KI; ++i)
+#pragma unroll
+                        for (int rg = 0; rg < RG; ++rg)
+                            if (pending & (1u << (i * RG + rg))) w[i][rg] = ld_relaxed_v4(src + i * src_group + rg * 128);
+                };
+                request();
+                unsigned char *dst = dst0 + i0 * kDstGroup;
+                const int last = min(KI, ngroups - i0);
+                int polls = 0, delivered = 0;
+                long long t_start = 0;
+                for (;;) {
+#pragma unroll
+                    for (int i = 0; i < KI; ++i)
+#pragma unroll
+                        for (int rg = 0; rg < RG; ++rg)
+                            if ((pending & (1u << (i * RG + rg))) && words_ready(w[i][rg], phase)) {
+                                store_piece(dst + i * kDstGroup + rg * 1024, w[i][rg], 0xbfffbfffu);
+                                pending &= ~(1u << (i * RG + rg));
+                            }
+                    const unsigned open = __reduce_or_sync(0xffffffffu, pending);
+                    // groups this warp has delivered
+                    int done = delivered;
+                    while (done < last && !(open & (((1u << RG) - 1u) << (done * RG)))) ++done;
+                    if (done > delivered) {
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        for (int gi = delivered; gi < done; ++gi) bar_arrive(kGroupBar + i0 + gi, (kPollers + 1) * 32);
+                        delivered = done;
+                    }
+                    if (!open) break;
+                    request();
+                    if ((++polls & 15) == 0) {
+                        const long long now = clock64();
+                        if (t_start == 0) t_start = now;
+                        if (*abort_v) pending = 0;
+                        else if (now - t_start > a.spin_limit || ld_volatile_s32(a.status) != kStatusOk) {
+                            *abort_v = 1;
+                            atomicExch(a.status, kStatusTimeout);
+                            pending = 0;
+                        }
+                    }
+                }
+            }
+        }
+
+        // ---- accumulators, partner's partial sums, gates, state
+        if (fin) {
+            mbar_wait(smem_u32(&accum_bar), (uint32_t)s & 1u, abort_v);
+            __syncwarp();
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t ta = acc_col + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)fb0;
+            float z[RS], zl[RS];
+            tmem_ld<RS>(ta, z);
+            tmem_ld<RS>(ta + (uint32_t)Bp, zl);
+            if (NACC > 1 && nissue > 1) {
+                float y[RS], yl[RS];
+                tmem_ld<RS>(ta + (uint32_t)N, y);
+                tmem_ld<RS>(ta + (uint32_t)(N + Bp), yl);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                for (int i = 0; i < RS; ++i) z[i] = (z[i] + y[i]) + (zl[i] + yl[i]);
+            } else {
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                for (int i = 0; i < RS; ++i) z[i] += zl[i];
+            }
+            if (pair) {
+                if (*abort_v) {
+                    // gave up: nothing is sent any more, so the partner must not wait for it
+                    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(abort_remote), "r"(1) : "memory");
+                } else if (row < RT && !mine) {
+                    const uint32_t dst = zs2_remote + (uint32_t)((s & 1) * RA * PZ) * 4u, bar = partial_remote + (uint32_t)(s & 1) * 8u;
+#pragma unroll
+                    for (int i = 0; i < RS; i += 4) st_async_v4(dst + i * 4, z[i], z[i + 1], z[i + 2], z[i + 3], bar);
+                }
+                __syncwarp();
+                if (__any_sync(0xffffffffu, mine)) {
+                    mbar_wait(smem_u32(&partial_bar[s & 1]), (uint32_t)(s >> 1) & 1u, abort_v);
+                    __syncwarp();
+                    if (mine) {
+                        const float *zp = zs2_mine + (s & 1) * RA * PZ;
+#pragma unroll
+                        for (int i = 0; i < RS; i += 4) {
+                            const float4 p = *reinterpret_cast<const float4 *>(zp + i);
+                            z[i] += p.x; z[i + 1] += p.y; z[i + 2] += p.z; z[i + 3] += p.w;
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < RS; ++i) z[i] = gate_fast(z[i] + g[i], act_k, act_sc, act_of);
+            unsigned *dst = out0 + (size_t)(s & 1) * slot_words;
+            const unsigned phase_out = word_phase(s);
+#pragma unroll
+            for (int m = 0; m < RS / 4; ++m) {
+                quad_transpose(z[4 * m], z[4 * m + 1], z[4 * m + 2], z[4 * m + 3], fq);
+                c[m] = fmaf(z[4 * m + 1], c[m], z[4 * m] * z[4 * m + 2]);
+                hn[m] = z[4 * m + 3] * tanh_fast(c[m]);
+                // (fb0 is a multiple of four: of eight where a thread has more than one item)
+                if (m < npub) st_relaxed_u32(dst + (m & 1) * 16 + (m >> 1) * 128, pack_word(hn[m], phase_out));
+            }
+        }
+        // Nobody polls or overwrites the operand before the whole CTA has published: early polls of words that are being
+        // written pull their lines to and fro between the two halves of the L2, and delay everyone.
+        bar_sync(1, kThreads);
+        if (yp) {
+#pragma unroll
+            for (int m = 0; m < RS / 4; ++m)
+                if (m < nout) yp[m * ystep] = hn[m];
+            yp += yadv;
+        }
+        if (xp) {
+#pragma unroll
+            for (int m = 0; m < RS / 4; ++m)
+                if (m < nout) {
+                    const __nv_bfloat16 hi = __float2bfloat16_rn(hn[m]);
+                    xp[m * xstep] = hi;
+                    xp[a.xb_plane + m * xstep] = __float2bfloat16_rn(hn[m] - __bfloat162float(hi));
+                }
+            xp += xadv;
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < RS / 4; ++m)
+        if (m < nout) {
+            if (a.hT) a.hT[state0 + (size_t)(fb0 + 4 * m + fq) * H] = hn[m];
+            if (a.cT) a.cT[state0 + (size_t)(fb0 + 4 * m + fq) * H] = c[m];
+        }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (__syncthreads_or(*abort_v)) {           // one answer for the whole CTA: the partner may raise the flag at any time
+        // a wait gave up: products and partial sums may still be in flight; they land within microseconds
+        if (tid == 0) atomicExch(a.status, kStatusTimeout);
+        const long long t0 = clock64();
+        while (clock64() - t0 < 200000) { }
+        __syncthreads();
+    }
+    if (warp == kIssuer) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base_s) : "memory");
+    }
     if (pair) cluster_sync_all();               // no CTA leaves while its partner may still write into its shared memory
 }
 
-// rows x cols bf16 matrix, row stride ld elements; box = 64 columns x box_rows, 128-byte swizzle, zero fill
-bool encode_2d(void *map, const void *base, long long rows, int cols, int ld, int box_rows)
+typedef void (*KernelFn)(const RecurTcArgs);
+KernelFn pick(int rg)
 {
-    return encode_tmap_bf16_2d(map, base, rows, cols, ld, box_rows);
+    switch (rg) {
+        case 1: return recur_tc_kernel<1>;
+        case 2: return recur_tc_kernel<2>;
+        case 3: return recur_tc_kernel<3>;
+        case 4: return recur_tc_kernel<4>;
+        case 5: return recur_tc_kernel<5>;
+        case 6: return recur_tc_kernel<6>;
+        case 7: return recur_tc_kernel<7>;
+        case 8: return recur_tc_kernel<8>;
+        default: return nullptr;
+    }
+}
+int groups_of(int rows) { return (rows + 7) / 8; }
+
+cudaLaunchConfig_t config(cudaLaunchAttribute (&attr)[2], int grid, size_t smem, int pair, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = pair ? 2 : 1;
+    return cfg;
 }
 
 }  // namespace
 
-static_assert(sizeof(CUtensorMap) == 128, "tensor map size");
-
-size_t recur_tc_smem_bytes(int RA, int nkb, int N, int stages, int kbs, int upc, int B, int pair)
+size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair)
 {
-    // pair mode: tiles of 2 RA rows, half of the K blocks (rounded up), and a second block of partial sums
-    const int RT = pair ? 2 * RA : RA, nkb_alloc = pair ? (nkb + 1) / 2 : nkb;
-    // the last weight tile is read as 128 rows: at least (128 - RT) * 128 bytes must follow it
-    const size_t scratch = (size_t)(4 * upc * B) * (pair ? 3 : 1) + (size_t)((upc * B + 3) & ~3);
-    const size_t after = (size_t)stages * kbs * N * 128 + scratch * 4 + 16;
-    const size_t need = (size_t)(128 - RT) * 128;
-    return 1024 + (size_t)nkb_alloc * RT * 128 + (after > need ? after : need);
+    const int rg = groups_of(rows);
+    return 1024 + (size_t)((KH + 63) / 64) * (16 * rg) * 128 + (pair ? (size_t)2 * 4 * upc * tc_partial_pitch(rg) * 4 : 0);
 }
 
-// Ring shape for one launch: stages of up to four K blocks (one mbarrier round trip per stage instead of per
-// block); a ring that holds the whole operand if one fits, else as many stages as fit, at least two.
-bool recur_tc_plan(int RA, int nkb, int N, int upc, int B, size_t max_smem, int pair, int *kbs_out, int *stages_out)
+// Partition of H units over at most max_cta CTAs, and the most batch rows (<= rows_wanted) a pass can take; false when
+// the slice does not fit tensor memory.
+bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, size_t max_smem, RecurTcPlan *p)
 {
-    const int nkb_cta = pair ? (nkb + 1) / 2 : nkb;
-    if (pair && (2 * RA > 128 || nkb < 2)) return false;
-    // first choice: a ring that holds a whole step's operand (all copies of a step are then issued together),
-    // in as few stages as possible
-    for (int kbs = nkb_cta < 4 ? nkb_cta : 4; kbs >= 1 && nkb_cta <= 32; --kbs) {
-        const int st = (nkb_cta + kbs - 1) / kbs;
-        if (st <= kMaxStages && recur_tc_smem_bytes(RA, nkb, N, st, kbs, upc, B, pair) <= max_smem) {
-            *kbs_out = kbs;
-            *stages_out = st;
-            return true;
-        }
+    if (pair && H <= 64) return false;                                  // both halves of K must exist
+    int upc = 4, n = 0;
+    for (; upc <= 16; upc += 4) {
+        n = (H + upc - 1) / upc;
+        if (pair) n = (n + 1) / 2 * 2;
+        if (n <= max_cta) break;
     }
-    for (int kbs = nkb_cta < 4 ? nkb_cta : 4; kbs >= 1; --kbs) {
-        const int groups = (nkb_cta + kbs - 1) / kbs;
-        for (int st = groups < kMaxStages ? groups : kMaxStages; st >= (groups > 1 ? 2 : 1); --st) {
-            if (recur_tc_smem_bytes(RA, nkb, N, st, kbs, upc, B, pair) <= max_smem) {
-                *kbs_out = kbs;
-                *stages_out = st;
-                return true;
-            }
+    if (upc > 16) return false;
+    const int KH = ((pair ? (H + 1) / 2 : H) + 15) / 16 * 16;
+    for (int rg = groups_of(rows_wanted < kTcMaxRows ? rows_wanted : kTcMaxRows); rg >= 1; --rg) {
+        if (KH / 2 + tc_acc_columns(rg) <= 512 && KH <= 16 * kPollers * kMaxGroups && recur_tc_smem_bytes(KH, upc, 8 * rg, pair) <= max_smem) {
+            p->upc = upc; p->ncta = n; p->KH = KH; p->pair = pair; p->rows = 8 * rg;
+            return true;
         }
     }
     return false;
 }
 
-bool recur_tc_encode_weights(void *map, const void *w, long long rows, int ld, int RA)
-{
-    return encode_2d(map, w, rows, ld, ld, RA);
-}
-bool recur_tc_encode_planes(void *map, const void *hbuf, int D, int H, int ldh, int B)
-{
-    // a box holds the 2B plane rows rounded up to a swizzle group of 8, not the MMA's N (a multiple of 16)
-    return encode_2d(map, hbuf, (long long)D * 2 * kTcPlaneRows, H, ldh, (2 * B + 7) & ~7);
-}
-
 cudaError_t recur_tc_prepare(int max_smem)
 {
-    return cudaFuncSetAttribute(recur_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+    for (int rg = 1; rg <= kTcMaxRows / 8; ++rg) {
+        const cudaError_t e = cudaFuncSetAttribute(pick(rg), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // Can `grid` CTAs of this kernel be co-resident as clusters of two (pair mode needs every pair on one GPC)?
-bool recur_tc_pair_supported(int grid, size_t smem)
+bool recur_tc_pair_supported(int grid, int rows, size_t smem)
 {
-    if (grid < 2 || (grid & 1)) return false;
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = config(attr, grid, smem, 1, nullptr);
+    cfg.attrs = attr + 1; cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)recur_tc_kernel, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)pick(groups_of(rows)), &cfg) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     return clusters * 2 >= grid;
 }
 
-cudaError_t launch_recur_tc(const void *tmap_w, const void *tmap_h, const RecurTcArgs &a, size_t smem, cudaStream_t st)
+cudaError_t launch_recur_tc(const RecurTcArgs &a, cudaStream_t st)
 {
-    CUtensorMap mw, mh;
-    memcpy(&mw, tmap_w, sizeof mw);
-    memcpy(&mh, tmap_h, sizeof mh);
+    KernelFn fn = pick(groups_of(a.B));
+    if (!fn) return cudaErrorInvalidValue;
     RecurTcArgs copy = a;
-    void *params[] = {&mw, &mh, &copy};
-    const int grid = a.ncta_dir * (a.ndirs ? a.ndirs : a.D);
-    if (!a.pair)
-        return cudaLaunchCooperativeKernel((const void *)recur_tc_kernel, dim3(grid), dim3(kThreads), params, smem, st);
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    void *params[] = {&copy};
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeCooperative;
-    attr[1].val.cooperative = 1;
-    cfg.attrs = attr; cfg.numAttrs = 2;
-    return cudaLaunchKernelExC(&cfg, (const void *)recur_tc_kernel, params);
+    const cudaLaunchConfig_t cfg = config(attr, a.ncta_dir * (a.ndirs ? a.ndirs : a.D), recur_tc_smem_bytes(a.KH, a.upc, a.B, a.pair), a.pair, st);
+    return cudaLaunchKernelExC(&cfg, (const void *)fn, params);
 }
 
 }  // namespace lstm
