@@ -57,11 +57,6 @@ constexpr int kGroupBar = 2;                    // named barrier of group 0: pol
 __host__ __device__ constexpr int tc_rows_per_thread(int rg) { return rg <= 2 ? 4 : rg <= 4 ? 8 : 16; }
 // operand groups a lane has in flight: 16-byte chunks of rg batch rows each, at most twelve (registers)
 __host__ __device__ constexpr int tc_groups_in_flight(int rg) { return 12 / rg < kMaxGroups ? 12 / rg : kMaxGroups; }
-// floats between the rows of received partial sums: a multiple of 4 off the bank period
-__host__ __device__ constexpr int tc_partial_pitch(int rg)
-{
-    return (8 * rg + tc_rows_per_thread(rg) - 1) / tc_rows_per_thread(rg) * tc_rows_per_thread(rg) + 4;
-}
 
 // ---- two-CTA cluster helpers: the partner's shared memory and barriers
 __device__ __forceinline__ uint32_t cluster_ctarank()
@@ -76,11 +71,11 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t local_smem_addr, uint32_
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_smem_addr), "r"(rank));
     return r;
 }
-// 16 bytes into another CTA's shared memory; the bytes are counted on that CTA's barrier
-__device__ __forceinline__ void st_async_v4(uint32_t remote_dst, float a, float b, float c, float d, uint32_t remote_bar)
+// one word into another CTA's shared memory; the bytes are counted on that CTA's barrier
+__device__ __forceinline__ void st_async(uint32_t remote_dst, float v, uint32_t remote_bar)
 {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
-                 ::"r"(remote_dst), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(__float_as_uint(c)), "r"(__float_as_uint(d)), "r"(remote_bar) : "memory");
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                 ::"r"(remote_dst), "r"(__float_as_uint(v)), "r"(remote_bar) : "memory");
 }
 __device__ __forceinline__ void cluster_sync_all()
 {
@@ -137,7 +132,7 @@ __device__ __forceinline__ void quad_transpose(float &v0, float &v1, float &v2, 
 template <int RG>
 __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs a)
 {
-    constexpr int Bp = 8 * RG, N = 2 * Bp, RS = tc_rows_per_thread(RG), NSUB = (Bp + RS - 1) / RS, PZ = tc_partial_pitch(RG);
+    constexpr int Bp = 8 * RG, N = 2 * Bp, RS = tc_rows_per_thread(RG), NSUB = (Bp + RS - 1) / RS;
     constexpr int KI = tc_groups_in_flight(RG), NACC = tc_accumulators(RG);
     constexpr uint32_t tmem = 0;                                            // all 512 columns are ours: they start at address 0
     constexpr uint32_t acc_col = 512u - tc_acc_columns(RG);                 // accumulators behind the weights
@@ -158,12 +153,12 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     const int ngroups = (nk16 + kPollers - 1) / kPollers;                   // warp w fetches piece w of every group
     const int nissue = min(NACC, ngroups);                                  // issuing warps, each with an accumulator
 
-    // shared memory: operand tiles of 64 columns [N rows][128 bytes, swizzled], then the partner's partial sums [2][RA][PZ]
+    // shared memory: operand tiles of 64 columns [N rows][128 bytes, swizzled], then the partner's partial sums [2][Bp][RA]
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     unsigned char *op = smem_raw + (base - smem_u32(smem_raw));
     const int tiles = (a.KH + 63) >> 6;
     float *zs2 = reinterpret_cast<float *>(op + (size_t)tiles * N * 128);
-    LSTM_CHECK_SMEM_END(reinterpret_cast<unsigned char *>(zs2 + (pair ? 2 * RA * PZ : 0)) - smem_raw, a.status);
+    LSTM_CHECK_SMEM_END(reinterpret_cast<unsigned char *>(zs2 + (pair ? 2 * RA * Bp : 0)) - smem_raw, a.status);
 
     if (tid == 0) {
         abort_s = 0;
@@ -190,9 +185,11 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     const unsigned slot_words = (unsigned)((H + 15) >> 4) * rgx * 128u;
     const size_t set_words = (size_t)2 * D * slot_words;
     auto chunk_word = [&](int q, int b) -> unsigned { return (((unsigned)(q >> 2) * rgx + (b >> 3)) * 32u + (q & 3) * 8u + (b & 7)) * 4u; };
-    unsigned *xch_d = a.xch + (size_t)a.set * set_words + (size_t)d * 2 * slot_words;
+    // (buffers by place in the launch, not by direction: launches that run the directions in turn share them)
+    const size_t xch_off = (size_t)(d - a.dir0) * 2 * slot_words;
+    unsigned *xch_d = a.xch + (size_t)a.set * set_words + xch_off;
     {
-        unsigned *other = a.xch + (size_t)(a.set ^ 1) * set_words + (size_t)d * 2 * slot_words;
+        unsigned *other = a.xch + (size_t)(a.set ^ 1) * set_words + xch_off;
         const int cq = cta * (upc >> 2), qn = max(0, min(upc >> 2, nq - cq));
         for (int i = tid; i < 2 * qn * a.clear_rows; i += kThreads) {
             const int sl = i / (qn * a.clear_rows), r = i - sl * qn * a.clear_rows, q = r / a.clear_rows, b = r - q * a.clear_rows;
@@ -241,13 +238,14 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     const bool fin = sub < NSUB && (warp & 3) * 32 < RT;                    // this warp reads accumulators
     const bool mine = row < RT && side == rank;
     const int u = lr >> 2, j = cta * upc + u;                               // unit of this row, if it is ours
+    const bool any_mine = __any_sync(0xffffffffu, mine);
     const bool own = mine && fin && j < Hq, real = own && j < H;
     const int fb0 = sub * RS;
     const float act_k = (fq == 2 ? -2.0f : -1.0f) * 1.4426950408889634f, act_sc = fq == 2 ? 2.0f : 1.0f, act_of = fq == 2 ? -1.0f : 0.0f;
-    const uint32_t zs2_remote = pair ? map_to_cta(smem_u32(zs2), (uint32_t)(rank ^ 1)) + (uint32_t)(lr * PZ + fb0) * 4u : 0u;
+    const uint32_t zs2_remote = pair ? map_to_cta(smem_u32(zs2), (uint32_t)(rank ^ 1)) + (uint32_t)(fb0 * RA + lr) * 4u : 0u;
     const uint32_t partial_remote = pair ? map_to_cta(smem_u32(partial_bar), (uint32_t)(rank ^ 1)) : 0u;
     const uint32_t abort_remote = pair ? map_to_cta(smem_u32(&abort_s), (uint32_t)(rank ^ 1)) : 0u;
-    const float *zs2_mine = zs2 + lr * PZ + fb0;
+    const float *zs2_mine = zs2 + fb0 * RA + lr;
     const size_t state0 = ((size_t)d * a.Bs + a.b0) * H + j;                // element of (pass row 0, unit j) in the state arrays
     // projection terms, outputs: pointers that advance by one timestep per step
     const long long gstep = (long long)D * 4 * H, dir = d ? -1 : 1;
@@ -272,10 +270,28 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
         hn[m] = 0.0f;
     }
 
-#pragma unroll 1
-    for (int s = 0; s < T; ++s) {
-        // ---- projection terms of this thread's row; the lines of a later step are requested into L2
-        float g[RS];
+    // outputs of a step: written while the next step's poll is under way
+    auto write_outputs = [&]() {
+        if (yp) {
+#pragma unroll
+            for (int m = 0; m < RS / 4; ++m)
+                if (m < nout) yp[m * ystep] = hn[m];
+            yp += yadv;
+        }
+        if (xp) {
+#pragma unroll
+            for (int m = 0; m < RS / 4; ++m)
+                if (m < nout) {
+                    const __nv_bfloat16 hi = __float2bfloat16_rn(hn[m]);
+                    xp[m * xstep] = hi;
+                    xp[a.xb_plane + m * xstep] = __float2bfloat16_rn(hn[m] - __bfloat162float(hi));
+                }
+            xp += xadv;
+        }
+    };
+    float g[RS];
+    auto load_g = [&](int s) {
+        // projection terms of this thread's row; the lines of a later step are requested into L2
 #pragma unroll
         for (int i = 0; i < RS; ++i) g[i] = i < nrow ? ld_nc_early(gp + i * gstep) : 0.0f;
         if (a.nsplit > 1)
@@ -286,8 +302,14 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
         if (pre && s + 2 < T) asm volatile("prefetch.global.L2 [%0];" ::"l"(gpre));
         gp += gadv;
         gpre += gadv;
+    };
+
+#pragma unroll 1
+    for (int s = 0; s < T; ++s) {
+        if (s > 0) write_outputs();
+        load_g(s);
         // (an aborted CTA opens no further phase: the open one never completes, and a second arrival would exceed its count)
-        if (pair && tid == 0 && !*abort_v) mbar_expect_tx(smem_u32(&partial_bar[s & 1]), (uint32_t)(RA * NSUB * RS * 4));
+        if (pair && tid == 0 && !*abort_v) mbar_expect_tx(smem_u32(&partial_bar[s & 1]), (uint32_t)(RA * Bp * 4));
 
         if (warp >= kIssuer && warp < kIssuer + nissue) {
             // ---- products: issuing warp w takes every nissue-th group, one elected thread, an accumulator of its own
@@ -299,17 +321,10 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
                 if (elect_one()) {
                     const uint64_t bd = bdesc0 + (uint64_t)(gi * (kDstGroup / 16));
                     const uint32_t ad = tmem + (uint32_t)(gi * kPollers * 8), acc = acc_col + (uint32_t)(w * N);
-                    if (n == kPollers) {
 #pragma unroll
-                        for (int t4 = 0; t4 < kPollers / 4; ++t4)
-#pragma unroll
-                            for (int kk = 0; kk < 4; ++kk)
-                                umma_bf16_ta(acc, ad + (t4 * 4 + kk) * 8, bd + (uint64_t)(t4 * (N * 128 / 16) + kk * 2), idesc, gi >= nissue || t4 + kk ? 1u : 0u);
-                    } else {
-#pragma unroll 1
-                        for (int k = 0; k < n; ++k)
+                    for (int k = 0; k < kPollers; ++k)
+                        if (k < n)
                             umma_bf16_ta(acc, ad + k * 8, bd + (uint64_t)((k >> 2) * (N * 128 / 16) + (k & 3) * 2), idesc, gi >= nissue || k ? 1u : 0u);
-                    }
                     if (gi + nissue >= ngroups) umma_commit(smem_u32(&accum_bar));
                 }
                 __syncwarp();
@@ -420,24 +435,24 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
                     // gave up: nothing is sent any more, so the partner must not wait for it
                     asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(abort_remote), "r"(1) : "memory");
                 } else if (row < RT && !mine) {
-                    const uint32_t dst = zs2_remote + (uint32_t)((s & 1) * RA * PZ) * 4u, bar = partial_remote + (uint32_t)(s & 1) * 8u;
+                    const uint32_t dst = zs2_remote + (uint32_t)((s & 1) * RA * Bp) * 4u, bar = partial_remote + (uint32_t)(s & 1) * 8u;
 #pragma unroll
-                    for (int i = 0; i < RS; i += 4) st_async_v4(dst + i * 4, z[i], z[i + 1], z[i + 2], z[i + 3], bar);
+                    for (int i = 0; i < RS; ++i)
+                        if (RS * NSUB == Bp || fb0 + i < Bp) st_async(dst + (uint32_t)(i * RA) * 4u, z[i], bar);
                 }
                 __syncwarp();
-                if (__any_sync(0xffffffffu, mine)) {
+                if (any_mine) {
                     mbar_wait(smem_u32(&partial_bar[s & 1]), (uint32_t)(s >> 1) & 1u, abort_v);
                     __syncwarp();
                     if (mine) {
-                        const float *zp = zs2_mine + (s & 1) * RA * PZ;
+                        const float *zp = zs2_mine + (s & 1) * RA * Bp;
 #pragma unroll
-                        for (int i = 0; i < RS; i += 4) {
-                            const float4 p = *reinterpret_cast<const float4 *>(zp + i);
-                            z[i] += p.x; z[i + 1] += p.y; z[i + 2] += p.z; z[i + 3] += p.w;
-                        }
+                        for (int i = 0; i < RS; ++i)
+                            if (RS * NSUB == Bp || fb0 + i < Bp) z[i] += zp[i * RA];
                     }
                 }
             }
+            if (any_mine) {
 #pragma unroll
             for (int i = 0; i < RS; ++i) z[i] = gate_fast(z[i] + g[i], act_k, act_sc, act_of);
             unsigned *dst = out0 + (size_t)(s & 1) * slot_words;
@@ -450,27 +465,13 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
                 // (fb0 is a multiple of four: of eight where a thread has more than one item)
                 if (m < npub) st_relaxed_u32(dst + (m & 1) * 16 + (m >> 1) * 128, pack_word(hn[m], phase_out));
             }
+            }
         }
         // Nobody polls or overwrites the operand before the whole CTA has published: early polls of words that are being
         // written pull their lines to and fro between the two halves of the L2, and delay everyone.
         bar_sync(1, kThreads);
-        if (yp) {
-#pragma unroll
-            for (int m = 0; m < RS / 4; ++m)
-                if (m < nout) yp[m * ystep] = hn[m];
-            yp += yadv;
-        }
-        if (xp) {
-#pragma unroll
-            for (int m = 0; m < RS / 4; ++m)
-                if (m < nout) {
-                    const __nv_bfloat16 hi = __float2bfloat16_rn(hn[m]);
-                    xp[m * xstep] = hi;
-                    xp[a.xb_plane + m * xstep] = __float2bfloat16_rn(hn[m] - __bfloat162float(hi));
-                }
-            xp += xadv;
-        }
     }
+    write_outputs();
 #pragma unroll
     for (int m = 0; m < RS / 4; ++m)
         if (m < nout) {
@@ -527,7 +528,7 @@ cudaLaunchConfig_t config(cudaLaunchAttribute (&attr)[2], int grid, size_t smem,
 size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair)
 {
     const int rg = groups_of(rows);
-    return 1024 + (size_t)((KH + 63) / 64) * (16 * rg) * 128 + (pair ? (size_t)2 * 4 * upc * tc_partial_pitch(rg) * 4 : 0);
+    return 1024 + (size_t)((KH + 63) / 64) * (16 * rg) * 128 + (pair ? (size_t)2 * 4 * upc * 8 * rg * 4 : 0);
 }
 
 // Partition of H units over at most max_cta CTAs, and the most batch rows (<= rows_wanted) a pass can take; false when
