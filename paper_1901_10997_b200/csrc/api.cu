@@ -71,6 +71,9 @@ struct lstm_handle {
     unsigned *tcb_xch = nullptr; int tcb_set = 0, tcb_dirty = 0;
     // H-LSTM cell: width of the hidden layer inside each gate (0: plain LSTM), pass-2 column tiles per warp
     int Hh = 0, hl_nkw2 = 0;
+    bool use_ht = false;               // H-LSTM on the tile kernel; else on the one that runs batch rows in turn
+    HlstmTilePlan ht = {0, 0, 0, 0, 0, 0};
+    unsigned *ht_hx = nullptr, *ht_rx = nullptr; int ht_set = 0;
     unsigned long long *rxch = nullptr; size_t rxch_words = 0;
     std::vector<Layer> layers;
     // workspace
@@ -399,6 +402,47 @@ std::vector<uint32_t> pack_fragments(const float *m, int U, int K, int ncta, int
     return f;
 }
 
+// One 16 x 16 operand-A tile with the lane's columns adjacent (4 * (lane & 3) .. + 3): rows r0 .. of an [R x K] matrix, zero
+// beyond row r_end and column K; 128 words.
+void pack_tile(const float *m, int K, int r0, int r_end, int k0, uint32_t *out)
+{
+    auto wv = [&](int r, int k) -> uint32_t { return r < r_end && k < K ? f32_to_bf16_rne(m[(size_t)r * K + k]) : 0u; };
+    for (int lane = 0; lane < 32; ++lane) {
+        const int r = r0 + (lane >> 2), k = k0 + 4 * (lane & 3);
+        *out++ = wv(r, k) | (wv(r, k + 1) << 16);
+        *out++ = wv(r + 8, k) | (wv(r + 8, k + 1) << 16);
+        *out++ = wv(r, k + 2) | (wv(r, k + 3) << 16);
+        *out++ = wv(r + 8, k + 2) | (wv(r + 8, k + 3) << 16);
+    }
+}
+// Uh [4Hh x H] and W [4H x Hh] (gate blocks) as the fragments of the H-LSTM tile kernel
+std::vector<uint32_t> pack_ht_hidden(const float *uh, const HlstmTilePlan &p)
+{
+    const int mt = (p.Hh + 15) / 16;
+    std::vector<uint32_t> f((size_t)p.ncta * 16 * p.kt * p.n1 * 128, 0u);
+    for (int c = 0; c < p.ncta; ++c)
+        for (int wp = 0; wp < 16; ++wp)
+            for (int i = 0; i < p.kt; ++i)
+                for (int n = 0; n < p.n1; ++n) {
+                    const int tile = c * p.n1 + n, q = tile / mt, k0 = (wp * p.kt + i) * 16;
+                    if (tile < 4 * mt && k0 < p.H)
+                        pack_tile(uh, p.H, q * p.Hh + (tile - q * mt) * 16, (q + 1) * p.Hh, k0, f.data() + (((size_t)(c * 16 + wp) * p.kt + i) * p.n1 + n) * 128);
+                }
+    return f;
+}
+std::vector<uint32_t> pack_ht_gates(const float *w, const HlstmTilePlan &p)
+{
+    const int kt2 = ((p.Hh + 15) / 16 + 3) / 4;
+    std::vector<uint32_t> f((size_t)p.ncta * 16 * kt2 * 128, 0u);
+    for (int c = 0; c * 16 < p.H; ++c)
+        for (int wp = 0; wp < 16; ++wp)
+            for (int i = 0; i < kt2; ++i) {
+                const int q = wp >> 2, k0 = ((wp & 3) * kt2 + i) * 16;
+                if (k0 < p.Hh) pack_tile(w, p.Hh, q * p.H + c * 16, (q + 1) * p.H, k0, f.data() + ((size_t)(c * 16 + wp) * kt2 + i) * 128);
+            }
+    return f;
+}
+
 // Rows of a [4H x H] recurrent matrix (row q*H + j) as the batched tensor-core kernel wants them: per CTA [8-column
 // piece of its K range][row 4 * unit + gate of its units, in pair mode of both CTAs' units] 8 bf16.
 std::vector<uint16_t> pack_tc_rows(const float *m, int H, const RecurTcPlan &p)
@@ -456,7 +500,7 @@ void free_all(lstm_handle *h)
         cudaFree(ly.bias_out); cudaFree(ly.wtc[0]); cudaFree(ly.wtc[1]);
     }
     cudaFree(h->G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
-    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); cudaFree(h->tcb_xch); cudaFree(h->status_dev);
+    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); cudaFree(h->tcb_xch); cudaFree(h->ht_hx); cudaFree(h->ht_rx); cudaFree(h->status_dev);
     for (int l = 0; l < kMaxWaveLayers; ++l) cudaFree(h->wave_frag[l]);
     cudaFree(h->wave_xch);
     cudaFree(h->cmap); cudaFree(h->rem_idx); cudaFree(h->rem_bias);
@@ -1043,9 +1087,14 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
     h->spin_limit_default = h->spin_limit;
     auto bail = [&](int code) { g_create_error = h->err; free_all(h); delete h; return code; };
 
-    // tiling: row tiles cover 4 x (units per CTA) of both passes; pass 1 keeps up to nkr column tiles per
-    // warp in registers, the rest and all of pass 2 in shared memory
     {
+        // LSTM_B200_RECUR=mma keeps the kernel that runs batch rows in turn
+        const char *env = getenv("LSTM_B200_RECUR");
+        h->use_ht = !(env && strcmp(env, "mma") == 0) && hlstm_tile_plan(H, Hh, h->sm_count / D, (size_t)h->smem_optin - 64, &h->ht);
+    }
+    // tiling of the other kernel: row tiles cover 4 x (units per CTA) of both passes; pass 1 keeps up to nkr column tiles per
+    // warp in registers, the rest and all of pass 2 in shared memory
+    if (!h->use_ht) {
         const int upch = (Hh + h->ncta_dir - 1) / h->ncta_dir;
         const int mt = (4 * std::max(h->upc, upch) + 15) / 16;
         const int nk1 = (H + 15) / 16, nk2 = (Hh + 15) / 16;
@@ -1110,8 +1159,8 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
                 if (bb) for (int j = 0; j < H; ++j) bias_o[(size_t)d * 4 * H + (size_t)j * 4 + q] = bb[q * H + j];
             }
             const int NW = h->mma_nw;
-            std::vector<uint32_t> f1 = pack_fragments(uh, Hh, H, h->ncta_dir, NW, h->mma_nkr + h->mma_nks, h->mma_mt);
-            std::vector<uint32_t> f2 = pack_fragments(ww, H, Hh, h->ncta_dir, NW, h->hl_nkw2, h->mma_mt);
+            const std::vector<uint32_t> f1 = h->use_ht ? pack_ht_hidden(uh, h->ht) : pack_fragments(uh, Hh, H, h->ncta_dir, NW, h->mma_nkr + h->mma_nks, h->mma_mt);
+            const std::vector<uint32_t> f2 = h->use_ht ? pack_ht_gates(ww, h->ht) : pack_fragments(ww, H, Hh, h->ncta_dir, NW, h->hl_nkw2, h->mma_mt);
             rc = upload(h, (uint32_t **)&ly.wfrag[d], f1.data(), f1.size() * 4, st, "hidden-layer recurrent fragments");
             if (rc == LSTM_OK) rc = upload(h, (uint32_t **)&ly.frag2[d], f2.data(), f2.size() * 4, st, "gate output fragments");
             if (rc == LSTM_OK) cudaStreamSynchronize(st);
@@ -1137,12 +1186,16 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
         for (int i = 0; i < 2 && rc == LSTM_OK; ++i) rc = dev_alloc(h, &h->ybuf[i], Mmax * D * H * 4, false, st, "layer activations");
     }
     h->xch_words = (size_t)D * 2 * max_B * H;
-    h->rxch_words = (size_t)D * 2 * max_B * 4 * Hh;
+    if (h->use_ht) {
+        h->xch_words = 1;
+        if (rc == LSTM_OK) rc = dev_alloc(h, &h->ht_hx, (size_t)2 * D * 2 * ((H + 15) / 16) * 256 * 4, true, st, "exchange words");
+        if (rc == LSTM_OK) rc = dev_alloc(h, &h->ht_rx, (size_t)2 * D * 2 * ((Hh + 15) / 16) * 1024 * 4, true, st, "hidden-layer exchange words");
+    } else h->rxch_words = (size_t)D * 2 * max_B * 4 * Hh;
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->xch, h->xch_words * 8, true, st, "exchange buffer");
-    if (rc == LSTM_OK) rc = dev_alloc(h, &h->rxch, h->rxch_words * 8, true, st, "hidden-layer exchange buffer");
+    if (rc == LSTM_OK && h->rxch_words) rc = dev_alloc(h, &h->rxch, h->rxch_words * 8, true, st, "hidden-layer exchange buffer");
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->status_dev, sizeof(int), true, st, "status word");
     if (rc == LSTM_OK) {
-        cudaError_t e = hlstm_mma_prepare(h->mma_mt, h->mma_nkr, h->mma_nw, h->smem_optin - 64);
+        cudaError_t e = h->use_ht ? hlstm_tile_prepare(h->ht) : hlstm_mma_prepare(h->mma_mt, h->mma_nkr, h->mma_nw, h->smem_optin - 64);
         if (e == cudaSuccess) e = proj_tc_prepare();
         if (e != cudaSuccess) rc = fail(h, LSTM_ERR_CUDA, "kernel set-up failed: %s", cudaGetErrorString(e));
     }
@@ -1319,6 +1372,37 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         // ---- recurrence: all directions in one launch, or one launch per direction
         const int npass = h->seq_dirs ? D : 1;
         for (int pass = 0; pass < npass; ++pass) {
+        if (h->use_ht) {
+            const int passes = (B + kHtRows - 1) / kHtRows;
+            for (int p = 0; p < passes; ++p) {
+                HlstmTileArgs m;
+                memset(&m, 0, sizeof m);
+                m.Bs = B; m.b0 = (int)((long long)B * p / passes); m.B = (int)((long long)B * (p + 1) / passes) - m.b0;
+                m.H = H; m.Hh = h->Hh; m.T = T; m.D = D; m.ncta_dir = h->ht.ncta; m.nsplit = nsplit;
+                m.spin_limit = h->spin_limit;
+                m.withhold_cta = h->withhold_cta < 0 ? -1 : h->withhold_cta % (h->ht.ncta * D);
+                for (int d = 0; d < D; ++d) { m.frag1[d] = ly.wfrag[d]; m.frag2[d] = ly.frag2[d]; }
+                m.G = h->G;
+                m.g_split_stride = (long long)M * N;
+                m.bias_out = ly.bias_out;
+                const size_t so = (size_t)l * D * B * H;
+                m.h0 = h0 ? h0 + so : nullptr; m.c0 = c0 ? c0 + so : nullptr;
+                m.hT = hT ? hT + so : nullptr; m.cT = cT ? cT + so : nullptr;
+                m.y = l == L - 1 ? y : nullptr;                  // the next layer reads the bf16 planes
+                m.xb_next = l < L - 1 ? h->xbn[l & 1] : nullptr;
+                m.xb_ld = h->ldn;
+                m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
+                m.hx = h->ht_hx; m.rx = h->ht_rx; m.set = h->ht_set;
+                m.status = h->status_dev;
+                if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+                e = launch_hlstm_tile(m, h->ht, st);
+                ++h->last_launches;
+                if (e == cudaSuccess) h->ht_set ^= 1;
+                if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+                if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
+            }
+            continue;
+        }
         if (h->Hh) {
             HlstmArgs m;
             memset(&m, 0, sizeof m);
@@ -1640,7 +1724,7 @@ int lstm_info(const lstm_handle *h, int64_t *out, int n)
         return cnt;
     }
     RecurShape shp = recur_shape(h, h->max_B, 0);
-    if (h->Hh) shp.smem = hlstm_mma_smem_bytes(h->mma_mt, h->mma_nkr, h->mma_nw, h->mma_nks, h->hl_nkw2, h->upc, h->max_B);
+    if (h->Hh && !h->use_ht) shp.smem = hlstm_mma_smem_bytes(h->mma_mt, h->mma_nkr, h->mma_nw, h->mma_nks, h->hl_nkw2, h->upc, h->max_B);
     const size_t wsize = h->dtype == LSTM_BF16W_F32S ? 2 : 4;
     int64_t rows_res = 0, rows_str = 0;
     if (h->use_mma) {

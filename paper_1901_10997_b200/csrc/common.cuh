@@ -262,6 +262,36 @@ cudaError_t hlstm_mma_prepare(int mt, int nkr, int nw, int max_smem);
 cudaError_t launch_hlstm_mma(const HlstmArgs &a, int mt, int nkr, int nw, size_t smem, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------
+// H-LSTM kernel for batches: row tiles of sixteen units of one gate, eight batch rows per operand-B tile (hlstm_tile.cu)
+// ---------------------------------------------------------------------------------------------------
+constexpr int kHtRows = 16;            // batch rows of one launch; larger calls run several
+struct HlstmTilePlan { int H, Hh, n1, kt, ncta; size_t max_smem; };     // hidden tiles per CTA, column tiles of h per warp, CTAs per direction
+struct HlstmTileArgs {
+    int H, Hh, B, T, D;
+    int Bs, b0;                 // batch rows of the call, first row of this launch
+    int ncta_dir, nsplit;
+    long long spin_limit;
+    int withhold_cta;
+    const uint4 *frag1[2];      // Uh per direction: [cta][warp][kt column tiles][n1 hidden tiles][lane]
+    const uint4 *frag2[2];      // W per direction: [cta][warp = 4 * gate + K quarter][column tile][lane]
+    const float *G;             // as in HlstmArgs
+    long long g_split_stride;
+    const float *bias_out;
+    const float *h0, *c0;
+    float *hT, *cT;
+    float *y;
+    __nv_bfloat16 *xb_next;
+    long long xb_plane;
+    int xb_ld;
+    unsigned *hx, *rx;          // exchange words [2 sets][D][2 slots][tile][2 row groups][128]: tiles of cell units; of 4 x hidden units
+    int set;                    // the set this launch uses; it clears the other one
+    int *status;
+};
+bool hlstm_tile_plan(int H, int Hh, int max_cta, size_t max_smem, HlstmTilePlan *p);
+cudaError_t hlstm_tile_prepare(const HlstmTilePlan &p);
+cudaError_t launch_hlstm_tile(const HlstmTileArgs &a, const HlstmTilePlan &p, cudaStream_t st);
+
+// ---------------------------------------------------------------------------------------------------
 // Row/column-pruned stacks: moving states and outputs between the full width H and the compact width Hc of the
 // surviving units, and the closed-form recurrence of the removed ones.
 // ---------------------------------------------------------------------------------------------------
