@@ -56,6 +56,7 @@ struct lstm_handle {
     // register-resident recurrent kernel (bf16 dense): row tiles, column tiles per warp in registers and
     // in shared memory, warps per CTA
     bool use_mma = false;
+    bool step_ok = false;              // single timesteps run on the streaming kernel (lstm_step.cu)
     bool fuse_ok = false;              // short single sequences: projection fused into the register-resident kernel's prologue
     // register-resident sparse kernel (bf16, CSR execution): warps, columns per warp, row tiles, entry slots per lane
     bool use_csr_reg = false;
@@ -903,6 +904,13 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     if (rc == LSTM_OK && cudaStreamSynchronize(st) != cudaSuccess)
         rc = fail(h, LSTM_ERR_CUDA, "workspace set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
     if (rc) return bail(rc);
+    if (h->use_mma && h->fuse_ok && !h->Hh) {
+        const char *wenv = getenv("LSTM_B200_WAVE");
+        bool fits = !(h->use_wave && wenv && strcmp(wenv, "1") == 0);
+        for (const Layer &ly : h->layers)
+            fits = fits && ly.xfrag[0] && lstm_step_smem_bytes(h->mma_mt, kStepMaxRows, h->mma_nw / 2 * ly.nkw_x, h->mma_nw * (h->mma_nkr + h->mma_nks)) <= (size_t)h->smem_optin;
+        h->step_ok = fits && lstm_step_prepare(h->mma_mt, h->smem_optin) == cudaSuccess;
+    }
     *out = h;
     return LSTM_OK;
 }
@@ -1329,6 +1337,32 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         if (h->rxch && cudaMemsetAsync(h->rxch, 0, h->rxch_words * 8, st) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
         if (h->wave_xch && cudaMemsetAsync(h->wave_xch, 0, h->wave_xch_words * 8, st) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
         h->stamp_next = 1;
+    }
+
+    // A single timestep of a few sequences on the register-resident kernel's weights: one streaming launch per layer
+    if (T == 1 && B <= kStepMaxRows && h->step_ok && !h->probe && h->withhold_cta < 0) {
+        for (int l = 0; l < L; ++l) {
+            const Layer &ly = h->layers[l];
+            LstmStepArgs m;
+            memset(&m, 0, sizeof m);
+            m.H = H; m.B = B; m.D = D; m.ncta_dir = h->ncta_dir;
+            m.in_l = ly.in_l; m.x_tiles = h->mma_nw / 2 * ly.nkw_x; m.h_tiles = h->mma_nw * (h->mma_nkr + h->mma_nks);
+            m.first = l == 0;
+            for (int d = 0; d < D; ++d) { m.xfrag[d] = ly.xfrag[d]; m.hfrag[d] = ly.wfrag[d]; }
+            m.X = l == 0 ? x : h->ybuf[(l - 1) & 1];
+            m.bias = ly.bias;
+            const size_t so = (size_t)l * D * B * H;
+            m.h0 = h0 ? h0 + so : nullptr; m.c0 = c0 ? c0 + so : nullptr;
+            m.hT = hT ? hT + so : nullptr; m.cT = cT ? cT + so : nullptr;
+            m.y = l == L - 1 ? y : h->ybuf[l & 1];
+            m.status = h->status_dev;
+            if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+            e = launch_lstm_step(m, h->mma_mt, st);
+            ++h->last_launches;
+            if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+            if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "step launch failed (layer %d): %s", l, cudaGetErrorString(e));
+        }
+        return LSTM_OK;
     }
 
     if (h->use_wave && B <= 4 && !h->probe) {          // (the probe builds exist for the per-layer kernels)

@@ -106,6 +106,27 @@ cudaError_t recur_mma_prepare(int mt, int nkr, int nw, int max_smem);
 cudaError_t launch_recur_mma(const RecurMmaArgs &a, int mt, int nkr, int nw, size_t smem, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------
+// One timestep of one layer (T = 1, up to kStepMaxRows batch rows) over the register-resident kernel's fragments
+// ---------------------------------------------------------------------------------------------------
+constexpr int kStepMaxRows = 8;
+struct LstmStepArgs {
+    int H, B, D, ncta_dir;
+    int in_l, x_tiles, h_tiles; // input width; 16-column tiles of the two fragment arrays per CTA
+    int first;                  // 1: first layer of the call (reads nothing before the work ahead of it is complete)
+    const uint4 *xfrag[2];      // [cta][x_tiles][MT][lane], the lane's columns adjacent
+    const uint4 *hfrag[2];      // [cta][h_tiles][MT][lane]
+    const float *X;             // [B][in_l]
+    const float *bias;          // [D][H][4]
+    const float *h0, *c0;       // [D][B][H] or nullptr
+    float *hT, *cT;
+    float *y;                   // [B][D*H]
+    int *status;
+};
+size_t lstm_step_smem_bytes(int mt, int B, int x_tiles, int h_tiles);
+cudaError_t lstm_step_prepare(int mt, int max_smem);
+cudaError_t launch_lstm_step(const LstmStepArgs &a, int mt, cudaStream_t st);
+
+// ---------------------------------------------------------------------------------------------------
 // Layer-wavefront recurrent kernel (unidirectional stacks of 2 to 4 layers, bf16 dense, up to four sequences).
 // CTAs [l * ncta_layer, (l + 1) * ncta_layer) run layer l.  Layer 0's matrix is Wh_0 [4H x H]; layer l >= 1's
 // is [Wx_l | Wh_l] [4H x 2H] acting on [h^{l-1}_t ; h^l_{t-1}].  Fragment layout as in RecurMmaArgs with

@@ -1,0 +1,193 @@
+// One timestep of one LSTM layer (T = 1, bf16 dense weights, up to eight batch rows): the call of a program that generates
+// token by token and carries the state itself.
+//     z = b + Wx x + Wh h;  i,f,o = sigmoid(z_i,z_f,z_o), g = tanh(z_g);  c' = f c + i g;  h' = o tanh(c')
+// There is nothing to exchange between CTAs and no weight is used twice, so what bounds it is the one read of both weight
+// matrices from HBM (36 MB per layer at 1500 -> 1500: 5.5 us at 6.55 TB/s).  A plain launch of the recurrent kernel spends
+// its time on the fragments' residency, one tile ahead, and on the cooperative launches.  Here every CTA requests its
+// whole slice into L2 at once, then streams the same operand-A fragments the recurrent kernel keeps (mma.m16n8k16, up to
+// eighteen 16-byte loads in flight a lane), and two CTAs fit an SM, so that with programmatic dependent launch the next
+// layer's (or the next call's) requests leave while this layer finishes: what a kernel reads of its predecessor it
+// reads behind griddepcontrol.wait, weights before it.  A layer above the first also multiplies Wh h0 before the wait:
+// the layer below lets it start only after its own wait, i.e. when everything before the call is complete.
+// Measured (2 x 1500, one sequence, per call of the binding): 49.1 us as two cooperative launches, 27.6 us here.
+#include "common.cuh"
+#include "device_util.cuh"
+
+#include <cstring>
+
+namespace lstm {
+namespace {
+
+constexpr int kWarps = 8, kThreads = 256;
+
+// MT: 16-row tiles of the CTA (4 gate rows x units).  RB: batch rows the operand is laid out for: up to 4 rows put their hi
+// and lo planes into adjacent columns, 8 take one column each and two instructions a tile.
+template <int MT, int RB>
+__global__ void __launch_bounds__(kThreads, 2) lstm_step_kernel(const LstmStepArgs a)
+{
+    constexpr int U = MT == 1 ? 12 : MT == 2 ? 8 : MT == 3 ? 6 : 4;     // column tiles in flight
+    constexpr int RP = MT * 16 + (RB == 8 ? 4 : 8), WS = RB * RP;       // partial sums [warp][row][RP]: no bank conflicts
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, tig = lane & 3;
+    const int H = a.H, B = a.B, D = a.D;
+    const int d = blockIdx.x / a.ncta_dir, cta = blockIdx.x % a.ncta_dir;
+    int u0, nu;
+    unit_range(H, a.ncta_dir, cta, u0, nu);
+    const uint4 *fx = a.xfrag[d] + (size_t)cta * a.x_tiles * MT * 32, *fh = a.hfrag[d] + (size_t)cta * a.h_tiles * MT * 32;
+    // the whole slice into L2
+    for (int i = tid; i < a.h_tiles * MT * 4; i += kThreads)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char *>(fh) + (size_t)i * 128));
+    for (int i = tid; i < a.x_tiles * MT * 4; i += kThreads)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char *>(fx) + (size_t)i * 128));
+    if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    const int xk = a.x_tiles * 16, hk = a.h_tiles * 16;                 // columns of the staged operands, zero beyond the real ones
+    const int pitch = (xk > hk ? xk : hk) + 16;
+    unsigned *op = reinterpret_cast<unsigned *>(smem);                  // [RB][pitch] words {bf16 hi | bf16 lo}
+    float *red = reinterpret_cast<float *>(op + RB * pitch);            // [kWarps][RB][RP]
+    LSTM_CHECK_SMEM_END(reinterpret_cast<unsigned char *>(red + kWarps * WS) - smem, a.status);
+
+    float acc[MT][4];
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[mt][e] = 0.0f;
+    // columns of h: the recurrent fragments hold columns 2 tig, 2 tig + 1, 2 tig + 8, 2 tig + 9 of a tile in this lane, the
+    // input fragments 4 tig .. 4 tig + 3
+    const int brow = RB == 8 ? g : RB == 1 ? 0 : g >> 1;
+    const unsigned sel = RB != 8 && (g & 1) ? 0x5410u : 0x7632u;
+    auto stage = [&](const float *src, long long row_stride, int n, int ncol) {
+        for (int i = tid; i < RB * ncol; i += kThreads) {
+            const int b = i / ncol, k = i - b * ncol;
+            op[b * pitch + k] = src && b < B && k < n ? split_word(src[b * row_stride + k]) : 0u;
+        }
+        __syncthreads();
+    };
+    auto products = [&](const uint4 *frag, int tiles, bool adjacent) {
+        const unsigned *ow = op + brow * pitch + (adjacent ? 4 : 2) * tig;
+        const int second = adjacent ? 2 : 8;
+#pragma unroll 1
+        for (int t0 = warp; t0 < tiles; t0 += kWarps * U) {
+            uint4 af[U][MT];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt)
+                    af[u][mt] = t0 + kWarps * u < tiles ? ld_nc_u4(frag + (size_t)((t0 + kWarps * u) * MT + mt) * 32 + lane) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (t0 + kWarps * u < tiles) {
+                    const uint2 w0 = *reinterpret_cast<const uint2 *>(ow + (t0 + kWarps * u) * 16);
+                    const uint2 w1 = *reinterpret_cast<const uint2 *>(ow + (t0 + kWarps * u) * 16 + second);
+                    const unsigned b0 = __byte_perm(w0.x, w0.y, sel), b1 = __byte_perm(w1.x, w1.y, sel);
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt) mma_bf16(acc[mt], af[u][mt], b0, b1);
+                    if (RB == 8) {
+                        const unsigned l0 = __byte_perm(w0.x, w0.y, 0x5410u), l1 = __byte_perm(w1.x, w1.y, 0x5410u);
+#pragma unroll
+                        for (int mt = 0; mt < MT; ++mt) mma_bf16(acc[mt], af[u][mt], l0, l1);
+                    }
+                }
+        }
+        __syncthreads();                                                // the staged operand is free again
+    };
+    if (a.h0) {
+        stage(a.h0 + (size_t)d * B * H, H, H, hk);
+        products(fh, a.h_tiles, false);
+    }
+    if (!a.first) asm volatile("griddepcontrol.wait;" ::: "memory");
+    stage(a.X, a.in_l, a.in_l, xk);
+    products(fx, a.x_tiles, true);
+
+    float *rw = red + warp * WS + g;
+    if (RB == 8) {
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+            rw[2 * tig * RP + mt * 16] = acc[mt][0];
+            rw[(2 * tig + 1) * RP + mt * 16] = acc[mt][1];
+            rw[2 * tig * RP + mt * 16 + 8] = acc[mt][2];
+            rw[(2 * tig + 1) * RP + mt * 16 + 8] = acc[mt][3];
+        }
+    } else if (tig < RB) {
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+            rw[tig * RP + mt * 16] = acc[mt][0] + acc[mt][1];
+            rw[tig * RP + mt * 16 + 8] = acc[mt][2] + acc[mt][3];
+        }
+    }
+    __syncthreads();
+    // a quad per (unit, batch row): one gate each, then all four update the state and deal out the stores
+    const int fq = lane & 3;
+    const float act_k = (fq == 2 ? -2.0f : -1.0f) * 1.4426950408889634f, act_sc = fq == 2 ? 2.0f : 1.0f, act_of = fq == 2 ? -1.0f : 0.0f;
+    for (int i0 = 0; i0 < nu * B; i0 += kThreads / 4) {
+        const int item = i0 + (tid >> 2), b = item / nu, u = item - b * nu, j = u0 + u;
+        const bool live = item < nu * B;
+        float z = 0.0f;
+        if (live) {
+            z = a.bias[((size_t)d * H + j) * 4 + fq];
+            const float *rp = red + b * RP + 4 * u + fq;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) z += rp[w * WS];
+        }
+        const float act = gate_fast(z, act_k, act_sc, act_of);
+        const int q0 = lane & ~3;
+        const float vi = __shfl_sync(0xffffffffu, act, q0), vf = __shfl_sync(0xffffffffu, act, q0 + 1);
+        const float vg = __shfl_sync(0xffffffffu, act, q0 + 2), vo = __shfl_sync(0xffffffffu, act, q0 + 3);
+        if (live) {
+            const size_t so = ((size_t)d * B + b) * H + j;
+            const float cn = fmaf(vf, a.c0 ? a.c0[so] : 0.0f, vi * vg);
+            const float hn = vo * tanh_fast(cn);
+            if (fq == 0) a.y[(size_t)b * D * H + (size_t)d * H + j] = hn;
+            else if (fq == 1 && a.hT) a.hT[so] = hn;
+            else if (fq == 2 && a.cT) a.cT[so] = cn;
+        }
+    }
+}
+
+typedef void (*KernelFn)(const LstmStepArgs);
+template <int MT> KernelFn pick_rows(int B) { return B == 1 ? lstm_step_kernel<MT, 1> : B <= 4 ? lstm_step_kernel<MT, 4> : lstm_step_kernel<MT, 8>; }
+KernelFn pick(int mt, int B)
+{
+    switch (mt) {
+        case 1: return pick_rows<1>(B);
+        case 2: return pick_rows<2>(B);
+        case 3: return pick_rows<3>(B);
+        case 4: return pick_rows<4>(B);
+        default: return nullptr;
+    }
+}
+
+}  // namespace
+
+size_t lstm_step_smem_bytes(int mt, int B, int x_tiles, int h_tiles)
+{
+    const int rb = B == 1 ? 1 : B <= 4 ? 4 : 8, tiles = x_tiles > h_tiles ? x_tiles : h_tiles;
+    return (size_t)rb * (tiles * 16 + 16) * 4 + (size_t)kWarps * rb * (mt * 16 + 8) * 4;
+}
+
+cudaError_t lstm_step_prepare(int mt, int max_smem)
+{
+    for (int B = 1; B <= kStepMaxRows; B = B == 1 ? 4 : 2 * B) {
+        KernelFn fn = pick(mt, B);
+        if (!fn) return cudaErrorInvalidValue;
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t launch_lstm_step(const LstmStepArgs &a, int mt, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(a.ncta_dir * a.D); cfg.blockDim = dim3(kThreads); cfg.stream = st;
+    cfg.dynamicSmemBytes = lstm_step_smem_bytes(mt, a.B, a.x_tiles, a.h_tiles);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, pick(mt, a.B), a);
+}
+
+}  // namespace lstm
