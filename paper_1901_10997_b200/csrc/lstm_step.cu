@@ -9,7 +9,8 @@
 // layer's (or the next call's) requests leave while this layer finishes: what a kernel reads of its predecessor it
 // reads behind griddepcontrol.wait, weights before it.  A layer above the first also multiplies Wh h0 before the wait:
 // the layer below lets it start only after its own wait, i.e. when everything before the call is complete.
-// Measured (2 x 1500, one sequence, per call of the binding): 49.1 us as two cooperative launches, 27.6 us here.
+// Measured (2 x 1500, one sequence, per call of the binding): 49.1 us as two cooperative launches, 23.1 us here (27.6 with
+// every load behind the wait).
 #include "common.cuh"
 #include "device_util.cuh"
 
@@ -39,13 +40,12 @@ __global__ void __launch_bounds__(kThreads, 2) lstm_step_kernel(const LstmStepAr
         asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char *>(fh) + (size_t)i * 128));
     for (int i = tid; i < a.x_tiles * MT * 4; i += kThreads)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char *>(fx) + (size_t)i * 128));
-    if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!a.first) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     const int xk = a.x_tiles * 16, hk = a.h_tiles * 16;                 // columns of the staged operands, zero beyond the real ones
-    const int pitch = (xk > hk ? xk : hk) + 16;
-    unsigned *op = reinterpret_cast<unsigned *>(smem);                  // [RB][pitch] words {bf16 hi | bf16 lo}
-    float *red = reinterpret_cast<float *>(op + RB * pitch);            // [kWarps][RB][RP]
+    unsigned *oph = reinterpret_cast<unsigned *>(smem);                 // [RB][hk + 16] words {bf16 hi | bf16 lo}
+    unsigned *opx = oph + RB * (hk + 16);                               // [RB][xk + 16]
+    float *red = reinterpret_cast<float *>(opx + RB * (xk + 16));       // [kWarps][RB][RP]
     LSTM_CHECK_SMEM_END(reinterpret_cast<unsigned char *>(red + kWarps * WS) - smem, a.status);
 
     float acc[MT][4];
@@ -57,24 +57,33 @@ __global__ void __launch_bounds__(kThreads, 2) lstm_step_kernel(const LstmStepAr
     // input fragments 4 tig .. 4 tig + 3
     const int brow = RB == 8 ? g : RB == 1 ? 0 : g >> 1;
     const unsigned sel = RB != 8 && (g & 1) ? 0x5410u : 0x7632u;
-    auto stage = [&](const float *src, long long row_stride, int n, int ncol) {
-        for (int i = tid; i < RB * ncol; i += kThreads) {
-            const int b = i / ncol, k = i - b * ncol;
-            op[b * pitch + k] = src && b < B && k < n ? split_word(src[b * row_stride + k]) : 0u;
-        }
-        __syncthreads();
+    auto stage = [&](unsigned *op, const float *src, long long row_stride, int n, int ncol) {
+#pragma unroll
+        for (int b = 0; b < RB; ++b)
+            for (int k0 = tid; k0 < ncol; k0 += 8 * kThreads) {
+                float v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = b < B && k0 + i * kThreads < n ? src[b * row_stride + k0 + i * kThreads] : 0.0f;
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (k0 + i * kThreads < ncol) op[b * (ncol + 16) + k0 + i * kThreads] = split_word(v[i]);
+            }
     };
-    auto products = [&](const uint4 *frag, int tiles, bool adjacent) {
+    // a warp takes every kWarps-th column tile, U of them in flight
+    uint4 af[U][MT];
+    auto load = [&](const uint4 *frag, int tiles, int t0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+                af[u][mt] = t0 + kWarps * u < tiles ? ld_nc_u4(frag + (size_t)((t0 + kWarps * u) * MT + mt) * 32 + lane) : make_uint4(0, 0, 0, 0);
+    };
+    // products of all tiles of a matrix whose first U are loaded; ends with the first U of `next` on their way
+    auto products = [&](const unsigned *op, int pitch, const uint4 *frag, int tiles, bool adjacent, const uint4 *next, int next_tiles) {
         const unsigned *ow = op + brow * pitch + (adjacent ? 4 : 2) * tig;
         const int second = adjacent ? 2 : 8;
 #pragma unroll 1
         for (int t0 = warp; t0 < tiles; t0 += kWarps * U) {
-            uint4 af[U][MT];
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
-                    af[u][mt] = t0 + kWarps * u < tiles ? ld_nc_u4(frag + (size_t)((t0 + kWarps * u) * MT + mt) * 32 + lane) : make_uint4(0, 0, 0, 0);
 #pragma unroll
             for (int u = 0; u < U; ++u)
                 if (t0 + kWarps * u < tiles) {
@@ -89,16 +98,29 @@ __global__ void __launch_bounds__(kThreads, 2) lstm_step_kernel(const LstmStepAr
                         for (int mt = 0; mt < MT; ++mt) mma_bf16(acc[mt], af[u][mt], l0, l1);
                     }
                 }
+            const bool more = t0 + kWarps * U < tiles;
+            if (more || next) load(more ? frag : next, more ? tiles : next_tiles, more ? t0 + kWarps * U : warp);
         }
-        __syncthreads();                                                // the staged operand is free again
     };
-    if (a.h0) {
-        stage(a.h0 + (size_t)d * B * H, H, H, hk);
-        products(fh, a.h_tiles, false);
+    // What depends on the kernel before this one is read behind the wait: for the first layer both operands, above it x.
+    const bool with_h = a.h0 != nullptr;
+    load(with_h ? fh : fx, with_h ? a.h_tiles : a.x_tiles, warp);
+    if (a.first) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        stage(opx, a.X, a.in_l, a.in_l, xk);
     }
-    if (!a.first) asm volatile("griddepcontrol.wait;" ::: "memory");
-    stage(a.X, a.in_l, a.in_l, xk);
-    products(fx, a.x_tiles, true);
+    if (with_h) {
+        stage(oph, a.h0 + (size_t)d * B * H, H, H, hk);
+        __syncthreads();
+        products(oph, hk + 16, fh, a.h_tiles, false, fx, a.x_tiles);
+    }
+    if (!a.first) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        stage(opx, a.X, a.in_l, a.in_l, xk);
+    }
+    __syncthreads();
+    products(opx, xk + 16, fx, a.x_tiles, true, nullptr, 0);
 
     float *rw = red + warp * WS + g;
     if (RB == 8) {
@@ -162,8 +184,8 @@ KernelFn pick(int mt, int B)
 
 size_t lstm_step_smem_bytes(int mt, int B, int x_tiles, int h_tiles)
 {
-    const int rb = B == 1 ? 1 : B <= 4 ? 4 : 8, tiles = x_tiles > h_tiles ? x_tiles : h_tiles;
-    return (size_t)rb * (tiles * 16 + 16) * 4 + (size_t)kWarps * rb * (mt * 16 + 8) * 4;
+    const int rb = B == 1 ? 1 : B <= 4 ? 4 : 8;
+    return (size_t)rb * ((x_tiles + h_tiles) * 16 + 32) * 4 + (size_t)kWarps * rb * (mt * 16 + 8) * 4;
 }
 
 cudaError_t lstm_step_prepare(int mt, int max_smem)
