@@ -70,6 +70,7 @@ struct lstm_handle {
     bool use_tcb = false;
     RecurTcPlan tcb = {0, 0, 0, 0, 0};
     unsigned *tcb_xch = nullptr; int tcb_set = 0, tcb_dirty = 0;
+    unsigned *f32_xch = nullptr; int f32_set = 0;      // fp32 dense, at most two units per CTA: exchange words (two sets)
     // H-LSTM cell: width of the hidden layer inside each gate (0: plain LSTM), pass-2 column tiles per warp
     int Hh = 0, hl_nkw2 = 0;
     bool use_ht = false;               // H-LSTM on the tile kernel; else on the one that runs batch rows in turn
@@ -501,7 +502,7 @@ void free_all(lstm_handle *h)
         cudaFree(ly.bias_out); cudaFree(ly.wtc[0]); cudaFree(ly.wtc[1]);
     }
     cudaFree(h->G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
-    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); cudaFree(h->tcb_xch); cudaFree(h->ht_hx); cudaFree(h->ht_rx); cudaFree(h->status_dev);
+    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); cudaFree(h->tcb_xch); cudaFree(h->ht_hx); cudaFree(h->f32_xch); cudaFree(h->ht_rx); cudaFree(h->status_dev);
     for (int l = 0; l < kMaxWaveLayers; ++l) cudaFree(h->wave_frag[l]);
     cudaFree(h->wave_xch);
     cudaFree(h->cmap); cudaFree(h->rem_idx); cudaFree(h->rem_bias);
@@ -882,6 +883,8 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         for (int i = 0; i < 2 && rc == LSTM_OK; ++i) rc = dev_alloc(h, &h->ybuf[i], Mmax * D * H * 4, false, st, "layer activations");
     h->xch_words = (size_t)D * 2 * max_B * H;
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->xch, h->xch_words * 8, true, st, "exchange buffer");
+    if (rc == LSTM_OK && dtype == LSTM_F32 && !csr && h->upc <= 2 && H <= kF32MaxUnits)
+        rc = dev_alloc(h, &h->f32_xch, (size_t)2 * D * 2 * H * 32 * sizeof(unsigned), true, st, "exchange words");
     if (rc == LSTM_OK && h->use_tcb) {
         rc = dev_alloc(h, &h->tcb_xch, (size_t)2 * D * 2 * round_up(H, 16) * h->tcb.rows * sizeof(unsigned), true, st, "exchange words");
     }
@@ -1533,6 +1536,29 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             e = launch_recur_csr_reg(m, h->csr_slots, h->csr_nw, smem, st);
             ++h->last_launches;
+            if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+            if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
+            continue;
+        }
+        if (h->f32_xch && B <= kF32MaxRows) {
+            RecurF32Args m;
+            memset(&m, 0, sizeof m);
+            m.dir0 = h->seq_dirs ? pass : 0; m.ndirs = h->seq_dirs ? 1 : D;
+            m.H = H; m.Hp8 = h->Hp8; m.B = B; m.T = T; m.D = D; m.ncta_dir = h->ncta_dir;
+            m.spin_limit = h->spin_limit;
+            m.withhold_cta = h->withhold_cta;
+            for (int d = 0; d < D; ++d) m.wh[d] = (const float *)ly.wh[d];
+            m.G = h->G;
+            const size_t so = (size_t)l * D * B * H;
+            m.h0 = h0 ? h0 + so : nullptr; m.c0 = c0 ? c0 + so : nullptr;
+            m.hT = hT ? hT + so : nullptr; m.cT = cT ? cT + so : nullptr;
+            m.y = l == L - 1 ? y : h->ybuf[l & 1];
+            m.xch = h->f32_xch; m.set = h->f32_set;
+            m.status = h->status_dev;
+            if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+            e = launch_recur_f32(m, st);
+            ++h->last_launches;
+            if (e == cudaSuccess) h->f32_set ^= 1;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             continue;

@@ -55,6 +55,27 @@ cudaError_t recur_dense_prepare(int max_smem);   // raises the dynamic shared-me
 cudaError_t recur_csr_prepare(int max_smem);
 
 // ---------------------------------------------------------------------------------------------------
+// fp32 recurrent kernel on the double-precision tensor instruction (at most two units per CTA, 32 batch rows)
+// ---------------------------------------------------------------------------------------------------
+constexpr int kF32MaxUnits = 296;     // widest layer: two units on each of 148 CTAs
+constexpr int kF32MaxRows = 32;
+struct RecurF32Args {
+    int dir0, ndirs;            // as in RecurArgs
+    int H, Hp8, B, T, D, ncta_dir;
+    long long spin_limit;
+    int withhold_cta;
+    const float *wh[2];         // [H][4][Hp8]
+    const float *G;             // [T*B][D][H][4]
+    const float *h0, *c0;
+    float *hT, *cT;
+    float *y;
+    unsigned *xch;              // exchange words [2 sets][D][2 slots][H][32 batch rows]
+    int set;                    // the set this launch uses; it clears the other one
+    int *status;
+};
+cudaError_t launch_recur_f32(const RecurF32Args &a, cudaStream_t st);
+
+// ---------------------------------------------------------------------------------------------------
 // Register-resident recurrent kernel (bf16 weights, dense).  Same CTA/unit partition and exchange
 // buffer as above.  The slice of a CTA is cut into 16 x 16 tiles: MT row tiles (4 gate rows per unit,
 // zero-padded) by NW * nkw column tiles; warp w owns column tiles [w * nkw, (w + 1) * nkw) of every row

@@ -34,12 +34,14 @@ __global__ void __launch_bounds__(256) proj_simt_kernel(const float *__restrict_
                                                         int ldw, const float *__restrict__ bias,
                                                         float *__restrict__ G, int M, int N, int K)
 {
-    __shared__ float xs[16][64 + 4];
-    __shared__ float ws[16][64 + 4];
+    typedef typename AccOf<WT>::T AT;
+    // operands in the type of the sums: converted once as they are stored, not at every use (a conversion to fp64 has a
+    // quarter of the rate of an fp64 multiply-add)
+    __shared__ AT xs[16][64 + 4];
+    __shared__ AT ws[16][64 + 4];
     const int tid = threadIdx.x;
     const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
     const int tm = (tid / 16) * 4, tn = (tid % 16) * 4;
-    typedef typename AccOf<WT>::T AT;
     AT acc[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -52,19 +54,19 @@ __global__ void __launch_bounds__(256) proj_simt_kernel(const float *__restrict_
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int k = k0 + kk + i;
-            xs[kk + i][r] = (m0 + r < M && k < K) ? X[(size_t)(m0 + r) * K + k] : 0.0f;
-            ws[kk + i][r] = (n0 + r < N && k < K) ? to_f32(W[(size_t)(n0 + r) * ldw + k]) : 0.0f;
+            xs[kk + i][r] = (AT)((m0 + r < M && k < K) ? X[(size_t)(m0 + r) * K + k] : 0.0f);
+            ws[kk + i][r] = (AT)((n0 + r < N && k < K) ? to_f32(W[(size_t)(n0 + r) * ldw + k]) : 0.0f);
         }
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
-            float xv[4], wv[4];
+            AT xv[4], wv[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) { xv[i] = xs[k][tm + i]; wv[i] = ws[k][tn + i]; }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma((AT)xv[i], (AT)wv[j], acc[i][j]);
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma(xv[i], wv[j], acc[i][j]);
         }
         __syncthreads();
     }
