@@ -25,23 +25,18 @@ __global__ void stage_bf16_kernel(const float *__restrict__ x, __nv_bfloat16 *__
 __device__ __forceinline__ float to_f32(float v) { return v; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-template <typename WT> struct AccOf { typedef float T; };
-template <> struct AccOf<float> { typedef double T; };   // fp32 storage accumulates in fp64
-
 // 64x64 output tile, K step 16, 256 threads, 4x4 outputs per thread.
 template <typename WT>
 __global__ void __launch_bounds__(256) proj_simt_kernel(const float *__restrict__ X, const WT *__restrict__ W,
                                                         int ldw, const float *__restrict__ bias,
                                                         float *__restrict__ G, int M, int N, int K)
 {
-    typedef typename AccOf<WT>::T AT;
-    // operands in the type of the sums: converted once as they are stored, not at every use (a conversion to fp64 has a
-    // quarter of the rate of an fp64 multiply-add)
-    __shared__ AT xs[16][64 + 4];
-    __shared__ AT ws[16][64 + 4];
+    __shared__ float xs[16][64 + 4];
+    __shared__ float ws[16][64 + 4];
     const int tid = threadIdx.x;
     const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
     const int tm = (tid / 16) * 4, tn = (tid % 16) * 4;
+    typedef float AT;
     AT acc[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -54,19 +49,19 @@ __global__ void __launch_bounds__(256) proj_simt_kernel(const float *__restrict_
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int k = k0 + kk + i;
-            xs[kk + i][r] = (AT)((m0 + r < M && k < K) ? X[(size_t)(m0 + r) * K + k] : 0.0f);
-            ws[kk + i][r] = (AT)((n0 + r < N && k < K) ? to_f32(W[(size_t)(n0 + r) * ldw + k]) : 0.0f);
+            xs[kk + i][r] = (m0 + r < M && k < K) ? X[(size_t)(m0 + r) * K + k] : 0.0f;
+            ws[kk + i][r] = (n0 + r < N && k < K) ? to_f32(W[(size_t)(n0 + r) * ldw + k]) : 0.0f;
         }
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
-            AT xv[4], wv[4];
+            float xv[4], wv[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) { xv[i] = xs[k][tm + i]; wv[i] = ws[k][tn + i]; }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(xv[i], wv[j], acc[i][j]);
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma((AT)xv[i], (AT)wv[j], acc[i][j]);
         }
         __syncthreads();
     }
@@ -80,6 +75,79 @@ __global__ void __launch_bounds__(256) proj_simt_kernel(const float *__restrict_
             if (n < N) G[(size_t)m * N + n] = (float)(acc[i][j] + (AT)(bias ? bias[n] : 0.0f));
         }
     }
+}
+
+// fp32 storage: sums in fp64 on the double-precision tensor instruction.  32 x 32 output tile, K step 16, four warps of 2 x 2
+// m8n8 tiles.  What bounds it is the fp64 rate (64 multiply-adds per clock and SM) once the operands are converted as they
+// are stored instead of at every use and a lane's operands are single conflict-free loads; the next K step is on its way
+// while this one is multiplied, and small tiles put several CTAs on an SM.  2000 x 800 x 200: 83 us with the fp64
+// multiply-adds of the tile kernel above, 50 us here.
+__device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b)
+{
+    asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+}
+__global__ void __launch_bounds__(128) proj_f64_kernel(const float *__restrict__ X, const float *__restrict__ W, int ldw,
+                                                       const float *__restrict__ bias, float *__restrict__ G, int M, int N, int K)
+{
+    constexpr int P = 36;                                      // doubles between K rows: a half warp's 4 x 4 operands hit all banks
+    __shared__ double xs[2][16][P], ws[2][16][P];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 32, wm = (warp >> 1) * 16, wn = (warp & 1) * 16;
+    const int r = tid >> 2, kk = (tid & 3) * 4;                // this thread loads 4 adjacent elements of row r of each tile
+    const bool xok = m0 + r < M, wok = n0 + r < N;
+    const bool vec = (K & 3) == 0 && (ldw & 3) == 0 && ((reinterpret_cast<size_t>(X) | reinterpret_cast<size_t>(W)) & 15) == 0;
+    const float *xp = X + (size_t)(m0 + r) * K + kk, *wp = W + (size_t)(n0 + r) * ldw + kk;
+    float4 xn, wv;
+    auto load = [&](const float *p, bool ok, int k0) -> float4 {
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (ok) {
+            const int left = K - k0 - kk;
+            if (vec) { if (left > 0) v = *reinterpret_cast<const float4 *>(p + k0); }
+            else {
+                if (left > 0) v.x = p[k0];
+                if (left > 1) v.y = p[k0 + 1];
+                if (left > 2) v.z = p[k0 + 2];
+                if (left > 3) v.w = p[k0 + 3];
+            }
+        }
+        return v;
+    };
+    double acc[2][2][2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
+    xn = load(xp, xok, 0);
+    wv = load(wp, wok, 0);
+    int buf = 0;
+    for (int k0 = 0; k0 < K; k0 += 16, buf ^= 1) {
+        xs[buf][kk][r] = xn.x; xs[buf][kk + 1][r] = xn.y; xs[buf][kk + 2][r] = xn.z; xs[buf][kk + 3][r] = xn.w;
+        ws[buf][kk][r] = wv.x; ws[buf][kk + 1][r] = wv.y; ws[buf][kk + 2][r] = wv.z; ws[buf][kk + 3][r] = wv.w;
+        __syncthreads();                                       // (two buffers: the one read two steps ago is written next)
+        if (k0 + 16 < K) { xn = load(xp, xok, k0 + 16); wv = load(wp, wok, k0 + 16); }
+#pragma unroll
+        for (int k = 0; k < 16; k += 4) {
+            double a[2], b[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                a[i] = xs[buf][k + (lane & 3)][wm + 8 * i + (lane >> 2)];
+                b[i] = ws[buf][k + (lane & 3)][wn + 8 * i + (lane >> 2)];
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) mma_f64(acc[i][j], a[i], b[j]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int m = m0 + wm + 8 * i + (lane >> 2), n = n0 + wn + 8 * j + 2 * (lane & 3) + e;
+                if (m < M && n < N) G[(size_t)m * N + n] = (float)(acc[i][j][e] + (double)(bias ? bias[n] : 0.0f));
+            }
 }
 
 // CSR projection: a CTA stages MT = 8 activation rows (transposed so that the 8 values of one column
@@ -199,7 +267,7 @@ cudaError_t launch_proj_simt(const float *X, const void *W, bool bf16, int ldw, 
     if (bf16)
         proj_simt_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(X, (const __nv_bfloat16 *)W, ldw, bias, G, M, N, K);
     else
-        proj_simt_kernel<float><<<grid, 256, 0, st>>>(X, (const float *)W, ldw, bias, G, M, N, K);
+        proj_f64_kernel<<<dim3((N + 31) / 32, (M + 31) / 32), 128, 0, st>>>(X, (const float *)W, ldw, bias, G, M, N, K);
     return cudaGetLastError();
 }
 
