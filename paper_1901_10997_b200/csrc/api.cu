@@ -69,7 +69,7 @@ struct lstm_handle {
     // batched tensor-core recurrence: partition and exchange words (two sets: a launch clears the other one)
     bool use_tcb = false;
     RecurTcPlan tcb = {0, 0, 0, 0, 0};
-    unsigned *tcb_xch = nullptr; int tcb_set = 0, tcb_dirty = 0;
+    unsigned *tcb_xch = nullptr; int tcb_set = 0; unsigned tcb_dirty = 0;
     unsigned *f32_xch = nullptr; int f32_set = 0;      // fp32 dense, at most two units per CTA: exchange words (two sets)
     // H-LSTM cell: width of the hidden layer inside each gate (0: plain LSTM), pass-2 column tiles per warp
     int Hh = 0, hl_nkw2 = 0;
@@ -101,7 +101,7 @@ struct lstm_handle {
     int ev_used = 0;
     int last_launches = 0;
     // layer-wavefront kernel (unidirectional stacks, up to four sequences): CTAs per layer, units per CTA, tiling
-    bool use_wave = false;
+    bool use_wave = false, wave_all = false;    // wave_all: LSTM_B200_WAVE=1, whatever else could serve the call
     int wave_ncta = 0, wave_upc = 0, wave_mt = 0, wave_nkr = 0, wave_nkw[kMaxWaveLayers] = {0, 0, 0, 0}, wave_nkw_max = 0;
     uint4 *wave_frag[kMaxWaveLayers] = {nullptr, nullptr, nullptr, nullptr};
     unsigned long long *wave_xch = nullptr; size_t wave_xch_words = 0;
@@ -445,6 +445,10 @@ std::vector<uint32_t> pack_ht_gates(const float *w, const HlstmTilePlan &p)
     return f;
 }
 
+// Fewest batch rows the batched tensor-core recurrence serves: from two on it beats the passes of up to four rows of the
+// register-resident kernel (2 x 1500, T = 35: two rows 288 us, @TC2@ us on the tensor cores) and of the layer-wavefront kernel.
+int tc_min_rows(const lstm_handle *) { return 2; }
+
 // Rows of a [4H x H] recurrent matrix (row q*H + j) as the batched tensor-core kernel wants them: per CTA [8-column
 // piece of its K range][row 4 * unit + gate of its units, in pair mode of both CTAs' units] 8 bf16.
 std::vector<uint16_t> pack_tc_rows(const float *m, int H, const RecurTcPlan &p)
@@ -476,6 +480,7 @@ void plan_wave(lstm_handle *h)
     if (h->D != 1 || h->L < 2 || h->L > kMaxWaveLayers || h->dtype != LSTM_BF16W_F32S || h->exec_mode != LSTM_DENSE || h->Hh) return;
     const char *env = getenv("LSTM_B200_WAVE");
     if (env && strcmp(env, "0") == 0) return;
+    h->wave_all = env && strcmp(env, "1") == 0;
     const int H = h->H;
     const int n = std::max(1, std::min(h->sm_count / h->L, H));
     const int upc = (H + n - 1) / n;
@@ -626,12 +631,12 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                              recur_csr_reg_fuse_smem_bytes(nw, kspan, mt, h->upc) <= (size_t)h->smem_optin - 64;
         }
     }
-    // Batched tensor-core recurrence (handles made for more than four sequences), with the current split of the SMs: as
+    // Batched tensor-core recurrence (handles made for several sequences), with the current split of the SMs: as
     // clusters of two where the device can co-schedule them, else every CTA alone.  bf16 CSR handles use it too, with the
     // zeros multiplied.
     auto plan_tcb = [&](int ncta, int dirs_side_by_side) -> bool {
         const char *env = getenv("LSTM_B200_RECUR");
-        if (!bf16 || (csr && !h->csr_dense_proj) || max_B <= 4 || (env && (strcmp(env, "mma") == 0 || strcmp(env, "simt") == 0))) return false;
+        if (!bf16 || (csr && !h->csr_dense_proj) || max_B < tc_min_rows(h) || (env && (strcmp(env, "mma") == 0 || strcmp(env, "simt") == 0))) return false;
         const size_t smem = (size_t)h->smem_optin - kTcStaticSmem;
         if (recur_tc_prepare((int)smem) != cudaSuccess) { cudaGetLastError(); return false; }
         if (!(env && strcmp(env, "tc1") == 0) && recur_tc_plan(H, ncta, max_B, 1, smem, &h->tcb) &&
@@ -886,7 +891,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     if (rc == LSTM_OK && dtype == LSTM_F32 && !csr && h->upc <= 2 && H <= kF32MaxUnits)
         rc = dev_alloc(h, &h->f32_xch, (size_t)2 * D * 2 * H * 32 * sizeof(unsigned), true, st, "exchange words");
     if (rc == LSTM_OK && h->use_tcb) {
-        rc = dev_alloc(h, &h->tcb_xch, (size_t)2 * D * 2 * round_up(H, 16) * h->tcb.rows * sizeof(unsigned), true, st, "exchange words");
+        rc = dev_alloc(h, &h->tcb_xch, 2 * (recur_tc_xch_words(H, h->tcb.rows, D) + kTcXchSlack) * sizeof(unsigned), true, st, "exchange words");
     }
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->status_dev, sizeof(int), true, st, "status word");
     if (rc == LSTM_OK && h->use_wave) {
@@ -908,8 +913,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         rc = fail(h, LSTM_ERR_CUDA, "workspace set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
     if (rc) return bail(rc);
     if (h->use_mma && h->fuse_ok && !h->Hh) {
-        const char *wenv = getenv("LSTM_B200_WAVE");
-        bool fits = !(h->use_wave && wenv && strcmp(wenv, "1") == 0);
+        bool fits = !(h->use_wave && h->wave_all);
         for (const Layer &ly : h->layers)
             fits = fits && ly.xfrag[0] && lstm_step_smem_bytes(h->mma_mt, kStepMaxRows, h->mma_nw / 2 * ly.nkw_x, h->mma_nw * (h->mma_nkr + h->mma_nks)) <= (size_t)h->smem_optin;
         h->step_ok = fits && lstm_step_prepare(h->mma_mt, h->smem_optin) == cudaSuccess;
@@ -1368,7 +1372,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         return LSTM_OK;
     }
 
-    if (h->use_wave && B <= 4 && !h->probe) {          // (the probe builds exist for the per-layer kernels)
+    if (h->use_wave && B <= (h->use_tcb && !h->wave_all ? 1 : 4) && !h->probe) {          // (the probe builds exist for the per-layer kernels)
         // all layers in one launch: layer 0's projection for all timesteps, then the wavefront kernel
         int nsplit = 1;
         { const int prc = run_projection(h, 0, x, x, M, D * 4 * H, &nsplit, st); if (prc != LSTM_OK) return prc; }
@@ -1471,7 +1475,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             continue;
         }
-        if (h->use_tcb && B > 4) {
+        if (h->use_tcb && B >= tc_min_rows(h)) {
             // passes of at most tcb.rows batch rows, as equal as possible
             const int passes = (B + h->tcb.rows - 1) / h->tcb.rows, dirs = h->seq_dirs ? 1 : D;
             for (int p = 0; p < passes; ++p) {
@@ -1493,12 +1497,12 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                 m.y = l == L - 1 ? y : m.xb_next ? nullptr : h->ybuf[l & 1];
                 m.xb_ld = h->ldn;
                 m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
-                m.xch = h->tcb_xch; m.set = h->tcb_set; m.xch_rows = h->tcb.rows; m.clear_rows = h->tcb_dirty;
+                m.xch = h->tcb_xch; m.set = h->tcb_set; m.set_words = recur_tc_xch_words(H, h->tcb.rows, D) + kTcXchSlack; m.clear_words = h->tcb_dirty;
                 m.status = h->status_dev;
                 if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 e = launch_recur_tc(m, st);
                 ++h->last_launches;
-                if (e == cudaSuccess) { h->tcb_set ^= 1; h->tcb_dirty = m.B; }
+                if (e == cudaSuccess) { h->tcb_set ^= 1; h->tcb_dirty = (unsigned)recur_tc_xch_words(H, m.B, dirs); }
                 if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             }
@@ -1796,7 +1800,7 @@ int lstm_info(const lstm_handle *h, int64_t *out, int n)
     }
     const Layer &l0 = h->layers[0];
     const int launches = h->last_launches > 0 ? h->last_launches : h->L * 2 + (h->use_tc ? 1 : 0);
-    const int tcb_at_max = h->use_tcb && h->max_B > 4 ? (h->tcb.pair ? 2 : 1) : 0;
+    const int tcb_at_max = h->use_tcb ? (h->tcb.pair ? 2 : 1) : 0;
     if (h->use_csr_reg) shp.smem = recur_csr_reg_smem_bytes(h->csr_nw, h->csr_kspan, h->csr_mt, h->upc, h->max_B);
     const int64_t vals[19] = {h->sm_count, h->ncta_dir, h->use_mma ? h->mma_nw * 32 : h->use_csr_reg ? h->csr_nw * 32 : h->threads, (int64_t)shp.smem,
                               rows_res, rows_str, (l0.plan_M >= 0) ? l0.plan.nsplit : 1, h->use_tc ? 1 : 0, launches,

@@ -257,12 +257,15 @@ struct RecurTcArgs {
     __nv_bfloat16 *xb_next;
     long long xb_plane;
     int xb_ld;
-    unsigned *xch;              // exchange words [2 sets][D][2 slots][16 columns][8 rows of xch_rows] blocks of 128
-    int set;                    // the set this launch uses; it clears the other one for the next launch
-    int xch_rows, clear_rows;   // rows allocated; rows the previous launch may have written
+    unsigned *xch;              // exchange words, 2 sets of [directions][2 slots][16 columns][8 batch rows] blocks of 128
+    size_t set_words;           // words from set to set
+    int set;                    // the set this launch uses; it clears the other one for the next launch ...
+    unsigned clear_words;       // ... as far as the previous launch may have written it
     int *status;
 };
 size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair);
+size_t recur_tc_xch_words(int H, int rows, int dirs);    // exchange words of one launch with `rows` batch rows
+constexpr size_t kTcXchSlack = 5 * 12 * 8 * 128;           // words a polling warp may read beyond them
 bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, size_t max_smem, RecurTcPlan *p);
 bool recur_tc_pair_supported(int grid, int rows, size_t smem);
 cudaError_t recur_tc_prepare(int max_smem);

@@ -32,8 +32,8 @@
 //     offset from a pointer that advances by one step.
 //
 // Per step (launch time / T, one layer), against the previous kernel (weights in shared memory as the A operand, h planes by
-// tensor copies behind one stamp per CTA, three "lane == 0" issuing threads): H = 1500, 20 rows 5.8 -> 4.5 us; two directions of
-// 800, 16 rows 4.7 -> 2.9 us; 50 rows in a pass 8.0 us (batches above 64 ran as passes of four rows before).
+// tensor copies behind one stamp per CTA, three "lane == 0" issuing threads): H = 1500, 20 rows 5.8 -> 3.6 us; two directions of
+// 800, 16 rows 4.7 -> 2.55 us; 50 rows in a pass 6.1 us (batches above 64 ran as passes of four rows before).
 //
 // Pair mode needs K for both halves and clusters of two; otherwise (narrow layers, or LSTM_B200_RECUR=tc1) a CTA works
 // alone on its own rows and all of K.  Every wait on another CTA is bounded; on expiry the CTA records a timeout status,
@@ -51,6 +51,10 @@ constexpr int kWarps = 16, kThreads = kWarps * 32;     // 128 registers a thread
 constexpr int kPollers = 12;                    // warps that fetch the operand (a multiple of 4 keeps their addresses linear)
 constexpr int kIssuer = 12;                     // first of the warps that issue the products; all warps finish
 constexpr int kMaxGroups = 5;                   // operand groups of 16 * kPollers columns
+// Clock ticks from the CTA's own barrier to its first poll: nothing can have arrived earlier, and loads that come too early
+// delay the words they wait for.  Measured us per step at 0 / 600 / 1000 ticks: H = 1500, 8 rows 2.40 / 2.30 / 2.47; two
+// directions of 800, 8 rows 1.97 / 1.97 / 2.11.
+constexpr unsigned kPollDelay = 600;
 constexpr int kGroupBar = 2;                    // named barrier of group 0: polling warps arrive, an issuing warp waits
 
 // batch rows a worker thread finishes per accumulator row
@@ -178,24 +182,16 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     volatile int *abort_v = &abort_s;
 
     // Exchange words: this launch's set starts with every phase bit at 0, the first words carry 1; the other set, which
-    // the next launch will use, is cleared here, every CTA its own words.
+    // the next launch will use, is cleared here as far as the launch before wrote it.
     // Block (16 columns, 8 batch rows) = 512 contiguous bytes, [column / 4][row][4 words]: a warp's load of a block is four
     // full lines, each by eight consecutive lanes.
-    const int Hq = (H + 3) & ~3, nq = Hq >> 2, rgx = a.xch_rows >> 3;       // chunks of four units; row groups allocated
-    const unsigned slot_words = (unsigned)((H + 15) >> 4) * rgx * 128u;
-    const size_t set_words = (size_t)2 * D * slot_words;
-    auto chunk_word = [&](int q, int b) -> unsigned { return (((unsigned)(q >> 2) * rgx + (b >> 3)) * 32u + (q & 3) * 8u + (b & 7)) * 4u; };
+    const int Hq = (H + 3) & ~3, nq = Hq >> 2;                              // chunks of four units
+    const unsigned slot_words = (unsigned)((H + 15) >> 4) * (RG * 128u);
+    auto chunk_word = [&](int q, int b) -> unsigned { return ((unsigned)(q >> 2) * RG + (b >> 3)) * 128u + (q & 3) * 32u + (b & 7) * 4u; };
     // (buffers by place in the launch, not by direction: launches that run the directions in turn share them)
-    const size_t xch_off = (size_t)(d - a.dir0) * 2 * slot_words;
-    unsigned *xch_d = a.xch + (size_t)a.set * set_words + xch_off;
-    {
-        unsigned *other = a.xch + (size_t)(a.set ^ 1) * set_words + xch_off;
-        const int cq = cta * (upc >> 2), qn = max(0, min(upc >> 2, nq - cq));
-        for (int i = tid; i < 2 * qn * a.clear_rows; i += kThreads) {
-            const int sl = i / (qn * a.clear_rows), r = i - sl * qn * a.clear_rows, q = r / a.clear_rows, b = r - q * a.clear_rows;
-            *reinterpret_cast<uint4 *>(other + (size_t)sl * slot_words + chunk_word(cq + q, b)) = make_uint4(0, 0, 0, 0);
-        }
-    }
+    unsigned *xch_d = a.xch + (size_t)a.set * a.set_words + (size_t)(d - a.dir0) * 2 * slot_words;
+    for (unsigned i = blockIdx.x * kThreads + tid; i < a.clear_words / 4u; i += gridDim.x * kThreads)
+        reinterpret_cast<uint4 *>(a.xch + (size_t)(a.set ^ 1) * a.set_words)[i] = make_uint4(0, 0, 0, 0);
     // weights into tensor memory: warp w writes lane quadrant w % 4, every fourth 8-column piece
     {
         const int row = (warp & 3) * 32 + lane, pieces = a.KH >> 3;
@@ -224,14 +220,15 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     // which the swizzle spreads over all banks.
     const int qq = lane >> 3, rr = lane & 7;
     const int q0 = (k_lo >> 2) + warp * 4 + qq;
-    const unsigned *src0 = xch_d + ((size_t)((k_lo >> 4) + warp) * rgx * 32 + lane) * 4;
-    const unsigned src_group = 128u * kPollers * (unsigned)rgx;             // words from group to group
+    const unsigned *src_even = xch_d + (size_t)((k_lo >> 4) + warp) * (RG * 128) + lane * 4, *src_odd = src_even + slot_words;
+    constexpr int kSrcGroup = kPollers * RG * 128;                          // words from group to group
     unsigned char *dst0 = op + (warp >> 2) * (N * 128) + rr * 128 + ((((warp & 3) * 32) + qq * 8) ^ (rr << 4));
     constexpr int kDstGroup = kPollers / 4 * N * 128;
-    int n_lane = 0;                                                         // groups this lane has a chunk in
-    for (int i = 0; i < ngroups; ++i)
-        if (warp < kPollers && i * kPollers + warp < nk16 && q0 + i * 4 * kPollers < nq) n_lane = i + 1;
-    const unsigned rg_mask = (1u << max(0, min(RG, (B - rr + 7) >> 3))) - 1u;
+    // groups this warp has a piece of, groups this lane has a chunk in, and whether its row of the last row group exists:
+    // what does not exist is read as the zeros the buffer holds there, and not waited for
+    const int n_warp = warp < kPollers ? (nk16 - warp + kPollers - 1) / kPollers : 0;
+    const int n_lane = min(n_warp, (nq - q0 + 4 * kPollers - 1) / (4 * kPollers));
+    const bool last_row = B - 8 * (RG - 1) > rr;
     // finishing: TMEM lane quadrant, accumulator row, batch rows [sub * RS, + RS)
     const int row = (warp & 3) * 32 + lane, sub = warp >> 2, fq = lane & 3;
     const int side = pair && row >= RA ? 1 : 0, lr = row - side * RA;
@@ -289,25 +286,30 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
             xp += xadv;
         }
     };
+    // Projection terms of this thread's row, requested between the last poll and the wait for the products, which hides the
+    // trip to L2; the lines are requested from HBM two steps ahead.  Requested ahead of the polls, or a whole step ahead,
+    // they delayed them: 2.63 -> 3.08 us per step (two directions of 800, 16 rows).
     float g[RS];
     auto load_g = [&](int s) {
-        // projection terms of this thread's row; the lines of a later step are requested into L2
 #pragma unroll
         for (int i = 0; i < RS; ++i) g[i] = i < nrow ? ld_nc_early(gp + i * gstep) : 0.0f;
         if (a.nsplit > 1)
-            for (int sp = 1; sp < a.nsplit; ++sp)
+            for (int sp = 1; sp < a.nsplit; ++sp) {
+                float v[RS];
 #pragma unroll
-                for (int i = 0; i < RS; ++i)
-                    if (i < nrow) g[i] += ld_nc_early(gp + sp * a.g_split_stride + i * gstep);
+                for (int i = 0; i < RS; ++i) v[i] = i < nrow ? ld_nc_early(gp + sp * a.g_split_stride + i * gstep) : 0.0f;
+#pragma unroll
+                for (int i = 0; i < RS; ++i) g[i] += v[i];
+            }
         if (pre && s + 2 < T) asm volatile("prefetch.global.L2 [%0];" ::"l"(gpre));
         gp += gadv;
         gpre += gadv;
     };
+    unsigned t_pub = 0;
 
 #pragma unroll 1
     for (int s = 0; s < T; ++s) {
         if (s > 0) write_outputs();
-        load_g(s);
         // (an aborted CTA opens no further phase: the open one never completes, and a second arrival would exceed its count)
         if (pair && tid == 0 && !*abort_v) mbar_expect_tx(smem_u32(&partial_bar[s & 1]), (uint32_t)(RA * Bp * 4));
 
@@ -338,11 +340,11 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
                 }
             };
             const unsigned phase = word_phase(s - 1);
-            const unsigned *src = src0 + (size_t)((s - 1) & 1) * slot_words;
+            const unsigned *src = (s & 1) ? src_even : src_odd;
             if (s == 0 && a.h0) {
                 for (int i = 0; i < n_lane; ++i)
                     for (int rg = 0; rg < RG; ++rg)
-                        if (rg_mask & (1u << rg)) {
+                        if (rg < RG - 1 || last_row) {
                             const int k = 4 * (q0 + i * 4 * kPollers);
                             const float *hp = a.h0 + ((size_t)d * a.Bs + a.b0 + rg * 8 + rr) * H + k;
                             uint4 v = make_uint4(split_word(hp[0]), 0, 0, 0);
@@ -352,65 +354,63 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
                             store_piece(dst0 + i * kDstGroup + rg * 1024, v, 0xffffffffu);
                         }
             }
+            if (s > 0) while ((unsigned)clock() - t_pub < kPollDelay) { }
 #pragma unroll 1
-            for (int i0 = 0; i0 < ngroups; i0 += KI, src += KI * src_group) {
-                unsigned pending = 0;                       // bit i * RG + rg: chunk not here yet
+            for (int i0 = 0; i0 < ngroups; i0 += KI, src += KI * kSrcGroup) {
                 uint4 w[KI][RG];
-                if (s > 0 && !*abort_v) {
-#pragma unroll
-                    for (int i = 0; i < KI; ++i)
-                        if (i0 + i < n_lane) pending |= rg_mask << (i * RG);
-                }
-                auto request = [&]() {
-#pragma unroll
-                    for (int i = 0; i < KI; ++i)
-#pragma unroll
-                        for (int rg = 0; rg < RG; ++rg)
-                            if (pending & (1u << (i * RG + rg))) w[i][rg] = ld_relaxed_v4(src + i * src_group + rg * 128);
-                };
-                request();
                 unsigned char *dst = dst0 + i0 * kDstGroup;
-                const int last = min(KI, ngroups - i0);
-                int polls = 0, delivered = 0;
-                long long t_start = 0;
-                for (;;) {
+                if (s > 0) {
 #pragma unroll
                     for (int i = 0; i < KI; ++i)
+                        if (i0 + i < n_warp) {
 #pragma unroll
-                        for (int rg = 0; rg < RG; ++rg)
-                            if ((pending & (1u << (i * RG + rg))) && words_ready(w[i][rg], phase)) {
-                                store_piece(dst + i * kDstGroup + rg * 1024, w[i][rg], 0xbfffbfffu);
-                                pending &= ~(1u << (i * RG + rg));
+                            for (int rg = 0; rg < RG; ++rg) w[i][rg] = ld_relaxed_v4(src + i * kSrcGroup + rg * 128);
+                        }
+                }
+#pragma unroll
+                for (int i = 0; i < KI; ++i)
+                    if (i0 + i < ngroups) {
+                        if (s > 0 && i0 + i < n_warp) {
+                            auto missing = [&]() -> unsigned {          // row groups of this piece that are not here yet
+                                unsigned m = 0;
+#pragma unroll
+                                for (int rg = 0; rg < RG; ++rg)
+                                    if (!words_ready(w[i][rg], phase) && (rg < RG - 1 || last_row)) m |= 1u << rg;
+                                return i0 + i < n_lane ? m : 0u;
+                            };
+                            unsigned pending = missing();
+                            int polls = 0;
+                            long long t_start = 0;
+                            while (__any_sync(0xffffffffu, pending)) {
+#pragma unroll
+                                for (int rg = 0; rg < RG; ++rg)
+                                    if (pending & (1u << rg)) w[i][rg] = ld_relaxed_v4(src + i * kSrcGroup + rg * 128);
+                                pending = missing();
+                                if ((++polls & 15) == 0 || *abort_v) {
+                                    const long long now = clock64();
+                                    if (t_start == 0) t_start = now;
+                                    if (*abort_v) pending = 0;
+                                    else if (now - t_start > a.spin_limit || ld_volatile_s32(a.status) != kStatusOk) {
+                                        *abort_v = 1;
+                                        atomicExch(a.status, kStatusTimeout);
+                                        pending = 0;
+                                    }
+                                }
                             }
-                    const unsigned open = __reduce_or_sync(0xffffffffu, pending);
-                    // groups this warp has delivered
-                    int done = delivered;
-                    while (done < last && !(open & (((1u << RG) - 1u) << (done * RG)))) ++done;
-                    if (done > delivered) {
+#pragma unroll
+                            for (int rg = 0; rg < RG; ++rg) store_piece(dst + i * kDstGroup + rg * 1024, w[i][rg], 0xbfffbfffu);
+                        }
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                         __syncwarp();
-                        for (int gi = delivered; gi < done; ++gi) bar_arrive(kGroupBar + i0 + gi, (kPollers + 1) * 32);
-                        delivered = done;
+                        bar_arrive(kGroupBar + i0 + i, (kPollers + 1) * 32);
                     }
-                    if (!open) break;
-                    request();
-                    if ((++polls & 15) == 0) {
-                        const long long now = clock64();
-                        if (t_start == 0) t_start = now;
-                        if (*abort_v) pending = 0;
-                        else if (now - t_start > a.spin_limit || ld_volatile_s32(a.status) != kStatusOk) {
-                            *abort_v = 1;
-                            atomicExch(a.status, kStatusTimeout);
-                            pending = 0;
-                        }
-                    }
-                }
             }
         }
 
         // ---- accumulators, partner's partial sums, gates, state
         if (fin) {
+            load_g(s);
             mbar_wait(smem_u32(&accum_bar), (uint32_t)s & 1u, abort_v);
             __syncwarp();
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -470,6 +470,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
         // Nobody polls or overwrites the operand before the whole CTA has published: early polls of words that are being
         // written pull their lines to and fro between the two halves of the L2, and delay everyone.
         bar_sync(1, kThreads);
+        t_pub = (unsigned)clock();
     }
     write_outputs();
 #pragma unroll
@@ -530,6 +531,8 @@ size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair)
     const int rg = groups_of(rows);
     return 1024 + (size_t)((KH + 63) / 64) * (16 * rg) * 128 + (pair ? (size_t)2 * 4 * upc * 8 * rg * 4 : 0);
 }
+
+size_t recur_tc_xch_words(int H, int rows, int dirs) { return (size_t)dirs * 2 * ((H + 15) / 16) * groups_of(rows) * 128; }
 
 // Partition of H units over at most max_cta CTAs, and the most batch rows (<= rows_wanted) a pass can take; false when
 // the slice does not fit tensor memory.
