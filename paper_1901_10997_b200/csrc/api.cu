@@ -446,7 +446,7 @@ std::vector<uint32_t> pack_ht_gates(const float *w, const HlstmTilePlan &p)
 }
 
 // Fewest batch rows the batched tensor-core recurrence serves: from two on it beats the passes of up to four rows of the
-// register-resident kernel (2 x 1500, T = 35: two rows 288 us, @TC2@ us on the tensor cores) and of the layer-wavefront kernel.
+// register-resident kernel (2 x 1500, T = 35: two rows 288 us, 208 us on the tensor cores).
 int tc_min_rows(const lstm_handle *) { return 2; }
 
 // Rows of a [4H x H] recurrent matrix (row q*H + j) as the batched tensor-core kernel wants them: per CTA [8-column
@@ -1372,7 +1372,9 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         return LSTM_OK;
     }
 
-    if (h->use_wave && B <= (h->use_tcb && !h->wave_all ? 1 : 4) && !h->probe) {          // (the probe builds exist for the per-layer kernels)
+    // The layer-wavefront kernel serves one sequence, and two where the step is short enough for its product per row (2 x 517, T = 23,
+    // two rows: 108 us against 127 us batched; 2 x 800, T = 35: 179 against 183; three rows: 144 against 135)
+    if (h->use_wave && B <= (!h->use_tcb || h->wave_all ? 4 : H <= 800 ? 2 : 1) && !h->probe) {          // (the probe builds exist for the per-layer kernels)
         // all layers in one launch: layer 0's projection for all timesteps, then the wavefront kernel
         int nsplit = 1;
         { const int prc = run_projection(h, 0, x, x, M, D * 4 * H, &nsplit, st); if (prc != LSTM_OK) return prc; }

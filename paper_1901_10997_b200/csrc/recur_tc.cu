@@ -293,14 +293,24 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     auto load_g = [&](int s) {
 #pragma unroll
         for (int i = 0; i < RS; ++i) g[i] = i < nrow ? ld_nc_early(gp + i * gstep) : 0.0f;
-        if (a.nsplit > 1)
-            for (int sp = 1; sp < a.nsplit; ++sp) {
-                float v[RS];
+        if (a.nsplit > 1) {
+            // further planes of a projection split along K: all of them on their way together
+            const float *p1 = gp + a.g_split_stride, *p2 = a.nsplit > 2 ? p1 + a.g_split_stride : p1, *p3 = a.nsplit > 3 ? p2 + a.g_split_stride : p1;
+            const int n2 = a.nsplit > 2 ? nrow : 0, n3 = a.nsplit > 3 ? nrow : 0;
+            constexpr int C = RS < 8 ? RS : 8;
 #pragma unroll
-                for (int i = 0; i < RS; ++i) v[i] = i < nrow ? ld_nc_early(gp + sp * a.g_split_stride + i * gstep) : 0.0f;
+            for (int i0 = 0; i0 < RS; i0 += C) {
+                float v[C], u[C], w[C];
 #pragma unroll
-                for (int i = 0; i < RS; ++i) g[i] += v[i];
+                for (int i = 0; i < C; ++i) {
+                    v[i] = i0 + i < nrow ? ld_nc_early(p1 + (i0 + i) * gstep) : 0.0f;
+                    u[i] = i0 + i < n2 ? ld_nc_early(p2 + (i0 + i) * gstep) : 0.0f;
+                    w[i] = i0 + i < n3 ? ld_nc_early(p3 + (i0 + i) * gstep) : 0.0f;
+                }
+#pragma unroll
+                for (int i = 0; i < C; ++i) g[i0 + i] += (v[i] + u[i]) + w[i];
             }
+        }
         if (pre && s + 2 < T) asm volatile("prefetch.global.L2 [%0];" ::"l"(gpre));
         gp += gadv;
         gpre += gadv;
