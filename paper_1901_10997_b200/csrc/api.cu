@@ -13,6 +13,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <thread>
 #include <vector>
 
 using namespace lstm;
@@ -373,14 +374,27 @@ int max_b_fits(const lstm_handle *h)
     return (size_t)2 * h->Hs * 4 + c_bytes + rp <= budget;
 }
 
+// fn(0) .. fn(n - 1) on the host's cores: packing is most of what creating a handle costs
+template <class Fn> void parallel_for(int n, Fn fn)
+{
+    const int nt = std::max(1, std::min({n, (int)std::thread::hardware_concurrency(), 8}));
+    std::vector<std::thread> pool;
+    auto work = [&](int t) { for (int i = t; i < n; i += nt) fn(i); };
+    for (int t = 1; t < nt; ++t) {
+        try { pool.emplace_back(work, t); } catch (...) { work(t); }
+    }
+    work(0);
+    for (auto &t : pool) t.join();
+}
+
 // Operand-A fragments of a [4U x K] matrix whose row q*U + u is gate q of unit u: per CTA (units split
 // evenly over ncta CTAs) [warp][column tile][row tile][lane] x 4 words, local row = 4 * unit + gate,
 // zero beyond the CTA's units and beyond column K.
 std::vector<uint32_t> pack_fragments(const float *m, int U, int K, int ncta, int NW, int nkw, int MT, bool adjacent = false)
 {
     std::vector<uint32_t> f((size_t)ncta * NW * nkw * MT * 32 * 4, 0u);
-    size_t o = 0;
-    for (int c = 0; c < ncta; ++c) {
+    parallel_for(ncta, [&](int c) {
+        size_t o = (size_t)c * NW * nkw * MT * 128;
         int u0, nu; unit_range_host(U, ncta, c, u0, nu);
         auto wv = [&](int r, int k) -> uint32_t {
             if (r >= 4 * nu || k >= K) return 0u;
@@ -400,7 +414,7 @@ std::vector<uint32_t> pack_fragments(const float *m, int U, int K, int ncta, int
                         f[o++] = wv(r0, kb) | (wv(r0, kb + 1) << 16);
                         f[o++] = wv(r1, kb) | (wv(r1, kb + 1) << 16);
                     }
-    }
+    });
     return f;
 }
 
@@ -422,7 +436,7 @@ std::vector<uint32_t> pack_ht_hidden(const float *uh, const HlstmTilePlan &p)
 {
     const int mt = (p.Hh + 15) / 16;
     std::vector<uint32_t> f((size_t)p.ncta * 16 * p.kt * p.n1 * 128, 0u);
-    for (int c = 0; c < p.ncta; ++c)
+    parallel_for(p.ncta, [&](int c) {
         for (int wp = 0; wp < 16; ++wp)
             for (int i = 0; i < p.kt; ++i)
                 for (int n = 0; n < p.n1; ++n) {
@@ -430,18 +444,20 @@ std::vector<uint32_t> pack_ht_hidden(const float *uh, const HlstmTilePlan &p)
                     if (tile < 4 * mt && k0 < p.H)
                         pack_tile(uh, p.H, q * p.Hh + (tile - q * mt) * 16, (q + 1) * p.Hh, k0, f.data() + (((size_t)(c * 16 + wp) * p.kt + i) * p.n1 + n) * 128);
                 }
+    });
     return f;
 }
 std::vector<uint32_t> pack_ht_gates(const float *w, const HlstmTilePlan &p)
 {
     const int kt2 = ((p.Hh + 15) / 16 + 3) / 4;
     std::vector<uint32_t> f((size_t)p.ncta * 16 * kt2 * 128, 0u);
-    for (int c = 0; c * 16 < p.H; ++c)
+    parallel_for((p.H + 15) / 16, [&](int c) {
         for (int wp = 0; wp < 16; ++wp)
             for (int i = 0; i < kt2; ++i) {
                 const int q = wp >> 2, k0 = ((wp & 3) * kt2 + i) * 16;
                 if (k0 < p.Hh) pack_tile(w, p.Hh, q * p.H + c * 16, (q + 1) * p.H, k0, f.data() + ((size_t)(c * 16 + wp) * kt2 + i) * 128);
             }
+    });
     return f;
 }
 
@@ -455,7 +471,7 @@ std::vector<uint16_t> pack_tc_rows(const float *m, int H, const RecurTcPlan &p)
 {
     const int units = p.pair ? 2 * p.upc : p.upc, rows = 4 * units, pieces = p.KH / 8;
     std::vector<uint16_t> out((size_t)p.ncta * pieces * rows * 8, 0);
-    for (int c = 0; c < p.ncta; ++c) {
+    parallel_for(p.ncta, [&](int c) {
         const int k0 = p.pair ? (c & 1) * p.KH : 0, k1 = std::min(H, k0 + p.KH), u0 = (p.pair ? c / 2 : c) * units;
         uint16_t *dst = out.data() + (size_t)c * pieces * rows * 8;
         const int nu = std::max(0, std::min(units, H - u0));
@@ -467,7 +483,7 @@ std::vector<uint16_t> pack_tc_rows(const float *m, int H, const RecurTcPlan &p)
                 for (int e = 0; e < n; ++e) d8[r * 8 + e] = f32_to_bf16_rne(src[e]);
             }
         }
-    }
+    });
     return out;
 }
 
@@ -704,13 +720,14 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                     if (rc == LSTM_OK) cudaStreamSynchronize(st);
                     if (rc) break;
                 }
-                for (int q = 0; q < 4; ++q)
+                parallel_for(4, [&](int q) {
                     for (int j = 0; j < H; ++j) {
                         const float *srow = m.data() + (size_t)(q * H + j) * ly.in_l;
                         const size_t drow = ((size_t)d * 4 * H + (size_t)j * 4 + q) * ly.ldk;
                         if (bf16) for (int k = 0; k < ly.in_l; ++k) wx16[drow + k] = f32_to_bf16_rne(srow[k]);
                         else memcpy(&wx32[drow], srow, sizeof(float) * ly.in_l);
                     }
+                });
                 snprintf(name, sizeof name, "wh[layer %d, dir %d]", l, d);
                 rc = matrix_to_dense(h, 4 * H, H, src.wh, src.mask_h, src.wh_rowptr, src.wh_col, src.wh_val, m, name);
                 if (rc) break;
