@@ -33,6 +33,9 @@ struct Layer {
     int *wh_ptr[2] = {nullptr, nullptr};   // CSR recurrence: padded entry offsets [4H+1]
     void *wh_ent[2] = {nullptr, nullptr};
     uint4 *wfrag[2] = {nullptr, nullptr};  // register-resident kernel: operand-A fragments
+    uint4 *ofrag[2] = {nullptr, nullptr};  // one-sequence kernel: Wh ...
+    uint4 *oxfrag[2] = {nullptr, nullptr}; //   ... and Wx (projection fused into the kernel's prologue)
+    int nkw_ox = 0;
     uint4 *xfrag[2] = {nullptr, nullptr};  //   and Wx in the same layout (projection fused into the kernel's prologue)
     int nkw_x = 0;
     uint4 *wtc[2] = {nullptr, nullptr};    // batched tensor-core kernel: [cta][8-column piece][row 4 * unit + gate]
@@ -57,6 +60,10 @@ struct lstm_handle {
     // register-resident recurrent kernel (bf16 dense): row tiles, column tiles per warp in registers and
     // in shared memory, warps per CTA
     bool use_mma = false;
+    // one sequence: its own partition (whole groups of four units per CTA), fragments and exchange words (two sets)
+    bool use_one = false, one_fuse = false;
+    RecurOnePlan one = {0, 0, 0, 0};
+    unsigned *one_xch = nullptr; int one_set = 0;
     bool step_ok = false;              // single timesteps run on the streaming kernel (lstm_step.cu)
     bool fuse_ok = false;              // short single sequences: projection fused into the register-resident kernel's prologue
     // register-resident sparse kernel (bf16, CSR execution): warps, columns per warp, row tiles, entry slots per lane
@@ -388,14 +395,15 @@ template <class Fn> void parallel_for(int n, Fn fn)
 }
 
 // Operand-A fragments of a [4U x K] matrix whose row q*U + u is gate q of unit u: per CTA (units split
-// evenly over ncta CTAs) [warp][column tile][row tile][lane] x 4 words, local row = 4 * unit + gate,
+// evenly over ncta CTAs, or upc units each) [warp][column tile][row tile][lane] x 4 words, local row = 4 * unit + gate,
 // zero beyond the CTA's units and beyond column K.
-std::vector<uint32_t> pack_fragments(const float *m, int U, int K, int ncta, int NW, int nkw, int MT, bool adjacent = false)
+std::vector<uint32_t> pack_fragments(const float *m, int U, int K, int ncta, int NW, int nkw, int MT, bool adjacent = false, int upc = 0)
 {
     std::vector<uint32_t> f((size_t)ncta * NW * nkw * MT * 32 * 4, 0u);
     parallel_for(ncta, [&](int c) {
         size_t o = (size_t)c * NW * nkw * MT * 128;
         int u0, nu; unit_range_host(U, ncta, c, u0, nu);
+        if (upc) { u0 = c * upc; nu = std::min(upc, U - u0); }
         auto wv = [&](int r, int k) -> uint32_t {
             if (r >= 4 * nu || k >= K) return 0u;
             return f32_to_bf16_rne(m[(size_t)((r & 3) * U + u0 + (r >> 2)) * K + k]);
@@ -519,11 +527,11 @@ void free_all(lstm_handle *h)
 {
     for (auto &ly : h->layers) {
         cudaFree(ly.wx); cudaFree(ly.bias); cudaFree(ly.wx_rowptr); cudaFree(ly.wx_ent);
-        for (int d = 0; d < 2; ++d) { cudaFree(ly.wh[d]); cudaFree(ly.wh_ptr[d]); cudaFree(ly.wh_ent[d]); cudaFree(ly.wfrag[d]); cudaFree(ly.xfrag[d]); cudaFree(ly.frag2[d]); cudaFree(ly.csr_reg_ent[d]); cudaFree(ly.csr_reg_rows[d]); }
+        for (int d = 0; d < 2; ++d) { cudaFree(ly.wh[d]); cudaFree(ly.wh_ptr[d]); cudaFree(ly.wh_ent[d]); cudaFree(ly.wfrag[d]); cudaFree(ly.ofrag[d]); cudaFree(ly.oxfrag[d]); cudaFree(ly.xfrag[d]); cudaFree(ly.frag2[d]); cudaFree(ly.csr_reg_ent[d]); cudaFree(ly.csr_reg_rows[d]); }
         cudaFree(ly.bias_out); cudaFree(ly.wtc[0]); cudaFree(ly.wtc[1]);
     }
     cudaFree(h->G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
-    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); cudaFree(h->tcb_xch); cudaFree(h->ht_hx); cudaFree(h->f32_xch); cudaFree(h->ht_rx); cudaFree(h->status_dev);
+    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); cudaFree(h->tcb_xch); cudaFree(h->ht_hx); cudaFree(h->f32_xch); cudaFree(h->one_xch); cudaFree(h->ht_rx); cudaFree(h->status_dev);
     for (int l = 0; l < kMaxWaveLayers; ++l) cudaFree(h->wave_frag[l]);
     cudaFree(h->wave_xch);
     cudaFree(h->cmap); cudaFree(h->rem_idx); cudaFree(h->rem_bias);
@@ -672,6 +680,11 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         if (h->use_mma) { h->seq_dirs = true; h->use_tcb = plan_tcb(h->ncta_dir, 1); }
         else { h->ncta_dir = nc; h->upc = up; h->threads = th; }
     }
+    {
+        const char *fenv = getenv("LSTM_B200_FUSE"), *renv = getenv("LSTM_B200_RECUR");
+        h->use_one = h->use_mma && !(renv && strcmp(renv, "mma") == 0) && recur_one_plan(H, h->ncta_dir, (size_t)h->smem_optin - 64, &h->one);
+        h->one_fuse = h->use_one && !(fenv && strcmp(fenv, "0") == 0) && recur_one_fuse_smem_bytes(h->one.mt, h->one.nks) <= (size_t)h->smem_optin - 64;
+    }
     h->layers.resize(layers);
     if (const char *env = getenv("LSTM_B200_SPIN_LIMIT")) { long long v = atoll(env); if (v > 0) h->spin_limit = v; }
     h->spin_limit_default = h->spin_limit;
@@ -710,6 +723,13 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                 if (rc) break;
                 std::vector<float> wave_x;
                 if (h->use_wave && l > 0) wave_x = m;                 // the wavefront kernel folds Wx of the upper layers into the step
+                if (h->one_fuse) {
+                    ly.nkw_ox = ((ly.in_l + 15) / 16 + 7) / 8;
+                    const std::vector<uint32_t> fx = pack_fragments(m.data(), H, ly.in_l, h->one.ncta, 8, ly.nkw_ox, h->one.mt, true, 4 * h->one.mt);
+                    rc = upload(h, (uint32_t **)&ly.oxfrag[d], fx.data(), fx.size() * 4, st, "input weight fragments");
+                    if (rc == LSTM_OK) cudaStreamSynchronize(st);
+                    if (rc) break;
+                }
                 if (h->use_mma && bf16 && h->fuse_ok) {
                     // the same matrix as operand-A fragments: short single sequences compute their projection in the
                     // recurrent kernel's prologue
@@ -747,6 +767,12 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                     }
                     const std::vector<uint32_t> f = pack_fragments(src_m, H, Kw, h->wave_ncta, 16, h->wave_nkw[l], h->wave_mt);
                     rc = upload(h, (uint32_t **)&h->wave_frag[l], f.data(), f.size() * 4, st, "wavefront weight fragments");
+                    if (rc == LSTM_OK) cudaStreamSynchronize(st);
+                    if (rc) break;
+                }
+                if (h->use_one) {
+                    const std::vector<uint32_t> f = pack_fragments(m.data(), H, H, h->one.ncta, 16, h->one.nkr + h->one.nks, h->one.mt, true, 4 * h->one.mt);
+                    rc = upload(h, (uint32_t **)&ly.ofrag[d], f.data(), f.size() * 4, st, "recurrent weight fragments");
                     if (rc == LSTM_OK) cudaStreamSynchronize(st);
                     if (rc) break;
                 }
@@ -905,6 +931,11 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         for (int i = 0; i < 2 && rc == LSTM_OK; ++i) rc = dev_alloc(h, &h->ybuf[i], Mmax * D * H * 4, false, st, "layer activations");
     h->xch_words = (size_t)D * 2 * max_B * H;
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->xch, h->xch_words * 8, true, st, "exchange buffer");
+    if (rc == LSTM_OK && h->use_one) {
+        rc = dev_alloc(h, &h->one_xch, (size_t)2 * D * 2 * h->one.ncta * 32 * sizeof(unsigned), true, st, "exchange words");
+        if (rc == LSTM_OK && recur_one_prepare(h->one, h->smem_optin - 64) != cudaSuccess)
+            rc = fail(h, LSTM_ERR_CUDA, "one-sequence kernel set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
+    }
     if (rc == LSTM_OK && dtype == LSTM_F32 && !csr && h->upc <= 2 && H <= kF32MaxUnits)
         rc = dev_alloc(h, &h->f32_xch, (size_t)2 * D * 2 * H * 32 * sizeof(unsigned), true, st, "exchange words");
     if (rc == LSTM_OK && h->use_tcb) {
@@ -1425,7 +1456,8 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         int nsplit = 1;
         // ---- input staging + projection (a single short sequence on the register-resident kernel computes its
         // projection inside that kernel's prologue instead: two launches and one round trip of G fewer per layer)
-        const bool fuse = (h->fuse_ok || (h->csr_fuse_ok && h->use_csr_reg)) && !h->Hh && B == 1 && T <= kFuseMaxT && !h->probe &&
+        const bool one = h->use_one && B == 1 && !h->probe;
+        const bool fuse = one ? h->one_fuse && T <= kFuseMaxT : (h->fuse_ok || (h->csr_fuse_ok && h->use_csr_reg)) && !h->Hh && B == 1 && T <= kFuseMaxT && !h->probe &&
                           ly.xfrag[0] != nullptr;
         if (!fuse) { const int prc = run_projection(h, l, l == 0 ? x : nullptr, Xf, M, N, &nsplit, st); if (prc != LSTM_OK) return prc; }
 
@@ -1559,6 +1591,36 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             e = launch_recur_csr_reg(m, h->csr_slots, h->csr_nw, smem, st);
             ++h->last_launches;
+            if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+            if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
+            continue;
+        }
+        if (one) {
+            RecurOneArgs m;
+            memset(&m, 0, sizeof m);
+            const int dirs = h->seq_dirs ? 1 : D;
+            m.dir0 = h->seq_dirs ? pass : 0; m.ndirs = dirs;
+            m.H = H; m.T = T; m.D = D; m.ncta_dir = h->one.ncta; m.nsplit = nsplit; m.nkw_smem = h->one.nks;
+            m.spin_limit = h->spin_limit;
+            m.withhold_cta = h->withhold_cta < 0 ? -1 : h->withhold_cta % (h->one.ncta * dirs);
+            m.in_l = ly.in_l; m.nkw_x = ly.nkw_ox; m.X = Xf; m.bias = ly.bias;
+            m.gs_off = (int)recur_one_gs_offset(h->one.mt, h->one.nks);
+            for (int d = 0; d < D; ++d) { m.wfrag[d] = ly.ofrag[d]; m.xfrag[d] = ly.oxfrag[d]; }
+            m.G = h->G;
+            m.g_split_stride = (long long)M * N;
+            const size_t so = (size_t)l * D * H;
+            m.h0 = h0 ? h0 + so : nullptr; m.c0 = c0 ? c0 + so : nullptr;
+            m.hT = hT ? hT + so : nullptr; m.cT = cT ? cT + so : nullptr;
+            m.y = l == L - 1 ? y : h->ybuf[l & 1];
+            m.xb_next = (l < L - 1 && h->use_tc && !fuse) ? h->xbn[l & 1] : nullptr;     // a fused next layer reads the fp32 activations
+            m.xb_ld = h->ldn;
+            m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
+            m.xch = h->one_xch; m.set = h->one_set;
+            m.status = h->status_dev;
+            if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+            e = launch_recur_one(m, h->one, fuse, st);
+            ++h->last_launches;
+            if (e == cudaSuccess) h->one_set ^= 1;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             continue;

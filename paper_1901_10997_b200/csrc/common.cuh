@@ -127,6 +127,40 @@ cudaError_t recur_mma_prepare(int mt, int nkr, int nw, int max_smem);
 cudaError_t launch_recur_mma(const RecurMmaArgs &a, int mt, int nkr, int nw, size_t smem, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------
+// Register-resident recurrent kernel for one sequence (recur_one.cu): CTA c owns units [c * 4 mt, (c + 1) * 4 mt)
+// ---------------------------------------------------------------------------------------------------
+struct RecurOnePlan { int mt, nkr, nks, ncta; };     // 16-row tiles; column tiles per warp in registers, in shared memory; CTAs per direction
+struct RecurOneArgs {
+    int dir0, ndirs;            // as in RecurArgs
+    int H, T, D, ncta_dir, nsplit;
+    int nkw_smem;
+    long long spin_limit;
+    int withhold_cta;
+    int in_l, nkw_x, gs_off;    // projection in the prologue: input width, column tiles of Wx per range, byte offset of its rows of G
+    const float *X;
+    const uint4 *xfrag[2];      // [cta][8 ranges][nkw_x][mt][lane], the lane's columns adjacent
+    const float *bias;
+    const uint4 *wfrag[2];      // [cta][warp][column tile][row tile][lane], the lane's columns adjacent
+    const float *G;
+    long long g_split_stride;
+    const float *h0, *c0;
+    float *hT, *cT;
+    float *y;
+    __nv_bfloat16 *xb_next;
+    long long xb_plane;
+    int xb_ld;
+    unsigned *xch;              // exchange words [2 sets][D][2 slots][ncta_dir][32]
+    int set;                    // the set this launch uses; it clears the other one
+    int *status;
+};
+size_t recur_one_smem_bytes(int mt, int nks);
+size_t recur_one_gs_offset(int mt, int nks);
+size_t recur_one_fuse_smem_bytes(int mt, int nks);
+bool recur_one_plan(int H, int max_cta, size_t max_smem, RecurOnePlan *p);
+cudaError_t recur_one_prepare(const RecurOnePlan &p, int max_smem);
+cudaError_t launch_recur_one(const RecurOneArgs &a, const RecurOnePlan &p, bool fuse, cudaStream_t st);
+
+// ---------------------------------------------------------------------------------------------------
 // One timestep of one layer (T = 1, up to kStepMaxRows batch rows) over the register-resident kernel's fragments
 // ---------------------------------------------------------------------------------------------------
 constexpr int kStepMaxRows = 8;
