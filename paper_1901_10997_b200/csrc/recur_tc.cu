@@ -25,15 +25,17 @@
 //   * The K range is handed to the issuing warps in groups as they arrive (a named barrier each: an issuing thread's
 //     mbarrier wait queues behind its own instructions), so the products overlap the fetch.
 //   * Accumulator row = 4 x unit + gate = TMEM lane: a thread reads its row's hi and lo columns for a few batch
-//     rows, sends them to the partner (st.async, completes on the partner's mbarrier) or adds what the partner sent,
-//     applies its gate's function, and a 4 x 4 transpose inside the quad gives every thread all four gates of a (unit,
-//     batch row) of its own; c stays in registers.
+//     rows of the partner and sends them (st.async, completes on the partner's mbarrier), then its own batch rows, adds what
+//     the partner sent, applies its gate's function, and a 4 x 4 transpose inside the quad gives every thread all four gates
+//     of a (unit, batch row) of its own; c stays in registers.  The pair splits this work by batch rows, not by units: all
+//     lanes of a warp then have gates to compute and a thread half as many (us per step, by units -> by rows: H = 1500, 20
+//     rows 3.70 -> 3.28, 50 rows 6.10 -> 5.03; H = 600, 50 rows 4.42 -> 3.34; two directions of 800, 16 rows 2.67 -> 2.40).
 //   * A step is bound by the instructions on this chain (16 warps on four schedulers), so every address is a fixed
 //     offset from a pointer that advances by one step.
 //
 // Per step (launch time / T, one layer), against the previous kernel (weights in shared memory as the A operand, h planes by
-// tensor copies behind one stamp per CTA, three "lane == 0" issuing threads): H = 1500, 20 rows 5.8 -> 3.6 us; two directions of
-// 800, 16 rows 4.7 -> 2.55 us; 50 rows in a pass 6.1 us (batches above 64 ran as passes of four rows before).
+// tensor copies behind one stamp per CTA, three "lane == 0" issuing threads): H = 1500, 20 rows 5.8 -> 3.3 us; two directions of
+// 800, 16 rows 4.7 -> 2.4 us; 50 rows in a pass 5.0 us (batches above 64 ran as passes of four rows before).
 //
 // Pair mode needs K for both halves and clusters of two; otherwise (narrow layers, or LSTM_B200_RECUR=tc1) a CTA works
 // alone on its own rows and all of K.  Every wait on another CTA is bounded; on expiry the CTA records a timeout status,
@@ -57,8 +59,12 @@ constexpr int kMaxGroups = 5;                   // operand groups of 16 * kPolle
 constexpr unsigned kPollDelay = 600;
 constexpr int kGroupBar = 2;                    // named barrier of group 0: polling warps arrive, an issuing warp waits
 
-// batch rows a worker thread finishes per accumulator row
-__host__ __device__ constexpr int tc_rows_per_thread(int rg) { return rg <= 2 ? 4 : rg <= 4 ? 8 : 16; }
+// Batch rows the first CTA of a pair finishes, for the units of both; the second one takes the rest, so that every lane of a
+// warp has gates to compute and the row groups of a line of exchange words keep one writer.  A single row group cannot be
+// split like that: there each CTA finishes its own units.  A CTA alone finishes all 8 rg.
+__host__ __device__ constexpr int tc_rows_of_first(int rg, bool pair) { return pair ? (rg + 1) / 2 * 8 : 8 * rg; }
+// batch rows a thread finishes per accumulator row: four warps share the rows of a lane quadrant
+__host__ __device__ constexpr int tc_rows_per_thread(int rows) { return rows <= 16 ? 4 : rows <= 32 ? 8 : 16; }
 // operand groups a lane has in flight: 16-byte chunks of rg batch rows each, at most twelve (registers)
 __host__ __device__ constexpr int tc_groups_in_flight(int rg) { return 12 / rg < kMaxGroups ? 12 / rg : kMaxGroups; }
 
@@ -133,10 +139,11 @@ __device__ __forceinline__ void quad_transpose(float &v0, float &v1, float &v2, 
 }
 
 // RG: groups of eight batch rows of a pass
-template <int RG>
+template <int RG, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs a)
 {
-    constexpr int Bp = 8 * RG, N = 2 * Bp, RS = tc_rows_per_thread(RG), NSUB = (Bp + RS - 1) / RS;
+    constexpr int Bp = 8 * RG, N = 2 * Bp, HB = tc_rows_of_first(RG, PAIR), RS = tc_rows_per_thread(HB);
+    constexpr bool UNITS = PAIR && RG == 1;
     constexpr int KI = tc_groups_in_flight(RG), NACC = tc_accumulators(RG);
     constexpr uint32_t tmem = 0;                                            // all 512 columns are ours: they start at address 0
     constexpr uint32_t acc_col = 512u - tc_acc_columns(RG);                 // accumulators behind the weights
@@ -149,20 +156,19 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     const int H = a.H, B = a.B, T = a.T, D = a.D, upc = a.upc;
     const int d = a.dir0 + blockIdx.x / a.ncta_dir;
     const int cta = blockIdx.x % a.ncta_dir;
-    const int pair = a.pair;
-    const int rank = pair ? (int)cluster_ctarank() : 0;
-    const int RA = 4 * upc, RT = pair ? 2 * RA : RA;                        // accumulator rows of one CTA's units; of the tile
+    const int rank = PAIR ? (int)cluster_ctarank() : 0;
+    const int RT = PAIR ? 8 * upc : 4 * upc;                                // accumulator rows of the tile
     const int k_lo = rank * a.KH, k_n = min(a.KH, H - k_lo);                // this CTA's K range
     const int nk16 = (k_n + 15) >> 4;
     const int ngroups = (nk16 + kPollers - 1) / kPollers;                   // warp w fetches piece w of every group
     const int nissue = min(NACC, ngroups);                                  // issuing warps, each with an accumulator
 
-    // shared memory: operand tiles of 64 columns [N rows][128 bytes, swizzled], then the partner's partial sums [2][Bp][RA]
+    // shared memory: operand tiles of 64 columns [N rows][128 bytes, swizzled], then the partner's partial sums [2][HB][RT]
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     unsigned char *op = smem_raw + (base - smem_u32(smem_raw));
     const int tiles = (a.KH + 63) >> 6;
     float *zs2 = reinterpret_cast<float *>(op + (size_t)tiles * N * 128);
-    LSTM_CHECK_SMEM_END(reinterpret_cast<unsigned char *>(zs2 + (pair ? 2 * RA * Bp : 0)) - smem_raw, a.status);
+    LSTM_CHECK_SMEM_END(reinterpret_cast<unsigned char *>(zs2 + (PAIR ? 2 * RT * HB : 0)) - smem_raw, a.status);
 
     if (tid == 0) {
         abort_s = 0;
@@ -212,7 +218,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (pair) cluster_sync_all();               // the partner's barriers are initialised before anything reaches them
+    if (PAIR) cluster_sync_all();               // the partner's barriers are initialised before anything reaches them
 
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     const uint64_t bdesc0 = umma_desc_sw128(base);
@@ -229,20 +235,20 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     const int n_warp = warp < kPollers ? (nk16 - warp + kPollers - 1) / kPollers : 0;
     const int n_lane = min(n_warp, (nq - q0 + 4 * kPollers - 1) / (4 * kPollers));
     const bool last_row = B - 8 * (RG - 1) > rr;
-    // finishing: TMEM lane quadrant, accumulator row, batch rows [sub * RS, + RS)
+    // finishing: TMEM lane quadrant, accumulator row, batch rows [fb0, + RS); of the partner's batch rows [sb0, + RS)
     const int row = (warp & 3) * 32 + lane, sub = warp >> 2, fq = lane & 3;
-    const int side = pair && row >= RA ? 1 : 0, lr = row - side * RA;
-    const bool fin = sub < NSUB && (warp & 3) * 32 < RT;                    // this warp reads accumulators
-    const bool mine = row < RT && side == rank;
-    const int u = lr >> 2, j = cta * upc + u;                               // unit of this row, if it is ours
-    const bool any_mine = __any_sync(0xffffffffu, mine);
-    const bool own = mine && fin && j < Hq, real = own && j < H;
-    const int fb0 = sub * RS;
+    const bool mine = row < RT && (!UNITS || (row >= RT / 2) == (rank != 0)), theirs = row < RT && (!UNITS || !mine);
+    const int my_lo = UNITS ? 0 : rank * HB, my_n = UNITS ? Bp : rank ? Bp - HB : HB;
+    const int other_lo = UNITS ? 0 : HB - my_lo, other_n = UNITS ? Bp : PAIR ? Bp - my_n : 0;
+    const bool fin = sub * RS < my_n && __any_sync(0xffffffffu, mine), snd = sub * RS < other_n && __any_sync(0xffffffffu, theirs);
+    const int fb0 = my_lo + sub * RS, sb0 = other_lo + sub * RS;
+    const int j = (PAIR ? cta & ~1 : cta) * upc + (row >> 2);               // unit of this row
+    const bool own = fin && mine && j < Hq, real = own && j < H;
     const float act_k = (fq == 2 ? -2.0f : -1.0f) * 1.4426950408889634f, act_sc = fq == 2 ? 2.0f : 1.0f, act_of = fq == 2 ? -1.0f : 0.0f;
-    const uint32_t zs2_remote = pair ? map_to_cta(smem_u32(zs2), (uint32_t)(rank ^ 1)) + (uint32_t)(fb0 * RA + lr) * 4u : 0u;
-    const uint32_t partial_remote = pair ? map_to_cta(smem_u32(partial_bar), (uint32_t)(rank ^ 1)) : 0u;
-    const uint32_t abort_remote = pair ? map_to_cta(smem_u32(&abort_s), (uint32_t)(rank ^ 1)) : 0u;
-    const float *zs2_mine = zs2 + fb0 * RA + lr;
+    const uint32_t zs2_remote = PAIR ? map_to_cta(smem_u32(zs2), (uint32_t)(rank ^ 1)) + (uint32_t)(sub * RS * RT + row) * 4u : 0u;
+    const uint32_t partial_remote = PAIR ? map_to_cta(smem_u32(partial_bar), (uint32_t)(rank ^ 1)) : 0u;
+    const uint32_t abort_remote = PAIR ? map_to_cta(smem_u32(&abort_s), (uint32_t)(rank ^ 1)) : 0u;
+    const float *zs2_mine = zs2 + sub * RS * RT + row;
     const size_t state0 = ((size_t)d * a.Bs + a.b0) * H + j;                // element of (pass row 0, unit j) in the state arrays
     // projection terms, outputs: pointers that advance by one timestep per step
     const long long gstep = (long long)D * 4 * H, dir = d ? -1 : 1;
@@ -250,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     const float *gp = a.G + m0 * gstep + (long long)d * 4 * H + 4 * (long long)j + fq;
     const int nrow = real ? max(0, min(RS, B - fb0)) : 0;
     const float *gpre = a.G + (m0 + 2 * dir * a.Bs + lane) * gstep + (long long)d * 4 * H + 4 * (long long)(j - (lane >> 2));
-    const bool pre = lane < RS && fb0 + lane < B && fin && mine && j - (lane >> 2) < H;
+    const bool pre = lane < RS && fb0 + lane < B && fin && j - (lane >> 2) < H;
     float *yp = a.y ? a.y + (m0 + fq) * D * H + (long long)d * H + j : nullptr;
     __nv_bfloat16 *xp = a.xb_next ? a.xb_next + (m0 + fq) * a.xb_ld + (long long)d * H + j : nullptr;
     const long long gadv = dir * a.Bs * gstep, yadv = dir * a.Bs * D * H, xadv = dir * a.Bs * a.xb_ld;
@@ -321,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     for (int s = 0; s < T; ++s) {
         if (s > 0) write_outputs();
         // (an aborted CTA opens no further phase: the open one never completes, and a second arrival would exceed its count)
-        if (pair && tid == 0 && !*abort_v) mbar_expect_tx(smem_u32(&partial_bar[s & 1]), (uint32_t)(RA * Bp * 4));
+        if (PAIR && tid == 0 && !*abort_v) mbar_expect_tx(smem_u32(&partial_bar[s & 1]), (uint32_t)((UNITS ? RT / 2 : RT) * my_n * 4));
 
         if (warp >= kIssuer && warp < kIssuer + nissue) {
             // ---- products: issuing warp w takes every nissue-th group, one elected thread, an accumulator of its own
@@ -419,62 +425,65 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
         }
 
         // ---- accumulators, partner's partial sums, gates, state
-        if (fin) {
+        if (fin || snd) {
             load_g(s);
             mbar_wait(smem_u32(&accum_bar), (uint32_t)s & 1u, abort_v);
             __syncwarp();
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t ta = acc_col + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)fb0;
-            float z[RS], zl[RS];
-            tmem_ld<RS>(ta, z);
-            tmem_ld<RS>(ta + (uint32_t)Bp, zl);
-            if (NACC > 1 && nissue > 1) {
-                float y[RS], yl[RS];
-                tmem_ld<RS>(ta + (uint32_t)N, y);
-                tmem_ld<RS>(ta + (uint32_t)(N + Bp), yl);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            float z[RS];
+            auto read_sums = [&](int b0) {                       // this row's sums for batch rows b0 .. b0 + RS - 1
+                const uint32_t ta = acc_col + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)b0;
+                float zl[RS];
+                tmem_ld<RS>(ta, z);
+                tmem_ld<RS>(ta + (uint32_t)Bp, zl);
+                if (NACC > 1 && nissue > 1) {
+                    float y[RS], yl[RS];
+                    tmem_ld<RS>(ta + (uint32_t)N, y);
+                    tmem_ld<RS>(ta + (uint32_t)(N + Bp), yl);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                for (int i = 0; i < RS; ++i) z[i] = (z[i] + y[i]) + (zl[i] + yl[i]);
-            } else {
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    for (int i = 0; i < RS; ++i) z[i] = (z[i] + y[i]) + (zl[i] + yl[i]);
+                } else {
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                for (int i = 0; i < RS; ++i) z[i] += zl[i];
-            }
-            if (pair) {
+                    for (int i = 0; i < RS; ++i) z[i] += zl[i];
+                }
+            };
+            if (PAIR && snd) {
+                read_sums(sb0);
                 if (*abort_v) {
                     // gave up: nothing is sent any more, so the partner must not wait for it
                     asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(abort_remote), "r"(1) : "memory");
-                } else if (row < RT && !mine) {
-                    const uint32_t dst = zs2_remote + (uint32_t)((s & 1) * RA * Bp) * 4u, bar = partial_remote + (uint32_t)(s & 1) * 8u;
+                } else if (theirs) {
+                    const uint32_t dst = zs2_remote + (uint32_t)((s & 1) * RT * HB) * 4u, bar = partial_remote + (uint32_t)(s & 1) * 8u;
 #pragma unroll
-                    for (int i = 0; i < RS; ++i)
-                        if (RS * NSUB == Bp || fb0 + i < Bp) st_async(dst + (uint32_t)(i * RA) * 4u, z[i], bar);
+                    for (int i = 0; i < RS; ++i) st_async(dst + (uint32_t)(i * RT) * 4u, z[i], bar);
                 }
                 __syncwarp();
-                if (any_mine) {
+            }
+            if (fin) {
+                if (!UNITS || !snd) read_sums(fb0);
+                if (PAIR) {
                     mbar_wait(smem_u32(&partial_bar[s & 1]), (uint32_t)(s >> 1) & 1u, abort_v);
                     __syncwarp();
                     if (mine) {
-                        const float *zp = zs2_mine + (s & 1) * RA * Bp;
+                        const float *zp = zs2_mine + (s & 1) * RT * HB;
 #pragma unroll
-                        for (int i = 0; i < RS; ++i)
-                            if (RS * NSUB == Bp || fb0 + i < Bp) z[i] += zp[i * RA];
+                        for (int i = 0; i < RS; ++i) z[i] += zp[i * RT];
                     }
                 }
-            }
-            if (any_mine) {
 #pragma unroll
-            for (int i = 0; i < RS; ++i) z[i] = gate_fast(z[i] + g[i], act_k, act_sc, act_of);
-            unsigned *dst = out0 + (size_t)(s & 1) * slot_words;
-            const unsigned phase_out = word_phase(s);
+                for (int i = 0; i < RS; ++i) z[i] = gate_fast(z[i] + g[i], act_k, act_sc, act_of);
+                unsigned *dst = out0 + (size_t)(s & 1) * slot_words;
+                const unsigned phase_out = word_phase(s);
 #pragma unroll
-            for (int m = 0; m < RS / 4; ++m) {
-                quad_transpose(z[4 * m], z[4 * m + 1], z[4 * m + 2], z[4 * m + 3], fq);
-                c[m] = fmaf(z[4 * m + 1], c[m], z[4 * m] * z[4 * m + 2]);
-                hn[m] = z[4 * m + 3] * tanh_fast(c[m]);
-                // (fb0 is a multiple of four: of eight where a thread has more than one item)
-                if (m < npub) st_relaxed_u32(dst + (m & 1) * 16 + (m >> 1) * 128, pack_word(hn[m], phase_out));
-            }
+                for (int m = 0; m < RS / 4; ++m) {
+                    quad_transpose(z[4 * m], z[4 * m + 1], z[4 * m + 2], z[4 * m + 3], fq);
+                    c[m] = fmaf(z[4 * m + 1], c[m], z[4 * m] * z[4 * m + 2]);
+                    hn[m] = z[4 * m + 3] * tanh_fast(c[m]);
+                    // (fb0 is a multiple of four: of eight where a thread has more than one item)
+                    if (m < npub) st_relaxed_u32(dst + (m & 1) * 16 + (m >> 1) * 128, pack_word(hn[m], phase_out));
+                }
             }
         }
         // Nobody polls or overwrites the operand before the whole CTA has published: early polls of words that are being
@@ -501,24 +510,26 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base_s) : "memory");
     }
-    if (pair) cluster_sync_all();               // no CTA leaves while its partner may still write into its shared memory
+    if (PAIR) cluster_sync_all();               // no CTA leaves while its partner may still write into its shared memory
 }
 
 typedef void (*KernelFn)(const RecurTcArgs);
-KernelFn pick(int rg)
+template <bool PAIR>
+KernelFn pick_p(int rg)
 {
     switch (rg) {
-        case 1: return recur_tc_kernel<1>;
-        case 2: return recur_tc_kernel<2>;
-        case 3: return recur_tc_kernel<3>;
-        case 4: return recur_tc_kernel<4>;
-        case 5: return recur_tc_kernel<5>;
-        case 6: return recur_tc_kernel<6>;
-        case 7: return recur_tc_kernel<7>;
-        case 8: return recur_tc_kernel<8>;
+        case 1: return recur_tc_kernel<1, PAIR>;
+        case 2: return recur_tc_kernel<2, PAIR>;
+        case 3: return recur_tc_kernel<3, PAIR>;
+        case 4: return recur_tc_kernel<4, PAIR>;
+        case 5: return recur_tc_kernel<5, PAIR>;
+        case 6: return recur_tc_kernel<6, PAIR>;
+        case 7: return recur_tc_kernel<7, PAIR>;
+        case 8: return recur_tc_kernel<8, PAIR>;
         default: return nullptr;
     }
 }
+KernelFn pick(int rg, bool pair) { return pair ? pick_p<true>(rg) : pick_p<false>(rg); }
 int groups_of(int rows) { return (rows + 7) / 8; }
 
 cudaLaunchConfig_t config(cudaLaunchAttribute (&attr)[2], int grid, size_t smem, int pair, cudaStream_t st)
@@ -539,7 +550,7 @@ cudaLaunchConfig_t config(cudaLaunchAttribute (&attr)[2], int grid, size_t smem,
 size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair)
 {
     const int rg = groups_of(rows);
-    return 1024 + (size_t)((KH + 63) / 64) * (16 * rg) * 128 + (pair ? (size_t)2 * 4 * upc * 8 * rg * 4 : 0);
+    return 1024 + (size_t)((KH + 63) / 64) * (16 * rg) * 128 + (pair ? (size_t)2 * 8 * upc * tc_rows_of_first(rg, true) * 4 : 0);
 }
 
 size_t recur_tc_xch_words(int H, int rows, int dirs) { return (size_t)dirs * 2 * ((H + 15) / 16) * groups_of(rows) * 128; }
@@ -569,8 +580,10 @@ bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, size_t max_sme
 cudaError_t recur_tc_prepare(int max_smem)
 {
     for (int rg = 1; rg <= kTcMaxRows / 8; ++rg) {
-        const cudaError_t e = cudaFuncSetAttribute(pick(rg), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
-        if (e != cudaSuccess) return e;
+        for (int pair = 0; pair < 2; ++pair) {
+            const cudaError_t e = cudaFuncSetAttribute(pick(rg, pair != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+            if (e != cudaSuccess) return e;
+        }
     }
     return cudaSuccess;
 }
@@ -582,7 +595,7 @@ bool recur_tc_pair_supported(int grid, int rows, size_t smem)
     cudaLaunchConfig_t cfg = config(attr, grid, smem, 1, nullptr);
     cfg.attrs = attr + 1; cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)pick(groups_of(rows)), &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)pick(groups_of(rows), true), &cfg) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -591,7 +604,7 @@ bool recur_tc_pair_supported(int grid, int rows, size_t smem)
 
 cudaError_t launch_recur_tc(const RecurTcArgs &a, cudaStream_t st)
 {
-    KernelFn fn = pick(groups_of(a.B));
+    KernelFn fn = pick(groups_of(a.B), a.pair != 0);
     if (!fn) return cudaErrorInvalidValue;
     RecurTcArgs copy = a;
     void *params[] = {&copy};
