@@ -53,7 +53,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int w_tile = blockIdx.x, x_tile = blockIdx.y, split = blockIdx.z;
     const int kb0 = (int)((long long)split * a.kblocks / a.nsplit);
     const int kb1 = (int)((long long)(split + 1) * a.kblocks / a.nsplit);
@@ -98,30 +98,28 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---- MMA issuer
-            // instruction descriptor: fp32 accumulate, bf16 x bf16, both K-major, M = 128, N = 2 * n_tile: the
-            // hi and the lo activation tiles lie back to back in the stage and form ONE operand of 2 * n_tile
-            // rows (an instruction of this size costs the same whatever N, so one is half the price of two);
-            // accumulator columns [0, n_tile) hold the hi product, [n_tile, 2 n_tile) the lo product
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * a.n_tile) >> 3) << 17) |
-                                   ((uint32_t)(kBM >> 4) << 24);
-            bool ok = true;
-            int s = 0;
-            uint32_t ph = 0;
-            for (int i = 0; i < nkb && ok; ++i) {
-                ok = mbar_wait(smem_u32(&full_bar[s]), ph, abort_flag);
-                if (!ok) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t sa = tiles + (uint32_t)s * stage_bytes;
-                const uint64_t adesc = umma_desc_sw128(sa), bdesc = umma_desc_sw128(sa + a_bytes);
+        // ---- MMA issuer: the whole warp waits, one elected lane issues
+        // instruction descriptor: fp32 accumulate, bf16 x bf16, both K-major, M = 128, N = 2 * n_tile: the
+        // hi and the lo activation tiles lie back to back in the stage and form ONE operand of 2 * n_tile rows;
+        // accumulator columns [0, n_tile) hold the hi product, [n_tile, 2 n_tile) the lo product
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * a.n_tile) >> 3) << 17) |
+                               ((uint32_t)(kBM >> 4) << 24);
+        int s = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < nkb; ++i) {
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full_bar[s]), ph, abort_flag))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t sa = tiles + (uint32_t)s * stage_bytes;
+            const uint64_t adesc = umma_desc_sw128(sa), bdesc = umma_desc_sw128(sa + a_bytes);
+            if (elect_one()) {
 #pragma unroll
                 for (int k = 0; k < kBK / 16; ++k)
                     umma_bf16(tmem_base, adesc + 2 * k, bdesc + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
                 umma_commit(smem_u32(&empty_bar[s]));      // frees the stage once these MMAs have read it
-                if (++s == S) { s = 0; ph ^= 1u; }
+                if (i == nkb - 1) umma_commit(smem_u32(&accum_bar));     // accumulator complete
             }
-            if (ok) umma_commit(smem_u32(&accum_bar));     // accumulator complete
+            __syncwarp();
+            if (++s == S) { s = 0; ph ^= 1u; }
         }
     } else {
         // ---- epilogue: warp w may touch TMEM lanes 32*(w % 4) .. +31
@@ -155,6 +153,8 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     if (tid == 0 && abort_s) atomicExch(a.status, kStatusTimeout);
 }
 
+// (Issued by "lane == 0" the products of 6400 x 6400 x 1312 / 1600, five layers, took 1106 us, by an elected lane 1022; 3500 x
+// 6000 x 1500, two layers, 251 -> 234; what is left is the read-back between two tiles and the last wave.)
 // Tensor-bound shapes (several activation tiles): a persistent kernel, one CTA per SM, whose tile is 256 weight
 // rows x n_tile activation rows: two M = 128 accumulators share each staged activation tile, so a K block costs
 // 32 KB of weights + 2 x n_tile x 128 B of activations for twice the products of the kernel above (whose 128-row
@@ -179,7 +179,7 @@ proj_tc_big_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int S = a.stages, nkb = a.kblocks;
     const int ntiles = a.wtiles * a.xtiles;
     const uint32_t a_bytes = kBM * kBK * 2, b_bytes = (uint32_t)a.n_tile * kBK * 2;
@@ -229,36 +229,38 @@ proj_tc_big_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---- MMA issuer: accumulator h (weight rows h*128 .. +127 of the tile) at TMEM column h * 2 * n_tile;
-            // columns [0, n_tile) of an accumulator hold the hi product, [n_tile, 2 n_tile) the lo product
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * a.n_tile) >> 3) << 17) |
-                                   ((uint32_t)(kBM >> 4) << 24);
-            const uint32_t acc1 = tmem_base + (uint32_t)(2 * a.n_tile);
-            bool ok = true;
-            int s = 0;
-            uint32_t ph = 0, tph = 0;
-            for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, tph ^= 1u) {
-                // the read-back warps have left the accumulators of the previous tile
-                ok = mbar_wait(smem_u32(&drained_bar), tph ^ 1u, abort_flag);
+        // ---- MMA issuer (the whole warp waits, one elected lane issues): accumulator h (weight rows h*128 .. +127 of the
+        // tile) at TMEM column h * 2 * n_tile; columns [0, n_tile) of an accumulator hold the hi product, [n_tile,
+        // 2 n_tile) the lo product
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * a.n_tile) >> 3) << 17) |
+                               ((uint32_t)(kBM >> 4) << 24);
+        const uint32_t acc1 = tmem_base + (uint32_t)(2 * a.n_tile);
+        bool ok = true;
+        int s = 0;
+        uint32_t ph = 0, tph = 0;
+        for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, tph ^= 1u) {
+            // the read-back warps have left the accumulators of the previous tile
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&drained_bar), tph ^ 1u, abort_flag));
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int i = 0; i < nkb; ++i) {
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&full_bar[s]), ph, abort_flag));
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                for (int i = 0; i < nkb && ok; ++i) {
-                    ok = mbar_wait(smem_u32(&full_bar[s]), ph, abort_flag);
-                    if (!ok) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t sa = tiles + (uint32_t)s * stage_bytes;
-                    const uint64_t adesc0 = umma_desc_sw128(sa), adesc1 = umma_desc_sw128(sa + a_bytes);
-                    const uint64_t bdesc = umma_desc_sw128(sa + 2 * a_bytes);
+                const uint32_t sa = tiles + (uint32_t)s * stage_bytes;
+                const uint64_t adesc0 = umma_desc_sw128(sa), adesc1 = umma_desc_sw128(sa + a_bytes);
+                const uint64_t bdesc = umma_desc_sw128(sa + 2 * a_bytes);
+                if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < kBK / 16; ++k) {
                         umma_bf16(tmem_base, adesc0 + 2 * k, bdesc + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
                         umma_bf16(acc1, adesc1 + 2 * k, bdesc + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
                     }
                     umma_commit(smem_u32(&empty_bar[s]));
-                    if (++s == S) { s = 0; ph ^= 1u; }
+                    if (i == nkb - 1) umma_commit(smem_u32(&accum_bar));
                 }
-                if (ok) umma_commit(smem_u32(&accum_bar));
+                __syncwarp();
+                if (++s == S) { s = 0; ph ^= 1u; }
             }
         }
     } else {
