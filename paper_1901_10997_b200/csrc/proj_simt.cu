@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(128) proj_f64_kernel(const float *__restrict__
     constexpr int P = 36;                                      // doubles between K rows: a half warp's 4 x 4 operands hit all banks
     __shared__ double xs[2][16][P], ws[2][16][P];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 32, wm = (warp >> 1) * 16, wn = (warp & 1) * 16;
+    const int m0 = blockIdx.x * 32, n0 = blockIdx.y * 32, wm = (warp >> 1) * 16, wn = (warp & 1) * 16;
     const int r = tid >> 2, kk = (tid & 3) * 4;                // this thread loads 4 adjacent elements of row r of each tile
     const bool xok = m0 + r < M, wok = n0 + r < N;
     const bool vec = (K & 3) == 0 && (ldw & 3) == 0 && ((reinterpret_cast<size_t>(X) | reinterpret_cast<size_t>(W)) & 15) == 0;
@@ -284,7 +284,8 @@ cudaError_t launch_proj_simt(const float *X, const void *W, bool bf16, int ldw, 
     if (bf16)
         proj_simt_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(X, (const __nv_bfloat16 *)W, ldw, bias, G, M, N, K);
     else
-        proj_f64_kernel<<<dim3((N + 31) / 32, (M + 31) / 32), 128, 0, st>>>(X, (const float *)W, ldw, bias, G, M, N, K);
+        // rows in x, which may have 2^31 blocks; y may have 65535 (columns: at most 2 x 4 x 65535 / 32)
+        proj_f64_kernel<<<dim3((M + 31) / 32, (N + 31) / 32), 128, 0, st>>>(X, (const float *)W, ldw, bias, G, M, N, K);
     return cudaGetLastError();
 }
 

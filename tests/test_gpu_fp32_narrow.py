@@ -22,3 +22,20 @@ def test_fp32_narrow(oracle, s):
     assert_close(run_gpu(w, weights, x, h0, c0), ref, "fp32", "fp32 narrow")
     if not bidir:
         assert_close(run_gpu(w, weights, x, h0, c0, chunks=[1, T - 1]), ref, "fp32", "fp32 narrow, chunked")
+
+
+def test_fp32_projection_of_more_rows_than_a_grid_has_in_y():
+    """T x B = 2 100 000 rows, more than 65535 tiles of 32; every row against the product in float64."""
+    import torch
+    import paper_1901_10997_b200 as pkg
+    T, K, H = 2_100_000, 3, 9
+    g = torch.Generator(device="cuda").manual_seed(5)
+    wx = torch.rand((4 * H, K), generator=g, device="cuda") - 0.5
+    m = pkg.LSTM([{"wx": wx, "wh": torch.zeros((4 * H, H), device="cuda")}], layers=1, in_dim=K, hidden=H, dtype="fp32", max_T=T, max_B=1)
+    try:
+        x = torch.randn((T, 1, K), generator=g, device="cuda")
+        got = m.input_projection(x).reshape(T, 4 * H)
+        ref = x.reshape(T, K).double() @ wx.double().T
+        assert float((got.double() - ref).abs().max()) <= 2.0 ** -24 * float(ref.abs().max())      # one rounding to fp32
+    finally:
+        m.close()
