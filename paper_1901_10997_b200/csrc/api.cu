@@ -63,7 +63,7 @@ struct lstm_handle {
     // one sequence: its own partition (whole groups of four units per CTA), fragments and exchange words (two sets)
     bool use_one = false, one_fuse = false;
     RecurOnePlan one = {0, 0, 0, 0};
-    unsigned *one_xch = nullptr; int one_set = 0;
+    unsigned *one_xch = nullptr, *one_turn = nullptr;
     bool step_ok = false;              // single timesteps run on the streaming kernel (lstm_step.cu)
     bool fuse_ok = false;              // short single sequences: projection fused into the register-resident kernel's prologue
     // register-resident sparse kernel (bf16, CSR execution): warps, columns per warp, row tiles, entry slots per lane
@@ -74,16 +74,16 @@ struct lstm_handle {
     long long csr_conflicts = 0;       // shared-memory wavefronts per step and CTA lost to bank conflicts (worst CTA, worst matrix)
     int mma_mt = 0, mma_nkr = 0, mma_nks = 0, mma_nw = 0;
     bool seq_dirs = false;             // bidirectional layers run one direction after the other, each on all SMs
-    // batched tensor-core recurrence: partition and exchange words (two sets: a launch clears the other one)
+    // batched tensor-core recurrence: partition and exchange words (two sets: a launch uses one and clears the other)
     bool use_tcb = false;
     RecurTcPlan tcb = {0, 0, 0, 0, 0};
-    unsigned *tcb_xch = nullptr; int tcb_set = 0; unsigned tcb_dirty = 0;
-    unsigned *f32_xch = nullptr; int f32_set = 0;      // fp32 dense, at most two units per CTA: exchange words (two sets)
+    unsigned *tcb_xch = nullptr, *tcb_turn = nullptr;
+    unsigned *f32_xch = nullptr, *f32_turn = nullptr;  // fp32 dense, at most two units per CTA: exchange words (two sets)
     // H-LSTM cell: width of the hidden layer inside each gate (0: plain LSTM), pass-2 column tiles per warp
     int Hh = 0, hl_nkw2 = 0;
     bool use_ht = false;               // H-LSTM on the tile kernel; else on the one that runs batch rows in turn
     HlstmTilePlan ht = {0, 0, 0, 0, 0, 0};
-    unsigned *ht_hx = nullptr, *ht_rx = nullptr; int ht_set = 0;
+    unsigned *ht_hx = nullptr, *ht_rx = nullptr, *ht_turn = nullptr;
     unsigned long long *rxch = nullptr; size_t rxch_words = 0;
     std::vector<Layer> layers;
     // workspace
@@ -268,6 +268,14 @@ int dev_alloc(lstm_handle *h, T **dst, size_t bytes, bool zero, cudaStream_t st,
     if (zero && bytes && cudaMemsetAsync(*dst, 0, bytes, st) != cudaSuccess)
         return fail(h, LSTM_ERR_CUDA, "clearing %s failed", what);
     return LSTM_OK;
+}
+
+// exchange words with a phase bit, two sets, and behind them the words that say whose turn the sets are (device_util.cuh)
+int alloc_xch(lstm_handle *h, unsigned **xch, unsigned **turn, size_t words, cudaStream_t st)
+{
+    const int rc = dev_alloc(h, xch, (words + 32) * sizeof(unsigned), true, st, "exchange words");
+    if (rc == LSTM_OK) *turn = *xch + words;
+    return rc;
 }
 
 inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
@@ -932,15 +940,13 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     h->xch_words = (size_t)D * 2 * max_B * H;
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->xch, h->xch_words * 8, true, st, "exchange buffer");
     if (rc == LSTM_OK && h->use_one) {
-        rc = dev_alloc(h, &h->one_xch, (size_t)2 * D * 2 * h->one.ncta * 32 * sizeof(unsigned), true, st, "exchange words");
+        rc = alloc_xch(h, &h->one_xch, &h->one_turn, (size_t)2 * D * 2 * h->one.ncta * 32, st);
         if (rc == LSTM_OK && recur_one_prepare(h->one, h->smem_optin - 64) != cudaSuccess)
             rc = fail(h, LSTM_ERR_CUDA, "one-sequence kernel set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
     }
     if (rc == LSTM_OK && dtype == LSTM_F32 && !csr && h->upc <= 2 && H <= kF32MaxUnits)
-        rc = dev_alloc(h, &h->f32_xch, (size_t)2 * D * 2 * H * 32 * sizeof(unsigned), true, st, "exchange words");
-    if (rc == LSTM_OK && h->use_tcb) {
-        rc = dev_alloc(h, &h->tcb_xch, 2 * (recur_tc_xch_words(H, h->tcb.rows, D) + kTcXchSlack) * sizeof(unsigned), true, st, "exchange words");
-    }
+        rc = alloc_xch(h, &h->f32_xch, &h->f32_turn, (size_t)2 * D * 2 * H * 32, st);
+    if (rc == LSTM_OK && h->use_tcb) rc = alloc_xch(h, &h->tcb_xch, &h->tcb_turn, 2 * (recur_tc_xch_words(H, h->tcb.rows, D) + kTcXchSlack), st);
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->status_dev, sizeof(int), true, st, "status word");
     if (rc == LSTM_OK && h->use_wave) {
         h->wave_xch_words = (size_t)layers * max_T * std::min(max_B, 4) * H;
@@ -1251,7 +1257,7 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
     h->xch_words = (size_t)D * 2 * max_B * H;
     if (h->use_ht) {
         h->xch_words = 1;
-        if (rc == LSTM_OK) rc = dev_alloc(h, &h->ht_hx, (size_t)2 * D * 2 * ((H + 15) / 16) * 256 * 4, true, st, "exchange words");
+        if (rc == LSTM_OK) rc = alloc_xch(h, &h->ht_hx, &h->ht_turn, (size_t)2 * D * 2 * ((H + 15) / 16) * 256, st);
         if (rc == LSTM_OK) rc = dev_alloc(h, &h->ht_rx, (size_t)2 * D * 2 * ((Hh + 15) / 16) * 1024 * 4, true, st, "hidden-layer exchange words");
     } else h->rxch_words = (size_t)D * 2 * max_B * 4 * Hh;
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->xch, h->xch_words * 8, true, st, "exchange buffer");
@@ -1484,12 +1490,11 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                 m.xb_next = l < L - 1 ? h->xbn[l & 1] : nullptr;
                 m.xb_ld = h->ldn;
                 m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
-                m.hx = h->ht_hx; m.rx = h->ht_rx; m.set = h->ht_set;
+                m.hx = h->ht_hx; m.rx = h->ht_rx; m.turn = h->ht_turn;
                 m.status = h->status_dev;
                 if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 e = launch_hlstm_tile(m, h->ht, st);
                 ++h->last_launches;
-                if (e == cudaSuccess) h->ht_set ^= 1;
                 if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             }
@@ -1548,12 +1553,11 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                 m.y = l == L - 1 ? y : m.xb_next ? nullptr : h->ybuf[l & 1];
                 m.xb_ld = h->ldn;
                 m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
-                m.xch = h->tcb_xch; m.set = h->tcb_set; m.set_words = recur_tc_xch_words(H, h->tcb.rows, D) + kTcXchSlack; m.clear_words = h->tcb_dirty;
+                m.xch = h->tcb_xch; m.set_words = recur_tc_xch_words(H, h->tcb.rows, D) + kTcXchSlack; m.used_words = (unsigned)recur_tc_xch_words(H, m.B, dirs); m.turn = h->tcb_turn;
                 m.status = h->status_dev;
                 if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 e = launch_recur_tc(m, st);
                 ++h->last_launches;
-                if (e == cudaSuccess) { h->tcb_set ^= 1; h->tcb_dirty = (unsigned)recur_tc_xch_words(H, m.B, dirs); }
                 if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             }
@@ -1615,12 +1619,11 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             m.xb_next = (l < L - 1 && h->use_tc && !fuse) ? h->xbn[l & 1] : nullptr;     // a fused next layer reads the fp32 activations
             m.xb_ld = h->ldn;
             m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
-            m.xch = h->one_xch; m.set = h->one_set;
+            m.xch = h->one_xch; m.turn = h->one_turn;
             m.status = h->status_dev;
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             e = launch_recur_one(m, h->one, fuse, st);
             ++h->last_launches;
-            if (e == cudaSuccess) h->one_set ^= 1;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             continue;
@@ -1638,12 +1641,11 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             m.h0 = h0 ? h0 + so : nullptr; m.c0 = c0 ? c0 + so : nullptr;
             m.hT = hT ? hT + so : nullptr; m.cT = cT ? cT + so : nullptr;
             m.y = l == L - 1 ? y : h->ybuf[l & 1];
-            m.xch = h->f32_xch; m.set = h->f32_set;
+            m.xch = h->f32_xch; m.turn = h->f32_turn;
             m.status = h->status_dev;
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             e = launch_recur_f32(m, st);
             ++h->last_launches;
-            if (e == cudaSuccess) h->f32_set ^= 1;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             continue;

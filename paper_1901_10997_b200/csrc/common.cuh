@@ -69,8 +69,8 @@ struct RecurF32Args {
     const float *h0, *c0;
     float *hT, *cT;
     float *y;
-    unsigned *xch;              // exchange words [2 sets][D][2 slots][H][32 batch rows]
-    int set;                    // the set this launch uses; it clears the other one
+    unsigned *xch;              // exchange words [2 sets][D][2 slots][H][32 batch rows]: a launch uses one set and clears the other
+    unsigned *turn;             // whose turn the sets are (device_util.cuh)
     int *status;
 };
 cudaError_t launch_recur_f32(const RecurF32Args &a, cudaStream_t st);
@@ -149,8 +149,8 @@ struct RecurOneArgs {
     __nv_bfloat16 *xb_next;
     long long xb_plane;
     int xb_ld;
-    unsigned *xch;              // exchange words [2 sets][D][2 slots][ncta_dir][32]
-    int set;                    // the set this launch uses; it clears the other one
+    unsigned *xch;              // exchange words [2 sets][D][2 slots][ncta_dir][32]: a launch uses one set and clears the other
+    unsigned *turn;             // whose turn the sets are (device_util.cuh)
     int *status;
 };
 size_t recur_one_smem_bytes(int mt, int nks);
@@ -293,8 +293,9 @@ struct RecurTcArgs {
     int xb_ld;
     unsigned *xch;              // exchange words, 2 sets of [directions][2 slots][16 columns][8 batch rows] blocks of 128
     size_t set_words;           // words from set to set
-    int set;                    // the set this launch uses; it clears the other one for the next launch ...
-    unsigned clear_words;       // ... as far as the previous launch may have written it
+    unsigned used_words;        // words of its set this launch may write
+    unsigned *turn;             // whose turn the sets are (device_util.cuh); [1 + set]: words the last launch on a set may have
+                                // written, which the next launch clears
     int *status;
 };
 size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair);
@@ -363,7 +364,7 @@ struct HlstmTileArgs {
     long long xb_plane;
     int xb_ld;
     unsigned *hx, *rx;          // exchange words [2 sets][D][2 slots][tile][2 row groups][128]: tiles of cell units; of 4 x hidden units
-    int set;                    // the set this launch uses; it clears the other one
+    unsigned *turn;             // whose turn the sets are (device_util.cuh): a launch uses one set and clears the other
     int *status;
 };
 bool hlstm_tile_plan(int H, int Hh, int max_cta, size_t max_smem, HlstmTilePlan *p);

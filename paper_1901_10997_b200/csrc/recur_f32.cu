@@ -44,9 +44,8 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
     // exchange words [set][direction of the launch][slot][unit][32 batch rows]; the other set is cleared for the next launch
     const unsigned slot_words = (unsigned)H * 32u;
     const size_t off = (size_t)(d - a.dir0) * 2 * slot_words, set_words = (size_t)2 * D * slot_words;
-    unsigned *xch = a.xch + (size_t)a.set * set_words + off;
-    for (int i = tid; i < nu * 64; i += kThreads)
-        a.xch[(size_t)(a.set ^ 1) * set_words + off + (size_t)(i & 1) * slot_words + u0 * 32 + (i >> 1)] = 0u;
+    const int set = xch_set(a.turn);
+    unsigned *xch = a.xch + (size_t)set * set_words + off;
 
     const int ksteps = (H + 3) >> 2, kper = (ksteps + KS - 1) / KS;
     const int nt = warp / KS, kq = warp - nt * KS;
@@ -59,6 +58,8 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
 #pragma unroll
         for (int i = 0; i < KW; ++i) af[i] = i < kn && u < nu && kcol + 4 * i < H ? (double)w[4 * i] : 0.0;
     }
+    for (int i = tid; i < nu * 64; i += kThreads)
+        a.xch[(size_t)(set ^ 1) * set_words + off + (size_t)(i & 1) * slot_words + u0 * 32 + (i >> 1)] = 0u;
     unsigned mine = 0;                                     // k4 steps in which this lane has a value to fetch
 #pragma unroll
     for (int i = 0; i < KW; ++i)
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
     }
     if (live && fq == 2 && a.hT) a.hT[so] = hn;
     if (live && fq == 3 && a.cT) a.cT[so] = c;
+    if (tid == 0) xch_done(a.turn);
 }
 
 typedef void (*KernelFn)(const RecurF32Args);

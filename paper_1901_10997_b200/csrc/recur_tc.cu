@@ -189,9 +189,9 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     const unsigned slot_words = (unsigned)((H + 15) >> 4) * (RG * 128u);
     auto chunk_word = [&](int q, int b) -> unsigned { return ((unsigned)(q >> 2) * RG + (b >> 3)) * 128u + (q & 3) * 32u + (b & 7) * 4u; };
     // (buffers by place in the launch, not by direction: launches that run the directions in turn share them)
-    unsigned *xch_d = a.xch + (size_t)a.set * a.set_words + (size_t)(d - a.dir0) * 2 * slot_words;
-    for (unsigned i = blockIdx.x * kThreads + tid; i < a.clear_words / 4u; i += gridDim.x * kThreads)
-        reinterpret_cast<uint4 *>(a.xch + (size_t)(a.set ^ 1) * a.set_words)[i] = make_uint4(0, 0, 0, 0);
+    const int set = xch_set(a.turn);
+    const unsigned clear_words = ld_relaxed_u32(a.turn + 1 + (set ^ 1));
+    unsigned *xch_d = a.xch + (size_t)set * a.set_words + (size_t)(d - a.dir0) * 2 * slot_words;
     // weights into tensor memory: warp w writes lane quadrant w % 4, every fourth 8-column piece
     {
         const int row = (warp & 3) * 32 + lane, pieces = a.KH >> 3;
@@ -207,6 +207,9 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
+    for (unsigned i = blockIdx.x * kThreads + tid; i < clear_words / 4u; i += gridDim.x * kThreads)
+        reinterpret_cast<uint4 *>(a.xch + (size_t)(set ^ 1) * a.set_words)[i] = make_uint4(0, 0, 0, 0);
+    if (blockIdx.x == 0 && tid == 0) a.turn[1 + set] = a.used_words;
     for (int i = tid; i < tiles * N * 8; i += kThreads) reinterpret_cast<uint4 *>(op)[i] = make_uint4(0, 0, 0, 0);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -492,6 +495,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
             if (a.hT) a.hT[state0 + (size_t)(fb0 + 4 * m + fq) * H] = hn[m];
             if (a.cT) a.cT[state0 + (size_t)(fb0 + 4 * m + fq) * H] = c[m];
         }
+    if (tid == 0) xch_done(a.turn);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     if (__syncthreads_or(*abort_v)) {           // one answer for the whole CTA: the partner may raise the flag at any time
         // a wait gave up: products and partial sums may still be in flight; they land within microseconds

@@ -1,0 +1,54 @@
+"""Calls recorded into a CUDA graph beside ordinary calls on the same handle: the exchange words of the kernels that count their
+sets on the device (batched, one wide sequence, narrow fp32, H-LSTM tiles), and single timesteps (needs a B200)."""
+import pytest
+
+import lstm_workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+# (kind, dtype, H, T, B): several steps and a single one of each kernel; pairs and passes of the batched one
+CASES = [("lstm", "bf16", 300, 6, 3), ("lstm", "bf16", 200, 4, 70), ("lstm", "bf16", 300, 1, 16), ("lstm", "bf16", 1201, 6, 1), ("lstm", "fp32", 100, 6, 3),
+         ("lstm", "fp32", 100, 1, 3), ("hlstm", "bf16", 150, 6, 3), ("hlstm", "bf16", 150, 1, 17), ("lstm", "bf16", 300, 1, 4)]
+
+
+@pytest.mark.parametrize("c", CASES, ids=lambda c: f"{c[0]}_{c[1]}_H{c[2]}_T{c[3]}_B{c[4]}")
+def test_recorded_calls_beside_ordinary_ones(c):
+    import torch
+    import paper_1901_10997_b200 as pkg
+    kind, dtype, H, T, B = c
+    w = wl.Workload("capture", 1, False, 40, H, 7, B, dtype, 0.05, seed=H + B)
+    if kind == "hlstm":
+        weights, x = wl.make_hlstm(w, 64)
+        m = pkg.HLSTM(weights, layers=1, in_dim=40, hidden=H, gate_hidden=64, dtype=dtype, max_T=7, max_B=B)
+    else:
+        weights, x = wl.make(w)
+        m = pkg.LSTM(weights, layers=1, in_dim=40, hidden=H, dtype=dtype, max_T=7, max_B=B)
+    try:
+        x = torch.from_numpy(x).cuda()
+        xg = x[:T].flip(0).contiguous()
+        expect = [[t.clone() for t in m.forward(xx)] for xx in (x, xg)]
+        out = tuple(torch.empty_like(t) for t in expect[1])
+        m.check()
+
+        def ordinary(what):
+            got = m.forward(x)
+            m.check()
+            assert all(torch.equal(a, b) for a, b in zip(got, expect[0])), what
+
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            m.forward(xg, out=out)
+        ordinary("after recording")
+        for i in range(3):
+            for _ in range(i + 1):
+                for t in out:
+                    t.zero_()
+                graph.replay()
+                m.check()
+                torch.cuda.synchronize()
+                assert all(torch.equal(a, b) for a, b in zip(out, expect[1])), f"replay {i}"
+            ordinary(f"after replay {i}")
+        ordinary("again")
+        del graph
+    finally:
+        m.close()
