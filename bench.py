@@ -343,16 +343,10 @@ def trimmed_mean(ms, drop=0.1):
     return float(sum(keep) / len(keep))
 
 
-def kernel_of(info, mode):
-    if mode == "hlstm":
-        return "hlstm_mma_kernel", "hlstm_mma.cu"
-    if mode == "csr":
-        return ("recur_csr_kernel", "recur_csr.cu") if info.get("recur_csr_register_resident") else ("recur_kernel", "recur.cu")
-    if info.get("recur_batched_tensor_core"):
-        return "recur_tc_kernel", "recur_tc.cu"
-    if info.get("recur_register_resident"):
-        return "recur_mma_kernel", "recur_mma.cu"
-    return "recur_kernel", "recur.cu"
+def kernel_of(pkg, info):
+    """The recurrent kernel of the last call and its source file."""
+    name = pkg.RECUR_KERNELS[info["kernel"]]
+    return name, name.removesuffix("_kernel") + ".cu"
 
 
 class GpuCase:
@@ -438,7 +432,7 @@ class GpuCase:
         rec_avg_ms = rec_ms / max(rec_n, 1)
         achieved = alg_bytes / (rec_avg_ms * 1e-3) / 1e9 if rec_avg_ms > 0 else None
         info = self.model.info()
-        kernel_name, kernel_src = kernel_of(info, self.mode)
+        kernel_name, kernel_src = kernel_of(self.pkg, info)
         traffic, source = measured_traffic(kernel_name, self.name, kernel_src)
         steps_per_launch = w.T * (2 if (w.dirs == 2 and info.get("ctas_per_dir") == info.get("sm_count")) else 1)
         return {"bound": "hbm", "kernel": f"{kernel_name} (one launch = one layer, all T steps" + (", its input projection in the prologue)" if fused else ")"),

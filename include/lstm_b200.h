@@ -244,27 +244,46 @@ LSTM_API int lstm_profile_read(lstm_handle *h, int *launches, float *ms);
 enum { LSTM_PROBE_NO_PRODUCTS = 1, LSTM_PROBE_NO_GATES = 2, LSTM_PROBE_NO_EXCHANGE = 4, LSTM_PROBE_WHOLE_STEP = 8 };
 LSTM_API int lstm_probe(lstm_handle *h, int parts_left_out);
 
+/* Recurrent kernels, as lstm_info reports the one that the last lstm_forward launched */
+enum {
+    LSTM_RAN_NONE        = 0,    /* no call yet */
+    LSTM_RAN_SHARED      = 1,    /* recur_kernel: weights in shared memory, streamed from L2 beyond it */
+    LSTM_RAN_REGISTERS   = 2,    /* recur_mma_kernel: weights in registers */
+    LSTM_RAN_ONE         = 3,    /* recur_one_kernel: one sequence of a wide layer */
+    LSTM_RAN_WAVE        = 4,    /* recur_wave_kernel: all layers in one launch */
+    LSTM_RAN_BATCHED     = 5,    /* recur_tc_kernel: several sequences, weights in tensor memory */
+    LSTM_RAN_SPARSE      = 6,    /* recur_csr_kernel: lists of surviving weights in registers */
+    LSTM_RAN_F32         = 7,    /* recur_f32_kernel: narrow fp32 layers */
+    LSTM_RAN_STEP        = 8,    /* lstm_step_kernel: a single timestep */
+    LSTM_RAN_HLSTM_ROWS  = 9,    /* hlstm_mma_kernel: H-LSTM, batch rows one after the other */
+    LSTM_RAN_HLSTM_TILES = 10    /* hlstm_tile_kernel: H-LSTM for batches */
+};
+
 /*
  * Read-only facts about how the handle runs (for reports): writes up to n values into out and
- * returns the number available.  Order: [0] SM count, [1] CTAs of the recurrent kernel per direction,
+ * returns the number available.  [1]..[5] and [9]..[11] describe the per-layer kernel that serves whatever no
+ * other kernel of the handle does; [19]..[22] describe what the last lstm_forward launched.
+ * Order: [0] SM count, [1] CTAs of the per-layer kernel per direction,
  * [2] threads per CTA, [3] dynamic shared memory bytes per CTA at max_B, [4] recurrent-matrix rows
  * resident in shared memory per CTA (max over CTAs), [5] rows streamed from L2 per CTA (max),
  * [6] split-K factor of the input projection at max_T*max_B, [7] 1 if the projection uses the tensor-core
  * (tcgen05) kernel, [8] kernels launched by the most recent lstm_forward (before the first call: the count expected),
  * [9] 1 if the recurrence keeps its weights in registers (bf16 dense), 0 for the shared-memory kernel,
  * [10] 16-column weight tiles per warp held in registers, [11] per warp held in shared memory,
- * [12] nonzero if a call at max_B runs the batched tensor-core (tcgen05) recurrence (2: as clusters of two CTAs
- * that split K, 1: every CTA on its own): bf16 dense LSTM handles use
- * it for batches of 5 to 64 sequences where its operand ring fits beside the resident slice, and the
- * register-resident kernel (passes of four sequences) otherwise,
+ * [12] nonzero if the handle has the batched tensor-core (tcgen05) recurrence (2: as clusters of two CTAs
+ * that split K, 1: every CTA on its own): bf16 LSTM handles, dense or CSR, made for two sequences or more, whose
+ * slices fit tensor memory.  Calls that another kernel runs faster do not use it,
  * [13] 1 if a CSR handle runs the register-resident sparse kernel (bf16 storage, at most 16 units per CTA,
  * lane lists short enough for registers), 0 for the shared-memory CSR kernel, [14] its entry slots per lane,
  * [15] shared-memory wavefronts per step and CTA that its gathers lose to bank conflicts (worst CTA),
  * [16] the compact width when the handle runs a row/column-pruned stack on its surviving units only (0: it does
  * not; then [0]..[15] describe the handle itself, otherwise the inner handle of that width), [17] the number
- * of (layer, direction, unit) triples removed, [18] 1 if calls with up to four sequences run the layer-wavefront
+ * of (layer, direction, unit) triples removed, [18] 1 if the handle has the layer-wavefront
  * kernel (unidirectional bf16 dense stacks of 2 to 4 layers whose slices fit on-chip with the SMs split between
- * the layers: all layers in one launch, layer l on timestep t beside layer l-1 on t+1).
+ * the layers: all layers in one launch, layer l on timestep t beside layer l-1 on t+1) for one sequence and, where it is
+ * faster than the batched kernel, for up to four,
+ * [19] the recurrent kernel the last lstm_forward launched (LSTM_RAN_*), [20] CTAs of that launch (the last one of the
+ * call), [21] its threads per CTA, [22] its dynamic shared memory per CTA in bytes.
  */
 LSTM_API int lstm_info(const lstm_handle *h, int64_t *out, int n);
 

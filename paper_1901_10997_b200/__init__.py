@@ -11,4 +11,6 @@ from .binding import (LSTM, HLSTM, LstmError, hlstm_create, lib_path, load_libra
                       LSTM_F32, LSTM_BF16W_F32S, LSTM_DENSE, LSTM_CSR, LSTM_OK, LSTM_ERR_INVALID,
                       LSTM_ERR_UNSUPPORTED, LSTM_ERR_CUDA, LSTM_ERR_NOMEM, LSTM_ERR_TIMEOUT, LSTM_ERR_INTERNAL,
                       LSTM_K_STAGE, LSTM_K_PROJ, LSTM_K_RECUR, LSTM_K_COUNT,
-                      LSTM_PROBE_NO_PRODUCTS, LSTM_PROBE_NO_GATES, LSTM_PROBE_NO_EXCHANGE, LSTM_PROBE_WHOLE_STEP)
+                      LSTM_PROBE_NO_PRODUCTS, LSTM_PROBE_NO_GATES, LSTM_PROBE_NO_EXCHANGE, LSTM_PROBE_WHOLE_STEP,
+                      LSTM_RAN_NONE, LSTM_RAN_SHARED, LSTM_RAN_REGISTERS, LSTM_RAN_ONE, LSTM_RAN_WAVE, LSTM_RAN_BATCHED, LSTM_RAN_SPARSE,
+                      LSTM_RAN_F32, LSTM_RAN_STEP, LSTM_RAN_HLSTM_ROWS, LSTM_RAN_HLSTM_TILES, RECUR_KERNELS)

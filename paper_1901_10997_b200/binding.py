@@ -16,6 +16,11 @@ LSTM_DENSE, LSTM_CSR = 0, 1
 LSTM_OK, LSTM_ERR_INVALID, LSTM_ERR_UNSUPPORTED, LSTM_ERR_CUDA, LSTM_ERR_NOMEM, LSTM_ERR_TIMEOUT, LSTM_ERR_INTERNAL = range(7)
 LSTM_K_STAGE, LSTM_K_PROJ, LSTM_K_RECUR, LSTM_K_COUNT = 0, 1, 2, 3
 LSTM_PROBE_NO_PRODUCTS, LSTM_PROBE_NO_GATES, LSTM_PROBE_NO_EXCHANGE, LSTM_PROBE_WHOLE_STEP = 1, 2, 4, 8
+(LSTM_RAN_NONE, LSTM_RAN_SHARED, LSTM_RAN_REGISTERS, LSTM_RAN_ONE, LSTM_RAN_WAVE, LSTM_RAN_BATCHED, LSTM_RAN_SPARSE, LSTM_RAN_F32,
+ LSTM_RAN_STEP, LSTM_RAN_HLSTM_ROWS, LSTM_RAN_HLSTM_TILES) = range(11)
+# names of the kernels, in that order
+RECUR_KERNELS = ("", "recur_kernel", "recur_mma_kernel", "recur_one_kernel", "recur_wave_kernel", "recur_tc_kernel", "recur_csr_kernel",
+                 "recur_f32_kernel", "lstm_step_kernel", "hlstm_mma_kernel", "hlstm_tile_kernel")
 
 import os as _os
 
@@ -166,7 +171,8 @@ def lstm_info(handle):
             "proj_splits", "proj_tensor_core", "launches_per_forward", "recur_register_resident",
             "col_tiles_in_registers", "col_tiles_in_smem", "recur_batched_tensor_core",
             "recur_csr_register_resident", "csr_slots_per_lane", "csr_bank_conflict_wavefronts",
-            "compact_hidden", "units_removed", "layer_wavefront"]
+            "compact_hidden", "units_removed", "layer_wavefront",
+            "kernel", "kernel_ctas", "kernel_threads", "kernel_smem_bytes"]
     return {k: int(out[i]) for i, k in enumerate(keys[:n])}
 
 

@@ -108,6 +108,8 @@ struct lstm_handle {
     std::vector<int> ev_kind;
     int ev_used = 0;
     int last_launches = 0;
+    int ran_kernel = LSTM_RAN_NONE, ran_ctas = 0, ran_threads = 0;     // recurrent kernel of the last forward call, as last launched
+    size_t ran_smem = 0;
     // layer-wavefront kernel (unidirectional stacks, up to four sequences): CTAs per layer, units per CTA, tiling
     bool use_wave = false, wave_all = false;    // wave_all: LSTM_B200_WAVE=1, whatever else could serve the call
     int wave_ncta = 0, wave_upc = 0, wave_mt = 0, wave_nkr = 0, wave_nkw[kMaxWaveLayers] = {0, 0, 0, 0}, wave_nkw_max = 0;
@@ -1275,6 +1277,11 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
     return LSTM_OK;
 }
 
+static void ran(lstm_handle *h, int kernel, int ctas, int threads, size_t smem)
+{
+    h->ran_kernel = kernel; h->ran_ctas = ctas; h->ran_threads = threads; h->ran_smem = smem;
+}
+
 static int record(lstm_handle *h, int kind, cudaStream_t st)
 {
     if (!h->prof) return 0;
@@ -1419,6 +1426,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             m.status = h->status_dev;
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             e = launch_lstm_step(m, h->mma_mt, st);
+            ran(h, LSTM_RAN_STEP, m.ncta_dir * D, kStepThreads, lstm_step_smem_bytes(h->mma_mt, B, m.x_tiles, m.h_tiles));
             ++h->last_launches;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "step launch failed (layer %d): %s", l, cudaGetErrorString(e));
@@ -1449,6 +1457,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         const size_t smem = recur_wave_smem_bytes(h->wave_mt, h->wave_nkr, h->wave_nkw_max, h->wave_upc, B);
         if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         e = launch_recur_wave(m, h->wave_mt, h->wave_nkr, smem, st);
+        ran(h, LSTM_RAN_WAVE, m.ncta_layer * L, 16 * 32, smem);
         ++h->last_launches;
         if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "wavefront launch failed: %s", cudaGetErrorString(e));
@@ -1494,6 +1503,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                 m.status = h->status_dev;
                 if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 e = launch_hlstm_tile(m, h->ht, st);
+                ran(h, LSTM_RAN_HLSTM_TILES, m.ncta_dir * D, kHtThreads, hlstm_tile_smem_bytes(h->ht, m.B));
                 ++h->last_launches;
                 if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
@@ -1526,6 +1536,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             const size_t smem = hlstm_mma_smem_bytes(h->mma_mt, h->mma_nkr, h->mma_nw, h->mma_nks, h->hl_nkw2, h->upc, B);
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             e = launch_hlstm_mma(m, h->mma_mt, h->mma_nkr, h->mma_nw, smem, st);
+            ran(h, LSTM_RAN_HLSTM_ROWS, m.ncta_dir * D, h->mma_nw * 32, smem);
             ++h->last_launches;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
@@ -1557,6 +1568,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                 m.status = h->status_dev;
                 if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 e = launch_recur_tc(m, st);
+                ran(h, LSTM_RAN_BATCHED, m.ncta_dir * dirs, kTcThreads, recur_tc_smem_bytes(m.KH, m.upc, m.B, m.pair));
                 ++h->last_launches;
                 if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
@@ -1594,6 +1606,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                                      : recur_csr_reg_smem_bytes(h->csr_nw, h->csr_kspan, h->csr_mt, h->upc, B);
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             e = launch_recur_csr_reg(m, h->csr_slots, h->csr_nw, smem, st);
+            ran(h, LSTM_RAN_SPARSE, m.ncta_dir * m.ndirs, h->csr_nw * 32, smem);
             ++h->last_launches;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
@@ -1623,6 +1636,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             m.status = h->status_dev;
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             e = launch_recur_one(m, h->one, fuse, st);
+            ran(h, LSTM_RAN_ONE, m.ncta_dir * dirs, kOneThreads, fuse ? recur_one_fuse_smem_bytes(h->one.mt, h->one.nks) : recur_one_smem_bytes(h->one.mt, h->one.nks));
             ++h->last_launches;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
@@ -1645,6 +1659,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             m.status = h->status_dev;
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             e = launch_recur_f32(m, st);
+            ran(h, LSTM_RAN_F32, m.ncta_dir * m.ndirs, kF32Threads, 0);
             ++h->last_launches;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
@@ -1676,8 +1691,10 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
             m.xch = h->xch;
             m.status = h->status_dev;
+            const size_t smem = fuse ? recur_mma_smem_bytes(h->mma_mt, h->mma_nkr, h->mma_nw, h->mma_nks, h->upc, 1, false, true) : shp.smem;
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
-            e = launch_recur_mma(m, h->mma_mt, h->mma_nkr, h->mma_nw, fuse ? recur_mma_smem_bytes(h->mma_mt, h->mma_nkr, h->mma_nw, h->mma_nks, h->upc, 1, false, true) : shp.smem, st);
+            e = launch_recur_mma(m, h->mma_mt, h->mma_nkr, h->mma_nw, smem, st);
+            ran(h, LSTM_RAN_REGISTERS, m.ncta_dir * m.ndirs, h->mma_nw * 32, smem);
             ++h->last_launches;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
@@ -1706,6 +1723,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         a.status = h->status_dev;
         if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         e = csr ? launch_recur_csr(a, bf16, shp.threads, shp.smem, st) : launch_recur_dense(a, bf16, shp.threads, shp.smem, st);
+        ran(h, LSTM_RAN_SHARED, a.ncta_dir * a.ndirs, shp.threads, shp.smem);
         ++h->last_launches;
         if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
@@ -1885,12 +1903,13 @@ int lstm_info(const lstm_handle *h, int64_t *out, int n)
     const int launches = h->last_launches > 0 ? h->last_launches : h->L * 2 + (h->use_tc ? 1 : 0);
     const int tcb_at_max = h->use_tcb ? (h->tcb.pair ? 2 : 1) : 0;
     if (h->use_csr_reg) shp.smem = recur_csr_reg_smem_bytes(h->csr_nw, h->csr_kspan, h->csr_mt, h->upc, h->max_B);
-    const int64_t vals[19] = {h->sm_count, h->ncta_dir, h->use_mma ? h->mma_nw * 32 : h->use_csr_reg ? h->csr_nw * 32 : h->threads, (int64_t)shp.smem,
+    const int64_t vals[23] = {h->sm_count, h->ncta_dir, h->use_mma ? h->mma_nw * 32 : h->use_csr_reg ? h->csr_nw * 32 : h->threads, (int64_t)shp.smem,
                               rows_res, rows_str, (l0.plan_M >= 0) ? l0.plan.nsplit : 1, h->use_tc ? 1 : 0, launches,
                               h->use_mma ? 1 : 0, h->use_mma ? h->mma_nkr : 0, h->use_mma ? h->mma_nks : 0, tcb_at_max,
-                              h->use_csr_reg ? 1 : 0, h->use_csr_reg ? h->csr_slots : 0, h->use_csr_reg ? h->csr_conflicts : 0, 0, 0, h->use_wave ? 1 : 0};
-    for (int i = 0; i < n && i < 19; ++i) out[i] = vals[i];
-    return 19;
+                              h->use_csr_reg ? 1 : 0, h->use_csr_reg ? h->csr_slots : 0, h->use_csr_reg ? h->csr_conflicts : 0, 0, 0, h->use_wave ? 1 : 0,
+                              h->ran_kernel, h->ran_ctas, h->ran_threads, (int64_t)h->ran_smem};
+    for (int i = 0; i < n && i < 23; ++i) out[i] = vals[i];
+    return 23;
 }
 
 }  // extern "C"

@@ -59,6 +59,7 @@ cudaError_t recur_csr_prepare(int max_smem);
 // ---------------------------------------------------------------------------------------------------
 constexpr int kF32MaxUnits = 296;     // widest layer: two units on each of 148 CTAs
 constexpr int kF32MaxRows = 32;
+constexpr int kF32Threads = 512;
 struct RecurF32Args {
     int dir0, ndirs;            // as in RecurArgs
     int H, Hp8, B, T, D, ncta_dir;
@@ -129,6 +130,7 @@ cudaError_t launch_recur_mma(const RecurMmaArgs &a, int mt, int nkr, int nw, siz
 // ---------------------------------------------------------------------------------------------------
 // Register-resident recurrent kernel for one sequence (recur_one.cu): CTA c owns units [c * 4 mt, (c + 1) * 4 mt)
 // ---------------------------------------------------------------------------------------------------
+constexpr int kOneThreads = 512;
 struct RecurOnePlan { int mt, nkr, nks, ncta; };     // 16-row tiles; column tiles per warp in registers, in shared memory; CTAs per direction
 struct RecurOneArgs {
     int dir0, ndirs;            // as in RecurArgs
@@ -164,6 +166,7 @@ cudaError_t launch_recur_one(const RecurOneArgs &a, const RecurOnePlan &p, bool 
 // One timestep of one layer (T = 1, up to kStepMaxRows batch rows) over the register-resident kernel's fragments
 // ---------------------------------------------------------------------------------------------------
 constexpr int kStepMaxRows = 8;
+constexpr int kStepThreads = 256;
 struct LstmStepArgs {
     int H, B, D, ncta_dir;
     int in_l, x_tiles, h_tiles; // input width; 16-column tiles of the two fragment arrays per CTA
@@ -266,6 +269,7 @@ cudaError_t launch_recur_csr_reg(const RecurCsrArgs &a, int slots, int nw, size_
 // the K range (KH columns each).  The weights go to tensor memory, h travels as phase-bit words in 16-byte chunks.
 // ---------------------------------------------------------------------------------------------------
 constexpr int kTcMaxRows = 64;        // batch rows of one pass; larger calls run several passes
+constexpr int kTcThreads = 512;
 constexpr int kTcStaticSmem = 1024;   // bytes kept free for the kernel's static shared memory (barriers, flags: under 100)
 // Accumulators (one issuing warp each) and the tensor-memory columns set aside for them with rg groups of eight batch
 // rows: an issuing warp needs about 370 cycles for a group of twelve instructions up to N = 32, 470 at N = 48, most of
@@ -345,6 +349,7 @@ cudaError_t launch_hlstm_mma(const HlstmArgs &a, int mt, int nkr, int nw, size_t
 // H-LSTM kernel for batches: row tiles of sixteen units of one gate, eight batch rows per operand-B tile (hlstm_tile.cu)
 // ---------------------------------------------------------------------------------------------------
 constexpr int kHtRows = 16;            // batch rows of one launch; larger calls run several
+constexpr int kHtThreads = 512;
 struct HlstmTilePlan { int H, Hh, n1, kt, ncta; size_t max_smem; };     // hidden tiles per CTA, column tiles of h per warp, CTAs per direction
 struct HlstmTileArgs {
     int H, Hh, B, T, D;
@@ -368,6 +373,7 @@ struct HlstmTileArgs {
     int *status;
 };
 bool hlstm_tile_plan(int H, int Hh, int max_cta, size_t max_smem, HlstmTilePlan *p);
+size_t hlstm_tile_smem_bytes(const HlstmTilePlan &p, int rows);
 cudaError_t hlstm_tile_prepare(const HlstmTilePlan &p);
 cudaError_t launch_hlstm_tile(const HlstmTileArgs &a, const HlstmTilePlan &p, cudaStream_t st);
 

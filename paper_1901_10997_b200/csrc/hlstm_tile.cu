@@ -24,7 +24,7 @@
 namespace lstm {
 namespace {
 
-constexpr int kWarps = 16, kThreads = 512;
+constexpr int kThreads = kHtThreads, kWarps = kThreads / 32;
 constexpr int kPitch = 20;                     // floats between the batch rows of a tile's partial sums: no bank conflicts
 constexpr int kTileRed = 8 * kPitch;           // partial sums of 16 rows x 8 batch rows
 constexpr unsigned kRPhase = 0x80000000u;
@@ -362,6 +362,8 @@ bool hlstm_tile_plan(int H, int Hh, int max_cta, size_t max_smem, HlstmTilePlan 
     return ut <= max_cta && (ut + 15) / 16 <= 6 && pick(p->n1, p->kt, 0) && smem_bytes(Hh, p->n1, kHtRows, 1) <= max_smem;
 }
 
+size_t hlstm_tile_smem_bytes(const HlstmTilePlan &p, int rows) { return smem_bytes(p.Hh, p.n1, rows, mode_of(p, rows, p.max_smem)); }
+
 cudaError_t hlstm_tile_prepare(const HlstmTilePlan &p)
 {
     for (int mode = 0; mode < 3; ++mode) {
@@ -377,7 +379,7 @@ cudaError_t launch_hlstm_tile(const HlstmTileArgs &a, const HlstmTilePlan &p, cu
     HlstmTileArgs copy = a;
     void *params[] = {&copy};
     return cudaLaunchCooperativeKernel((const void *)pick(p.n1, p.kt, mode), dim3(a.ncta_dir * a.D), dim3(kThreads), params,
-                                       smem_bytes(a.Hh, p.n1, a.B, mode), st);
+                                       hlstm_tile_smem_bytes(p, a.B), st);
 }
 
 }  // namespace lstm

@@ -19,7 +19,7 @@
 namespace lstm {
 namespace {
 
-constexpr int kWarps = 8, kThreads = 256;
+constexpr int kThreads = kStepThreads, kWarps = kThreads / 32;
 
 // MT: 16-row tiles of the CTA (4 gate rows x units).  RB: batch rows the operand is laid out for: up to 4 rows put their hi
 // and lo planes into adjacent columns, 8 take one column each and two instructions a tile.

@@ -19,7 +19,7 @@
 namespace lstm {
 namespace {
 
-constexpr int kWarps = 16, kThreads = 512;
+constexpr int kThreads = kF32Threads, kWarps = kThreads / 32;
 
 __device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b)
 {

@@ -26,7 +26,7 @@
 namespace lstm {
 namespace {
 
-constexpr int kNW = 16, kNT = kNW * 32;
+constexpr int kNT = kOneThreads, kNW = kNT / 32;
 constexpr int kMaxSplit = 4, kOneMinUnits = 1025;
 
 template <int MT, int NKR, bool FUSE>

@@ -49,7 +49,7 @@
 namespace lstm {
 namespace {
 
-constexpr int kWarps = 16, kThreads = kWarps * 32;     // 128 registers a thread
+constexpr int kThreads = kTcThreads;            // 128 registers a thread
 constexpr int kPollers = 12;                    // warps that fetch the operand (a multiple of 4 keeps their addresses linear)
 constexpr int kIssuer = 12;                     // first of the warps that issue the products; all warps finish
 constexpr int kMaxGroups = 5;                   // operand groups of 16 * kPollers columns

@@ -1,0 +1,59 @@
+"""Which recurrent kernel serves which call, as the library reports it after the call (needs a B200)."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def forward(kind, dtype, bidir, L, H, T, B, density=1.0, max_B=None):
+    """One call on fresh weights; the handle's report after it."""
+    import torch
+    import paper_1901_10997_b200 as pkg
+    D, n = 2 if bidir else 1, 24
+    g = torch.Generator(device="cuda").manual_seed(H + B)
+    ws = []
+    for layer in range(L):
+        for _ in range(D):
+            k = n if layer == 0 else D * H
+            if kind == "hlstm":
+                ws.append({"ux": torch.randn(4 * 64, k, generator=g, device="cuda"), "uh": torch.randn(4 * 64, H, generator=g, device="cuda"),
+                           "w": torch.randn(4 * H, 64, generator=g, device="cuda")})
+            else:
+                w = {"wx": torch.randn(4 * H, k, generator=g, device="cuda"), "wh": torch.randn(4 * H, H, generator=g, device="cuda")}
+                if density < 1:
+                    w["mask_x"] = (torch.rand(4 * H, k, generator=g, device="cuda") < density).to(torch.uint8)
+                    w["mask_h"] = (torch.rand(4 * H, H, generator=g, device="cuda") < density).to(torch.uint8)
+                ws.append(w)
+    shape = dict(layers=L, in_dim=n, hidden=H, bidir=bidir, dtype=dtype, max_T=T, max_B=max_B or B)
+    m = pkg.HLSTM(ws, gate_hidden=64, **shape) if kind == "hlstm" else pkg.LSTM(ws, exec_mode="csr" if density < 1 else "dense", **shape)
+    try:
+        assert m.info()["kernel"] == pkg.LSTM_RAN_NONE
+        m.forward(torch.randn(T, B, n, generator=g, device="cuda"))
+        m.check()
+        return m.info()
+    finally:
+        m.close()
+
+
+# (kind, dtype, bidir, layers, H, T, B, density) -> kernel, threads
+CASES = [
+    (("lstm", "fp32", False, 1, 200, 3, 20, 1.0), "F32", 512),
+    (("lstm", "fp32", False, 1, 400, 3, 2, 1.0), "SHARED", None),
+    (("lstm", "bf16", False, 1, 300, 3, 1, 1.0), "REGISTERS", 256),
+    (("lstm", "bf16", False, 1, 1300, 3, 1, 1.0), "ONE", 512),
+    (("lstm", "bf16", False, 2, 300, 3, 1, 1.0), "WAVE", 512),
+    (("lstm", "bf16", False, 2, 300, 3, 9, 1.0), "BATCHED", 512),
+    (("lstm", "bf16", False, 1, 1300, 3, 5, 1.0), "BATCHED", 512),
+    (("lstm", "bf16", False, 1, 600, 3, 16, 0.1), "BATCHED", 512),
+    (("lstm", "bf16", False, 1, 600, 3, 1, 0.1), "SPARSE", 512),
+    (("lstm", "bf16", False, 2, 300, 1, 8, 1.0), "STEP", 256),
+    (("hlstm", "bf16", False, 1, 300, 3, 9, 1.0), "HLSTM_TILES", 512),
+]
+
+
+@pytest.mark.parametrize("case,kernel,threads", CASES, ids=lambda v: "-".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_kernel_of_a_call(case, kernel, threads):
+    import paper_1901_10997_b200 as pkg
+    info = forward(*case)
+    assert pkg.RECUR_KERNELS[info["kernel"]] == pkg.RECUR_KERNELS[getattr(pkg, "LSTM_RAN_" + kernel)]
+    assert info["kernel_ctas"] >= 1 and (threads is None or info["kernel_threads"] == threads)
+    assert info["kernel_smem_bytes"] <= 227 * 1024
