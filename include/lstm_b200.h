@@ -229,8 +229,8 @@ LSTM_API int lstm_profile_enable(lstm_handle *h, int on);
 LSTM_API int lstm_profile_read(lstm_handle *h, int *launches, float *ms);
 
 /*
- * Step-cost probe of the register-resident recurrent kernel (bf16 dense LSTM handles, calls with one sequence;
- * calls with more run normally).  A recurrent step is a chain: wait for the other CTAs' h words -> tensor-core products ->
+ * Step-cost probe of the register-resident recurrent kernels (LSTM_RAN_REGISTERS, _ONE and _SPARSE, whichever the handle
+ * runs layer by layer; calls with one sequence; calls with more run normally).  A recurrent step is a chain: wait for the other CTAs' h words -> tensor-core products ->
  * CTA barrier, reduction, gate functions -> publish.  With a non-zero mask the following lstm_forward calls
  * leave parts of that chain out, so that timing them shows what each part costs (the "empty step": exchange
  * only, is the floor no kernel of this structure can go below).  Bits: LSTM_PROBE_NO_PRODUCTS (no tensor

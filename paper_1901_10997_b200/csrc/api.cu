@@ -1471,8 +1471,8 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         int nsplit = 1;
         // ---- input staging + projection (a single short sequence on the register-resident kernel computes its
         // projection inside that kernel's prologue instead: two launches and one round trip of G fewer per layer)
-        const bool one = h->use_one && B == 1 && !h->probe;
-        const bool fuse = one ? h->one_fuse && T <= kFuseMaxT : (h->fuse_ok || (h->csr_fuse_ok && h->use_csr_reg)) && !h->Hh && B == 1 && T <= kFuseMaxT && !h->probe &&
+        const bool one = h->use_one && B == 1;
+        const bool fuse = one ? h->one_fuse && T <= kFuseMaxT && !h->probe : (h->fuse_ok || (h->csr_fuse_ok && h->use_csr_reg)) && !h->Hh && B == 1 && T <= kFuseMaxT && !h->probe &&
                           ly.xfrag[0] != nullptr;
         if (!fuse) { const int prc = run_projection(h, l, l == 0 ? x : nullptr, Xf, M, N, &nsplit, st); if (prc != LSTM_OK) return prc; }
 
@@ -1617,7 +1617,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             memset(&m, 0, sizeof m);
             const int dirs = h->seq_dirs ? 1 : D;
             m.dir0 = h->seq_dirs ? pass : 0; m.ndirs = dirs;
-            m.H = H; m.T = T; m.D = D; m.ncta_dir = h->one.ncta; m.nsplit = nsplit; m.nkw_smem = h->one.nks;
+            m.H = H; m.T = T; m.D = D; m.ncta_dir = h->one.ncta; m.nsplit = nsplit; m.nkw_smem = h->one.nks; m.probe = h->probe;
             m.spin_limit = h->spin_limit;
             m.withhold_cta = h->withhold_cta < 0 ? -1 : h->withhold_cta % (h->one.ncta * dirs);
             m.in_l = ly.in_l; m.nkw_x = ly.nkw_ox; m.X = Xf; m.bias = ly.bias;

@@ -138,6 +138,7 @@ struct RecurOneArgs {
     int nkw_smem;
     long long spin_limit;
     int withhold_cta;
+    int probe;                  // measurement: parts of the step to leave out (LSTM_PROBE_*), 0 in normal operation
     int in_l, nkw_x, gs_off;    // projection in the prologue: input width, column tiles of Wx per range, byte offset of its rows of G
     const float *X;
     const uint4 *xfrag[2];      // [cta][8 ranges][nkw_x][mt][lane], the lane's columns adjacent

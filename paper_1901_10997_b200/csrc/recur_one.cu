@@ -29,9 +29,11 @@ namespace {
 constexpr int kNT = kOneThreads, kNW = kNT / 32;
 constexpr int kMaxSplit = 4, kOneMinUnits = 1025;
 
-template <int MT, int NKR, bool FUSE>
+// FUSE: projection in the prologue; PROBE: measurement build that leaves parts of the step out
+template <int MT, int NKR, bool FUSE, bool PROBE>
 __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
 {
+    const int probe = PROBE ? a.probe : 0;
     constexpr int UPC = 4 * MT, RP = MT * 16 + 4;              // units per CTA; floats between the warps' partial sums
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int abort_s;
@@ -128,7 +130,7 @@ __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
             const unsigned phase = word_phase(s - 1);
             const unsigned *p = src + ((s - 1) & 1) * slot_words;
             if (has) w = ld_relaxed_v4(p);
-            bool wait = has && !words_ready(w, phase);
+            bool wait = has && !words_ready(w, phase) && !(probe & 4);
             int polls = 0;
             long long t_start = 0;
             while (wait) {
@@ -158,16 +160,18 @@ __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
         for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[mt][e] = 0.0f;
+        if (!(probe & 1)) {
 #pragma unroll
-        for (int i = 0; i < NKR; ++i) {
-            const uint2 b = hl[4 * i];
+            for (int i = 0; i < NKR; ++i) {
+                const uint2 b = hl[4 * i];
 #pragma unroll
-            for (int mt = 0; mt < MT; ++mt) mma_bf16(acc[mt], areg[i][mt], b.x, b.y);
-        }
-        for (int i = 0; i < nks; ++i) {
-            const uint2 b = hl[4 * (NKR + i)];
+                for (int mt = 0; mt < MT; ++mt) mma_bf16(acc[mt], areg[i][mt], b.x, b.y);
+            }
+            for (int i = 0; i < nks; ++i) {
+                const uint2 b = hl[4 * (NKR + i)];
 #pragma unroll
-            for (int mt = 0; mt < MT; ++mt) mma_bf16(acc[mt], As_w[(size_t)(i * MT + mt) * 32], b.x, b.y);
+                for (int mt = 0; mt < MT; ++mt) mma_bf16(acc[mt], As_w[(size_t)(i * MT + mt) * 32], b.x, b.y);
+            }
         }
         // accumulator columns 0 and 1 are the hi and lo products (the other columns repeat them)
         if (tig == 0) {
@@ -180,7 +184,7 @@ __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
         }
         // projection term of this lane's gate: one value per split-K plane, on its way until the sums are there
         float v[kMaxSplit] = {0.0f, 0.0f, 0.0f, 0.0f};
-        if (real && (lane & 1) == 0) {
+        if (real && (lane & 1) == 0 && !(probe & 2)) {
             if (FUSE) v[0] = *gs;
             else {
 #pragma unroll
@@ -191,10 +195,12 @@ __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
         }
         gp += gadv;
         gs += FUSE ? (int)dir * GP : 0;
-        if (fin && s > 0) write_outputs();
+        if (fin && s > 0 && !(probe & 2)) write_outputs();
         bar_sync(1, nbar);
 
-        if (fin) {
+        if (probe & 2) {
+            if (publish) st_relaxed_u32(out + (s & 1) * slot_words, pack_word(0.0f, word_phase(s)));
+        } else if (fin) {
             const float *rp = red + ((s & 1) * kNW + (lane & 1) * 8) * RP + 4 * fu + fq;
             float p[4];
 #pragma unroll
@@ -221,16 +227,19 @@ __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
 }
 
 typedef void (*KernelFn)(const RecurOneArgs);
-template <bool FUSE>
+template <bool FUSE, bool PROBE>
 KernelFn pick_f(int mt, int nkr)
 {
     switch (mt * 16 + nkr) {
-        case 48 + 6: return recur_one_kernel<3, 6, FUSE>;
-        case 64 + 4: return recur_one_kernel<4, 4, FUSE>;
+        case 48 + 6: return recur_one_kernel<3, 6, FUSE, PROBE>;
+        case 64 + 4: return recur_one_kernel<4, 4, FUSE, PROBE>;
         default: return nullptr;
     }
 }
-KernelFn pick(int mt, int nkr, bool fuse) { return fuse ? pick_f<true>(mt, nkr) : pick_f<false>(mt, nkr); }
+KernelFn pick(int mt, int nkr, bool fuse, bool probe)
+{
+    return probe ? pick_f<false, true>(mt, nkr) : fuse ? pick_f<true, false>(mt, nkr) : pick_f<false, false>(mt, nkr);
+}
 
 }  // namespace
 
@@ -256,13 +265,13 @@ bool recur_one_plan(int H, int max_cta, size_t max_smem, RecurOnePlan *p)
     p->nkr = p->mt == 4 ? 4 : 6;
     p->nks = std::max(0, need - p->nkr);
     p->ncta = (H + upc - 1) / upc;
-    return H >= kOneMinUnits && p->mt >= 3 && pick(p->mt, p->nkr, false) && p->nkr + p->nks <= 8 && recur_one_smem_bytes(p->mt, p->nks) <= max_smem;
+    return H >= kOneMinUnits && p->mt >= 3 && pick(p->mt, p->nkr, false, false) && p->nkr + p->nks <= 8 && recur_one_smem_bytes(p->mt, p->nks) <= max_smem;
 }
 
 cudaError_t recur_one_prepare(const RecurOnePlan &p, int max_smem)
 {
-    for (int fuse = 0; fuse < 2; ++fuse) {
-        const cudaError_t e = cudaFuncSetAttribute(pick(p.mt, p.nkr, fuse != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+    for (int i = 0; i < 3; ++i) {
+        const cudaError_t e = cudaFuncSetAttribute(pick(p.mt, p.nkr, i == 1, i == 2), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -272,7 +281,7 @@ cudaError_t launch_recur_one(const RecurOneArgs &a, const RecurOnePlan &p, bool 
 {
     RecurOneArgs copy = a;
     void *params[] = {&copy};
-    return cudaLaunchCooperativeKernel((const void *)pick(p.mt, p.nkr, fuse), dim3(a.ncta_dir * (a.ndirs ? a.ndirs : a.D)), dim3(kNT), params,
+    return cudaLaunchCooperativeKernel((const void *)pick(p.mt, p.nkr, fuse, a.probe != 0), dim3(a.ncta_dir * (a.ndirs ? a.ndirs : a.D)), dim3(kNT), params,
                                        fuse ? recur_one_fuse_smem_bytes(p.mt, p.nks) : recur_one_smem_bytes(p.mt, p.nks), st);
 }
 

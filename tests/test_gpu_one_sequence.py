@@ -20,3 +20,23 @@ def test_one_sequence_wide_layers(oracle, s):
     h0, c0 = wl.make_states(w)
     ref = oracle.forward(weights, x, h0, c0, layers=L, bidir=bidir, hidden=H)
     assert_close(run_gpu(w, weights, x, h0, c0), ref, "bf16", "one")
+
+
+def test_probe_measures_the_kernel_that_serves_the_call(oracle):
+    import torch
+    import paper_1901_10997_b200 as pkg
+    w = wl.Workload("one_probe", 1, False, 40, 1201, 7, 1, "bf16", 0.03, seed=3)
+    weights, x = wl.make(w)
+    ref = oracle.forward(weights, x, layers=1, bidir=False, hidden=w.hidden)
+    m = pkg.LSTM(weights, layers=1, in_dim=40, hidden=w.hidden, dtype="bf16", max_T=7, max_B=1)
+    try:
+        xd = torch.from_numpy(x).cuda()
+        for mask in (1, 2, 4, 1 | 2, 4 | 2, pkg.LSTM_PROBE_WHOLE_STEP, 0):
+            m.probe(mask)
+            got = m.forward(xd)
+            m.check()
+            assert m.info()["kernel"] == pkg.LSTM_RAN_ONE
+            if mask in (0, pkg.LSTM_PROBE_WHOLE_STEP):
+                assert_close([t.cpu().numpy() for t in got], ref, "bf16", f"one/probe {mask}")
+    finally:
+        m.close()
