@@ -104,7 +104,7 @@ typedef struct {
  * Environment switches read at create time (for measurements and tests; unset = the library chooses):
  *   LSTM_B200_RECUR = simt  shared-memory recurrent kernel instead of the register-resident one (bf16 dense or CSR)
  *                   = mma   no batched tensor-core recurrence (batches above four run as passes of four); H-LSTM: batch
- *                           rows one after the other
+ *                           rows one after the other, as one row is by default
  *                   = tc1   batched tensor-core recurrence without cluster pairs
  *   LSTM_B200_FUSE  = 0     never compute the input projection inside the recurrent kernel (single sequences of up
  *                           to 40 steps on the register-resident kernel do so by default)

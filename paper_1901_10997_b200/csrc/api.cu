@@ -40,6 +40,7 @@ struct Layer {
     int nkw_x = 0;
     uint4 *wtc[2] = {nullptr, nullptr};    // batched tensor-core kernel: [cta][8-column piece][row 4 * unit + gate]
     uint4 *frag2[2] = {nullptr, nullptr};  // H-LSTM: fragments of the gate output matrices W
+    uint4 *tfrag[2] = {nullptr, nullptr}, *tfrag2[2] = {nullptr, nullptr};     //   the tile kernel's fragments of Uh and W
     float *bias_out = nullptr;             // H-LSTM: [D][H][4] bias of the gate pre-activations
     int csr_max_slice_entries = 0;     // largest per-CTA slice (entries, padded)
     unsigned *csr_reg_ent[2] = {nullptr, nullptr};   // register-resident sparse kernel: [cta][warp][slots][32] entry words
@@ -81,7 +82,7 @@ struct lstm_handle {
     unsigned *f32_xch = nullptr, *f32_turn = nullptr;  // fp32 dense, at most two units per CTA: exchange words (two sets)
     // H-LSTM cell: width of the hidden layer inside each gate (0: plain LSTM), pass-2 column tiles per warp
     int Hh = 0, hl_nkw2 = 0;
-    bool use_ht = false;               // H-LSTM on the tile kernel; else on the one that runs batch rows in turn
+    bool use_ht = false;               // H-LSTM: the tile kernel serves calls with several rows (use_mma: the row kernel the others)
     HlstmTilePlan ht = {0, 0, 0, 0, 0, 0};
     unsigned *ht_hx = nullptr, *ht_rx = nullptr, *ht_turn = nullptr;
     unsigned long long *rxch = nullptr; size_t rxch_words = 0;
@@ -537,7 +538,7 @@ void free_all(lstm_handle *h)
 {
     for (auto &ly : h->layers) {
         cudaFree(ly.wx); cudaFree(ly.bias); cudaFree(ly.wx_rowptr); cudaFree(ly.wx_ent);
-        for (int d = 0; d < 2; ++d) { cudaFree(ly.wh[d]); cudaFree(ly.wh_ptr[d]); cudaFree(ly.wh_ent[d]); cudaFree(ly.wfrag[d]); cudaFree(ly.ofrag[d]); cudaFree(ly.oxfrag[d]); cudaFree(ly.xfrag[d]); cudaFree(ly.frag2[d]); cudaFree(ly.csr_reg_ent[d]); cudaFree(ly.csr_reg_rows[d]); }
+        for (int d = 0; d < 2; ++d) { cudaFree(ly.wh[d]); cudaFree(ly.wh_ptr[d]); cudaFree(ly.wh_ent[d]); cudaFree(ly.wfrag[d]); cudaFree(ly.ofrag[d]); cudaFree(ly.oxfrag[d]); cudaFree(ly.xfrag[d]); cudaFree(ly.frag2[d]); cudaFree(ly.tfrag[d]); cudaFree(ly.tfrag2[d]); cudaFree(ly.csr_reg_ent[d]); cudaFree(ly.csr_reg_rows[d]); }
         cudaFree(ly.bias_out); cudaFree(ly.wtc[0]); cudaFree(ly.wtc[1]);
     }
     cudaFree(h->G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
@@ -1163,9 +1164,14 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
         const char *env = getenv("LSTM_B200_RECUR");
         h->use_ht = !(env && strcmp(env, "mma") == 0) && hlstm_tile_plan(H, Hh, h->sm_count / D, (size_t)h->smem_optin - 64, &h->ht);
     }
-    // tiling of the other kernel: row tiles cover 4 x (units per CTA) of both passes; pass 1 keeps up to nkr column tiles per
+    // The row kernel serves one sequence, for which its step is the shorter one, and everything where the tile kernel does not
+    // fit.  us per call, T = 35, row kernel / tile kernel: H = Hh = 800 152 / 191, 1500 240 / 283, H = 1200 with Hh = 320
+    // 140 / 147, two directions of 400 with Hh = 200 105 / 137; equal or up to 8 % the other way for a few narrow shapes (H = 600
+    // with Hh = 600, 100 with 50).  Two rows: 286 / 196 at H = Hh = 800.
+    // Its tiling: row tiles cover 4 x (units per CTA) of both passes; pass 1 keeps up to nkr column tiles per
     // warp in registers, the rest and all of pass 2 in shared memory
-    if (!h->use_ht) {
+    const int row_B = h->use_ht ? 1 : max_B;
+    {
         const int upch = (Hh + h->ncta_dir - 1) / h->ncta_dir;
         const int mt = (4 * std::max(h->upc, upch) + 15) / 16;
         const int nk1 = (H + 15) / 16, nk2 = (Hh + 15) / 16;
@@ -1180,13 +1186,14 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
             ok = nkr > 0 && recur_mma_shape_ok(mt, nkr, nw);
         }
         const int nks1 = ok && need1 > nkr ? need1 - nkr : 0;
-        if (ok) ok = hlstm_mma_smem_bytes(mt, nkr, nw, nks1, need2, h->upc, max_B) <= (size_t)h->smem_optin - 64;
-        if (!ok) {
+        if (ok) ok = hlstm_mma_smem_bytes(mt, nkr, nw, nks1, need2, h->upc, row_B) <= (size_t)h->smem_optin - 64;
+        if (!ok && !h->use_ht) {
             fail(h, LSTM_ERR_UNSUPPORTED, "hidden=%d gate_hidden=%d max_B=%d: the per-CTA slices do not fit registers and shared memory", H, Hh, max_B);
             return bail(LSTM_ERR_UNSUPPORTED);
         }
-        h->use_mma = true;
-        h->mma_mt = mt; h->mma_nkr = nkr; h->mma_nks = nks1; h->mma_nw = nw; h->hl_nkw2 = need2;
+        h->use_mma = ok;
+        if (ok) { h->mma_mt = mt; h->mma_nkr = nkr; h->mma_nks = nks1; h->mma_nw = nw; h->hl_nkw2 = need2; }
+        if (ok && max_B == 1) h->use_ht = false;
     }
 
     int rc = LSTM_OK;
@@ -1220,7 +1227,7 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
             };
             if (!masked(ux, src.mask_ux, (size_t)4 * Hh * ly.in_l, ux_m) || !masked(uh, src.mask_uh, (size_t)4 * Hh * H, uh_m) ||
                 !masked(ww, src.mask_w, (size_t)4 * H * Hh, w_m)) { rc = fail(h, LSTM_ERR_CUDA, "reading masks"); break; }
-            for (int q = 0; q < 4; ++q) {
+            parallel_for(4, [&](int q) {
                 for (int m = 0; m < Hh; ++m) {
                     const size_t prow = (size_t)d * 4 * Hh + (size_t)m * 4 + q;           // unit-major, gates adjacent
                     if (ba) bias_p[prow] = ba[q * Hh + m];
@@ -1228,13 +1235,19 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
                     for (int k = 0; k < ly.in_l; ++k) wx16[prow * ly.ldk + k] = f32_to_bf16_rne(srow[k]);
                 }
                 if (bb) for (int j = 0; j < H; ++j) bias_o[(size_t)d * 4 * H + (size_t)j * 4 + q] = bb[q * H + j];
+            });
+            auto put = [&](uint4 **dst, const std::vector<uint32_t> &f, const char *what) {
+                if (rc == LSTM_OK) rc = upload(h, (uint32_t **)dst, f.data(), f.size() * 4, st, what);
+                if (rc == LSTM_OK) cudaStreamSynchronize(st);
+            };
+            if (h->use_ht) {
+                put(&ly.tfrag[d], pack_ht_hidden(uh, h->ht), "hidden-layer recurrent tiles");
+                put(&ly.tfrag2[d], pack_ht_gates(ww, h->ht), "gate output tiles");
             }
-            const int NW = h->mma_nw;
-            const std::vector<uint32_t> f1 = h->use_ht ? pack_ht_hidden(uh, h->ht) : pack_fragments(uh, Hh, H, h->ncta_dir, NW, h->mma_nkr + h->mma_nks, h->mma_mt);
-            const std::vector<uint32_t> f2 = h->use_ht ? pack_ht_gates(ww, h->ht) : pack_fragments(ww, H, Hh, h->ncta_dir, NW, h->hl_nkw2, h->mma_mt);
-            rc = upload(h, (uint32_t **)&ly.wfrag[d], f1.data(), f1.size() * 4, st, "hidden-layer recurrent fragments");
-            if (rc == LSTM_OK) rc = upload(h, (uint32_t **)&ly.frag2[d], f2.data(), f2.size() * 4, st, "gate output fragments");
-            if (rc == LSTM_OK) cudaStreamSynchronize(st);
+            if (h->use_mma) {
+                put(&ly.wfrag[d], pack_fragments(uh, Hh, H, h->ncta_dir, h->mma_nw, h->mma_nkr + h->mma_nks, h->mma_mt), "hidden-layer recurrent fragments");
+                put(&ly.frag2[d], pack_fragments(ww, H, Hh, h->ncta_dir, h->mma_nw, h->hl_nkw2, h->mma_mt), "gate output fragments");
+            }
         }
         if (rc) break;
         rc = upload(h, &ly.bias, bias_p.data(), bias_p.size() * 4, st, "hidden-layer bias");
@@ -1256,17 +1269,18 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
         for (int i = 0; i < 2 && rc == LSTM_OK; ++i) rc = dev_alloc(h, &h->xbn[i], 2 * Mmax * h->ldn * 2, true, st, "bf16 layer activations");
         for (int i = 0; i < 2 && rc == LSTM_OK; ++i) rc = dev_alloc(h, &h->ybuf[i], Mmax * D * H * 4, false, st, "layer activations");
     }
-    h->xch_words = (size_t)D * 2 * max_B * H;
+    h->xch_words = (size_t)D * 2 * row_B * H;
+    h->rxch_words = (size_t)D * 2 * row_B * 4 * Hh;
     if (h->use_ht) {
-        h->xch_words = 1;
         if (rc == LSTM_OK) rc = alloc_xch(h, &h->ht_hx, &h->ht_turn, (size_t)2 * D * 2 * ((H + 15) / 16) * 256, st);
         if (rc == LSTM_OK) rc = dev_alloc(h, &h->ht_rx, (size_t)2 * D * 2 * ((Hh + 15) / 16) * 1024 * 4, true, st, "hidden-layer exchange words");
-    } else h->rxch_words = (size_t)D * 2 * max_B * 4 * Hh;
+    }
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->xch, h->xch_words * 8, true, st, "exchange buffer");
-    if (rc == LSTM_OK && h->rxch_words) rc = dev_alloc(h, &h->rxch, h->rxch_words * 8, true, st, "hidden-layer exchange buffer");
+    if (rc == LSTM_OK) rc = dev_alloc(h, &h->rxch, h->rxch_words * 8, true, st, "hidden-layer exchange buffer");
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->status_dev, sizeof(int), true, st, "status word");
     if (rc == LSTM_OK) {
-        cudaError_t e = h->use_ht ? hlstm_tile_prepare(h->ht) : hlstm_mma_prepare(h->mma_mt, h->mma_nkr, h->mma_nw, h->smem_optin - 64);
+        cudaError_t e = h->use_ht ? hlstm_tile_prepare(h->ht) : cudaSuccess;
+        if (e == cudaSuccess && h->use_mma) e = hlstm_mma_prepare(h->mma_mt, h->mma_nkr, h->mma_nw, h->smem_optin - 64);
         if (e == cudaSuccess) e = proj_tc_prepare();
         if (e != cudaSuccess) rc = fail(h, LSTM_ERR_CUDA, "kernel set-up failed: %s", cudaGetErrorString(e));
     }
@@ -1479,7 +1493,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         // ---- recurrence: all directions in one launch, or one launch per direction
         const int npass = h->seq_dirs ? D : 1;
         for (int pass = 0; pass < npass; ++pass) {
-        if (h->use_ht) {
+        if (h->use_ht && (B > 1 || !h->use_mma)) {
             const int passes = (B + kHtRows - 1) / kHtRows;
             for (int p = 0; p < passes; ++p) {
                 HlstmTileArgs m;
@@ -1488,7 +1502,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                 m.H = H; m.Hh = h->Hh; m.T = T; m.D = D; m.ncta_dir = h->ht.ncta; m.nsplit = nsplit;
                 m.spin_limit = h->spin_limit;
                 m.withhold_cta = h->withhold_cta < 0 ? -1 : h->withhold_cta % (h->ht.ncta * D);
-                for (int d = 0; d < D; ++d) { m.frag1[d] = ly.wfrag[d]; m.frag2[d] = ly.frag2[d]; }
+                for (int d = 0; d < D; ++d) { m.frag1[d] = ly.tfrag[d]; m.frag2[d] = ly.tfrag2[d]; }
                 m.G = h->G;
                 m.g_split_stride = (long long)M * N;
                 m.bias_out = ly.bias_out;
@@ -1889,7 +1903,7 @@ int lstm_info(const lstm_handle *h, int64_t *out, int n)
         return cnt;
     }
     RecurShape shp = recur_shape(h, h->max_B, 0);
-    if (h->Hh && !h->use_ht) shp.smem = hlstm_mma_smem_bytes(h->mma_mt, h->mma_nkr, h->mma_nw, h->mma_nks, h->hl_nkw2, h->upc, h->max_B);
+    if (h->Hh && h->use_mma) shp.smem = hlstm_mma_smem_bytes(h->mma_mt, h->mma_nkr, h->mma_nw, h->mma_nks, h->hl_nkw2, h->upc, h->use_ht ? 1 : h->max_B);
     const size_t wsize = h->dtype == LSTM_BF16W_F32S ? 2 : 4;
     int64_t rows_res = 0, rows_str = 0;
     if (h->use_mma) {

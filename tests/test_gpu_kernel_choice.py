@@ -47,6 +47,10 @@ CASES = [
     (("lstm", "bf16", False, 1, 600, 3, 1, 0.1), "SPARSE", 512),
     (("lstm", "bf16", False, 2, 300, 1, 8, 1.0), "STEP", 256),
     (("hlstm", "bf16", False, 1, 300, 3, 9, 1.0), "HLSTM_TILES", 512),
+    (("hlstm", "bf16", False, 1, 300, 3, 2, 1.0), "HLSTM_TILES", 512),
+    # one sequence, on a handle made for one and on one made for several
+    (("hlstm", "bf16", False, 1, 300, 3, 1, 1.0), "HLSTM_ROWS", None),
+    (("hlstm", "bf16", True, 1, 300, 3, 1, 1.0, 20), "HLSTM_ROWS", None),
 ]
 
 
