@@ -77,7 +77,7 @@ struct lstm_handle {
     bool seq_dirs = false;             // bidirectional layers run one direction after the other, each on all SMs
     // batched tensor-core recurrence: partition and exchange words (two sets: a launch uses one and clears the other)
     bool use_tcb = false;
-    RecurTcPlan tcb = {0, 0, 0, 0, 0};
+    RecurTcPlan tcb = {0, 0, 0, 0, 0, 0};
     unsigned *tcb_xch = nullptr, *tcb_turn = nullptr;
     unsigned *f32_xch = nullptr, *f32_turn = nullptr;  // fp32 dense, at most two units per CTA: exchange words (two sets)
     // H-LSTM cell: width of the hidden layer inside each gate (0: plain LSTM), pass-2 column tiles per warp
@@ -668,15 +668,16 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     }
     // Batched tensor-core recurrence (handles made for several sequences), with the current split of the SMs: as
     // clusters of two where the device can co-schedule them, else every CTA alone.  bf16 CSR handles use it too, with the
-    // zeros multiplied.
+    // zeros multiplied and all 24 bits of h, as their lists do.
+    const int tc_terms = csr ? 3 : 2;
     auto plan_tcb = [&](int ncta, int dirs_side_by_side) -> bool {
         const char *env = getenv("LSTM_B200_RECUR");
         if (!bf16 || (csr && !h->csr_dense_proj) || max_B < tc_min_rows(h) || (env && (strcmp(env, "mma") == 0 || strcmp(env, "simt") == 0))) return false;
         const size_t smem = (size_t)h->smem_optin - kTcStaticSmem;
-        if (recur_tc_prepare((int)smem) != cudaSuccess) { cudaGetLastError(); return false; }
-        if (!(env && strcmp(env, "tc1") == 0) && recur_tc_plan(H, ncta, max_B, 1, smem, &h->tcb) &&
-            recur_tc_pair_supported(h->tcb.ncta * dirs_side_by_side, h->tcb.rows, recur_tc_smem_bytes(h->tcb.KH, h->tcb.upc, h->tcb.rows, 1))) return true;
-        return recur_tc_plan(H, ncta, max_B, 0, smem, &h->tcb);
+        if (recur_tc_prepare(tc_terms, (int)smem) != cudaSuccess) { cudaGetLastError(); return false; }
+        if (!(env && strcmp(env, "tc1") == 0) && recur_tc_plan(H, ncta, max_B, 1, tc_terms, smem, &h->tcb) &&
+            recur_tc_pair_supported(h->tcb.ncta * dirs_side_by_side, h->tcb)) return true;
+        return recur_tc_plan(H, ncta, max_B, 0, tc_terms, smem, &h->tcb);
     };
     h->use_tcb = plan_tcb(h->ncta_dir, D);
     if (D == 2 && bf16 && !csr && !h->use_mma && !h->use_tcb) {
@@ -1565,7 +1566,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                 m.dir0 = h->seq_dirs ? pass : 0; m.ndirs = dirs;
                 m.Bs = B; m.b0 = (int)((long long)B * p / passes); m.B = (int)((long long)B * (p + 1) / passes) - m.b0;
                 m.H = H; m.T = T; m.D = D; m.nsplit = nsplit;
-                m.ncta_dir = h->tcb.ncta; m.upc = h->tcb.upc; m.KH = h->tcb.KH; m.pair = h->tcb.pair;
+                m.ncta_dir = h->tcb.ncta; m.upc = h->tcb.upc; m.KH = h->tcb.KH; m.pair = h->tcb.pair; m.terms = h->tcb.terms;
                 m.spin_limit = h->spin_limit;
                 m.withhold_cta = h->withhold_cta < 0 ? -1 : h->withhold_cta % (h->tcb.ncta * dirs);
                 m.wpack[0] = ly.wtc[0]; m.wpack[1] = ly.wtc[1];
@@ -1582,7 +1583,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                 m.status = h->status_dev;
                 if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 e = launch_recur_tc(m, st);
-                ran(h, LSTM_RAN_BATCHED, m.ncta_dir * dirs, kTcThreads, recur_tc_smem_bytes(m.KH, m.upc, m.B, m.pair));
+                ran(h, LSTM_RAN_BATCHED, m.ncta_dir * dirs, kTcThreads, recur_tc_smem_bytes(m.KH, m.upc, m.B, m.pair, m.terms));
                 ++h->last_launches;
                 if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));

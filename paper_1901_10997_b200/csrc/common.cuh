@@ -272,17 +272,25 @@ cudaError_t launch_recur_csr_reg(const RecurCsrArgs &a, int slots, int nw, size_
 constexpr int kTcMaxRows = 64;        // batch rows of one pass; larger calls run several passes
 constexpr int kTcThreads = 512;
 constexpr int kTcStaticSmem = 1024;   // bytes kept free for the kernel's static shared memory (barriers, flags: under 100)
-// Accumulators (one issuing warp each) and the tensor-memory columns set aside for them with rg groups of eight batch
-// rows: an issuing warp needs about 370 cycles for a group of twelve instructions up to N = 32, 470 at N = 48, most of
-// it between the instructions, so two of them share the work; from N = 80 on the tensor cores are the limit.
-__host__ __device__ constexpr int tc_accumulators(int rg) { return rg <= 4 ? 2 : 1; }
-__host__ __device__ constexpr int tc_acc_columns(int rg) { return rg <= 4 ? 32 * rg : 128; }
-struct RecurTcPlan { int upc, ncta, KH, pair, rows; };   // units per CTA, CTAs per direction, K columns per CTA, clusters of two, rows per pass
+// h enters the products as `terms` bf16 terms: two (16 bits of h) for dense handles, three (all 24) for pruned ones, whose
+// lists multiply h as it is.  Columns of the operand with rg groups of eight batch rows (a multiple of 16):
+__host__ __device__ constexpr int tc_columns(int rg, int terms) { return (8 * rg * terms + 15) / 16 * 16; }
+// Accumulators (one issuing warp each) and the tensor-memory columns set aside for them: an issuing warp needs about 370
+// cycles for a group of twelve instructions up to N = 32, 470 at N = 48, most of it between the instructions, so two of
+// them share the work; from N = 80 on the tensor cores are the limit.
+__host__ __device__ constexpr int tc_accumulators(int rg, int terms) { return tc_columns(rg, terms) <= 64 ? 2 : 1; }
+__host__ __device__ constexpr int tc_acc_columns(int rg, int terms)
+{
+    const int n = tc_accumulators(rg, terms) * tc_columns(rg, terms);
+    return tc_accumulators(rg, terms) == 2 || n > 128 ? n : 128;
+}
+// units per CTA, CTAs per direction, K columns per CTA, clusters of two, rows per pass, terms of h
+struct RecurTcPlan { int upc, ncta, KH, pair, rows, terms; };
 struct RecurTcArgs {
     int dir0, ndirs;            // directions this launch runs: dir0 .. dir0 + ndirs - 1 (ndirs = 0 means all D)
     int H, B, T, D;             // B: batch rows of this pass ...
     int Bs, b0;                 // ... of the call's Bs, starting at row b0
-    int ncta_dir, upc, KH, pair;
+    int ncta_dir, upc, KH, pair, terms;
     int nsplit;
     long long spin_limit;
     int withhold_cta;
@@ -303,12 +311,12 @@ struct RecurTcArgs {
                                 // written, which the next launch clears
     int *status;
 };
-size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair);
+size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair, int terms);
 size_t recur_tc_xch_words(int H, int rows, int dirs);    // exchange words of one launch with `rows` batch rows
 constexpr size_t kTcXchSlack = 5 * 12 * 8 * 128;           // words a polling warp may read beyond them
-bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, size_t max_smem, RecurTcPlan *p);
-bool recur_tc_pair_supported(int grid, int rows, size_t smem);
-cudaError_t recur_tc_prepare(int max_smem);
+bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, int terms, size_t max_smem, RecurTcPlan *p);
+bool recur_tc_pair_supported(int grid, const RecurTcPlan &p);
+cudaError_t recur_tc_prepare(int terms, int max_smem);
 cudaError_t launch_recur_tc(const RecurTcArgs &a, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------

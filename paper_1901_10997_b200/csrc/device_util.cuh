@@ -89,6 +89,9 @@ __device__ __forceinline__ unsigned split_word(float h)
     return ((unsigned)__bfloat16_as_ushort(hi) << 16) | (unsigned)__bfloat16_as_ushort(lo);
 }
 __device__ __forceinline__ unsigned pack_word(float h, unsigned phase) { return (split_word(h) & ~kPhaseBit) | phase; }
+// Exchange words that carry h as its own 32 bits (narrow fp32 layers, pruned layers): without bit 30 a NaN reads as 1.5 or more,
+// which no h is (a fast tanh may pass 1 by a rounding), and gets the bit back.
+constexpr float kMaskedNan = 1.25f;
 __device__ __forceinline__ bool words_ready(const uint4 &w, unsigned phase)
 {
     return (((w.x ^ phase) | (w.y ^ phase) | (w.z ^ phase) | (w.w ^ phase)) & kPhaseBit) == 0;

@@ -9,7 +9,7 @@
 // split (row tile of eight batch rows) x (K range); the weights of a warp's K range sit in registers as doubles.  A lane's
 // operand is ONE value of h, so it polls that word straight into its fragment: no staging, no reduction across lanes (a
 // dot product per warp needed 160 shuffles a unit).  h travels as its own 32 bits: |h| <= 1, so bit 30 is free for the phase
-// (device_util.cuh), and a NaN is still told from every h without it; a unit's 32 batch rows are one line with one writer.  After one barrier a quad per (unit, batch row) adds
+// (device_util.cuh); a unit's 32 batch rows are one line with one writer.  After one barrier a quad per (unit, batch row) adds
 // the K ranges' sums, one gate each, and applies the gate functions, each from one exponential and one division.
 // Measured (2 x 200, batch 20, T = 35, per call): 480 us with recur.cu, 234 us here.
 // Every wait is bounded; on expiry the CTA records a timeout status, stops waiting and runs to the end.
@@ -123,17 +123,17 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
         }
         __syncwarp();
         if (s > 0) {
-            // the words without their phase.  A NaN without bit 30 reads as 1 < |h| < 2, which no h is: it gets the bit back.
+            // the words without their phase
             float top = 0.0f;
 #pragma unroll
             for (int i = 0; i < KW; ++i) {
                 w[i] &= ~kPhaseBit;
                 top = fmaxf(top, fabsf(__uint_as_float(w[i])));
             }
-            if (top > 1.0f) {
+            if (top > kMaskedNan) {
 #pragma unroll
                 for (int i = 0; i < KW; ++i)
-                    if (fabsf(__uint_as_float(w[i])) > 1.0f) w[i] |= kPhaseBit;
+                    if (fabsf(__uint_as_float(w[i])) > kMaskedNan) w[i] |= kPhaseBit;
             }
         }
         double acc0[2] = {0.0, 0.0}, acc1[2] = {0.0, 0.0};      // two chains: the instruction's latency exceeds its rate

@@ -18,8 +18,12 @@
 //     same loop entered by "lane == 0" with per-thread operands took 8260.
 //   * h travels between the CTAs as 32-bit words with a phase bit (device_util.cuh), in 16-byte chunks of four units
 //     of one batch row; the consumers poll the words themselves, twelve warps with all their chunks in
-//     flight, split them into the bf16 hi and lo planes and store those as the swizzled B operand (rows 0 .. Bp-1 hi,
-//     Bp .. 2 Bp - 1 lo).  A step has no stamps, no release or acquire fence and no second trip for the data.
+//     flight, split them into bf16 planes and store those as the swizzled B operand (rows 0 .. Bp - 1 hi, Bp .. 2 Bp - 1
+//     lo).  Pruned layers have a third plane: their lists (recur_csr.cu) multiply h in fp32, so a batch of them carries h
+//     as its own 32 bits and splits it into three terms that hold all 24: with two terms the recurrent products alone were
+//     off by 9e-7 (1.5e-7 with three, as with the lists).  The split and the third plane cost 2 - 17 % of a call
+//     (2 x 1500, T = 35: 4 rows 233 -> 236 us, 16 rows 249 -> 286; 2 x 800, 16 rows 198 -> 219).  A step has no
+//     stamps, no release or acquire fence and no second trip for the data.
 //     LDG.128 reads a row range that all SMs share at 55 - 60 bytes per clock and SM (24 when a quarter warp's 128 bytes
 //     straddle two lines), a tensor copy at about 20.
 //   * The K range is handed to the issuing warps in groups as they arrive (a named barrier each: an issuing thread's
@@ -132,15 +136,15 @@ __device__ __forceinline__ void quad_transpose(float &v0, float &v1, float &v2, 
     if (o2) { v0 = r2; v1 = r3; } else { v2 = r2; v3 = r3; }
 }
 
-// RG: groups of eight batch rows of a pass
-template <int RG, bool PAIR>
+// RG: groups of eight batch rows of a pass; TERMS: bf16 terms of h, two from words {hi | lo}, three from words that are h itself
+template <int RG, bool PAIR, int TERMS>
 __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs a)
 {
-    constexpr int Bp = 8 * RG, N = 2 * Bp, HB = tc_rows_of_first(RG, PAIR), RS = tc_rows_per_thread(HB);
+    constexpr int Bp = 8 * RG, N = tc_columns(RG, TERMS), HB = tc_rows_of_first(RG, PAIR), RS = tc_rows_per_thread(HB);
     constexpr bool UNITS = PAIR && RG == 1;
-    constexpr int KI = tc_groups_in_flight(RG), NACC = tc_accumulators(RG);
+    constexpr int KI = tc_groups_in_flight(RG), NACC = tc_accumulators(RG, TERMS);
     constexpr uint32_t tmem = 0;                                            // all 512 columns are ours: they start at address 0
-    constexpr uint32_t acc_col = 512u - tc_acc_columns(RG);                 // accumulators behind the weights
+    constexpr uint32_t acc_col = 512u - tc_acc_columns(RG, TERMS);                 // accumulators behind the weights
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long accum_bar, partial_bar[2];
     __shared__ uint32_t tmem_base_s;
@@ -346,12 +350,34 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
             }
         } else if (warp < kPollers) {
             // ---- operand: h_{s-1} of this CTA's K range, KI groups at a time
-            auto store_piece = [&](unsigned char *dst, const uint4 &w, unsigned keep) {
-                if (LSTM_CHECK_INDEX(dst - op + Bp * 128 + 7, tiles * N * 128, a.status)) {
+            auto store_piece = [&](unsigned char *dst, uint4 w, bool polled) {
+                if (!LSTM_CHECK_INDEX(dst - op + (TERMS - 1) * Bp * 128 + 7, tiles * N * 128, a.status)) return;
+                if constexpr (TERMS == 2) {
+                    const unsigned keep = polled ? 0xbfffbfffu : 0xffffffffu;
                     *reinterpret_cast<uint2 *>(dst) = make_uint2(__byte_perm(w.x, w.y, 0x7632u) & keep, __byte_perm(w.z, w.w, 0x7632u) & keep);
                     *reinterpret_cast<uint2 *>(dst + Bp * 128) = make_uint2(__byte_perm(w.x, w.y, 0x5410u), __byte_perm(w.z, w.w, 0x5410u));
+                } else {
+                    if (polled) {
+                        w.x &= ~kPhaseBit; w.y &= ~kPhaseBit; w.z &= ~kPhaseBit; w.w &= ~kPhaseBit;
+                        auto size = [](unsigned v) { return fabsf(__uint_as_float(v)); };
+                        if (fmaxf(fmaxf(size(w.x), size(w.y)), fmaxf(size(w.z), size(w.w))) > kMaskedNan) {
+                            if (size(w.x) > kMaskedNan) w.x |= kPhaseBit;
+                            if (size(w.y) > kMaskedNan) w.y |= kPhaseBit;
+                            if (size(w.z) > kMaskedNan) w.z |= kPhaseBit;
+                            if (size(w.w) > kMaskedNan) w.w |= kPhaseBit;
+                        }
+                    }
+                    // each term takes the upper half of what is left, eight bits of it: three hold all 24, nothing is rounded
+#pragma unroll
+                    for (int t = 0; t < 3; ++t) {
+                        *reinterpret_cast<uint2 *>(dst + t * Bp * 128) = make_uint2(__byte_perm(w.x, w.y, 0x7632u), __byte_perm(w.z, w.w, 0x7632u));
+                        if (t == 2) break;
+                        auto rest = [](unsigned v) { return __float_as_uint(__uint_as_float(v) - __uint_as_float(v & 0xffff0000u)); };
+                        w = make_uint4(rest(w.x), rest(w.y), rest(w.z), rest(w.w));
+                    }
                 }
             };
+            auto word_of = [](float h) { return TERMS == 2 ? split_word(h) : __float_as_uint(h); };
             const unsigned phase = word_phase(s - 1);
             const unsigned *src = (s & 1) ? src_even : src_odd;
             if (s == 0 && a.h0) {
@@ -360,11 +386,11 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
                         if (rg < RG - 1 || last_row) {
                             const int k = 4 * (q0 + i * 4 * kPollers);
                             const float *hp = a.h0 + ((size_t)d * a.Bs + a.b0 + rg * 8 + rr) * H + k;
-                            uint4 v = make_uint4(split_word(hp[0]), 0, 0, 0);
-                            if (k + 1 < H) v.y = split_word(hp[1]);
-                            if (k + 2 < H) v.z = split_word(hp[2]);
-                            if (k + 3 < H) v.w = split_word(hp[3]);
-                            store_piece(dst0 + i * kDstGroup + rg * 1024, v, 0xffffffffu);
+                            uint4 v = make_uint4(word_of(hp[0]), 0, 0, 0);
+                            if (k + 1 < H) v.y = word_of(hp[1]);
+                            if (k + 2 < H) v.z = word_of(hp[2]);
+                            if (k + 3 < H) v.w = word_of(hp[3]);
+                            store_piece(dst0 + i * kDstGroup + rg * 1024, v, false);
                         }
             }
             if (s > 0) while ((unsigned)clock() - t_pub < kPollDelay) { }
@@ -411,7 +437,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
                                 }
                             }
 #pragma unroll
-                            for (int rg = 0; rg < RG; ++rg) store_piece(dst + i * kDstGroup + rg * 1024, w[i][rg], 0xbfffbfffu);
+                            for (int rg = 0; rg < RG; ++rg) store_piece(dst + i * kDstGroup + rg * 1024, w[i][rg], true);
                         }
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -431,6 +457,47 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
             auto read_sums = [&](int b0) {                       // this row's sums for batch rows b0 .. b0 + RS - 1
                 const uint32_t ta = acc_col + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)b0;
                 float zl[RS];
+                if constexpr (TERMS == 3 && RG == 1) {           // (with more rows the two waits below are faster: 219 against 235 us per
+                    float v[6][RS];                              // call at 2 x 800, 16 rows)
+#pragma unroll
+                    for (int t = 0; t < 3; ++t) tmem_ld<RS>(ta + (uint32_t)(t * Bp), v[t]);
+                    if (nissue > 1) {
+#pragma unroll
+                        for (int t = 0; t < 3; ++t) tmem_ld<RS>(ta + (uint32_t)(N + t * Bp), v[3 + t]);
+                    }
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int i = 0; i < RS; ++i)
+                        z[i] = nissue > 1 ? (v[0][i] + v[3][i]) + ((v[1][i] + v[4][i]) + (v[2][i] + v[5][i])) : v[0][i] + (v[1][i] + v[2][i]);
+                    return;
+                }
+                if constexpr (TERMS == 3) {                      // the last two terms first: their sum takes the place of the second
+                    float zt[RS];
+                    tmem_ld<RS>(ta + (uint32_t)Bp, zl);
+                    tmem_ld<RS>(ta + (uint32_t)(2 * Bp), zt);
+                    if (NACC > 1 && nissue > 1) {
+                        float y[RS], yt[RS];
+                        tmem_ld<RS>(ta + (uint32_t)(N + Bp), y);
+                        tmem_ld<RS>(ta + (uint32_t)(N + 2 * Bp), yt);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int i = 0; i < RS; ++i) zl[i] = (zl[i] + y[i]) + (zt[i] + yt[i]);
+                        tmem_ld<RS>(ta + (uint32_t)N, y);
+                        tmem_ld<RS>(ta, z);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int i = 0; i < RS; ++i) z[i] = (z[i] + y[i]) + zl[i];
+                    } else {
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int i = 0; i < RS; ++i) zl[i] += zt[i];
+                        tmem_ld<RS>(ta, z);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int i = 0; i < RS; ++i) z[i] += zl[i];
+                    }
+                    return;
+                }
                 tmem_ld<RS>(ta, z);
                 tmem_ld<RS>(ta + (uint32_t)Bp, zl);
                 if (NACC > 1 && nissue > 1) {
@@ -479,7 +546,9 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
                     c[m] = fmaf(z[4 * m + 1], c[m], z[4 * m] * z[4 * m + 2]);
                     hn[m] = z[4 * m + 3] * tanh_fast(c[m]);
                     // (fb0 is a multiple of four: of eight where a thread has more than one item)
-                    if (m < npub) st_relaxed_u32(dst + (m & 1) * 16 + (m >> 1) * 128, pack_word(hn[m], phase_out));
+                    if (m < npub)
+                        st_relaxed_u32(dst + (m & 1) * 16 + (m >> 1) * 128,
+                                       TERMS == 2 ? pack_word(hn[m], phase_out) : (__float_as_uint(hn[m]) & ~kPhaseBit) | phase_out);
                 }
             }
         }
@@ -512,22 +581,25 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
 }
 
 typedef void (*KernelFn)(const RecurTcArgs);
-template <bool PAIR>
+template <bool PAIR, int TERMS>
 KernelFn pick_p(int rg)
 {
     switch (rg) {
-        case 1: return recur_tc_kernel<1, PAIR>;
-        case 2: return recur_tc_kernel<2, PAIR>;
-        case 3: return recur_tc_kernel<3, PAIR>;
-        case 4: return recur_tc_kernel<4, PAIR>;
-        case 5: return recur_tc_kernel<5, PAIR>;
-        case 6: return recur_tc_kernel<6, PAIR>;
-        case 7: return recur_tc_kernel<7, PAIR>;
-        case 8: return recur_tc_kernel<8, PAIR>;
+        case 1: return recur_tc_kernel<1, PAIR, TERMS>;
+        case 2: return recur_tc_kernel<2, PAIR, TERMS>;
+        case 3: return recur_tc_kernel<3, PAIR, TERMS>;
+        case 4: return recur_tc_kernel<4, PAIR, TERMS>;
+        case 5: return recur_tc_kernel<5, PAIR, TERMS>;
+        case 6: return recur_tc_kernel<6, PAIR, TERMS>;
+        case 7: return recur_tc_kernel<7, PAIR, TERMS>;
+        case 8: return recur_tc_kernel<8, PAIR, TERMS>;
         default: return nullptr;
     }
 }
-KernelFn pick(int rg, bool pair) { return pair ? pick_p<true>(rg) : pick_p<false>(rg); }
+KernelFn pick(int rg, bool pair, int terms)
+{
+    return terms == 3 ? (pair ? pick_p<true, 3>(rg) : pick_p<false, 3>(rg)) : (pair ? pick_p<true, 2>(rg) : pick_p<false, 2>(rg));
+}
 int groups_of(int rows) { return (rows + 7) / 8; }
 
 cudaLaunchConfig_t config(cudaLaunchAttribute (&attr)[2], int grid, size_t smem, int pair, cudaStream_t st)
@@ -545,17 +617,17 @@ cudaLaunchConfig_t config(cudaLaunchAttribute (&attr)[2], int grid, size_t smem,
 
 }  // namespace
 
-size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair)
+size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair, int terms)
 {
     const int rg = groups_of(rows);
-    return 1024 + (size_t)((KH + 63) / 64) * (16 * rg) * 128 + (pair ? (size_t)2 * 8 * upc * tc_rows_of_first(rg, true) * 4 : 0);
+    return 1024 + (size_t)((KH + 63) / 64) * tc_columns(rg, terms) * 128 + (pair ? (size_t)2 * 8 * upc * tc_rows_of_first(rg, true) * 4 : 0);
 }
 
 size_t recur_tc_xch_words(int H, int rows, int dirs) { return (size_t)dirs * 2 * ((H + 15) / 16) * groups_of(rows) * 128; }
 
 // Partition of H units over at most max_cta CTAs, and the most batch rows (<= rows_wanted) a pass can take; false when
 // the slice does not fit tensor memory.
-bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, size_t max_smem, RecurTcPlan *p)
+bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, int terms, size_t max_smem, RecurTcPlan *p)
 {
     if (pair && H <= 64) return false;                                  // both halves of K must exist
     int upc = 4, n = 0;
@@ -567,19 +639,19 @@ bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, size_t max_sme
     if (upc > 16) return false;
     const int KH = ((pair ? (H + 1) / 2 : H) + 15) / 16 * 16;
     for (int rg = groups_of(rows_wanted < kTcMaxRows ? rows_wanted : kTcMaxRows); rg >= 1; --rg) {
-        if (KH / 2 + tc_acc_columns(rg) <= 512 && KH <= 16 * kPollers * kMaxGroups && recur_tc_smem_bytes(KH, upc, 8 * rg, pair) <= max_smem) {
-            p->upc = upc; p->ncta = n; p->KH = KH; p->pair = pair; p->rows = 8 * rg;
+        if (KH / 2 + tc_acc_columns(rg, terms) <= 512 && KH <= 16 * kPollers * kMaxGroups && recur_tc_smem_bytes(KH, upc, 8 * rg, pair, terms) <= max_smem) {
+            p->upc = upc; p->ncta = n; p->KH = KH; p->pair = pair; p->rows = 8 * rg; p->terms = terms;
             return true;
         }
     }
     return false;
 }
 
-cudaError_t recur_tc_prepare(int max_smem)
+cudaError_t recur_tc_prepare(int terms, int max_smem)
 {
     for (int rg = 1; rg <= kTcMaxRows / 8; ++rg) {
         for (int pair = 0; pair < 2; ++pair) {
-            const cudaError_t e = cudaFuncSetAttribute(pick(rg, pair != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+            const cudaError_t e = cudaFuncSetAttribute(pick(rg, pair != 0, terms), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
             if (e != cudaSuccess) return e;
         }
     }
@@ -587,13 +659,13 @@ cudaError_t recur_tc_prepare(int max_smem)
 }
 
 // Can `grid` CTAs of this kernel be co-resident as clusters of two (pair mode needs every pair on one GPC)?
-bool recur_tc_pair_supported(int grid, int rows, size_t smem)
+bool recur_tc_pair_supported(int grid, const RecurTcPlan &p)
 {
     cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = config(attr, grid, smem, 1, nullptr);
+    cudaLaunchConfig_t cfg = config(attr, grid, recur_tc_smem_bytes(p.KH, p.upc, p.rows, 1, p.terms), 1, nullptr);
     cfg.attrs = attr + 1; cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)pick(groups_of(rows), true), &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)pick(groups_of(p.rows), true, p.terms), &cfg) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -602,12 +674,12 @@ bool recur_tc_pair_supported(int grid, int rows, size_t smem)
 
 cudaError_t launch_recur_tc(const RecurTcArgs &a, cudaStream_t st)
 {
-    KernelFn fn = pick(groups_of(a.B), a.pair != 0);
+    KernelFn fn = pick(groups_of(a.B), a.pair != 0, a.terms);
     if (!fn) return cudaErrorInvalidValue;
     RecurTcArgs copy = a;
     void *params[] = {&copy};
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = config(attr, a.ncta_dir * (a.ndirs ? a.ndirs : a.D), recur_tc_smem_bytes(a.KH, a.upc, a.B, a.pair), a.pair, st);
+    const cudaLaunchConfig_t cfg = config(attr, a.ncta_dir * (a.ndirs ? a.ndirs : a.D), recur_tc_smem_bytes(a.KH, a.upc, a.B, a.pair, a.terms), a.pair, st);
     return cudaLaunchKernelExC(&cfg, (const void *)fn, params);
 }
 
