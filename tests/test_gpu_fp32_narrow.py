@@ -24,6 +24,18 @@ def test_fp32_narrow(oracle, s):
         assert_close(run_gpu(w, weights, x, h0, c0, chunks=[1, T - 1]), ref, "fp32", "fp32 narrow, chunked")
 
 
+@pytest.mark.parametrize("size", [1e-6, 1e-12, 1e-30])
+def test_fp32_narrow_keeps_the_digits_of_small_values(oracle, size):
+    """Gate pre-activations of this size: tanh z = z and logistic = 1/2 to all digits, every value keeps its fp32 precision."""
+    import numpy as np
+    w = wl.Workload("small", 1, False, 24, 100, 3, 12, "fp32", 0.1, seed=3)
+    weights, x = wl.make(w)
+    for q in weights:
+        q["wx"], q["b"] = np.float32(q["wx"] * size), np.float32(q["b"] * size)
+    ref = oracle.forward(weights, x, layers=1, bidir=False, hidden=100)
+    assert_close(run_gpu(w, weights, x), ref, "fp32", f"small values {size}")
+
+
 def test_fp32_projection_of_more_rows_than_a_grid_has_in_y():
     """T x B = 2 100 000 rows, more than 65535 tiles of 32; every row against the product in float64."""
     import torch
