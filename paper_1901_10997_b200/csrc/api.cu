@@ -38,7 +38,7 @@ struct Layer {
     int nkw_ox = 0;
     uint4 *xfrag[2] = {nullptr, nullptr};  //   and Wx in the same layout (projection fused into the kernel's prologue)
     int nkw_x = 0;
-    uint4 *wtc[2] = {nullptr, nullptr};    // batched tensor-core kernel: [cta][8-column piece][row 4 * unit + gate]
+    uint4 *wtc[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // batched tensor-core kernel, by plan and direction: [cta][8-column piece][row 4 * unit + gate]
     uint4 *frag2[2] = {nullptr, nullptr};  // H-LSTM: fragments of the gate output matrices W
     uint4 *tfrag[2] = {nullptr, nullptr}, *tfrag2[2] = {nullptr, nullptr};     //   the tile kernel's fragments of Uh and W
     float *bias_out = nullptr;             // H-LSTM: [D][H][4] bias of the gate pre-activations
@@ -75,10 +75,11 @@ struct lstm_handle {
     long long csr_conflicts = 0;       // shared-memory wavefronts per step and CTA lost to bank conflicts (worst CTA, worst matrix)
     int mma_mt = 0, mma_nkr = 0, mma_nks = 0, mma_nw = 0;
     bool seq_dirs = false;             // bidirectional layers run one direction after the other, each on all SMs
-    // batched tensor-core recurrence: partition and exchange words (two sets: a launch uses one and clears the other)
-    bool use_tcb = false;
-    RecurTcPlan tcb = {0, 0, 0, 0, 0, 0};
-    unsigned *tcb_xch = nullptr, *tcb_turn = nullptr;
+    // batched tensor-core recurrence: partition and exchange words (two sets: a launch uses one and clears the other).  Narrow
+    // layers have a second plan, every CTA on its own, for calls with up to tc_single_rows rows.
+    bool use_tcb = false, use_tc1 = false;
+    RecurTcPlan tcb[2] = {{0, 0, 0, 0, 0, 0}, {0, 0, 0, 0, 0, 0}};
+    unsigned *tcb_xch[2] = {nullptr, nullptr}, *tcb_turn[2] = {nullptr, nullptr};
     unsigned *f32_xch = nullptr, *f32_turn = nullptr;  // fp32 dense, at most two units per CTA: exchange words (two sets)
     // H-LSTM cell: width of the hidden layer inside each gate (0: plain LSTM), pass-2 column tiles per warp
     int Hh = 0, hl_nkw2 = 0;
@@ -484,6 +485,17 @@ std::vector<uint32_t> pack_ht_gates(const float *w, const HlstmTilePlan &p)
 // register-resident kernel (2 x 1500, T = 35: two rows 288 us, 208 us on the tensor cores).
 int tc_min_rows(const lstm_handle *) { return 2; }
 
+// Most rows for which the batched kernel runs narrow layers without cluster pairs: the products are short there, and the
+// partner's partial sums cost more than half of them saves.  Pairs / single CTAs, time per call of one layer, T = 35: H = 128
+// with 2, 8, 32, 48 rows 1.19, 1.03, 1.03, 0.96; 256 1.04, 1.09, 0.99, 0.92; 400 1.04, 1.03, 0.97, 0.85; 512 1.05, 1.05, 0.92,
+// 0.80; 600 with 2 rows 0.95.  Two directions the same up to 256, then even.  Pruned layers (three terms of h, so twice the
+// splitting in a CTA alone): 256 with 2, 8, 16, 24 rows 1.10, 1.09, 1.05, 0.96; 512 1.09, 1.05, 0.94, 0.86.
+int tc_single_rows(int H, int D, int terms)
+{
+    if (terms == 3) return H <= 256 ? 16 : H <= 512 ? 8 : 0;
+    return H <= 256 ? 32 : D == 2 ? 0 : H <= 400 ? 24 : H <= 512 ? 16 : 0;
+}
+
 // Rows of a [4H x H] recurrent matrix (row q*H + j) as the batched tensor-core kernel wants them: per CTA [8-column
 // piece of its K range][row 4 * unit + gate of its units, in pair mode of both CTAs' units] 8 bf16.
 std::vector<uint16_t> pack_tc_rows(const float *m, int H, const RecurTcPlan &p)
@@ -539,10 +551,11 @@ void free_all(lstm_handle *h)
     for (auto &ly : h->layers) {
         cudaFree(ly.wx); cudaFree(ly.bias); cudaFree(ly.wx_rowptr); cudaFree(ly.wx_ent);
         for (int d = 0; d < 2; ++d) { cudaFree(ly.wh[d]); cudaFree(ly.wh_ptr[d]); cudaFree(ly.wh_ent[d]); cudaFree(ly.wfrag[d]); cudaFree(ly.ofrag[d]); cudaFree(ly.oxfrag[d]); cudaFree(ly.xfrag[d]); cudaFree(ly.frag2[d]); cudaFree(ly.tfrag[d]); cudaFree(ly.tfrag2[d]); cudaFree(ly.csr_reg_ent[d]); cudaFree(ly.csr_reg_rows[d]); }
-        cudaFree(ly.bias_out); cudaFree(ly.wtc[0]); cudaFree(ly.wtc[1]);
+        cudaFree(ly.bias_out);
+        for (int i = 0; i < 4; ++i) cudaFree(ly.wtc[i >> 1][i & 1]);
     }
     cudaFree(h->G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
-    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); cudaFree(h->tcb_xch); cudaFree(h->ht_hx); cudaFree(h->f32_xch); cudaFree(h->one_xch); cudaFree(h->ht_rx); cudaFree(h->status_dev);
+    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); cudaFree(h->tcb_xch[0]); cudaFree(h->tcb_xch[1]); cudaFree(h->ht_hx); cudaFree(h->f32_xch); cudaFree(h->one_xch); cudaFree(h->ht_rx); cudaFree(h->status_dev);
     for (int l = 0; l < kMaxWaveLayers; ++l) cudaFree(h->wave_frag[l]);
     cudaFree(h->wave_xch);
     cudaFree(h->cmap); cudaFree(h->rem_idx); cudaFree(h->rem_bias);
@@ -675,9 +688,13 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         if (!bf16 || (csr && !h->csr_dense_proj) || max_B < tc_min_rows(h) || (env && (strcmp(env, "mma") == 0 || strcmp(env, "simt") == 0))) return false;
         const size_t smem = (size_t)h->smem_optin - kTcStaticSmem;
         if (recur_tc_prepare(tc_terms, (int)smem) != cudaSuccess) { cudaGetLastError(); return false; }
-        if (!(env && strcmp(env, "tc1") == 0) && recur_tc_plan(H, ncta, max_B, 1, tc_terms, smem, &h->tcb) &&
-            recur_tc_pair_supported(h->tcb.ncta * dirs_side_by_side, h->tcb)) return true;
-        return recur_tc_plan(H, ncta, max_B, 0, tc_terms, smem, &h->tcb);
+        if (!(env && strcmp(env, "tc1") == 0) && recur_tc_plan(H, ncta, max_B, 1, tc_terms, smem, &h->tcb[0]) &&
+            recur_tc_pair_supported(h->tcb[0].ncta * dirs_side_by_side, h->tcb[0])) {
+            const int rows = std::min(max_B, tc_single_rows(H, D, tc_terms));
+            h->use_tc1 = rows > 0 && recur_tc_plan(H, ncta, rows, 0, tc_terms, smem, &h->tcb[1]);
+            return true;
+        }
+        return recur_tc_plan(H, ncta, max_B, 0, tc_terms, smem, &h->tcb[0]);
     };
     h->use_tcb = plan_tcb(h->ncta_dir, D);
     if (D == 2 && bf16 && !csr && !h->use_mma && !h->use_tcb) {
@@ -811,9 +828,10 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                     rc = upload(h, &ly.wh[d], p.data(), n * 4, st, "recurrent weights");
                     if (rc == LSTM_OK) cudaStreamSynchronize(st);
                 }
-                if (rc == LSTM_OK && h->use_tcb) {
-                    const std::vector<uint16_t> p = pack_tc_rows(m.data(), H, h->tcb);
-                    rc = upload(h, (uint16_t **)&ly.wtc[d], p.data(), p.size() * 2, st, "recurrent weight rows");
+                for (int i = 0; i < 2 && rc == LSTM_OK; ++i) {
+                    if (!(i ? h->use_tc1 : h->use_tcb)) continue;
+                    const std::vector<uint16_t> p = pack_tc_rows(m.data(), H, h->tcb[i]);
+                    rc = upload(h, (uint16_t **)&ly.wtc[i][d], p.data(), p.size() * 2, st, "recurrent weight rows");
                     if (rc == LSTM_OK) cudaStreamSynchronize(st);
                 }
             } else {
@@ -852,9 +870,11 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                     std::vector<float> m((size_t)4 * H * H, 0.0f);
                     for (int r = 0; r < 4 * H; ++r)
                         for (int e = ch.rowptr[r]; e < ch.rowptr[r + 1]; ++e) m[(size_t)r * H + ch.col[e]] = ch.val[e];
-                    const std::vector<uint16_t> p = pack_tc_rows(m.data(), H, h->tcb);
-                    rc = upload(h, (uint16_t **)&ly.wtc[d], p.data(), p.size() * 2, st, "recurrent weight rows");
-                    if (rc == LSTM_OK) cudaStreamSynchronize(st);
+                    for (int i = 0; i < (h->use_tc1 ? 2 : 1) && rc == LSTM_OK; ++i) {
+                        const std::vector<uint16_t> p = pack_tc_rows(m.data(), H, h->tcb[i]);
+                        rc = upload(h, (uint16_t **)&ly.wtc[i][d], p.data(), p.size() * 2, st, "recurrent weight rows");
+                        if (rc == LSTM_OK) cudaStreamSynchronize(st);
+                    }
                     if (rc) break;
                 }
                 if (h->use_csr_reg) {
@@ -950,7 +970,8 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     }
     if (rc == LSTM_OK && dtype == LSTM_F32 && !csr && h->upc <= 2 && H <= kF32MaxUnits)
         rc = alloc_xch(h, &h->f32_xch, &h->f32_turn, (size_t)2 * D * 2 * H * 32, st);
-    if (rc == LSTM_OK && h->use_tcb) rc = alloc_xch(h, &h->tcb_xch, &h->tcb_turn, 2 * (recur_tc_xch_words(H, h->tcb.rows, D) + kTcXchSlack), st);
+    for (int i = 0; i < 2 && rc == LSTM_OK; ++i)
+        if (i ? h->use_tc1 : h->use_tcb) rc = alloc_xch(h, &h->tcb_xch[i], &h->tcb_turn[i], 2 * (recur_tc_xch_words(H, h->tcb[i].rows, D) + kTcXchSlack), st);
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->status_dev, sizeof(int), true, st, "status word");
     if (rc == LSTM_OK && h->use_wave) {
         h->wave_xch_words = (size_t)layers * max_T * std::min(max_B, 4) * H;
@@ -1558,18 +1579,20 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             continue;
         }
         if (h->use_tcb && B >= tc_min_rows(h)) {
-            // passes of at most tcb.rows batch rows, as equal as possible
-            const int passes = (B + h->tcb.rows - 1) / h->tcb.rows, dirs = h->seq_dirs ? 1 : D;
+            // passes of at most plan.rows batch rows, as equal as possible
+            const int which = h->use_tc1 && B <= h->tcb[1].rows ? 1 : 0;
+            const RecurTcPlan &plan = h->tcb[which];
+            const int passes = (B + plan.rows - 1) / plan.rows, dirs = h->seq_dirs ? 1 : D;
             for (int p = 0; p < passes; ++p) {
                 RecurTcArgs m;
                 memset(&m, 0, sizeof m);
                 m.dir0 = h->seq_dirs ? pass : 0; m.ndirs = dirs;
                 m.Bs = B; m.b0 = (int)((long long)B * p / passes); m.B = (int)((long long)B * (p + 1) / passes) - m.b0;
                 m.H = H; m.T = T; m.D = D; m.nsplit = nsplit;
-                m.ncta_dir = h->tcb.ncta; m.upc = h->tcb.upc; m.KH = h->tcb.KH; m.pair = h->tcb.pair; m.terms = h->tcb.terms;
+                m.ncta_dir = plan.ncta; m.upc = plan.upc; m.KH = plan.KH; m.pair = plan.pair; m.terms = plan.terms;
                 m.spin_limit = h->spin_limit;
-                m.withhold_cta = h->withhold_cta < 0 ? -1 : h->withhold_cta % (h->tcb.ncta * dirs);
-                m.wpack[0] = ly.wtc[0]; m.wpack[1] = ly.wtc[1];
+                m.withhold_cta = h->withhold_cta < 0 ? -1 : h->withhold_cta % (plan.ncta * dirs);
+                m.wpack[0] = ly.wtc[which][0]; m.wpack[1] = ly.wtc[which][1];
                 m.G = h->G;
                 m.g_split_stride = (long long)M * N;
                 const size_t so = (size_t)l * D * B * H;
@@ -1579,7 +1602,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                 m.y = l == L - 1 ? y : m.xb_next ? nullptr : h->ybuf[l & 1];
                 m.xb_ld = h->ldn;
                 m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
-                m.xch = h->tcb_xch; m.set_words = recur_tc_xch_words(H, h->tcb.rows, D) + kTcXchSlack; m.used_words = (unsigned)recur_tc_xch_words(H, m.B, dirs); m.turn = h->tcb_turn;
+                m.xch = h->tcb_xch[which]; m.set_words = recur_tc_xch_words(H, plan.rows, D) + kTcXchSlack; m.used_words = (unsigned)recur_tc_xch_words(H, m.B, dirs); m.turn = h->tcb_turn[which];
                 m.status = h->status_dev;
                 if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 e = launch_recur_tc(m, st);
@@ -1916,7 +1939,7 @@ int lstm_info(const lstm_handle *h, int64_t *out, int n)
     }
     const Layer &l0 = h->layers[0];
     const int launches = h->last_launches > 0 ? h->last_launches : h->L * 2 + (h->use_tc ? 1 : 0);
-    const int tcb_at_max = h->use_tcb ? (h->tcb.pair ? 2 : 1) : 0;
+    const int tcb_at_max = h->use_tcb ? (h->tcb[0].pair ? 2 : 1) : 0;
     if (h->use_csr_reg) shp.smem = recur_csr_reg_smem_bytes(h->csr_nw, h->csr_kspan, h->csr_mt, h->upc, h->max_B);
     const int64_t vals[23] = {h->sm_count, h->ncta_dir, h->use_mma ? h->mma_nw * 32 : h->use_csr_reg ? h->csr_nw * 32 : h->threads, (int64_t)shp.smem,
                               rows_res, rows_str, (l0.plan_M >= 0) ? l0.plan.nsplit : 1, h->use_tc ? 1 : 0, launches,
