@@ -109,7 +109,8 @@ typedef struct {
  *   LSTM_B200_FUSE  = 0     never compute the input projection inside the recurrent kernel (single sequences of up
  *                           to 40 steps on the register-resident kernel do so by default)
  *   LSTM_B200_WAVE  = 0     one launch per layer even where the layer-wavefront kernel would serve the stack
- *                   = 1     the layer-wavefront kernel for single timesteps too, where it serves the stack
+ *                   = 1     the layer-wavefront kernel for every call of up to four sequences, single timesteps
+ *                           included, where it serves the stack
  *   LSTM_B200_PROJ  = simt  CUDA-core input projection instead of the tensor-core one
  *                   = csr   CSR handles walk the lists of Wx in the projection too (by default bf16 CSR handles keep a
  *                           dense copy of Wx and project on the tensor cores; the recurrence stays sparse)

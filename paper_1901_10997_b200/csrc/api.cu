@@ -496,6 +496,25 @@ int tc_single_rows(int H, int D, int terms)
     return H <= 256 ? 32 : D == 2 ? 0 : H <= 400 ? 24 : H <= 512 ? 16 : 0;
 }
 
+// Does the layer-wavefront kernel serve a call?  One sequence always; two to four where one chain of T + L - 1 steps, with a product
+// per row and only layer 0's projection, beats L times T steps and projections of the batched kernel.  Time per call, wavefront /
+// batched: two layers, H = 128, 3 rows, T = 35 95 / 135 us; 256, 4 rows, T = 70 202 / 239; 512, T = 35 with 2, 3, 4 rows 0.68,
+// 0.92, 1.18, T = 70 with 3 rows 1.10 (3 T > 128 rows take the unsplit projection, which favours the batched kernel), T = 20
+// with 4 rows 1.02; 600 with 2 rows 0.89 - 0.94, with 3 rows 0.92 at T = 8, 1.06 at 23; 800 with 2 rows 0.91 at T = 16, 0.98 at
+// 23, 1.06 at 50; 900 1.21.  Three layers, T = 70: 512 with 4 rows 0.90, 600 with 3 rows 0.94, with 4 1.16, 760 with 2 rows 0.86,
+// with 3 1.10.  Four layers: 0.5 - 0.93 up to the widest (H = 592).
+bool wave_serves(const lstm_handle *h, int T, int B)
+{
+    if (!h->use_wave || B > 4 || h->probe) return false;          // (the probe builds exist for the per-layer kernels)
+    if (B == 1 || h->wave_all || !h->use_tcb || h->L >= 4) return true;
+    const int H = h->H, M = T * B;
+    if (h->L == 3) return H <= 512 || B <= (H <= 640 ? 3 : 2) || M <= 32;
+    if (H <= 256) return true;
+    if (H <= 512) return B == 2 || M <= (B == 3 ? 128 : 80);
+    if (H <= 640) return B == 2 || (B == 3 && T <= 8);
+    return H <= 800 && B == 2 && T <= 24;
+}
+
 // Rows of a [4H x H] recurrent matrix (row q*H + j) as the batched tensor-core kernel wants them: per CTA [8-column
 // piece of its K range][row 4 * unit + gate of its units, in pair mode of both CTAs' units] 8 bf16.
 std::vector<uint16_t> pack_tc_rows(const float *m, int H, const RecurTcPlan &p)
@@ -1470,9 +1489,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         return LSTM_OK;
     }
 
-    // The layer-wavefront kernel serves one sequence, and two where the step is short enough for its product per row (2 x 517, T = 23,
-    // two rows: 108 us against 127 us batched; 2 x 800, T = 35: 179 against 183; three rows: 144 against 135)
-    if (h->use_wave && B <= (!h->use_tcb || h->wave_all ? 4 : H <= 800 ? 2 : 1) && !h->probe) {          // (the probe builds exist for the per-layer kernels)
+    if (wave_serves(h, T, B)) {
         // all layers in one launch: layer 0's projection for all timesteps, then the wavefront kernel
         int nsplit = 1;
         { const int prc = run_projection(h, 0, x, x, M, D * 4 * H, &nsplit, st); if (prc != LSTM_OK) return prc; }

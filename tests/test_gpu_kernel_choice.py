@@ -48,6 +48,15 @@ CASES = [
     (("lstm", "bf16", False, 2, 300, 1, 8, 1.0), "STEP", 256),
     (("hlstm", "bf16", False, 1, 300, 3, 9, 1.0), "HLSTM_TILES", 512),
     (("hlstm", "bf16", False, 1, 300, 3, 2, 1.0), "HLSTM_TILES", 512),
+    # two to four rows of stacks that fit the wavefront kernel, and just beyond where it is the faster one
+    (("lstm", "bf16", False, 2, 200, 40, 4, 1.0), "WAVE", 512),
+    (("lstm", "bf16", False, 2, 300, 40, 3, 1.0), "WAVE", 512),
+    (("lstm", "bf16", False, 2, 300, 45, 3, 1.0), "BATCHED", 512),
+    (("lstm", "bf16", False, 2, 300, 30, 4, 1.0), "BATCHED", 512),
+    (("lstm", "bf16", False, 2, 700, 24, 2, 1.0), "WAVE", 512),
+    (("lstm", "bf16", False, 2, 700, 25, 2, 1.0), "BATCHED", 512),
+    (("lstm", "bf16", False, 3, 400, 40, 4, 1.0), "WAVE", 512),
+    (("lstm", "bf16", False, 4, 300, 40, 4, 1.0, 9), "WAVE", 512),
     # one sequence, on a handle made for one and on one made for several
     (("hlstm", "bf16", False, 1, 300, 3, 1, 1.0), "HLSTM_ROWS", None),
     (("hlstm", "bf16", True, 1, 300, 3, 1, 1.0, 20), "HLSTM_ROWS", None),
