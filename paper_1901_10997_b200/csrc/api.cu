@@ -515,6 +515,12 @@ bool wave_serves(const lstm_handle *h, int T, int B)
     return H <= 800 && B == 2 && T <= 24;
 }
 
+// Does the list kernel serve a call of a pruned handle?  One sequence always; a few rows for a few steps, where reading the whole
+// dense slice does not pay.  Time per call, lists / batched (the better of its plans), two layers, density 0.1: one step with 2 - 4
+// rows 0.82 - 0.98; two steps with 2, 4 rows 0.87 - 0.99, 0.96 - 1.01; three and four steps with 2 rows 0.89 - 0.98, with 3 rows
+// 1.00 - 1.09; six steps with 2 rows 0.95 - 1.07; one step with 5 rows 1.00 - 1.08.
+bool lists_serve(const lstm_handle *h, int T, int B) { return h->use_csr_reg && (B == 1 || !h->use_tcb || (B <= 4 && T * B <= 8)); }
+
 // Rows of a [4H x H] recurrent matrix (row q*H + j) as the batched tensor-core kernel wants them: per CTA [8-column
 // piece of its K range][row 4 * unit + gate of its units, in pair mode of both CTAs' units] 8 bf16.
 std::vector<uint16_t> pack_tc_rows(const float *m, int H, const RecurTcPlan &p)
@@ -1595,7 +1601,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             continue;
         }
-        if (h->use_tcb && B >= tc_min_rows(h)) {
+        if (h->use_tcb && B >= tc_min_rows(h) && !lists_serve(h, T, B)) {
             // passes of at most plan.rows batch rows, as equal as possible
             const int which = h->use_tc1 && B <= h->tcb[1].rows ? 1 : 0;
             const RecurTcPlan &plan = h->tcb[which];

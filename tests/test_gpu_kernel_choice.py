@@ -57,6 +57,11 @@ CASES = [
     (("lstm", "bf16", False, 2, 700, 25, 2, 1.0), "BATCHED", 512),
     (("lstm", "bf16", False, 3, 400, 40, 4, 1.0), "WAVE", 512),
     (("lstm", "bf16", False, 4, 300, 40, 4, 1.0, 9), "WAVE", 512),
+    # a few rows of a pruned handle for a few steps
+    (("lstm", "bf16", False, 2, 600, 1, 4, 0.1), "SPARSE", 512),
+    (("lstm", "bf16", True, 1, 600, 4, 2, 0.1, 16), "SPARSE", 512),
+    (("lstm", "bf16", False, 2, 600, 3, 3, 0.1), "BATCHED", 512),
+    (("lstm", "bf16", False, 2, 600, 1, 5, 0.1), "BATCHED", 512),
     # one sequence, on a handle made for one and on one made for several
     (("hlstm", "bf16", False, 1, 300, 3, 1, 1.0), "HLSTM_ROWS", None),
     (("hlstm", "bf16", True, 1, 300, 3, 1, 1.0, 20), "HLSTM_ROWS", None),
