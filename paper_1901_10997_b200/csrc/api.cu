@@ -1530,7 +1530,11 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         int nsplit = 1;
         // ---- input staging + projection (a single short sequence on the register-resident kernel computes its
         // projection inside that kernel's prologue instead: two launches and one round trip of G fewer per layer)
-        const bool one = h->use_one && B == 1;
+        // Directions in turn: every launch pays the prologue, which is longer on fewer CTAs with larger slices; the shorter step makes
+        // up for it from about twenty steps on where they are nearly all SMs.  Time per call, one layer, recur_mma / recur_one:
+        // H = 1700 (142 CTAs) T = 2, 10, 20, 35, 100 0.80, 0.99, 1.07, 1.12, 1.07; 1500 (125) 0.75, 0.92, 1.01, 1.03, 1.01;
+        // 1300 (109) 0.82, 0.90, 0.96, 0.99, 1.01; 1190 (100) 0.83, 0.91, 0.94, 0.97, 0.97.
+        const bool one = h->use_one && B == 1 && (!h->seq_dirs || (T >= 20 && 5 * h->one.ncta >= 4 * h->sm_count));
         const bool fuse = one ? h->one_fuse && T <= kFuseMaxT && !h->probe : (h->fuse_ok || (h->csr_fuse_ok && h->use_csr_reg)) && !h->Hh && B == 1 && T <= kFuseMaxT && !h->probe &&
                           ly.xfrag[0] != nullptr;
         if (!fuse) { const int prc = run_projection(h, l, l == 0 ? x : nullptr, Xf, M, N, &nsplit, st); if (prc != LSTM_OK) return prc; }

@@ -62,6 +62,11 @@ CASES = [
     (("lstm", "bf16", True, 1, 600, 4, 2, 0.1, 16), "SPARSE", 512),
     (("lstm", "bf16", False, 2, 600, 3, 3, 0.1), "BATCHED", 512),
     (("lstm", "bf16", False, 2, 600, 1, 5, 0.1), "BATCHED", 512),
+    # wide directions in turn: short calls, and widths that would leave a quarter of the SMs idle
+    (("lstm", "bf16", True, 1, 1500, 19, 1, 1.0), "REGISTERS", 512),
+    (("lstm", "bf16", True, 1, 1500, 20, 1, 1.0), "ONE", 512),
+    (("lstm", "bf16", True, 1, 1300, 41, 1, 1.0), "REGISTERS", 512),
+    (("lstm", "bf16", True, 1, 1100, 3, 1, 1.0), "ONE", 512),
     # one sequence, on a handle made for one and on one made for several
     (("hlstm", "bf16", False, 1, 300, 3, 1, 1.0), "HLSTM_ROWS", None),
     (("hlstm", "bf16", True, 1, 300, 3, 1, 1.0, 20), "HLSTM_ROWS", None),
