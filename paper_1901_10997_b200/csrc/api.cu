@@ -482,8 +482,9 @@ std::vector<uint32_t> pack_ht_gates(const float *w, const HlstmTilePlan &p)
 }
 
 // Fewest batch rows the batched tensor-core recurrence serves: from two on it beats the passes of up to four rows of the
-// register-resident kernel (2 x 1500, T = 35: two rows 288 us, 208 us on the tensor cores).
-int tc_min_rows(const lstm_handle *) { return 2; }
+// register-resident kernel (time per call of one layer, T = 35, that kernel / batched, two rows: H = 128 1.07, 256 0.96, 400 1.15,
+// 512 0.99, 800 1.28, 1024 1.33; two directions 1.04, 0.95, 1.03, 1.01, 1.40, 1.54).
+constexpr int kTcMinRows = 2;
 
 // Most rows for which the batched kernel runs narrow layers without cluster pairs: the products are short there, and the
 // partner's partial sums cost more than half of them saves.  Pairs / single CTAs, time per call of one layer, T = 35: H = 128
@@ -521,9 +522,9 @@ bool wave_serves(const lstm_handle *h, int T, int B)
 // 1.00 - 1.09; six steps with 2 rows 0.95 - 1.07; one step with 5 rows 1.00 - 1.08.
 bool lists_serve(const lstm_handle *h, int T, int B) { return h->use_csr_reg && (B == 1 || !h->use_tcb || (B <= 4 && T * B <= 8)); }
 
-// Rows of a [4H x H] recurrent matrix (row q*H + j) as the batched tensor-core kernel wants them: per CTA [8-column
+// Rows of a [4H x H] recurrent matrix (row q*H + j, dense or as lists) as the batched tensor-core kernel wants them: per CTA [8-column
 // piece of its K range][row 4 * unit + gate of its units, in pair mode of both CTAs' units] 8 bf16.
-std::vector<uint16_t> pack_tc_rows(const float *m, int H, const RecurTcPlan &p)
+std::vector<uint16_t> pack_tc_rows(const float *m, const HostCsr *lists, int H, const RecurTcPlan &p)
 {
     const int units = p.pair ? 2 * p.upc : p.upc, rows = 4 * units, pieces = p.KH / 8;
     std::vector<uint16_t> out((size_t)p.ncta * pieces * rows * 8, 0);
@@ -531,6 +532,16 @@ std::vector<uint16_t> pack_tc_rows(const float *m, int H, const RecurTcPlan &p)
         const int k0 = p.pair ? (c & 1) * p.KH : 0, k1 = std::min(H, k0 + p.KH), u0 = (p.pair ? c / 2 : c) * units;
         uint16_t *dst = out.data() + (size_t)c * pieces * rows * 8;
         const int nu = std::max(0, std::min(units, H - u0));
+        if (lists) {
+            for (int r = 0; r < 4 * nu; ++r) {
+                const int row = (r & 3) * H + u0 + (r >> 2);
+                const int *col = lists->col.data();
+                const int e1 = lists->rowptr[row + 1];
+                for (int e = (int)(std::lower_bound(col + lists->rowptr[row], col + e1, k0) - col); e < e1 && col[e] < k1; ++e)
+                    dst[((size_t)((col[e] - k0) >> 3) * rows + r) * 8 + ((col[e] - k0) & 7)] = f32_to_bf16_rne(lists->val[e]);
+            }
+            return;
+        }
         for (int k = k0; k < k1; k += 8) {                      // reads run down the rows, writes are contiguous
             const int n = std::min(8, k1 - k);
             uint16_t *d8 = dst + (size_t)((k - k0) >> 3) * rows * 8;
@@ -710,7 +721,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     const int tc_terms = csr ? 3 : 2;
     auto plan_tcb = [&](int ncta, int dirs_side_by_side) -> bool {
         const char *env = getenv("LSTM_B200_RECUR");
-        if (!bf16 || (csr && !h->csr_dense_proj) || max_B < tc_min_rows(h) || (env && (strcmp(env, "mma") == 0 || strcmp(env, "simt") == 0))) return false;
+        if (!bf16 || (csr && !h->csr_dense_proj) || max_B < kTcMinRows || (env && (strcmp(env, "mma") == 0 || strcmp(env, "simt") == 0))) return false;
         const size_t smem = (size_t)h->smem_optin - kTcStaticSmem;
         if (recur_tc_prepare(tc_terms, (int)smem) != cudaSuccess) { cudaGetLastError(); return false; }
         if (!(env && strcmp(env, "tc1") == 0) && recur_tc_plan(H, ncta, max_B, 1, tc_terms, smem, &h->tcb[0]) &&
@@ -855,7 +866,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                 }
                 for (int i = 0; i < 2 && rc == LSTM_OK; ++i) {
                     if (!(i ? h->use_tc1 : h->use_tcb)) continue;
-                    const std::vector<uint16_t> p = pack_tc_rows(m.data(), H, h->tcb[i]);
+                    const std::vector<uint16_t> p = pack_tc_rows(m.data(), nullptr, H, h->tcb[i]);
                     rc = upload(h, (uint16_t **)&ly.wtc[i][d], p.data(), p.size() * 2, st, "recurrent weight rows");
                     if (rc == LSTM_OK) cudaStreamSynchronize(st);
                 }
@@ -892,11 +903,8 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                 rc = matrix_to_csr(h, 4 * H, H, src.wh, src.mask_h, src.wh_rowptr, src.wh_col, src.wh_val, ch, name);
                 if (rc) break;
                 if (h->use_tcb) {
-                    std::vector<float> m((size_t)4 * H * H, 0.0f);
-                    for (int r = 0; r < 4 * H; ++r)
-                        for (int e = ch.rowptr[r]; e < ch.rowptr[r + 1]; ++e) m[(size_t)r * H + ch.col[e]] = ch.val[e];
                     for (int i = 0; i < (h->use_tc1 ? 2 : 1) && rc == LSTM_OK; ++i) {
-                        const std::vector<uint16_t> p = pack_tc_rows(m.data(), H, h->tcb[i]);
+                        const std::vector<uint16_t> p = pack_tc_rows(nullptr, &ch, H, h->tcb[i]);
                         rc = upload(h, (uint16_t **)&ly.wtc[i][d], p.data(), p.size() * 2, st, "recurrent weight rows");
                         if (rc == LSTM_OK) cudaStreamSynchronize(st);
                     }
@@ -1605,7 +1613,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             continue;
         }
-        if (h->use_tcb && B >= tc_min_rows(h) && !lists_serve(h, T, B)) {
+        if (h->use_tcb && B >= kTcMinRows && !lists_serve(h, T, B)) {
             // passes of at most plan.rows batch rows, as equal as possible
             const int which = h->use_tc1 && B <= h->tcb[1].rows ? 1 : 0;
             const RecurTcPlan &plan = h->tcb[which];
