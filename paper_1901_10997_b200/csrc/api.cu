@@ -50,6 +50,17 @@ struct Layer {
     int plan_M = -1;
 };
 
+// Exchange words with a phase bit: [2 sets]; a launch uses one set and clears the other for the next launch.  A launch that is being
+// recorded into a graph runs later, or several times, or never: it uses a second pair of sets, which the graph itself clears
+// before the launch, so that it neither meets words of an earlier run nor changes what ordinary launches find.
+struct PhaseWords {
+    unsigned *words = nullptr;         // [2 sets][set_words], ordinary launches
+    unsigned *recorded = nullptr;      // the same for recorded ones
+    size_t set_words = 0;
+    int set = 0;                       // ordinary launches: whose turn it is
+    unsigned dirty = 0;                // ... and how much of the other set the last one may have written
+};
+
 }  // namespace
 
 struct lstm_handle {
@@ -64,7 +75,7 @@ struct lstm_handle {
     // one sequence: its own partition (whole groups of four units per CTA), fragments and exchange words (two sets)
     bool use_one = false, one_fuse = false;
     RecurOnePlan one = {0, 0, 0, 0};
-    unsigned *one_xch = nullptr, *one_turn = nullptr;
+    PhaseWords one_xch;
     bool step_ok = false;              // single timesteps run on the streaming kernel (lstm_step.cu)
     bool fuse_ok = false;              // short single sequences: projection fused into the register-resident kernel's prologue
     // register-resident sparse kernel (bf16, CSR execution): warps, columns per warp, row tiles, entry slots per lane
@@ -75,17 +86,17 @@ struct lstm_handle {
     long long csr_conflicts = 0;       // shared-memory wavefronts per step and CTA lost to bank conflicts (worst CTA, worst matrix)
     int mma_mt = 0, mma_nkr = 0, mma_nks = 0, mma_nw = 0;
     bool seq_dirs = false;             // bidirectional layers run one direction after the other, each on all SMs
-    // batched tensor-core recurrence: partition and exchange words (two sets: a launch uses one and clears the other).  Narrow
+    // batched tensor-core recurrence: partition and exchange words.  Narrow
     // layers have a second plan, every CTA on its own, for calls with up to tc_single_rows rows.
     bool use_tcb = false, use_tc1 = false;
     RecurTcPlan tcb[2] = {{0, 0, 0, 0, 0, 0}, {0, 0, 0, 0, 0, 0}};
-    unsigned *tcb_xch[2] = {nullptr, nullptr}, *tcb_turn[2] = {nullptr, nullptr};
-    unsigned *f32_xch = nullptr, *f32_turn = nullptr;  // fp32 dense, at most two units per CTA: exchange words (two sets)
+    PhaseWords tcb_xch[2];
+    PhaseWords f32_xch;                // fp32 dense, at most two units per CTA
     // H-LSTM cell: width of the hidden layer inside each gate (0: plain LSTM), pass-2 column tiles per warp
     int Hh = 0, hl_nkw2 = 0;
     bool use_ht = false;               // H-LSTM: the tile kernel serves calls with several rows (use_mma: the row kernel the others)
     HlstmTilePlan ht = {0, 0, 0, 0, 0, 0};
-    unsigned *ht_hx = nullptr, *ht_rx = nullptr, *ht_turn = nullptr;
+    PhaseWords ht_hx, ht_rx;
     unsigned long long *rxch = nullptr; size_t rxch_words = 0;
     std::vector<Layer> layers;
     // workspace
@@ -274,12 +285,39 @@ int dev_alloc(lstm_handle *h, T **dst, size_t bytes, bool zero, cudaStream_t st,
     return LSTM_OK;
 }
 
-// exchange words with a phase bit, two sets, and behind them the words that say whose turn the sets are (device_util.cuh)
-int alloc_xch(lstm_handle *h, unsigned **xch, unsigned **turn, size_t words, cudaStream_t st)
+int alloc_phase_words(lstm_handle *h, PhaseWords &x, size_t set_words, cudaStream_t st)
 {
-    const int rc = dev_alloc(h, xch, (words + 32) * sizeof(unsigned), true, st, "exchange words");
-    if (rc == LSTM_OK) *turn = *xch + words;
+    x.set_words = set_words;
+    return dev_alloc(h, &x.words, 2 * set_words * sizeof(unsigned), true, st, "exchange words");
+}
+// (last of a handle's allocations: what a step touches stays close together)
+int alloc_recorded_words(lstm_handle *h, cudaStream_t st)
+{
+    int rc = LSTM_OK;
+    for (PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->f32_xch, &h->ht_hx, &h->ht_rx})
+        if (rc == LSTM_OK && x->words) rc = dev_alloc(h, &x->recorded, 2 * x->set_words * sizeof(unsigned), true, st, "exchange words");
     return rc;
+}
+
+bool recording(cudaStream_t st)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &status) != cudaSuccess) { cudaGetLastError(); return false; }
+    return status == cudaStreamCaptureStatusActive;
+}
+// The sets of the next launch (rec: it is being recorded): base, the set it uses, and how much of the other one it clears.
+cudaError_t phase_sets(const PhaseWords &x, bool rec, cudaStream_t st, unsigned **base, int *set, unsigned *clear_words)
+{
+    *base = rec ? x.recorded : x.words;
+    *set = rec ? 0 : x.set;
+    if (clear_words) *clear_words = rec ? 0 : x.dirty;
+    return rec ? cudaMemsetAsync(*base, 0, x.set_words * sizeof(unsigned), st) : cudaSuccess;
+}
+void phase_launched(PhaseWords &x, bool rec, unsigned used_words)
+{
+    if (rec) return;
+    x.set ^= 1;
+    x.dirty = used_words;
 }
 
 inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
@@ -489,12 +527,12 @@ constexpr int kTcMinRows = 2;
 // Most rows for which the batched kernel runs narrow layers without cluster pairs: the products are short there, and the
 // partner's partial sums cost more than half of them saves.  Pairs / single CTAs, time per call of one layer, T = 35: H = 128
 // with 2, 8, 32, 48 rows 1.19, 1.03, 1.03, 0.96; 256 1.04, 1.09, 0.99, 0.92; 400 1.04, 1.03, 0.97, 0.85; 512 1.05, 1.05, 0.92,
-// 0.80; 600 with 2 rows 0.95.  Two directions the same up to 256, then even.  Pruned layers (three terms of h, so twice the
+// 0.80 (16 rows 0.99); 600 with 2 rows 0.95.  Two directions the same up to 256, then even.  Pruned layers (three terms of h, so twice the
 // splitting in a CTA alone): 256 with 2, 8, 16, 24 rows 1.10, 1.09, 1.05, 0.96; 512 1.09, 1.05, 0.94, 0.86.
 int tc_single_rows(int H, int D, int terms)
 {
     if (terms == 3) return H <= 256 ? 16 : H <= 512 ? 8 : 0;
-    return H <= 256 ? 32 : D == 2 ? 0 : H <= 400 ? 24 : H <= 512 ? 16 : 0;
+    return H <= 256 ? 32 : D == 2 ? 0 : H <= 400 ? 24 : H <= 512 ? 8 : 0;
 }
 
 // Does the layer-wavefront kernel serve a call?  One sequence always; two to four where one chain of T + L - 1 steps, with a product
@@ -591,7 +629,9 @@ void free_all(lstm_handle *h)
         for (int i = 0; i < 4; ++i) cudaFree(ly.wtc[i >> 1][i & 1]);
     }
     cudaFree(h->G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
-    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); cudaFree(h->tcb_xch[0]); cudaFree(h->tcb_xch[1]); cudaFree(h->ht_hx); cudaFree(h->f32_xch); cudaFree(h->one_xch); cudaFree(h->ht_rx); cudaFree(h->status_dev);
+    cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); 
+    for (const PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->f32_xch, &h->ht_hx, &h->ht_rx}) { cudaFree(x->words); cudaFree(x->recorded); }
+    cudaFree(h->status_dev);
     for (int l = 0; l < kMaxWaveLayers; ++l) cudaFree(h->wave_frag[l]);
     cudaFree(h->wave_xch);
     cudaFree(h->cmap); cudaFree(h->rem_idx); cudaFree(h->rem_bias);
@@ -997,14 +1037,14 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     h->xch_words = (size_t)D * 2 * max_B * H;
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->xch, h->xch_words * 8, true, st, "exchange buffer");
     if (rc == LSTM_OK && h->use_one) {
-        rc = alloc_xch(h, &h->one_xch, &h->one_turn, (size_t)2 * D * 2 * h->one.ncta * 32, st);
+        rc = alloc_phase_words(h, h->one_xch, (size_t)D * 2 * h->one.ncta * 32, st);
         if (rc == LSTM_OK && recur_one_prepare(h->one, h->smem_optin - 64) != cudaSuccess)
             rc = fail(h, LSTM_ERR_CUDA, "one-sequence kernel set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
     }
     if (rc == LSTM_OK && dtype == LSTM_F32 && !csr && h->upc <= 2 && H <= kF32MaxUnits)
-        rc = alloc_xch(h, &h->f32_xch, &h->f32_turn, (size_t)2 * D * 2 * H * 32, st);
+        rc = alloc_phase_words(h, h->f32_xch, (size_t)D * 2 * H * 32, st);
     for (int i = 0; i < 2 && rc == LSTM_OK; ++i)
-        if (i ? h->use_tc1 : h->use_tcb) rc = alloc_xch(h, &h->tcb_xch[i], &h->tcb_turn[i], 2 * (recur_tc_xch_words(H, h->tcb[i].rows, D) + kTcXchSlack), st);
+        if (i ? h->use_tc1 : h->use_tcb) rc = alloc_phase_words(h, h->tcb_xch[i], recur_tc_xch_words(H, h->tcb[i].rows, D) + kTcXchSlack, st);
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->status_dev, sizeof(int), true, st, "status word");
     if (rc == LSTM_OK && h->use_wave) {
         h->wave_xch_words = (size_t)layers * max_T * std::min(max_B, 4) * H;
@@ -1021,6 +1061,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         if (e == cudaSuccess && csr) e = proj_csr_prepare(h->smem_optin - 64);
         if (e != cudaSuccess) rc = fail(h, LSTM_ERR_CUDA, "kernel set-up failed: %s", cudaGetErrorString(e));
     }
+    if (rc == LSTM_OK) rc = alloc_recorded_words(h, st);
     if (rc == LSTM_OK && cudaStreamSynchronize(st) != cudaSuccess)
         rc = fail(h, LSTM_ERR_CUDA, "workspace set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
     if (rc) return bail(rc);
@@ -1327,8 +1368,8 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
     h->xch_words = (size_t)D * 2 * row_B * H;
     h->rxch_words = (size_t)D * 2 * row_B * 4 * Hh;
     if (h->use_ht) {
-        if (rc == LSTM_OK) rc = alloc_xch(h, &h->ht_hx, &h->ht_turn, (size_t)2 * D * 2 * ((H + 15) / 16) * 256, st);
-        if (rc == LSTM_OK) rc = dev_alloc(h, &h->ht_rx, (size_t)2 * D * 2 * ((Hh + 15) / 16) * 1024 * 4, true, st, "hidden-layer exchange words");
+        if (rc == LSTM_OK) rc = alloc_phase_words(h, h->ht_hx, (size_t)D * 2 * ((H + 15) / 16) * 256, st);
+        if (rc == LSTM_OK) rc = alloc_phase_words(h, h->ht_rx, (size_t)D * 2 * ((Hh + 15) / 16) * 1024, st);
     }
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->xch, h->xch_words * 8, true, st, "exchange buffer");
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->rxch, h->rxch_words * 8, true, st, "hidden-layer exchange buffer");
@@ -1339,6 +1380,7 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
         if (e == cudaSuccess) e = proj_tc_prepare();
         if (e != cudaSuccess) rc = fail(h, LSTM_ERR_CUDA, "kernel set-up failed: %s", cudaGetErrorString(e));
     }
+    if (rc == LSTM_OK) rc = alloc_recorded_words(h, st);
     if (rc == LSTM_OK && cudaStreamSynchronize(st) != cudaSuccess)
         rc = fail(h, LSTM_ERR_CUDA, "workspace set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
     if (rc) return bail(rc);
@@ -1531,6 +1573,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         return LSTM_OK;
     }
 
+    const bool rec = recording(st);
     for (int l = 0; l < L; ++l) {
         Layer &ly = h->layers[l];
         const float *Xf = l == 0 ? x : h->ybuf[(l - 1) & 1];
@@ -1570,10 +1613,12 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                 m.xb_next = l < L - 1 ? h->xbn[l & 1] : nullptr;
                 m.xb_ld = h->ldn;
                 m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
-                m.hx = h->ht_hx; m.rx = h->ht_rx; m.turn = h->ht_turn;
+                if (phase_sets(h->ht_hx, rec, st, &m.hx, &m.set, nullptr) != cudaSuccess || phase_sets(h->ht_rx, rec, st, &m.rx, &m.set, nullptr) != cudaSuccess)
+                    return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
                 m.status = h->status_dev;
                 if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 e = launch_hlstm_tile(m, h->ht, st);
+                if (e == cudaSuccess) { phase_launched(h->ht_hx, rec, 0); phase_launched(h->ht_rx, rec, 0); }
                 ran(h, LSTM_RAN_HLSTM_TILES, m.ncta_dir * D, kHtThreads, hlstm_tile_smem_bytes(h->ht, m.B));
                 ++h->last_launches;
                 if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
@@ -1637,10 +1682,12 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
                 m.y = l == L - 1 ? y : m.xb_next ? nullptr : h->ybuf[l & 1];
                 m.xb_ld = h->ldn;
                 m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
-                m.xch = h->tcb_xch[which]; m.set_words = recur_tc_xch_words(H, plan.rows, D) + kTcXchSlack; m.used_words = (unsigned)recur_tc_xch_words(H, m.B, dirs); m.turn = h->tcb_turn[which];
+                m.set_words = h->tcb_xch[which].set_words;
+                if (phase_sets(h->tcb_xch[which], rec, st, &m.xch, &m.set, &m.clear_words) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
                 m.status = h->status_dev;
                 if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
                 e = launch_recur_tc(m, st);
+                if (e == cudaSuccess) phase_launched(h->tcb_xch[which], rec, (unsigned)recur_tc_xch_words(H, m.B, dirs));
                 ran(h, LSTM_RAN_BATCHED, m.ncta_dir * dirs, kTcThreads, recur_tc_smem_bytes(m.KH, m.upc, m.B, m.pair, m.terms));
                 ++h->last_launches;
                 if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
@@ -1705,17 +1752,18 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             m.xb_next = (l < L - 1 && h->use_tc && !fuse) ? h->xbn[l & 1] : nullptr;     // a fused next layer reads the fp32 activations
             m.xb_ld = h->ldn;
             m.xb_plane = (long long)h->max_T * h->max_B * h->ldn;
-            m.xch = h->one_xch; m.turn = h->one_turn;
+            if (phase_sets(h->one_xch, rec, st, &m.xch, &m.set, nullptr) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
             m.status = h->status_dev;
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             e = launch_recur_one(m, h->one, fuse, st);
+            if (e == cudaSuccess) phase_launched(h->one_xch, rec, 0);
             ran(h, LSTM_RAN_ONE, m.ncta_dir * dirs, kOneThreads, fuse ? recur_one_fuse_smem_bytes(h->one.mt, h->one.nks) : recur_one_smem_bytes(h->one.mt, h->one.nks));
             ++h->last_launches;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "recurrent launch failed (layer %d): %s", l, cudaGetErrorString(e));
             continue;
         }
-        if (h->f32_xch && B <= kF32MaxRows) {
+        if (h->f32_xch.words && B <= kF32MaxRows) {
             RecurF32Args m;
             memset(&m, 0, sizeof m);
             m.dir0 = h->seq_dirs ? pass : 0; m.ndirs = h->seq_dirs ? 1 : D;
@@ -1728,10 +1776,11 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             m.h0 = h0 ? h0 + so : nullptr; m.c0 = c0 ? c0 + so : nullptr;
             m.hT = hT ? hT + so : nullptr; m.cT = cT ? cT + so : nullptr;
             m.y = l == L - 1 ? y : h->ybuf[l & 1];
-            m.xch = h->f32_xch; m.turn = h->f32_turn;
+            if (phase_sets(h->f32_xch, rec, st, &m.xch, &m.set, nullptr) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
             m.status = h->status_dev;
             if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
             e = launch_recur_f32(m, st);
+            if (e == cudaSuccess) phase_launched(h->f32_xch, rec, 0);
             ran(h, LSTM_RAN_F32, m.ncta_dir * m.ndirs, kF32Threads, 0);
             ++h->last_launches;
             if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");

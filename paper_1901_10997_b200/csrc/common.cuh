@@ -70,8 +70,8 @@ struct RecurF32Args {
     const float *h0, *c0;
     float *hT, *cT;
     float *y;
-    unsigned *xch;              // exchange words [2 sets][D][2 slots][H][32 batch rows]: a launch uses one set and clears the other
-    unsigned *turn;             // whose turn the sets are (device_util.cuh)
+    unsigned *xch;              // exchange words [2 sets][D][2 slots][H][32 batch rows]
+    int set;                    // the set this launch uses; it clears the other one
     int *status;
 };
 cudaError_t launch_recur_f32(const RecurF32Args &a, cudaStream_t st);
@@ -132,13 +132,14 @@ cudaError_t launch_recur_mma(const RecurMmaArgs &a, int mt, int nkr, int nw, siz
 // ---------------------------------------------------------------------------------------------------
 constexpr int kOneThreads = 512;
 struct RecurOnePlan { int mt, nkr, nks, ncta; };     // 16-row tiles; column tiles per warp in registers, in shared memory; CTAs per direction
+// (New fields go to the end of a kernel's arguments: they are read through the constant cache, and four bytes ahead of the
+// pointers cost this kernel 1.7 us a launch.)
 struct RecurOneArgs {
     int dir0, ndirs;            // as in RecurArgs
     int H, T, D, ncta_dir, nsplit;
     int nkw_smem;
     long long spin_limit;
     int withhold_cta;
-    int probe;                  // measurement: parts of the step to leave out (LSTM_PROBE_*), 0 in normal operation
     int in_l, nkw_x, gs_off;    // projection in the prologue: input width, column tiles of Wx per range, byte offset of its rows of G
     const float *X;
     const uint4 *xfrag[2];      // [cta][8 ranges][nkw_x][mt][lane], the lane's columns adjacent
@@ -152,9 +153,10 @@ struct RecurOneArgs {
     __nv_bfloat16 *xb_next;
     long long xb_plane;
     int xb_ld;
-    unsigned *xch;              // exchange words [2 sets][D][2 slots][ncta_dir][32]: a launch uses one set and clears the other
-    unsigned *turn;             // whose turn the sets are (device_util.cuh)
+    unsigned *xch;              // exchange words [2 sets][D][2 slots][ncta_dir][32]
+    int set;                    // the set this launch uses; it clears the other one
     int *status;
+    int probe;                  // measurement: parts of the step to leave out (LSTM_PROBE_*), 0 in normal operation
 };
 size_t recur_one_smem_bytes(int mt, int nks);
 size_t recur_one_gs_offset(int mt, int nks);
@@ -290,7 +292,7 @@ struct RecurTcArgs {
     int dir0, ndirs;            // directions this launch runs: dir0 .. dir0 + ndirs - 1 (ndirs = 0 means all D)
     int H, B, T, D;             // B: batch rows of this pass ...
     int Bs, b0;                 // ... of the call's Bs, starting at row b0
-    int ncta_dir, upc, KH, pair, terms;
+    int ncta_dir, upc, KH, pair;
     int nsplit;
     long long spin_limit;
     int withhold_cta;
@@ -306,10 +308,10 @@ struct RecurTcArgs {
     int xb_ld;
     unsigned *xch;              // exchange words, 2 sets of [directions][2 slots][16 columns][8 batch rows] blocks of 128
     size_t set_words;           // words from set to set
-    unsigned used_words;        // words of its set this launch may write
-    unsigned *turn;             // whose turn the sets are (device_util.cuh); [1 + set]: words the last launch on a set may have
-                                // written, which the next launch clears
+    int set;                    // the set this launch uses; it clears the other one for the next launch ...
+    unsigned clear_words;       // ... as far as the previous launch may have written it
     int *status;
+    int terms;                  // bf16 terms of h: 2 or 3
 };
 size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair, int terms);
 size_t recur_tc_xch_words(int H, int rows, int dirs);    // exchange words of one launch with `rows` batch rows
@@ -378,7 +380,7 @@ struct HlstmTileArgs {
     long long xb_plane;
     int xb_ld;
     unsigned *hx, *rx;          // exchange words [2 sets][D][2 slots][tile][2 row groups][128]: tiles of cell units; of 4 x hidden units
-    unsigned *turn;             // whose turn the sets are (device_util.cuh): a launch uses one set and clears the other
+    int set;                    // the set this launch uses; it clears the other one
     int *status;
 };
 bool hlstm_tile_plan(int H, int Hh, int max_cta, size_t max_smem, HlstmTilePlan *p);

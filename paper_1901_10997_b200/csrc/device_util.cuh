@@ -77,11 +77,6 @@ __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v)
 // keeps its lo term (a NaN), so it still reaches every product.
 // ---------------------------------------------------------------------------------------------------
 constexpr unsigned kPhaseBit = 0x40000000u;
-// Whose turn the two sets of exchange words are is counted on the device, by the launches that ran: a recorded launch that has
-// not run yet, or runs again later, then still meets a set that the launch before it cleared.  Every CTA adds one to turn[0]
-// when it is done, modulo twice the CTAs of a launch; a CTA that has not read it has not added to it, so all read the same half.
-__device__ __forceinline__ int xch_set(const unsigned *turn) { return ld_relaxed_u32(turn) >= gridDim.x ? 1 : 0; }
-__device__ __forceinline__ void xch_done(unsigned *turn) { atomicInc(turn, 2u * gridDim.x - 1u); }
 __device__ __forceinline__ unsigned word_phase(int s) { return ((s >> 1) & 1) ? 0u : kPhaseBit; }
 __device__ __forceinline__ unsigned split_word(float h)
 {
@@ -90,7 +85,7 @@ __device__ __forceinline__ unsigned split_word(float h)
 }
 __device__ __forceinline__ unsigned pack_word(float h, unsigned phase) { return (split_word(h) & ~kPhaseBit) | phase; }
 // Exchange words that carry h as its own 32 bits (narrow fp32 layers, pruned layers): without bit 30 a NaN reads as 1.5 or more,
-// which no h is (a fast tanh may pass 1 by a rounding), and gets the bit back.
+// which no h is (a fast tanh may pass 1 by a rounding): its reader puts the bit back or marks the batch row.
 constexpr float kMaskedNan = 1.25f;
 __device__ __forceinline__ bool words_ready(const uint4 &w, unsigned phase)
 {

@@ -61,8 +61,13 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
 
     // exchange words: [set][D][slot][tile][2 row groups][128]; the other set is cleared for the next launch
     const unsigned hslot = (unsigned)uth * 256u, rslot = (unsigned)mth * 1024u;
-    const int set = xch_set(a.turn);
-    unsigned *hx = a.hx + ((size_t)set * D + d) * 2 * hslot, *rx = a.rx + ((size_t)set * D + d) * 2 * rslot;
+    unsigned *hx = a.hx + ((size_t)a.set * D + d) * 2 * hslot, *rx = a.rx + ((size_t)a.set * D + d) * 2 * rslot;
+    {
+        unsigned *ho = a.hx + ((size_t)(a.set ^ 1) * D + d) * 2 * hslot, *ro = a.rx + ((size_t)(a.set ^ 1) * D + d) * 2 * rslot;
+        for (int i = tid; i < 512; i += kThreads)
+            if (has2) ho[(size_t)(i >> 8) * hslot + cta * 256 + (i & 255)] = 0u;
+        for (int i = tid; i < 512 * nt; i += kThreads) ro[(size_t)(i & 1) * rslot + t0 * 256 + (i >> 1)] = 0u;
+    }
     uint4 areg[KT][N1];
     {
         const uint4 *src = a.frag1[d] + ((size_t)(cta * kWarps + warp) * KT * N1) * 32 + lane;
@@ -74,12 +79,6 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
     if (has2) {
         const uint4 *src = a.frag2[d] + (size_t)cta * kWarps * KT2 * 32;
         for (int i = tid; i < kWarps * KT2 * 32; i += kThreads) A2[i] = __ldg(src + i);
-    }
-    {
-        unsigned *ho = a.hx + ((size_t)(set ^ 1) * D + d) * 2 * hslot, *ro = a.rx + ((size_t)(set ^ 1) * D + d) * 2 * rslot;
-        for (int i = tid; i < 512; i += kThreads)
-            if (has2) ho[(size_t)(i >> 8) * hslot + cta * 256 + (i & 255)] = 0u;
-        for (int i = tid; i < 512 * nt; i += kThreads) ro[(size_t)(i & 1) * rslot + t0 * 256 + (i >> 1)] = 0u;
     }
     for (int i = tid; i < 16 * B; i += kThreads) {
         const int b = i >> 4, u = cta * 16 + (i & 15);
@@ -316,7 +315,6 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
             }
         }
     }
-    if (tid == 0) xch_done(a.turn);
 }
 
 typedef void (*KernelFn)(const HlstmTileArgs);

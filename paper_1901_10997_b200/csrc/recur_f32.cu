@@ -31,8 +31,9 @@ __device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b)
 // (off by less than 2 z^4 / 15 of it).  expm1 in place of both costs 0.4 us a step.
 __device__ __forceinline__ double gate_f64(double z, double k, double sc, double of)
 {
-    const double small = fma(z * z, z * (-1.0 / 3.0), z), act = sc / (1.0 + exp(k * z)) + of;
-    return of != 0.0 && fabs(z) < 1e-4 ? small : act;
+    double act = sc / (1.0 + exp(k * z)) + of;
+    if (of != 0.0 && (__double2hiint(z) & 0x7fffffff) < 0x3f1a36e2) act = fma(z * z, z * (-1.0 / 3.0), z);       // |z| < 1e-4
+    return act;
 }
 
 // NT: tiles of eight batch rows
@@ -44,6 +45,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
     constexpr int RB = NT * 8, P = RB + 2;                 // doubles between rows of partial sums
     __shared__ double red[KS * 8 * P];
     __shared__ int abort_s;
+    __shared__ int nan_s[32];                              // batch rows with a NaN in h: every sum of theirs is one, from then on
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int H = a.H, B = a.B, T = a.T, D = a.D;
     const int d = a.dir0 + blockIdx.x / a.ncta_dir, cta = blockIdx.x % a.ncta_dir;
@@ -53,8 +55,9 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
     // exchange words [set][direction of the launch][slot][unit][32 batch rows]; the other set is cleared for the next launch
     const unsigned slot_words = (unsigned)H * 32u;
     const size_t off = (size_t)(d - a.dir0) * 2 * slot_words, set_words = (size_t)2 * D * slot_words;
-    const int set = xch_set(a.turn);
-    unsigned *xch = a.xch + (size_t)set * set_words + off;
+    unsigned *xch = a.xch + (size_t)a.set * set_words + off;
+    for (int i = tid; i < nu * 64; i += kThreads)
+        a.xch[(size_t)(a.set ^ 1) * set_words + off + (size_t)(i & 1) * slot_words + u0 * 32 + (i >> 1)] = 0u;
 
     const int ksteps = (H + 3) >> 2, kper = (ksteps + KS - 1) / KS;
     const int nt = warp / KS, kq = warp - nt * KS;
@@ -67,8 +70,6 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
 #pragma unroll
         for (int i = 0; i < KW; ++i) af[i] = i < kn && u < nu && kcol + 4 * i < H ? (double)w[4 * i] : 0.0;
     }
-    for (int i = tid; i < nu * 64; i += kThreads)
-        a.xch[(size_t)(set ^ 1) * set_words + off + (size_t)(i & 1) * slot_words + u0 * 32 + (i >> 1)] = 0u;
     unsigned mine = 0;                                     // k4 steps in which this lane has a value to fetch
 #pragma unroll
     for (int i = 0; i < KW; ++i)
@@ -89,6 +90,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
     unsigned *out = xch + (size_t)j * 32 + fb;
     const double *rp = red + (fu * 4 + fq) * P + fb;
     if (tid == 0) abort_s = 0;
+    if (tid < 32) nan_s[tid] = 0;
     __syncthreads();
     volatile int *abort_v = &abort_s;
 
@@ -131,18 +133,12 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
             }
         }
         __syncwarp();
+        float top = 0.0f;
         if (s > 0) {
-            // the words without their phase
-            float top = 0.0f;
 #pragma unroll
             for (int i = 0; i < KW; ++i) {
                 w[i] &= ~kPhaseBit;
                 top = fmaxf(top, fabsf(__uint_as_float(w[i])));
-            }
-            if (top > kMaskedNan) {
-#pragma unroll
-                for (int i = 0; i < KW; ++i)
-                    if (fabsf(__uint_as_float(w[i])) > kMaskedNan) w[i] |= kPhaseBit;
             }
         }
         double acc0[2] = {0.0, 0.0}, acc1[2] = {0.0, 0.0};      // two chains: the instruction's latency exceeds its rate
@@ -154,11 +150,13 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
             r[0] = acc0[0] + acc1[0];
             r[1] = acc0[1] + acc1[1];
         }
+        if (top > kMaskedNan) nan_s[b_lane] = 1;       // (h of the first step keeps all its bits: no mark needed)
         __syncthreads();
         if (fin) {
             double z = (double)g;
 #pragma unroll
             for (int k = 0; k < KS; ++k) z += rp[k * 8 * P];
+            if (nan_s[fb]) z = nan("");
             const double act = gate_f64(z, act_k, act_sc, act_of);
             const int ql = lane & ~3;
             const double vi = __shfl_sync(0xffffffffu, act, ql), vf = __shfl_sync(0xffffffffu, act, ql + 1);
@@ -175,7 +173,6 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
     }
     if (live && fq == 2 && a.hT) a.hT[so] = hn;
     if (live && fq == 3 && a.cT) a.cT[so] = c;
-    if (tid == 0) xch_done(a.turn);
 }
 
 typedef void (*KernelFn)(const RecurF32Args);

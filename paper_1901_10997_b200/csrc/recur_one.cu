@@ -56,8 +56,8 @@ __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
     // is cleared for the next launch
     const unsigned slot_words = 32u * a.ncta_dir;
     const size_t off = (size_t)(d - a.dir0) * 2 * slot_words, set_words = (size_t)2 * D * slot_words;     // a line per CTA and slot
-    const int set = xch_set(a.turn);
-    unsigned *xch = a.xch + (size_t)set * set_words + off;
+    unsigned *xch = a.xch + (size_t)a.set * set_words + off;
+    if (tid < 2 * UPC) a.xch[(size_t)(a.set ^ 1) * set_words + off + (size_t)(tid & 1) * slot_words + cta * 32 + (tid >> 1)] = 0u;
 
     const uint4 *wsrc = a.wfrag[d] + ((size_t)(cta * kNW + warp) * nkw) * MT * 32 + lane;
     if (FUSE) {
@@ -73,7 +73,6 @@ __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
         for (int mt = 0; mt < MT; ++mt) areg[i][mt] = ld_nc_u4(wsrc + (size_t)(i * MT + mt) * 32);
     uint4 *As_w = As + (size_t)warp * nks * MT * 32 + lane;
     for (int i = 0; i < nks * MT; ++i) As_w[(size_t)i * 32] = __ldg(wsrc + (size_t)(NKR * MT + i) * 32);
-    if (tid < 2 * UPC) a.xch[(size_t)(set ^ 1) * set_words + off + (size_t)(tid & 1) * slot_words + cta * 32 + (tid >> 1)] = 0u;
     for (int i = tid; i < 2 * kNW * RP; i += kNT) red[i] = 0.0f;
     hs[lane] = make_uint2(0, 0);
     hs[32 + lane] = make_uint2(0, 0);
@@ -223,7 +222,6 @@ __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
         if (real && role == 4 && a.hT) a.hT[(size_t)d * H + j] = hn;
         if (real && role == 5 && a.cT) a.cT[(size_t)d * H + j] = c;
     }
-    if (tid == 0) xch_done(a.turn);
 }
 
 typedef void (*KernelFn)(const RecurOneArgs);

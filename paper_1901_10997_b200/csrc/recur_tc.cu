@@ -21,8 +21,8 @@
 //     flight, split them into bf16 planes and store those as the swizzled B operand (rows 0 .. Bp - 1 hi, Bp .. 2 Bp - 1
 //     lo).  Pruned layers have a third plane: their lists (recur_csr.cu) multiply h in fp32, so a batch of them carries h
 //     as its own 32 bits and splits it into three terms that hold all 24: with two terms the recurrent products alone were
-//     off by 9e-7 (1.5e-7 with three, as with the lists).  The split and the third plane cost 2 - 17 % of a call
-//     (2 x 1500, T = 35: 4 rows 233 -> 236 us, 16 rows 249 -> 286; 2 x 800, 16 rows 198 -> 219).  A step has no
+//     off by 9e-7 (1.5e-7 with three, as with the lists).  The split and the third plane cost 5 - 16 % of a call
+//     (2 x 1500, T = 35: 4 rows 233 -> 245 us, 16 rows 249 -> 286; 2 x 800, 16 rows 198 -> 219).  A step has no
 //     stamps, no release or acquire fence and no second trip for the data.
 //     LDG.128 reads a row range that all SMs share at 55 - 60 bytes per clock and SM (24 when a quarter warp's 128 bytes
 //     straddle two lines), a tensor copy at about 20.
@@ -193,9 +193,9 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
     const unsigned slot_words = (unsigned)((H + 15) >> 4) * (RG * 128u);
     auto chunk_word = [&](int q, int b) -> unsigned { return ((unsigned)(q >> 2) * RG + (b >> 3)) * 128u + (q & 3) * 32u + (b & 7) * 4u; };
     // (buffers by place in the launch, not by direction: launches that run the directions in turn share them)
-    const int set = xch_set(a.turn);
-    const unsigned clear_words = ld_relaxed_u32(a.turn + 1 + (set ^ 1));
-    unsigned *xch_d = a.xch + (size_t)set * a.set_words + (size_t)(d - a.dir0) * 2 * slot_words;
+    unsigned *xch_d = a.xch + (size_t)a.set * a.set_words + (size_t)(d - a.dir0) * 2 * slot_words;
+    for (unsigned i = blockIdx.x * kThreads + tid; i < a.clear_words / 4u; i += gridDim.x * kThreads)
+        reinterpret_cast<uint4 *>(a.xch + (size_t)(a.set ^ 1) * a.set_words)[i] = make_uint4(0, 0, 0, 0);
     // weights into tensor memory: warp w writes lane quadrant w % 4, every fourth 8-column piece
     {
         const int row = (warp & 3) * 32 + lane, pieces = a.KH >> 3;
@@ -211,9 +211,6 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
-    for (unsigned i = blockIdx.x * kThreads + tid; i < clear_words / 4u; i += gridDim.x * kThreads)
-        reinterpret_cast<uint4 *>(a.xch + (size_t)(set ^ 1) * a.set_words)[i] = make_uint4(0, 0, 0, 0);
-    if (blockIdx.x == 0 && tid == 0) a.turn[1 + set] = a.used_words;
     for (int i = tid; i < tiles * N * 8; i += kThreads) reinterpret_cast<uint4 *>(op)[i] = make_uint4(0, 0, 0, 0);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -457,20 +454,6 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
             auto read_sums = [&](int b0) {                       // this row's sums for batch rows b0 .. b0 + RS - 1
                 const uint32_t ta = acc_col + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)b0;
                 float zl[RS];
-                if constexpr (TERMS == 3 && RG == 1) {           // (with more rows the two waits below are faster: 219 against 235 us per
-                    float v[6][RS];                              // call at 2 x 800, 16 rows)
-#pragma unroll
-                    for (int t = 0; t < 3; ++t) tmem_ld<RS>(ta + (uint32_t)(t * Bp), v[t]);
-                    if (nissue > 1) {
-#pragma unroll
-                        for (int t = 0; t < 3; ++t) tmem_ld<RS>(ta + (uint32_t)(N + t * Bp), v[3 + t]);
-                    }
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                    for (int i = 0; i < RS; ++i)
-                        z[i] = nissue > 1 ? (v[0][i] + v[3][i]) + ((v[1][i] + v[4][i]) + (v[2][i] + v[5][i])) : v[0][i] + (v[1][i] + v[2][i]);
-                    return;
-                }
                 if constexpr (TERMS == 3) {                      // the last two terms first: their sum takes the place of the second
                     float zt[RS];
                     tmem_ld<RS>(ta + (uint32_t)Bp, zl);
@@ -564,7 +547,6 @@ __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs
             if (a.hT) a.hT[state0 + (size_t)(fb0 + 4 * m + fq) * H] = hn[m];
             if (a.cT) a.cT[state0 + (size_t)(fb0 + 4 * m + fq) * H] = c[m];
         }
-    if (tid == 0) xch_done(a.turn);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     if (__syncthreads_or(*abort_v)) {           // one answer for the whole CTA: the partner may raise the flag at any time
         // a wait gave up: products and partial sums may still be in flight; they land within microseconds
