@@ -1044,7 +1044,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     if (rc == LSTM_OK && dtype == LSTM_F32 && !csr && h->upc <= 2 && H <= kF32MaxUnits)
         rc = alloc_phase_words(h, h->f32_xch, (size_t)D * 2 * H * 32, st);
     for (int i = 0; i < 2 && rc == LSTM_OK; ++i)
-        if (i ? h->use_tc1 : h->use_tcb) rc = alloc_phase_words(h, h->tcb_xch[i], recur_tc_xch_words(H, h->tcb[i].rows, D) + kTcXchSlack, st);
+        if (i ? h->use_tc1 : h->use_tcb) rc = alloc_phase_words(h, h->tcb_xch[i], recur_tc_xch_words(H, h->tcb[i].rows, D), st);
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->status_dev, sizeof(int), true, st, "status word");
     if (rc == LSTM_OK && h->use_wave) {
         h->wave_xch_words = (size_t)layers * max_T * std::min(max_B, 4) * H;

@@ -315,7 +315,6 @@ struct RecurTcArgs {
 };
 size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair, int terms);
 size_t recur_tc_xch_words(int H, int rows, int dirs);    // exchange words of one launch with `rows` batch rows
-constexpr size_t kTcXchSlack = 5 * 12 * 8 * 128;           // words a polling warp may read beyond them
 bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, int terms, size_t max_smem, RecurTcPlan *p);
 bool recur_tc_pair_supported(int grid, const RecurTcPlan &p);
 cudaError_t recur_tc_prepare(int terms, int max_smem);

@@ -62,12 +62,6 @@ __device__ __forceinline__ void st_relaxed_u32(unsigned *p, unsigned v)
 {
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-// release store at GPU scope: what this thread wrote, and what it observed others write (a CTA barrier counts),
-// is visible to whoever reads the value with acquire semantics or fences after reading it
-__device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v)
-{
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 // ---------------------------------------------------------------------------------------------------
 // Exchange words: one hidden value in 32 bits, {bf16 hi : 16 | bf16 lo : 16} with hi = bf16(h), lo = bf16(h - hi), the
 // two terms the tensor cores multiply.  |h| = |o tanh(c)| <= 1, so bit 30 (the top exponent bit of hi) is always 0 in a
@@ -117,14 +111,6 @@ __device__ __forceinline__ float ld_nc_early(const float *p)
     asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ float4 ld_nc_f4(const float4 *p)
-{
-    float4 v;
-    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
-    return v;
-}
-// release / acquire fence at GPU scope (lighter than the sequentially consistent __threadfence)
-__device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 // 16-byte asynchronous copy global -> shared through L2 only (never a stale L1 line)
 __device__ __forceinline__ void cp_async_16(void *smem_dst, const void *gsrc)
@@ -140,6 +126,11 @@ __device__ __forceinline__ void cp_async_wait_all()
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
+// D += A (8x4, row) * B (4x8, col) in double precision
+__device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b)
+{
+    asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+}
 // D += A (16x16, row) * B (16x8, col), bf16 inputs, fp32 accumulation
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint4 &a, unsigned b0, unsigned b1)
 {

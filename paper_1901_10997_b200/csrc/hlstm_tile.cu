@@ -325,10 +325,10 @@ KernelFn pick_mode(int n1, int kt)
         case 1 * 16 + 4: return hlstm_tile_kernel<1, 4, MODE>;
         case 2 * 16 + 4: return hlstm_tile_kernel<2, 4, MODE>;
         case 3 * 16 + 4: return hlstm_tile_kernel<3, 4, MODE>;
-        case 4 * 16 + 4: return hlstm_tile_kernel<4, 4, MODE>;
+        case 4 * 16 + 4: if constexpr (MODE != 2) return hlstm_tile_kernel<4, 4, MODE>; else return nullptr;     // (mode_of: n1 * kt <= 12)
         case 1 * 16 + 6: return hlstm_tile_kernel<1, 6, MODE>;
         case 2 * 16 + 6: return hlstm_tile_kernel<2, 6, MODE>;
-        case 3 * 16 + 6: return hlstm_tile_kernel<3, 6, MODE>;
+        case 3 * 16 + 6: if constexpr (MODE != 2) return hlstm_tile_kernel<3, 6, MODE>; else return nullptr;
         default: return nullptr;
     }
 }
@@ -365,6 +365,7 @@ size_t hlstm_tile_smem_bytes(const HlstmTilePlan &p, int rows) { return smem_byt
 cudaError_t hlstm_tile_prepare(const HlstmTilePlan &p)
 {
     for (int mode = 0; mode < 3; ++mode) {
+        if (!pick(p.n1, p.kt, mode)) continue;
         const cudaError_t e = cudaFuncSetAttribute(pick(p.n1, p.kt, mode), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.max_smem);
         if (e != cudaSuccess) return e;
     }

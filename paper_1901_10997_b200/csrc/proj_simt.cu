@@ -3,6 +3,7 @@
 // computed for all timesteps at once).  The fp32 storage type uses the tiled FFMA kernel; pruned
 // weights in CSR form use the sparse kernel.  The bf16 tensor-core kernel lives in proj_tc.cu.
 #include "common.cuh"
+#include "device_util.cuh"
 
 #include <algorithm>
 
@@ -101,10 +102,6 @@ __global__ void __launch_bounds__(256) proj_simt_kernel(const float *__restrict_
 // are stored instead of at every use and a lane's operands are single conflict-free loads; the next K step is on its way
 // while this one is multiplied, and small tiles put several CTAs on an SM.  2000 x 800 x 200: 83 us with the fp64
 // multiply-adds of the tile kernel above, 50 us here.
-__device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b)
-{
-    asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
-}
 __global__ void __launch_bounds__(128) proj_f64_kernel(const float *__restrict__ X, const float *__restrict__ W, int ldw,
                                                        const float *__restrict__ bias, float *__restrict__ G, int M, int N, int K)
 {

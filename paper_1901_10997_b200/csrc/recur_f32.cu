@@ -21,11 +21,6 @@ namespace {
 
 constexpr int kThreads = kF32Threads, kWarps = kThreads / 32;
 
-__device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b)
-{
-    asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
-}
-
 // sc / (1 + e^(k z)) + of: the logistic function (k, sc, of = -1, 1, 0) or tanh (-2, 2, -1).  tanh of a small z is the
 // difference of two nearby numbers there, which loses the digits of z (all of them near 1e-16): below 1e-4 it is z - z^3 / 3
 // (off by less than 2 z^4 / 15 of it).  expm1 in place of both costs 0.4 us a step.
