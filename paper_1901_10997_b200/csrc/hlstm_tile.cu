@@ -117,7 +117,8 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
     }
 
     // polls w[i][rg] = the lane's 16 bytes of tile i, row group rg0 + rg (`src`: tile 0), waiting for `phase` in `bit`
-    auto fetch = [&](auto &w, const unsigned *src, int tiles, int rg0, unsigned phase, unsigned bit) {
+    // (`base`, `words`: the exchange words that src lies in)
+    auto fetch = [&](auto &w, const unsigned *src, const unsigned *base, unsigned words, int tiles, int rg0, unsigned phase, unsigned bit) {
         constexpr int NT = sizeof(w) / sizeof(w[0]);
         unsigned pending = 0;
 #pragma unroll
@@ -135,7 +136,8 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
             for (int i = 0; i < NT; ++i)
 #pragma unroll
                 for (int rg = 0; rg < RGS; ++rg)
-                    if (pending & (1u << (i * RGS + rg))) w[i][rg] = ld_relaxed_v4(src + i * 256 + (rg0 + rg) * 128);
+                    if ((pending & (1u << (i * RGS + rg))) && LSTM_CHECK_INDEX(src - base + i * 256 + (rg0 + rg) * 128 + 3, words, a.status))
+                        w[i][rg] = ld_relaxed_v4(src + i * 256 + (rg0 + rg) * 128);
 #pragma unroll
             for (int i = 0; i < NT; ++i)
 #pragma unroll
@@ -164,6 +166,7 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
         }
     };
     auto leave_sums = [&](float *dst, const float (&acc)[4]) {
+        if (!LSTM_CHECK_INDEX(dst - red + (MODE == 0 ? 3 : 7) * kPitch + 15, c_s - red, a.status)) return;
         if (MODE == 0) {
             dst[tig * kPitch + g] = acc[0] + acc[1];
             dst[tig * kPitch + g + 8] = acc[2] + acc[3];
@@ -213,7 +216,7 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
                         }
                     __syncwarp();
                 } else {
-                    fetch(w, hx + (size_t)((s - 1) & 1) * hslot + warp * KT * 256 + lane_word, k_tiles, rg0, h_phase, kPhaseBit);
+                    fetch(w, hx + (size_t)((s - 1) & 1) * hslot + warp * KT * 256 + lane_word, hx, 2 * hslot, k_tiles, rg0, h_phase, kPhaseBit);
                 }
                 const unsigned keep = s == 0 ? 0xffffffffu : 0xbfffbfffu;
                 float acc[N1][RGS][4];
@@ -246,7 +249,7 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
                         p[w4] = (rp[w4 * N1 * RGS * kTileRed] + rp[(w4 + 4) * N1 * RGS * kTileRed]) +
                                 (rp[(w4 + 8) * N1 * RGS * kTileRed] + rp[(w4 + 12) * N1 * RGS * kTileRed]);
                     const float r = fmaxf(((p[0] + p[1]) + (p[2] + p[3])) + gv[f], 0.0f);
-                    if (publish)
+                    if (publish && LSTM_CHECK_INDEX((size_t)(s & 1) * rslot + rword[f] + (rg0 + frg) * 128, 2 * rslot, a.status))
                         st_relaxed_u32(rx + (size_t)(s & 1) * rslot + rword[f] + (rg0 + frg) * 128, (split_word(r) & ~kRPhase) | r_phase);
                 }
             }
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
 #pragma unroll 1
                 for (int k0 = 0; k0 < m_tiles; k0 += KB) {
                     uint4 w[KB][RGS];
-                    fetch(w, src + (size_t)k0 * 256, m_tiles - k0, rg0, r_phase, kRPhase);
+                    fetch(w, src + (size_t)k0 * 256, rx, 2 * rslot, m_tiles - k0, rg0, r_phase, kRPhase);
 #pragma unroll
                     for (int i = 0; i < KB; ++i)
                         if (k0 + i < m_tiles) {
@@ -294,7 +297,7 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
                 const bool real = u2 < H;
                 cn = real ? fmaf(gf, c_s[b * 16 + frow], gi * gg) : 0.0f;
                 hn = real ? go * tanh_fast(cn) : 0.0f;
-                if (publish)
+                if (publish && LSTM_CHECK_INDEX((size_t)(s & 1) * hslot + cta * 256 + (rg0 + frg) * 128 + fb * 16 + frow, 2 * hslot, a.status))
                     st_relaxed_u32(hx + (size_t)(s & 1) * hslot + cta * 256 + (rg0 + frg) * 128 + fb * 16 + frow, pack_word(hn, word_phase(s)));
                 c_s[b * 16 + frow] = cn;
             }

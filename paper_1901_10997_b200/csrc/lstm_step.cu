@@ -66,7 +66,8 @@ __global__ void __launch_bounds__(kThreads, 2) lstm_step_kernel(const LstmStepAr
                 for (int i = 0; i < 8; ++i) v[i] = b < B && k0 + i * kThreads < n ? src[b * row_stride + k0 + i * kThreads] : 0.0f;
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
-                    if (k0 + i * kThreads < ncol) op[b * (ncol + 16) + k0 + i * kThreads] = split_word(v[i]);
+                    if (k0 + i * kThreads < ncol && LSTM_CHECK_INDEX(&op[b * (ncol + 16) + k0 + i * kThreads] - oph, reinterpret_cast<unsigned *>(red) - oph, a.status))
+                        op[b * (ncol + 16) + k0 + i * kThreads] = split_word(v[i]);
             }
     };
     // a warp takes every kWarps-th column tile, U of them in flight
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(kThreads, 2) lstm_step_kernel(const LstmStepAr
         for (int t0 = warp; t0 < tiles; t0 += kWarps * U) {
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (t0 + kWarps * u < tiles) {
+                if (t0 + kWarps * u < tiles && LSTM_CHECK_INDEX(ow + (t0 + kWarps * u) * 16 + second + 1 - oph, reinterpret_cast<unsigned *>(red) - oph, a.status)) {
                     const uint2 w0 = *reinterpret_cast<const uint2 *>(ow + (t0 + kWarps * u) * 16);
                     const uint2 w1 = *reinterpret_cast<const uint2 *>(ow + (t0 + kWarps * u) * 16 + second);
                     const unsigned b0 = __byte_perm(w0.x, w0.y, sel), b1 = __byte_perm(w1.x, w1.y, sel);
@@ -123,7 +124,8 @@ __global__ void __launch_bounds__(kThreads, 2) lstm_step_kernel(const LstmStepAr
     products(opx, xk + 16, fx, a.x_tiles, true, nullptr, 0);
 
     float *rw = red + warp * WS + g;
-    if (RB == 8) {
+    if (!LSTM_CHECK_INDEX(rw - red + (RB == 8 ? 7 : RB - 1) * RP + (MT - 1) * 16 + 8, kWarps * WS, a.status)) {
+    } else if (RB == 8) {
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
             rw[2 * tig * RP + mt * 16] = acc[mt][0];

@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
             while (pending) {
 #pragma unroll
                 for (int i = 0; i < KW; ++i)
-                    if (pending & (1u << i)) w[i] = ld_relaxed_u32(src + i * 128);
+                    if ((pending & (1u << i)) && LSTM_CHECK_INDEX(src - xch + i * 128, 2 * slot_words, a.status)) w[i] = ld_relaxed_u32(src + i * 128);
 #pragma unroll
                 for (int i = 0; i < KW; ++i)
                     if ((pending & (1u << i)) && ((w[i] ^ phase) & kPhaseBit) == 0) pending &= ~(1u << i);
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
 #pragma unroll
         for (int i = 0; i < KW; ++i)
             if (i < kn) mma_f64(i & 1 ? acc1 : acc0, af[i], (double)__uint_as_float(w[i]));
-        if (nt < NT) {
+        if (nt < NT && LSTM_CHECK_INDEX((kq * 8 + (lane >> 2)) * P + nt * 8 + 2 * (lane & 3) + 1, KS * 8 * P, a.status)) {
             double *r = red + (kq * 8 + (lane >> 2)) * P + nt * 8 + 2 * (lane & 3);
             r[0] = acc0[0] + acc1[0];
             r[1] = acc0[1] + acc1[1];
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Ar
             const double cn = fma(vf, (double)c, vi * vg);
             hn = (float)(vo * gate_f64(cn, -2.0, 2.0, -1.0));
             c = (float)cn;
-            if (live && fq == 0 && (int)blockIdx.x != a.withhold_cta)
+            if (live && fq == 0 && (int)blockIdx.x != a.withhold_cta && LSTM_CHECK_INDEX(out - xch + (s & 1) * slot_words, 2 * slot_words, a.status))
                 st_relaxed_u32(out + (s & 1) * slot_words, (__float_as_uint(hn) & ~kPhaseBit) | word_phase(s));
         }
         __syncthreads();                    // nobody polls before the CTA has published; the sums are free again

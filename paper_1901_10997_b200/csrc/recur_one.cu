@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
         } else {
             const unsigned phase = word_phase(s - 1);
             const unsigned *p = src + ((s - 1) & 1) * slot_words;
-            if (has) w = ld_relaxed_v4(p);
+            if (has && LSTM_CHECK_INDEX(p - xch + 3, 2 * slot_words, a.status)) w = ld_relaxed_v4(p);
             bool wait = has && !words_ready(w, phase) && !(probe & 4);
             int polls = 0;
             long long t_start = 0;
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
             }
         }
         // accumulator columns 0 and 1 are the hi and lo products (the other columns repeat them)
-        if (tig == 0) {
+        if (tig == 0 && LSTM_CHECK_INDEX(((s & 1) * kNW + warp) * RP + g + (MT - 1) * 16 + 8, 2 * kNW * RP, a.status)) {
             float *rw = red + ((s & 1) * kNW + warp) * RP + g;
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt) {
@@ -212,7 +212,8 @@ __global__ void __launch_bounds__(kNT, 1) recur_one_kernel(const RecurOneArgs a)
             const float vg = __shfl_sync(0xffffffffu, act, q0 + 4), vo = __shfl_sync(0xffffffffu, act, q0 + 6);
             c = fmaf(vf, c, vi * vg);
             hn = vo * tanh_fast(c);
-            if (publish) st_relaxed_u32(out + (s & 1) * slot_words, pack_word(hn, word_phase(s)));
+            if (publish && LSTM_CHECK_INDEX(out - xch + (s & 1) * slot_words, 2 * slot_words, a.status))
+                st_relaxed_u32(out + (s & 1) * slot_words, pack_word(hn, word_phase(s)));
         }
         __syncwarp();
         bar_sync(2, nbar);

@@ -1,5 +1,5 @@
 """The code paths the environment switches select instead of the defaults must stay correct: they are what the
-defaults are measured against (issuing threads of the batched recurrence, 128-row projection tiles, the
+defaults are measured against (128-row projection tiles, no cluster pairs in the batched recurrence, the
 list-walking projection of CSR handles), and some are the only path for shapes the default does not serve."""
 import numpy as np
 import pytest
@@ -26,20 +26,19 @@ def _forward(pkg, w, weights, x, h0, c0, exec_mode="dense"):
         m.close()
 
 
-@pytest.mark.parametrize("issuers", ["1", "2"])
-def test_batched_recurrence_with_fewer_issuing_threads(oracle, issuers, monkeypatch):
-    """One and two issuing threads (one and two accumulators) instead of three; pair mode and both directions,
-    and a slice whose ring does not hold a whole step's operand."""
+@pytest.mark.parametrize("shape", [(True, 300, 20), (True, 1100, 20), (False, 1600, 9), (False, 1100, 40)], ids=lambda s: f"D{1 + s[0]}_H{s[1]}_B{s[2]}")
+def test_batched_recurrence_with_one_and_two_issuing_warps(oracle, shape):
+    """A K range of one operand group (192 columns) has one issuing warp, a longer one two with an accumulator each, and more than
+    32 rows one again; cluster pairs, K halves of unequal size."""
     import paper_1901_10997_b200 as pkg
-    monkeypatch.setenv("LSTM_B200_TC_ISSUE", issuers)
-    for w in (small("tci_h600_b20", 1, True, 24, 600, 3, 20, "bf16", scale=0.05),
-              small("tci_h1600_b9", 1, False, 32, 1600, 2, 9, "bf16", scale=0.03)):
-        weights, x = wl.make(w)
-        h0, c0 = wl.make_states(w)
-        ref = oracle.forward(weights, x, h0, c0, layers=w.layers, bidir=w.bidir, hidden=w.hidden)
-        got, info = _forward(pkg, w, weights, x, h0, c0)
-        assert info["recur_batched_tensor_core"] >= 1
-        assert_close(got, ref, "bf16", f"{w.name}/issuers={issuers}")
+    bidir, H, B = shape
+    w = small("tci", 1, bidir, 24, H, 3, B, "bf16", scale=0.05 if H < 1000 else 0.03)
+    weights, x = wl.make(w)
+    h0, c0 = wl.make_states(w)
+    ref = oracle.forward(weights, x, h0, c0, layers=w.layers, bidir=w.bidir, hidden=w.hidden)
+    got, info = _forward(pkg, w, weights, x, h0, c0)
+    assert info["kernel"] == pkg.LSTM_RAN_BATCHED
+    assert_close(got, ref, "bf16", f"{w.name}/H={H}/B={B}")
 
 
 def test_batched_recurrence_without_cluster_pairs(oracle, monkeypatch):

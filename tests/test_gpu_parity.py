@@ -248,9 +248,8 @@ def test_batched_tensor_core_recurrence(oracle, w):
 
 @pytest.mark.parametrize("B", [6, 20])
 def test_first_call_of_a_fresh_handle_sees_a_nonzero_initial_state(oracle, B):
-    """The batched kernel publishes h0 under the call's first stamp; on a fresh handle (cleared flags and
-    planes) a consumer must still wait for that stamp instead of taking the cleared planes for h0.  Several
-    fresh handles in a row, one step each, so that a CTA that starts early would read zeros."""
+    """A single step from a non-zero h0 on several fresh handles in a row: a CTA that took the cleared exchange words of a
+    fresh handle for h0 would read zeros.  Six rows run the single-step kernel, twenty the batched one."""
     import torch
     import paper_1901_10997_b200 as pkg
     w = small("fresh_h0", 1, False, 24, 600, 1, B, "bf16", scale=0.05, seed=41)
@@ -297,8 +296,8 @@ def test_batched_recurrence_chunked_calls_carry_state(oracle):
 
 @pytest.mark.parametrize("dtype,mode,B", [("bf16", "dense", 2), ("fp32", "dense", 2), ("bf16", "csr", 2), ("bf16", "dense", 6)])
 def test_withheld_exchange_words_end_in_a_timeout_status_not_a_hang(oracle, dtype, mode, B):
-    """One CTA withholds its h values (B = 6: its stamp, in the batched kernel); the waits of the others run
-    out after a millisecond, the call reports LSTM_ERR_TIMEOUT, and the same handle computes correctly
+    """One CTA withholds its h values (all bf16 cases here run the batched kernel; every kernel has a case in
+    test_gpu_timeouts.py); the waits of the others run out after a millisecond, the call reports LSTM_ERR_TIMEOUT, and the same handle computes correctly
     again afterwards."""
     import torch
     import paper_1901_10997_b200 as pkg
