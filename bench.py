@@ -7,10 +7,11 @@ A step is one lstm_forward over the large language-model workload (2 layers, 150
 batch 1, bf16 weights / fp32 state): input projection for all timesteps + serial recurrence, every
 layer.  `value` is microseconds per sequence with inputs resident in device memory; `e2e` is the same
 through lstm_forward_host with pinned host buffers (copies inside the timed region).  At one GPU the
-line also carries short device-timed `legs` for the other workloads (batches of 20 and 16 sequences, the
-pruned stack dense-with-zeros against CSR, the speech-shaped stack, the small fp32 stack), the on-chip
+line also carries the time per sequence of short device-timed legs for the other workloads (batches of 20 and 16
+sequences, the pruned stack dense-with-zeros against CSR, the speech-shaped stack, the small fp32 stack), the on-chip
 yardstick of the recurrent step (`roofline.on_chip`: the exchange-only step measured by the library's own
-probe modes) and the fp64 CPU oracle timed on the host cores (all threads and one thread).
+probe modes) and the fp64 CPU oracle timed on the host cores (all threads and one thread).  The whole record, with every
+leg's spread, roofline, clocks and what the library reports, goes to DIR/bench.json.
 With N > 1 each rank runs an independent replica (batch columns and sequences never interact): no
 collective on the data path, N sequences per step.  Started without a launcher, `--gpus N` starts the N
 ranks itself (one process per GPU, rendezvous on 127.0.0.1).
@@ -23,7 +24,7 @@ Other modes:
     --workload NAME      cfg1 | cfg2 | cfg2_b20 | cfg4_10 | cfg4_05 | cfg4_10_csr | cfg4_05_csr |
                          cfg5 | cfg5_b16 | hlstm_ptb | hlstm_ds2 (default cfg2)
     --no-legs            headline workload only
-    --out DIR            where the sweeps write their tables (default bench_out)
+    --out DIR            where the whole record and the sweeps' tables are written (default bench_out)
 """
 from __future__ import annotations
 
@@ -617,11 +618,28 @@ def run_gpu(args):
         case.close()
         if world == 1 and not args.no_legs and args.workload == "cfg2":
             line["legs"] = run_legs(torch, pkg, dev, flush_buf, cache, peak, peak_kind)
-        print(json.dumps(line))
+        outdir = Path(args.out)
+        outdir.mkdir(parents=True, exist_ok=True)
+        (outdir / "bench.json").write_text(json.dumps(line, indent=1))
+        print(json.dumps(short_line(line)))
     else:
         case.close()
     if dist is not None:
         dist.destroy_process_group()
+
+
+def short_line(line):
+    """The line that is printed, short enough (about 2 KB) to survive in a log that keeps the end of the output: the headline and its
+    roofline, and of every leg the time per sequence in microseconds.  Everything else is in the file."""
+    out = {k: v for k, v in line.items() if k not in ("library", "legs", "roofline", "kernel_ms_per_forward", "sequences_per_sec")}
+    roof = line["roofline"]
+    out["roofline"] = {k: roof[k] for k in ("bound", "kernel", "achieved", "peak", "unit", "frac", "peak_kind", "traffic",
+                                            "algorithmic_bytes_per_launch", "us_per_timestep")}
+    if "on_chip" in roof:
+        out["roofline"]["on_chip"] = {k: roof["on_chip"][k] for k in ("step_us", "empty_step_us")}
+    if "legs" in line:
+        out["legs_us_per_sequence"] = {k: round(v["us_per_sequence"], 2) if "us_per_sequence" in v else v for k, v in line["legs"].items()}
+    return out
 
 
 def run_legs(torch, pkg, dev, flush_buf, cache, peak, peak_kind):
