@@ -16,7 +16,8 @@
 // bit of hi).  A block of sixteen units x eight batch rows is 512 contiguous bytes in operand-B order with ONE writer: a
 // lane's 16-byte load is its fragment, nothing is staged or converted.
 // Measured (one layer 1500 -> 1200, Hh = 320, T = 70, 16 rows, projection included): 354 us per call against 3825 us for the
-// kernel that runs the batch rows one after the other (hlstm_mma.cu, which still serves slices that do not fit here).
+// kernel that runs the batch rows one after the other (hlstm_mma.cu, which still serves one row, for which it is the faster one,
+// and slices that do not fit here).
 // Every wait is bounded; on expiry the CTA records a timeout status, stops waiting and runs to the end.
 #include "common.cuh"
 #include "device_util.cuh"

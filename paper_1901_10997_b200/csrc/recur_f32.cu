@@ -11,7 +11,7 @@
 // dot product per warp needed 160 shuffles a unit).  h travels as its own 32 bits: |h| <= 1, so bit 30 is free for the phase
 // (device_util.cuh); a unit's 32 batch rows are one line with one writer.  After one barrier a quad per (unit, batch row) adds
 // the K ranges' sums, one gate each, and applies the gate functions, each from one exponential and one division.
-// Measured (2 x 200, batch 20, T = 35, per call): 480 us with recur.cu, 234 us here.
+// Measured (2 x 200, batch 20, T = 35, per call): 480 us with recur.cu, 209 us here.
 // Every wait is bounded; on expiry the CTA records a timeout status, stops waiting and runs to the end.
 #include "common.cuh"
 #include "device_util.cuh"

@@ -12,7 +12,7 @@
 // memory.  What a step does, and why it is laid out like this:
 //
 //   * The weights sit in TENSOR MEMORY as the A operand (row = lane, two bf16 per column) for the whole sequence:
-//     128 rows by up to 896 columns.  Shared memory is then free for the B operand of a whole step, and an
+//     128 rows by up to 960 columns.  Shared memory is then free for the B operand of a whole step, and an
 //     instruction reads only its small B tile from it.  The issuing thread must be elected from a converged warp and
 //     take its operands from warp-uniform values: measured for 48 instructions of N = 16 / 48, 970 / 1370 cycles; the
 //     same loop entered by "lane == 0" with per-thread operands took 8260.
@@ -41,8 +41,8 @@
 // tensor copies behind one stamp per CTA, three "lane == 0" issuing threads): H = 1500, 20 rows 5.8 -> 3.3 us; two directions of
 // 800, 16 rows 4.7 -> 2.4 us; 50 rows in a pass 5.0 us (batches above 64 ran as passes of four rows before).
 //
-// Pair mode needs K for both halves and clusters of two; otherwise (narrow layers, or LSTM_B200_RECUR=tc1) a CTA works
-// alone on its own rows and all of K.  Every wait on another CTA is bounded; on expiry the CTA records a timeout status,
+// Pair mode needs K for both halves and clusters of two; without it (few rows of narrow layers, tc_single_rows in api.cu, or
+// LSTM_B200_RECUR=tc1) a CTA works alone on its own rows and all of K.  Every wait on another CTA is bounded; on expiry the CTA records a timeout status,
 // stops waiting for the rest of the launch and runs to the common exit, where tensor memory is released.
 #include "common.cuh"
 #include "device_util.cuh"
