@@ -686,10 +686,10 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
 
     if (allow_compact) {
         // row/column-pruned weights: run on the surviving units only (LSTM_B200_COMPACT=0 keeps the zeros)
-        // Unset: only handles made for batches (max_B of five or more), where the step is bound by throughput and a
-        // narrower model is faster; for up to four sequences the step is bound by the exchange latency, the narrower
-        // model gains nothing and the extra scatter kernel costs a few microseconds (measured: 172.7 against 164.6 us
-        // per sequence at width 1500 -> 1197).  LSTM_B200_COMPACT=1 compacts always, =0 never.
+        // Unset: only handles made for batches (max_B of five or more).  us per call, T = 35, zeros kept / compacted, 1500 -> 1197
+        // with 1, 2, 4, 8 rows: 138 / 146, 200 / 201, 224 / 212, 231 / 220; 1500 -> 800: 137 / 101, 199 / 184, 223 / 186, 233 / 194;
+        // 800 -> 600: 89 / 90, 172 / 164, 170 / 173, 176 / 177: few rows gain only where much is removed.
+        // LSTM_B200_COMPACT=1 compacts always, =0 never.
         const char *env = getenv("LSTM_B200_COMPACT");
         const bool want = env ? strcmp(env, "0") != 0 : max_B >= 5;
         if (want) {
