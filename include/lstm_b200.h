@@ -172,10 +172,8 @@ LSTM_API int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden,
  * 0 <= T <= max_T, 0 <= B <= max_B (T = 0 or B = 0: nothing is launched; hT,cT receive h0,c0).
  * Work is enqueued on cuda_stream and the call returns without synchronising; a device-side timeout
  * of this call is reported by lstm_status on the handle.
- * Stream capture: the launches of a call may be recorded into a CUDA graph and replayed beside ordinary calls on the same stream
- * if the call has one timestep or runs on one of the kernels LSTM_RAN_ONE, _BATCHED, _F32, _STEP, _HLSTM_TILES (lstm_info says
- * which kernel a call runs); the other kernels stamp their exchange words per call, and a second replay would meet the first
- * one's stamps.
+ * Stream capture: the launches of a call may be recorded into a CUDA graph and replayed, beside ordinary calls on the same stream:
+ * a recorded call has exchange words or stamps of its own, and the graph clears them before it uses them.
  * Non-finite values: a NaN in h reaches every unit of its batch row in the next step, also where pruned weights are zero if the
  * batch runs on LSTM_RAN_BATCHED (there and in the projection the zeros are multiplied; the lists skip them).
  * Steps, in order, per layer: input staging (bf16 mode), input projection for all timesteps at once

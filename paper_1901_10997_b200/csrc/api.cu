@@ -106,7 +106,7 @@ struct lstm_handle {
     float *ybuf[2] = {nullptr, nullptr};
     unsigned long long *xch = nullptr; size_t xch_words = 0;
     int *status_dev = nullptr;
-    unsigned stamp_next = 1;           // stamps start at 1: a cleared exchange word or flag (0) never matches or exceeds a wanted stamp
+    unsigned stamp_next = 1;           // of ordinary calls; starts at 1: a cleared exchange word (0) never carries a wanted stamp
     long long spin_limit = 2000000000LL;
     long long spin_limit_default = 2000000000LL;
     int withhold_cta = -1;             // failure-path self-test (lstm_selftest_timeout)
@@ -319,6 +319,8 @@ void phase_launched(PhaseWords &x, bool rec, unsigned used_words)
     x.set ^= 1;
     x.dirty = used_words;
 }
+
+constexpr unsigned kRecordedStamps = 0x80000000u;       // the first stamp of a recorded call
 
 inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
@@ -1510,13 +1512,26 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
     const bool csr = h->exec_mode == LSTM_CSR;
     cudaError_t e = cudaSuccess;
 
-    // stamps of the exchange words must stay unique: restart from a cleared buffer before wrapping
-    if ((unsigned long long)h->stamp_next + (unsigned long long)L * D * ((unsigned long long)T + 1ull) + 2ull >= 0xffffffffull) {
-        if (cudaMemsetAsync(h->xch, 0, h->xch_words * 8, st) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
-        if (h->rxch && cudaMemsetAsync(h->rxch, 0, h->rxch_words * 8, st) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
-        if (h->wave_xch && cudaMemsetAsync(h->wave_xch, 0, h->wave_xch_words * 8, st) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
+    // Stamps of the exchange words must stay unique.  Ordinary calls count up to the upper half of the numbers and restart from cleared
+    // words.  A call that is being recorded into a graph takes the upper half and clears the words first, with nodes of that graph: a
+    // replay writes the stamps of its recording again and would take the words of the replay before for its own.
+    const bool rec = recording(st);
+    auto clear_stamped = [&] {
+        return cudaMemsetAsync(h->xch, 0, h->xch_words * 8, st) == cudaSuccess &&
+               (!h->rxch || cudaMemsetAsync(h->rxch, 0, h->rxch_words * 8, st) == cudaSuccess) &&
+               (!h->wave_xch || cudaMemsetAsync(h->wave_xch, 0, h->wave_xch_words * 8, st) == cudaSuccess);
+    };
+    if (!rec && (unsigned long long)h->stamp_next + (unsigned long long)L * D * ((unsigned long long)T + 1ull) + 2ull >= kRecordedStamps) {
+        if (!clear_stamped()) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
         h->stamp_next = 1;
     }
+    unsigned recorded_next = kRecordedStamps;
+    auto take_stamps = [&](unsigned *base) {
+        unsigned &next = rec ? recorded_next : h->stamp_next;
+        *base = next;
+        next += (unsigned)T + 1u;
+        return *base != kRecordedStamps || clear_stamped();
+    };
 
     // A single timestep of a few sequences on the register-resident kernel's weights: one streaming launch per layer
     if (T == 1 && B <= kStepMaxRows && h->step_ok && !h->probe && h->withhold_cta < 0) {
@@ -1554,8 +1569,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         m.L = L; m.H = H; m.B = B; m.T = T; m.ncta_layer = h->wave_ncta; m.nsplit = nsplit;
         for (int l = 0; l < L; ++l) { m.nkw[l] = h->wave_nkw[l]; m.wfrag[l] = h->wave_frag[l]; m.bias[l] = h->layers[l].bias; }
         m.nkw_max = h->wave_nkw_max;
-        m.stamp_base = h->stamp_next;
-        h->stamp_next += (unsigned)T + 1u;
+        if (!take_stamps(&m.stamp_base)) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
         m.spin_limit = h->spin_limit;
         m.withhold_cta = h->withhold_cta;
         m.G = h->G;
@@ -1573,7 +1587,6 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         return LSTM_OK;
     }
 
-    const bool rec = recording(st);
     for (int l = 0; l < L; ++l) {
         Layer &ly = h->layers[l];
         const float *Xf = l == 0 ? x : h->ybuf[(l - 1) & 1];
@@ -1632,8 +1645,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             m.dir0 = h->seq_dirs ? pass : 0; m.ndirs = h->seq_dirs ? 1 : D;
             m.H = H; m.Hh = h->Hh; m.B = B; m.T = T; m.D = D; m.ncta_dir = h->ncta_dir; m.nsplit = nsplit;
             m.nks1 = h->mma_nks; m.nkw2 = h->hl_nkw2;
-            m.stamp_base = h->stamp_next;
-            h->stamp_next += (unsigned)T + 1u;
+            if (!take_stamps(&m.stamp_base)) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
             m.spin_limit = h->spin_limit;
             m.withhold_cta = h->withhold_cta;
             for (int d = 0; d < D; ++d) { m.frag1[d] = ly.wfrag[d]; m.frag2[d] = ly.frag2[d]; }
@@ -1701,8 +1713,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             m.dir0 = h->seq_dirs ? pass : 0; m.ndirs = h->seq_dirs ? 1 : D;
             m.H = H; m.B = B; m.T = T; m.D = D; m.ncta_dir = h->ncta_dir; m.nsplit = nsplit;
             m.kspan = h->csr_kspan; m.mt = h->csr_mt;
-            m.stamp_base = h->stamp_next;
-            h->stamp_next += (unsigned)T + 1u;
+            if (!take_stamps(&m.stamp_base)) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
             m.spin_limit = h->spin_limit;
             m.withhold_cta = h->withhold_cta;
             m.probe = B == 1 ? h->probe : 0;
@@ -1793,8 +1804,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             memset(&m, 0, sizeof m);
             m.dir0 = h->seq_dirs ? pass : 0; m.ndirs = h->seq_dirs ? 1 : D;
             m.H = H; m.B = B; m.T = T; m.D = D; m.ncta_dir = h->ncta_dir; m.nsplit = nsplit; m.nkw_smem = h->mma_nks; m.staged = shp.staged ? 1 : 0;
-            m.stamp_base = h->stamp_next;
-            h->stamp_next += (unsigned)T + 1u;
+            if (!take_stamps(&m.stamp_base)) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
             m.spin_limit = h->spin_limit;
             m.withhold_cta = h->withhold_cta;
             m.probe = B == 1 ? h->probe : 0;
@@ -1827,8 +1837,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         a.dir0 = h->seq_dirs ? pass : 0; a.ndirs = h->seq_dirs ? 1 : D;
         a.H = H; a.Hp8 = h->Hp8; a.Hs = h->Hs; a.B = B; a.T = T; a.D = D;
         a.ncta_dir = h->ncta_dir; a.nsplit = nsplit; a.BT = shp.BT; a.w_smem_bytes = shp.w_smem_bytes; a.stage_all = shp.stage_all ? 1 : 0;
-        a.stamp_base = h->stamp_next;
-        h->stamp_next += (unsigned)T + 1u;
+        if (!take_stamps(&a.stamp_base)) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
         a.spin_limit = h->spin_limit;
         a.withhold_cta = h->withhold_cta;
         for (int d = 0; d < D; ++d) { a.wh[d] = ly.wh[d]; a.csr_ptr[d] = ly.wh_ptr[d]; a.csr_ent[d] = ly.wh_ent[d]; }

@@ -25,3 +25,18 @@ def test_nan_in_one_unit(oracle, c):
         assert np.array_equal(np.isnan(got), np.isnan(want)), name
         ok = ~np.isnan(want)
         assert np.abs(got - want)[ok].max(initial=0) <= wl.TOLERANCE[dtype], name
+
+
+@pytest.mark.parametrize("H,B", [(300, 5), (600, 3), (600, 20)])
+def test_nan_in_one_unit_of_a_pruned_batch(oracle, H, B):
+    # (all 24 bits of h in a word; the removed weights are multiplied, so the NaN reaches the whole row one step later)
+    w = wl.Workload("nan", 1, False, 24, H, 6, B, "bf16", min(0.3, 1 / H ** 0.5), density=0.3, seed=H + B)
+    weights, x = wl.make(w)
+    h0, c0 = wl.make_states(w)
+    ref = oracle.forward(weights, x, h0, c0, layers=1, bidir=False, hidden=H)
+    c0[0, B - 1, H // 3] = np.nan
+    y, hT, cT = run_gpu(w, csr_weights(oracle, weights), x, h0, c0, exec_mode="csr")
+    assert np.isnan(y[0]).sum() == 1 and np.isnan(y[0, B - 1, H // 3])
+    assert np.isnan(y[2:, B - 1]).all() and np.isnan(hT[0, B - 1]).all() and np.isnan(cT[0, B - 1]).all()
+    for got, want in ((y[:, :-1], ref[0][:, :-1]), (hT[:, :-1], ref[1][:, :-1]), (cT[:, :-1], ref[2][:, :-1])):
+        assert np.abs(got - want).max() <= wl.TOLERANCE["bf16"]
