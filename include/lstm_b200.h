@@ -258,7 +258,7 @@ enum {
     LSTM_RAN_WAVE        = 4,    /* recur_wave_kernel: all layers in one launch */
     LSTM_RAN_BATCHED     = 5,    /* recur_tc_kernel: several sequences, weights in tensor memory */
     LSTM_RAN_SPARSE      = 6,    /* recur_csr_kernel: lists of surviving weights in registers */
-    LSTM_RAN_F32         = 7,    /* recur_f32_kernel: narrow fp32 layers */
+    LSTM_RAN_F32         = 7,    /* recur_f32_kernel: narrow fp32 layers; recur_f32_wave_kernel: all layers of a stack of them */
     LSTM_RAN_STEP        = 8,    /* lstm_step_kernel: a single timestep */
     LSTM_RAN_HLSTM_ROWS  = 9,    /* hlstm_mma_kernel: H-LSTM, batch rows one after the other */
     LSTM_RAN_HLSTM_TILES = 10    /* hlstm_tile_kernel: H-LSTM for batches */

@@ -92,6 +92,8 @@ struct lstm_handle {
     RecurTcPlan tcb[2] = {{0, 0, 0, 0, 0, 0}, {0, 0, 0, 0, 0, 0}};
     PhaseWords tcb_xch[2];
     PhaseWords f32_xch;                // fp32 dense, at most two units per CTA
+    int f32w_upc = 0;                  // fp32 stacks, all layers in one launch: units per CTA (0: not served) and exchange words
+    PhaseWords f32w_xch;
     // H-LSTM cell: width of the hidden layer inside each gate (0: plain LSTM), pass-2 column tiles per warp
     int Hh = 0, hl_nkw2 = 0;
     bool use_ht = false;               // H-LSTM: the tile kernel serves calls with several rows (use_mma: the row kernel the others)
@@ -294,7 +296,7 @@ int alloc_phase_words(lstm_handle *h, PhaseWords &x, size_t set_words, cudaStrea
 int alloc_recorded_words(lstm_handle *h, cudaStream_t st)
 {
     int rc = LSTM_OK;
-    for (PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->f32_xch, &h->ht_hx, &h->ht_rx})
+    for (PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->f32_xch, &h->f32w_xch, &h->ht_hx, &h->ht_rx})
         if (rc == LSTM_OK && x->words) rc = dev_alloc(h, &x->recorded, 2 * x->set_words * sizeof(unsigned), true, st, "exchange words");
     return rc;
 }
@@ -632,7 +634,7 @@ void free_all(lstm_handle *h)
     }
     cudaFree(h->G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
     cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); 
-    for (const PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->f32_xch, &h->ht_hx, &h->ht_rx}) { cudaFree(x->words); cudaFree(x->recorded); }
+    for (const PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->f32_xch, &h->f32w_xch, &h->ht_hx, &h->ht_rx}) { cudaFree(x->words); cudaFree(x->recorded); }
     cudaFree(h->status_dev);
     for (int l = 0; l < kMaxWaveLayers; ++l) cudaFree(h->wave_frag[l]);
     cudaFree(h->wave_xch);
@@ -1045,6 +1047,16 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     }
     if (rc == LSTM_OK && dtype == LSTM_F32 && !csr && h->upc <= 2 && H <= kF32MaxUnits)
         rc = alloc_phase_words(h, h->f32_xch, (size_t)D * 2 * H * 32, st);
+    {
+        const char *env = getenv("LSTM_B200_WAVE");
+        const int upc = dtype == LSTM_F32 && !csr && D == 1 && !(env && strcmp(env, "0") == 0) ? recur_f32_wave_units(layers, H, in_dim, h->sm_count) : 0;
+        if (rc == LSTM_OK && upc) {
+            rc = alloc_phase_words(h, h->f32w_xch, (size_t)layers * std::min(max_T, kF32WaveMaxT) * H * 32, st);
+            if (rc == LSTM_OK && recur_f32_wave_prepare(in_dim, H, upc) != cudaSuccess)
+                rc = fail(h, LSTM_ERR_CUDA, "fp32 stack kernel set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
+            h->f32w_upc = upc;
+        }
+    }
     for (int i = 0; i < 2 && rc == LSTM_OK; ++i)
         if (i ? h->use_tc1 : h->use_tcb) rc = alloc_phase_words(h, h->tcb_xch[i], recur_tc_xch_words(H, h->tcb[i].rows, D), st);
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->status_dev, sizeof(int), true, st, "status word");
@@ -1584,6 +1596,35 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         ++h->last_launches;
         if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "wavefront launch failed: %s", cudaGetErrorString(e));
+        return LSTM_OK;
+    }
+
+    if (h->f32w_upc && B <= kF32MaxRows && T <= kF32WaveMaxT) {
+        // fp32 stack: all layers and their projections in one launch
+        RecurF32WaveArgs m;
+        memset(&m, 0, sizeof m);
+        m.L = L; m.H = H; m.Hp8 = h->Hp8; m.B = B; m.T = T; m.in_dim = h->in_dim; m.upc = h->f32w_upc;
+        m.ncta = (H + m.upc - 1) / m.upc;
+        m.spin_limit = h->spin_limit;
+        m.withhold_cta = h->withhold_cta < 0 ? -1 : h->withhold_cta % (m.ncta * L);
+        m.x = x;
+        for (int l = 0; l < L; ++l) {
+            const Layer &ly = h->layers[l];
+            m.wx[l] = (const float *)ly.wx; m.ldx[l] = ly.ldk; m.wh[l] = (const float *)ly.wh[0]; m.bias[l] = ly.bias;
+        }
+        m.h0 = h0; m.c0 = c0; m.hT = hT; m.cT = cT; m.y = y;
+        m.slots = std::min(h->max_T, kF32WaveMaxT);
+        unsigned clear_T = 0;
+        if (phase_sets(h->f32w_xch, rec, st, &m.xch, &m.set, &clear_T) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
+        m.clear_T = (int)clear_T;
+        m.status = h->status_dev;
+        if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+        e = launch_recur_f32_wave(m, st);
+        if (e == cudaSuccess) phase_launched(h->f32w_xch, rec, (unsigned)T);
+        ran(h, LSTM_RAN_F32, m.ncta * L, kF32Threads, 0);
+        ++h->last_launches;
+        if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+        if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "stack launch failed: %s", cudaGetErrorString(e));
         return LSTM_OK;
     }
 

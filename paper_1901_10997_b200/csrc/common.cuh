@@ -220,6 +220,32 @@ cudaError_t recur_wave_prepare(int mt, int nkr, int max_smem);
 cudaError_t launch_recur_wave(const RecurWaveArgs &a, int mt, int nkr, size_t smem, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------
+// All layers of a unidirectional fp32 stack in one launch (recur_f32_wave.cu): CTAs [l * ncta, (l + 1) * ncta) run layer l, upc
+// units each, on [x_t or the layer below's h_t ; h_{t-1}].
+// ---------------------------------------------------------------------------------------------------
+constexpr int kF32WaveMaxT = 256;     // longest call: the exchange words have a slot for every timestep
+struct RecurF32WaveArgs {
+    int L, H, Hp8, B, T, in_dim, ncta, upc;
+    long long spin_limit;
+    int withhold_cta;
+    const float *x;                     // [T][B][in_dim]
+    const float *wx[kMaxWaveLayers];    // [H][4] rows of ldx elements
+    const float *wh[kMaxWaveLayers];    // [H][4] rows of Hp8 elements
+    const float *bias[kMaxWaveLayers];  // [H][4]
+    int ldx[kMaxWaveLayers];
+    const float *h0, *c0;               // [L][B][H] or nullptr
+    float *hT, *cT;
+    float *y;                           // [T][B][H]: the top layer's h
+    unsigned *xch;                      // exchange words [2 sets][L][slots][H][32 batch rows]
+    int slots;                          // timesteps there is room for
+    int set, clear_T;                   // the set this launch uses; it clears the other one as far as clear_T timesteps
+    int *status;
+};
+int recur_f32_wave_units(int L, int H, int in_dim, int max_cta);
+cudaError_t recur_f32_wave_prepare(int in_dim, int H, int upc);
+cudaError_t launch_recur_f32_wave(const RecurF32WaveArgs &a, cudaStream_t st);
+
+// ---------------------------------------------------------------------------------------------------
 // Register-resident sparse recurrent kernel (bf16 weights, CSR execution).  Same CTA/unit partition,
 // exchange buffer and finishing role as the dense register-resident kernel.  Warp w of a CTA owns the
 // columns [w * kspan, (w + 1) * kspan) of h; inside the warp every lane owns up to two of the CTA's 4 * units

@@ -158,6 +158,16 @@ __device__ __forceinline__ float gate_fast(float z, float neg_k_log2e, float sc,
 __device__ __forceinline__ float sigmoid_fast(float z) { return __fdividef(1.0f, 1.0f + ex2_fast(-1.4426950408889634f * z)); }
 __device__ __forceinline__ float tanh_fast(float z) { return fmaf(2.0f, __fdividef(1.0f, 1.0f + ex2_fast(-2.8853900817779268f * z)), -1.0f); }
 
+// sc / (1 + e^(k z)) + of: the logistic function (k, sc, of = -1, 1, 0) or tanh (-2, 2, -1).  tanh of a small z is the
+// difference of two nearby numbers there, which loses the digits of z (all of them near 1e-16): below 1e-4 it is z - z^3 / 3
+// (off by less than 2 z^4 / 15 of it).  expm1 in place of both costs 0.4 us a step.
+__device__ __forceinline__ double gate_f64(double z, double k, double sc, double of)
+{
+    double act = sc / (1.0 + exp(k * z)) + of;
+    if (of != 0.0 && (__double2hiint(z) & 0x7fffffff) < 0x3f1a36e2) act = fma(z * z, z * (-1.0 / 3.0), z);       // |z| < 1e-4
+    return act;
+}
+
 // hidden units [u0, u0 + n) of CTA c when H units are split evenly over nc CTAs
 __host__ __device__ __forceinline__ void unit_range(int H, int nc, int c, int &u0, int &n)
 {

@@ -21,16 +21,6 @@ namespace {
 
 constexpr int kThreads = kF32Threads, kWarps = kThreads / 32;
 
-// sc / (1 + e^(k z)) + of: the logistic function (k, sc, of = -1, 1, 0) or tanh (-2, 2, -1).  tanh of a small z is the
-// difference of two nearby numbers there, which loses the digits of z (all of them near 1e-16): below 1e-4 it is z - z^3 / 3
-// (off by less than 2 z^4 / 15 of it).  expm1 in place of both costs 0.4 us a step.
-__device__ __forceinline__ double gate_f64(double z, double k, double sc, double of)
-{
-    double act = sc / (1.0 + exp(k * z)) + of;
-    if (of != 0.0 && (__double2hiint(z) & 0x7fffffff) < 0x3f1a36e2) act = fma(z * z, z * (-1.0 / 3.0), z);       // |z| < 1e-4
-    return act;
-}
-
 // NT: tiles of eight batch rows
 template <int NT>
 __global__ void __launch_bounds__(kThreads, 1) recur_f32_kernel(const RecurF32Args a)
