@@ -108,7 +108,7 @@ typedef struct {
  *                   = tc1   batched tensor-core recurrence without cluster pairs
  *   LSTM_B200_FUSE  = 0     never compute the input projection inside the recurrent kernel (single sequences of up
  *                           to 40 steps on the register-resident kernel do so by default)
- *   LSTM_B200_WAVE  = 0     one launch per layer even where the layer-wavefront kernel would serve the stack
+ *   LSTM_B200_WAVE  = 0     one launch per layer even where a kernel that runs the layers of a stack side by side would serve it
  *                   = 1     the layer-wavefront kernel for every call of up to four sequences, single timesteps
  *                           included, where it serves the stack
  *   LSTM_B200_PROJ  = simt  CUDA-core input projection instead of the tensor-core one
@@ -256,7 +256,7 @@ enum {
     LSTM_RAN_REGISTERS   = 2,    /* recur_mma_kernel: weights in registers */
     LSTM_RAN_ONE         = 3,    /* recur_one_kernel: one sequence of a wide layer */
     LSTM_RAN_WAVE        = 4,    /* recur_wave_kernel: all layers in one launch */
-    LSTM_RAN_BATCHED     = 5,    /* recur_tc_kernel: several sequences, weights in tensor memory */
+    LSTM_RAN_BATCHED     = 5,    /* recur_tc_kernel: several sequences, weights in tensor memory; recur_stack_kernel: two layers of them */
     LSTM_RAN_SPARSE      = 6,    /* recur_csr_kernel: lists of surviving weights in registers */
     LSTM_RAN_F32         = 7,    /* recur_f32_kernel: narrow fp32 layers; recur_f32_wave_kernel: all layers of a stack of them */
     LSTM_RAN_STEP        = 8,    /* lstm_step_kernel: a single timestep */

@@ -12,7 +12,7 @@ CSRC = PKG / "csrc"
 LIB = PKG / "liblstm_b200.so"
 LIB_CHECKED = PKG / "liblstm_b200_checked.so"       # same sources with -DLSTM_B200_CHECKED: index checks inside the kernels
 INCLUDE = PKG.parent / "include"
-SOURCES = ["api.cu", "recur.cu", "recur_f32.cu", "recur_f32_wave.cu", "proj_simt.cu", "proj_tc.cu", "noalloc.cu", "recur_mma.cu", "recur_one.cu", "hlstm_mma.cu", "hlstm_tile.cu", "lstm_step.cu", "recur_tc.cu", "host_tools.cu", "recur_csr.cu", "csr_pack.cu", "compact.cu", "recur_wave.cu"]
+SOURCES = ["api.cu", "recur.cu", "recur_f32.cu", "recur_f32_wave.cu", "proj_simt.cu", "proj_tc.cu", "noalloc.cu", "recur_mma.cu", "recur_one.cu", "hlstm_mma.cu", "hlstm_tile.cu", "lstm_step.cu", "recur_tc.cu", "recur_stack.cu", "host_tools.cu", "recur_csr.cu", "csr_pack.cu", "compact.cu", "recur_wave.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "--use_fast_math=false"]
 

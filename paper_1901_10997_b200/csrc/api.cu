@@ -39,6 +39,7 @@ struct Layer {
     uint4 *xfrag[2] = {nullptr, nullptr};  //   and Wx in the same layout (projection fused into the kernel's prologue)
     int nkw_x = 0;
     uint4 *wtc[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // batched tensor-core kernel, by plan and direction: [cta][8-column piece][row 4 * unit + gate]
+    uint4 *wst = nullptr;                  //   the same for a stack of two layers in one launch
     uint4 *frag2[2] = {nullptr, nullptr};  // H-LSTM: fragments of the gate output matrices W
     uint4 *tfrag[2] = {nullptr, nullptr}, *tfrag2[2] = {nullptr, nullptr};     //   the tile kernel's fragments of Uh and W
     float *bias_out = nullptr;             // H-LSTM: [D][H][4] bias of the gate pre-activations
@@ -91,6 +92,13 @@ struct lstm_handle {
     bool use_tcb = false, use_tc1 = false;
     RecurTcPlan tcb[2] = {{0, 0, 0, 0, 0, 0}, {0, 0, 0, 0, 0, 0}};
     PhaseWords tcb_xch[2];
+    // two layers of a batch side by side: partition, exchange words behind the counts, the upper layer's G, and the projecting
+    // CTAs' work for calls of stack_T x stack_B
+    bool use_stack = false;
+    RecurTcPlan stack = {0, 0, 0, 0, 0, 0};
+    PhaseWords stack_xch;
+    float *stack_G = nullptr; int stack_M = 0;
+    StackProjArgs stack_proj; StackProjMaps stack_maps; int stack_chunk = 0, stack_T = 0, stack_B = 0;
     PhaseWords f32_xch;                // fp32 dense, at most two units per CTA
     int f32w_upc = 0;                  // fp32 stacks, all layers in one launch: units per CTA (0: not served) and exchange words
     PhaseWords f32w_xch;
@@ -296,7 +304,7 @@ int alloc_phase_words(lstm_handle *h, PhaseWords &x, size_t set_words, cudaStrea
 int alloc_recorded_words(lstm_handle *h, cudaStream_t st)
 {
     int rc = LSTM_OK;
-    for (PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->f32_xch, &h->f32w_xch, &h->ht_hx, &h->ht_rx})
+    for (PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->stack_xch, &h->f32_xch, &h->f32w_xch, &h->ht_hx, &h->ht_rx})
         if (rc == LSTM_OK && x->words) rc = dev_alloc(h, &x->recorded, 2 * x->set_words * sizeof(unsigned), true, st, "exchange words");
     return rc;
 }
@@ -564,6 +572,21 @@ bool wave_serves(const lstm_handle *h, int T, int B)
 // 1.00 - 1.09; six steps with 2 rows 0.95 - 1.07; one step with 5 rows 1.00 - 1.08.
 bool lists_serve(const lstm_handle *h, int T, int B) { return h->use_csr_reg && (B == 1 || !h->use_tcb || (B <= 4 && T * B <= 8)); }
 
+// Do two layers of a batch run side by side?  The lag of the upper layer, one chunk and its projection, has to be earned back.  Time per
+// call, side by side / one after the other, T = 4, 8, 16, 35, 70: H = 200 with 8, 32 rows 0.86, 0.82, 0.79, 0.75, 0.74 and 0.78,
+// 0.75, 0.72, 0.68, 0.67; 517 with 3, 20 rows 0.80, 0.76, 0.68, 0.70, 0.70 and 0.86, 0.75, 0.72, 0.67, 0.64; 1000 with 2, 32 rows
+// 0.96, 0.84, 0.75, 0.67, 0.64 and 1.00, 0.84, 0.77, 0.71, 0.66.  Wider layers, whose pairs have a second block of rows: 1250 with 2,
+// 20 rows 1.06, 0.97, 0.88, 0.84, 0.81 and 1.14, 1.04, 0.96, 0.91, 0.84; 1500 with 4, 20, 24, 32 rows 1.12, 1.05, 0.95, 0.82, 0.75;
+// 1.20, 0.98, 0.93, 0.88, 0.82; 1.15, 1.00, 0.99, 0.92, 0.91; 1.12, 1.04, 1.07, 1.06, 1.06 (three blocks of rows on each projecting CTA,
+// which no longer keep up).  Pruned layers the same: 800 with 2, 16 rows, T = 8 0.80, 0.72; 1500 with 16 rows, T = 35 0.84.
+bool stack_serves(const lstm_handle *h, int T, int B)
+{
+    if (!h->use_stack || h->probe || B < kStackMinRows || B > h->stack.rows || (long long)T * B > h->stack_M || T > kStackMaxChunks || lists_serve(h, T, B)) return false;
+    if (8 * h->stack.upc <= 128) return T >= 4;
+    const int blocks = (4 * h->H + 128 * (h->sm_count / 2 * 2 - 2 * h->stack.ncta) - 1) / (128 * (h->sm_count / 2 * 2 - 2 * h->stack.ncta));
+    return T >= 16 && (blocks < 3 || B <= 24);
+}
+
 // Rows of a [4H x H] recurrent matrix (row q*H + j, dense or as lists) as the batched tensor-core kernel wants them: per CTA [8-column
 // piece of its K range][row 4 * unit + gate of its units, in pair mode of both CTAs' units] 8 bf16.
 std::vector<uint16_t> pack_tc_rows(const float *m, const HostCsr *lists, int H, const RecurTcPlan &p)
@@ -631,10 +654,11 @@ void free_all(lstm_handle *h)
         for (int d = 0; d < 2; ++d) { cudaFree(ly.wh[d]); cudaFree(ly.wh_ptr[d]); cudaFree(ly.wh_ent[d]); cudaFree(ly.wfrag[d]); cudaFree(ly.ofrag[d]); cudaFree(ly.oxfrag[d]); cudaFree(ly.xfrag[d]); cudaFree(ly.frag2[d]); cudaFree(ly.tfrag[d]); cudaFree(ly.tfrag2[d]); cudaFree(ly.csr_reg_ent[d]); cudaFree(ly.csr_reg_rows[d]); }
         cudaFree(ly.bias_out);
         for (int i = 0; i < 4; ++i) cudaFree(ly.wtc[i >> 1][i & 1]);
+        cudaFree(ly.wst);
     }
-    cudaFree(h->G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
+    cudaFree(h->G); cudaFree(h->stack_G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
     cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); 
-    for (const PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->f32_xch, &h->f32w_xch, &h->ht_hx, &h->ht_rx}) { cudaFree(x->words); cudaFree(x->recorded); }
+    for (const PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->stack_xch, &h->f32_xch, &h->f32w_xch, &h->ht_hx, &h->ht_rx}) { cudaFree(x->words); cudaFree(x->recorded); }
     cudaFree(h->status_dev);
     for (int l = 0; l < kMaxWaveLayers; ++l) cudaFree(h->wave_frag[l]);
     cudaFree(h->wave_xch);
@@ -789,6 +813,14 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         if (h->use_mma) { h->seq_dirs = true; h->use_tcb = plan_tcb(h->ncta_dir, 1); }
         else { h->ncta_dir = nc; h->upc = up; h->threads = th; }
     }
+    if (h->use_tcb && D == 1 && layers == 2 && h->use_tc && !getenv("LSTM_B200_WAVE") && !getenv("LSTM_B200_RECUR")) {
+        const int smem = h->smem_optin - kTcStaticSmem;
+        bool fits = false;
+        h->use_stack = recur_stack_plan(H, h->sm_count, max_B, tc_terms, (size_t)smem, &h->stack) &&
+                       recur_stack_prepare(h->stack, h->sm_count, smem, &fits) == cudaSuccess && fits;
+        if (!h->use_stack) cudaGetLastError();
+        h->stack_M = std::min(max_T * std::min(max_B, h->stack.rows), kStackMaxRows);
+    }
     {
         const char *fenv = getenv("LSTM_B200_FUSE"), *renv = getenv("LSTM_B200_RECUR");
         h->use_one = h->use_mma && !(renv && strcmp(renv, "mma") == 0) && recur_one_plan(H, h->ncta_dir, (size_t)h->smem_optin - 64, &h->one);
@@ -914,6 +946,11 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                     rc = upload(h, (uint16_t **)&ly.wtc[i][d], p.data(), p.size() * 2, st, "recurrent weight rows");
                     if (rc == LSTM_OK) cudaStreamSynchronize(st);
                 }
+                if (rc == LSTM_OK && h->use_stack) {
+                    const std::vector<uint16_t> p = pack_tc_rows(m.data(), nullptr, H, h->stack);
+                    rc = upload(h, (uint16_t **)&ly.wst, p.data(), p.size() * 2, st, "recurrent weight rows");
+                    if (rc == LSTM_OK) cudaStreamSynchronize(st);
+                }
             } else {
                 HostCsr cx, ch;
                 snprintf(name, sizeof name, "wx[layer %d, dir %d]", l, d);
@@ -950,6 +987,11 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                     for (int i = 0; i < (h->use_tc1 ? 2 : 1) && rc == LSTM_OK; ++i) {
                         const std::vector<uint16_t> p = pack_tc_rows(nullptr, &ch, H, h->tcb[i]);
                         rc = upload(h, (uint16_t **)&ly.wtc[i][d], p.data(), p.size() * 2, st, "recurrent weight rows");
+                        if (rc == LSTM_OK) cudaStreamSynchronize(st);
+                    }
+                    if (rc == LSTM_OK && h->use_stack) {
+                        const std::vector<uint16_t> p = pack_tc_rows(nullptr, &ch, H, h->stack);
+                        rc = upload(h, (uint16_t **)&ly.wst, p.data(), p.size() * 2, st, "recurrent weight rows");
                         if (rc == LSTM_OK) cudaStreamSynchronize(st);
                     }
                     if (rc) break;
@@ -1059,6 +1101,10 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     }
     for (int i = 0; i < 2 && rc == LSTM_OK; ++i)
         if (i ? h->use_tc1 : h->use_tcb) rc = alloc_phase_words(h, h->tcb_xch[i], recur_tc_xch_words(H, h->tcb[i].rows, D), st);
+    if (rc == LSTM_OK && h->use_stack) {
+        rc = alloc_phase_words(h, h->stack_xch, 2 * kStackMaxChunks + 2 * recur_tc_xch_words(H, h->stack.rows, 1), st);
+        if (rc == LSTM_OK) rc = dev_alloc(h, &h->stack_G, (size_t)h->stack_M * 4 * H * 4, false, st, "upper layer's projection");
+    }
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->status_dev, sizeof(int), true, st, "status word");
     if (rc == LSTM_OK && h->use_wave) {
         h->wave_xch_words = (size_t)layers * max_T * std::min(max_B, 4) * H;
@@ -1622,6 +1668,64 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         e = launch_recur_f32_wave(m, st);
         if (e == cudaSuccess) phase_launched(h->f32w_xch, rec, (unsigned)T);
         ran(h, LSTM_RAN_F32, m.ncta * L, kF32Threads, 0);
+        ++h->last_launches;
+        if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+        if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "stack launch failed: %s", cudaGetErrorString(e));
+        return LSTM_OK;
+    }
+
+    if (stack_serves(h, T, B)) {
+        // two layers of a batch: the lower one's projection, then both recurrences and the upper one's projection in one launch
+        const Layer &up = h->layers[1];
+        const RecurTcPlan &plan = h->stack;
+        const long long plane = (long long)h->max_T * h->max_B * h->ldn;
+        if (h->stack_T != T || h->stack_B != B) {
+            memset(&h->stack_proj, 0, sizeof h->stack_proj);
+            h->stack_T = 0;
+            if (!recur_stack_proj_plan(plan, H, T, B, h->sm_count, (size_t)h->smem_optin - kTcStaticSmem, &h->stack_proj, &h->stack_chunk) ||
+                !stack_proj_maps(&h->stack_maps, (const __nv_bfloat16 *)up.wx, h->xbn[0], h->xbn[0] + plane, h->stack_proj, H, up.ldk, h->ldn))
+                return fail(h, LSTM_ERR_CUDA, "stack projection plan failed");
+            h->stack_T = T; h->stack_B = B;
+        }
+        int nsplit = 1;
+        { const int prc = run_projection(h, 0, x, x, M, 4 * H, &nsplit, st); if (prc != LSTM_OK) return prc; }
+        RecurStackArgs s;
+        memset(&s, 0, sizeof s);
+        unsigned *base = nullptr;
+        int set = 0;
+        if (phase_sets(h->stack_xch, rec, st, &base, &set, &s.clear_words) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
+        unsigned *counts = base + (size_t)set * h->stack_xch.set_words;
+        s.other_set = base + (size_t)(set ^ 1) * h->stack_xch.set_words;
+        for (int l = 0; l < 2; ++l) {
+            RecurTcArgs &m = s.layer[l];
+            m.ndirs = 1; m.H = H; m.B = m.Bs = B; m.T = T; m.D = 1;
+            m.ncta_dir = plan.ncta; m.upc = plan.upc; m.KH = plan.KH; m.pair = 1; m.terms = plan.terms;
+            m.nsplit = l ? 1 : nsplit;
+            m.spin_limit = h->spin_limit;
+            m.withhold_cta = h->withhold_cta < 0 ? -1 : h->withhold_cta % (2 * plan.ncta);
+            m.wpack[0] = h->layers[l].wst;
+            m.G = l ? h->stack_G : h->G;
+            m.g_split_stride = (long long)M * 4 * H;
+            const size_t so = (size_t)l * B * H;
+            m.h0 = h0 ? h0 + so : nullptr; m.c0 = c0 ? c0 + so : nullptr;
+            m.hT = hT ? hT + so : nullptr; m.cT = cT ? cT + so : nullptr;
+            if (l) m.y = y;
+            else { m.xb_next = h->xbn[0]; m.xb_ld = h->ldn; m.xb_plane = plane; }
+            m.xch = base + 2 * kStackMaxChunks + l * recur_tc_xch_words(H, B, 1);
+            m.set_words = h->stack_xch.set_words;
+            m.set = set;
+            m.status = h->status_dev;
+        }
+        s.proj = h->stack_proj;
+        s.proj.bias = up.bias; s.proj.G = h->stack_G;
+        s.proj.stored = s.proj.stored_out = counts; s.proj.n_stored = (unsigned)plan.ncta;
+        s.proj.ready = counts + kStackMaxChunks;
+        s.proj.spin_limit = h->spin_limit; s.proj.status = h->status_dev;
+        s.chunk = h->stack_chunk;
+        if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
+        e = launch_recur_stack(s, h->stack_maps, plan, h->sm_count, st);
+        if (e == cudaSuccess) phase_launched(h->stack_xch, rec, (unsigned)(2 * kStackMaxChunks + 2 * recur_tc_xch_words(H, B, 1)));
+        ran(h, LSTM_RAN_BATCHED, h->sm_count / 2 * 2, kTcThreads, recur_stack_smem_bytes(plan, B, s.proj));
         ++h->last_launches;
         if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "stack launch failed: %s", cudaGetErrorString(e));

@@ -347,6 +347,43 @@ cudaError_t recur_tc_prepare(int terms, int max_smem);
 cudaError_t launch_recur_tc(const RecurTcArgs &a, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------
+// Two stacked layers of a batch in one launch (recur_stack.cu): the pairs of layer[0], those of layer[1], and the CTAs that project
+// chunks of the lower layer's h onto the upper layer's gates (stack_proj.cuh).
+// ---------------------------------------------------------------------------------------------------
+constexpr int kStackMaxChunks = 256;
+constexpr int kStackMinProj = 16;     // projecting CTAs, at least
+constexpr int kStackMinRows = 2;
+constexpr int kStackMaxRows = 8192;   // rows (timesteps x sequences) of a call, at most
+struct StackProjArgs {
+    int M, N, kblocks;          // rows of X, columns of G, 64-column blocks of K
+    int rb, mb;                 // rows of Wx per block (multiple of 8, at most 128), blocks per CTA
+    int chunk_rows, nrp, nchunks;       // rows of X per chunk; the same as a multiple of 8
+    int stages;
+    const float *bias;
+    float *G;                   // [M][N]
+    const unsigned *stored;     // [chunk] CTAs of the lower layer that have stored their part of X; complete at n_stored
+    unsigned *stored_out;       //   (the same, for the lower layer)
+    unsigned n_stored;
+    unsigned *ready;            // [chunk] projecting CTAs that have stored their rows of G
+    long long spin_limit;
+    int *status;
+};
+struct RecurStackArgs {
+    RecurTcArgs layer[2];
+    StackProjArgs proj;
+    int chunk;                  // timesteps
+    unsigned *other_set;        // exchange words and counts of the next launch, cleared as far as the previous one wrote them
+    unsigned clear_words;
+};
+struct StackProjMaps { alignas(64) unsigned char w[128], x[128], xlo[128]; };
+bool recur_stack_plan(int H, int sm_count, int rows_wanted, int terms, size_t max_smem, RecurTcPlan *p);
+cudaError_t recur_stack_prepare(const RecurTcPlan &p, int sm_count, int max_smem, bool *fits);
+bool recur_stack_proj_plan(const RecurTcPlan &p, int H, int T, int B, int sm_count, size_t max_smem, StackProjArgs *a, int *chunk);
+bool stack_proj_maps(StackProjMaps *m, const __nv_bfloat16 *W, const __nv_bfloat16 *X, const __nv_bfloat16 *Xlo, const StackProjArgs &a, int K, int ldk, int ldx);
+size_t recur_stack_smem_bytes(const RecurTcPlan &p, int rows, const StackProjArgs &a);
+cudaError_t launch_recur_stack(const RecurStackArgs &a, const StackProjMaps &maps, const RecurTcPlan &p, int sm_count, cudaStream_t st);
+
+// ---------------------------------------------------------------------------------------------------
 // H-LSTM recurrent kernel (one ReLU hidden layer of width Hh inside each gate; bf16 weights, dense).
 // Pass 1 works on the four Uh_q [Hh x H] (hidden units split over the CTAs, fragments in registers and,
 // beyond nkr tiles per warp, in shared memory), pass 2 on the four W_q [H x Hh] (cell units split over the

@@ -1,0 +1,162 @@
+// Two stacked layers of a batch in one launch (paper, Section 5.1: the language model is two stacked recurrent layers): the upper
+// layer's recurrence runs some timesteps behind the lower one's, on SMs of its own, instead of after it.  A recurrence is bound by
+// the latency of its step and not by the SMs it runs on, so T steps plus the lag take little more than half of 2 T.
+//
+// Three groups of CTAs: the lower layer's and the upper layer's recurrence, each the CTA pairs of recur_tc.cu with its weights
+// resident (up to 192 accumulator rows a pair: the first 128 from tensor memory, the others from shared memory), and
+// between them the CTAs of stack_proj.cuh, which turn a chunk of timesteps of the lower layer's h into rows of the upper layer's G.
+// All three of the matrices do not fit the chip at 1500 x 1500; the one without a recurrence is streamed once per chunk.
+// Measured (us per call, one after the other -> here): 2 x 517, 3 rows, T = 23 137 -> 93; 2 x 1000, 8 rows, T = 35 206 -> 134; 2 x 1500, 20
+// rows, T = 35 296 -> 259; pruned, 16 rows 294 -> 244.  At 1500 and 20 rows a step takes 5.1 us (products 2650 clocks: 47 of 128 and
+// 47 of 64 rows at N = 48) and a chunk of four steps 22 us of the projecting CTAs, whose products are bound by shared memory:
+// 167 KB a K block, weights once in and once out, activations once in and three times out.
+// The groups meet through counts in global memory, one per chunk: "planes of X stored" and "rows of G stored".
+// All CTAs of the launch are resident (cooperative launch); every wait is bounded.
+#include "recur_tc_role.cuh"
+#include "stack_proj.cuh"
+
+#include <algorithm>
+#include <cstring>
+
+namespace lstm {
+namespace {
+
+template <int RG, int TERMS, int MB>
+__global__ void __launch_bounds__(kThreads, 1)
+recur_stack_kernel(const __grid_constant__ RecurStackArgs a, const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
+                   const __grid_constant__ CUtensorMap tmap_xlo)
+{
+    extern __shared__ __align__(16) unsigned char smem_stack[];
+    // the other set of exchange words and counts, for the next launch
+    for (unsigned i = blockIdx.x * kThreads + threadIdx.x; i < a.clear_words / 4u; i += gridDim.x * kThreads)
+        reinterpret_cast<uint4 *>(a.other_set)[i] = make_uint4(0, 0, 0, 0);
+    const int n = a.layer[0].ncta_dir, b = blockIdx.x;
+    if (b < n) recur_tc_role<RG, true, TERMS, MB, kTcLower>(a.layer[0], b, TcLink{a.chunk, a.proj.stored_out, nullptr, 0});
+    else if (b < 2 * n) recur_tc_role<RG, true, TERMS, MB, kTcUpper>(a.layer[1], b - n, TcLink{a.chunk, nullptr, a.proj.ready, (unsigned)(gridDim.x - 2 * n)});
+    else stack_proj_role(smem_stack, &tmap_w, &tmap_x, &tmap_xlo, a.proj, b - 2 * n);
+}
+
+typedef void (*KernelFn)(const RecurStackArgs, const CUtensorMap, const CUtensorMap, const CUtensorMap);
+template <int TERMS, int MB> KernelFn pick_m(int rg)
+{
+    switch (rg) {
+        case 1: return recur_stack_kernel<1, TERMS, MB>;
+        case 2: return recur_stack_kernel<2, TERMS, MB>;
+        case 3: if constexpr (TERMS == 2) return recur_stack_kernel<3, TERMS, MB>; else return nullptr;
+        case 4: if constexpr (TERMS == 2) return recur_stack_kernel<4, TERMS, MB>; else return nullptr;
+        default: return nullptr;
+    }
+}
+KernelFn pick(int rg, int terms, int mb)
+{
+    return terms == 3 ? (mb == 2 ? pick_m<3, 2>(rg) : pick_m<3, 1>(rg)) : (mb == 2 ? pick_m<2, 2>(rg) : pick_m<2, 1>(rg));
+}
+int groups_of(int rows) { return (rows + 7) / 8; }
+int blocks_of(int upc) { return 8 * upc > 128 ? 2 : 1; }
+
+size_t role_smem(int KH, int upc, int rows, int terms)
+{
+    const int rg = groups_of(rows), tiles = (KH + 63) / 64;
+    return 1024 + (size_t)tiles * (std::max(0, 8 * upc - 128) + tc_columns(rg, terms)) * 128 + (size_t)2 * 8 * upc * tc_rows_of_first(rg, true) * 4;
+}
+constexpr size_t kProjFixedSmem = 1024 + 120 * 128;            // alignment; the last block of a stage is read as 128 rows
+size_t proj_smem(const StackProjArgs &a) { return kProjFixedSmem + (size_t)a.stages * (a.mb * a.rb + 2 * a.nrp) * 128; }
+
+cudaLaunchConfig_t config(cudaLaunchAttribute (&attr)[2], int grid, size_t smem, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeCooperative;
+    attr[1].val.cooperative = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    return cfg;
+}
+
+}  // namespace
+
+size_t recur_stack_smem_bytes(const RecurTcPlan &p, int rows, const StackProjArgs &a) { return std::max(role_smem(p.KH, p.upc, rows, p.terms), proj_smem(a)); }
+
+// Partition of a stack whose calls have up to rows_wanted rows: CTA pairs of each layer, the others project.
+bool recur_stack_plan(int H, int sm_count, int rows_wanted, int terms, size_t max_smem, RecurTcPlan *p)
+{
+    if (H <= 64) return false;
+    const int KH = ((H + 1) / 2 + 15) / 16 * 16;
+    for (int upc = 4; upc <= 24; upc += 4) {
+        const int n = (H + 2 * upc - 1) / (2 * upc) * 2, mb = blocks_of(upc);
+        if (2 * n + kStackMinProj > sm_count) continue;
+        for (int rg = std::min(terms == 3 ? 2 : 4, groups_of(rows_wanted)); rg >= 1; --rg) {
+            const int acc = mb == 2 ? 2 * tc_columns(rg, terms) : tc_acc_columns(rg, terms);
+            if (KH / 2 + acc > 512 || KH > 16 * kPollers * kMaxGroups || role_smem(KH, upc, 8 * rg, terms) > max_smem) continue;
+            p->upc = upc; p->ncta = n; p->KH = KH; p->pair = 1; p->rows = 8 * rg; p->terms = terms;
+            return true;
+        }
+    }
+    return false;
+}
+
+cudaError_t recur_stack_prepare(const RecurTcPlan &p, int sm_count, int max_smem, bool *fits)
+{
+    *fits = true;
+    for (int rg = 1; rg <= p.rows / 8; ++rg) {
+        KernelFn fn = pick(rg, p.terms, blocks_of(p.upc));
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+        if (e != cudaSuccess) return e;
+        cudaLaunchAttribute attr[2];
+        cudaLaunchConfig_t cfg = config(attr, sm_count / 2 * 2, max_smem, nullptr);
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)fn, &cfg) != cudaSuccess) { cudaGetLastError(); clusters = 0; }
+        if (clusters < sm_count / 2) *fits = false;
+    }
+    return cudaSuccess;
+}
+
+// Rows, blocks and chunk of the projecting CTAs of a call: the shortest chunk that keeps up with the recurrences, or the longest there is
+// room for; false when there is none.
+bool recur_stack_proj_plan(const RecurTcPlan &p, int H, int T, int B, int sm_count, size_t max_smem, StackProjArgs *a, int *chunk)
+{
+    const int nproj = sm_count / 2 * 2 - 2 * p.ncta;
+    a->M = T * B; a->N = 4 * H; a->kblocks = (H + 63) / 64;
+    const int rows = (a->N + nproj - 1) / nproj;
+    a->mb = (rows + 127) / 128;
+    a->rb = ((rows + a->mb - 1) / a->mb + 7) / 8 * 8;
+    a->nrp = 0;
+    const int step = blocks_of(p.upc) == 2 ? 7000 : 4500;           // clock ticks of a step of the recurrence, roughly
+    for (int c = 1; c <= T; ++c) {
+        const int nrp = (c * B + 7) / 8 * 8;
+        if (nrp > 128 || a->mb * 2 * nrp > 512) break;
+        a->nrp = nrp;
+        a->chunk_rows = c * B;
+        *chunk = c;
+        const int bytes = a->mb * a->rb * 128 + 2 * nrp * 128;
+        const int cost = a->kblocks * std::max(bytes / 48, a->mb * 4 * std::max(32, nrp)) + 4000;
+        if (cost * 10 < 9 * c * step) break;
+    }
+    if (a->nrp == 0) return false;
+    a->nchunks = (T + *chunk - 1) / *chunk;
+    a->stages = std::min(kSpStages, (int)((max_smem - kProjFixedSmem) / ((a->mb * a->rb + 2 * a->nrp) * 128)));
+    return a->stages >= 2 && a->nchunks <= kStackMaxChunks;
+}
+
+bool stack_proj_maps(StackProjMaps *m, const __nv_bfloat16 *W, const __nv_bfloat16 *X, const __nv_bfloat16 *Xlo, const StackProjArgs &a, int K, int ldk, int ldx)
+{
+    return encode_tmap_bf16_2d(m->w, W, a.N, K, ldk, a.rb) && encode_tmap_bf16_2d(m->x, X, a.M, K, ldx, a.nrp) &&
+           encode_tmap_bf16_2d(m->xlo, Xlo, a.M, K, ldx, a.nrp);
+}
+
+cudaError_t launch_recur_stack(const RecurStackArgs &a, const StackProjMaps &maps, const RecurTcPlan &p, int sm_count, cudaStream_t st)
+{
+    KernelFn fn = pick(groups_of(a.layer[0].B), p.terms, blocks_of(p.upc));
+    if (!fn) return cudaErrorInvalidValue;
+    RecurStackArgs copy = a;
+    StackProjMaps m = maps;
+    void *params[] = {&copy, m.w, m.x, m.xlo};
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = config(attr, sm_count / 2 * 2, recur_stack_smem_bytes(p, a.layer[0].B, a.proj), st);
+    return cudaLaunchKernelExC(&cfg, (const void *)fn, params);
+}
+
+}  // namespace lstm

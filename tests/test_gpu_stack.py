@@ -1,0 +1,99 @@
+"""Two layers of a batch in one launch: edges of the partition (units per pair, the second block of accumulator rows, halves of K),
+of the row groups, of the chunks and of the rule that takes calls there, dense and pruned, against the oracle (needs a B200)."""
+import numpy as np
+import pytest
+
+import lstm_workloads as wl
+from gpu_util import assert_close, csr_weights, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+# (in_dim, H, T, B, density)
+SHAPES = [(5, 65, 4, 5, 1.0), (40, 128, 5, 8, 1.0), (33, 129, 9, 9, 1.0), (64, 301, 47, 3, 1.0), (70, 517, 7, 24, 1.0), (24, 600, 11, 32, 1.0), (20, 600, 6, 33, 1.0),
+          (30, 1056, 5, 2, 1.0), (30, 1057, 16, 2, 1.0), (16, 1280, 17, 9, 1.0), (24, 1281, 16, 17, 1.0), (40, 1500, 18, 20, 1.0), (16, 1500, 16, 25, 1.0), (16, 1536, 16, 3, 1.0),
+          (64, 300, 4, 7, 0.3), (48, 700, 9, 16, 0.1), (32, 1300, 16, 9, 0.1)]
+
+
+def make(s, seed=0):
+    in_dim, H, T, B, density = s
+    w = wl.Workload("stack", 2, False, in_dim, H, T, B, "bf16", min(0.3, 1.5 / (H * density) ** 0.5), density=density, seed=H + B + seed)
+    return (w, *wl.make(w), *wl.make_states(w))
+
+
+@pytest.mark.parametrize("s", SHAPES, ids=lambda s: "in{}_H{}_T{}_B{}_p{}".format(*s))
+def test_small_shapes_of_stacks(oracle, s):
+    w, weights, x, h0, c0 = make(s)
+    ref = oracle.forward(weights, x, h0, c0, layers=2, bidir=False, hidden=w.hidden)
+    mode, ws = ("dense", weights) if w.density == 1 else ("csr", csr_weights(oracle, weights))
+    assert_close(run_gpu(w, ws, x, h0, c0, exec_mode=mode), ref, "bf16", "stack")
+    if w.T == 9:
+        assert_close(run_gpu(w, ws, x, h0, c0, exec_mode=mode, chunks=[4, 5]), ref, "bf16", "stack, chunked")
+
+
+# H, T, B -> launches: beside each other three, one after the other five
+@pytest.mark.parametrize("H,T,B,launches", [(300, 4, 9, 3), (300, 3, 9, 5), (300, 4, 32, 3), (300, 4, 33, 5), (1200, 16, 9, 3), (1200, 15, 9, 5), (1500, 16, 24, 3), (1500, 16, 25, 5)])
+def test_calls_that_run_two_layers_at_once(H, T, B, launches):
+    import torch
+    import paper_1901_10997_b200 as pkg
+    g = torch.Generator(device="cuda").manual_seed(H)
+    ws = [{"wx": torch.randn(4 * H, n, generator=g, device="cuda"), "wh": torch.randn(4 * H, H, generator=g, device="cuda")} for n in (16, H)]
+    m = pkg.LSTM(ws, layers=2, in_dim=16, hidden=H, dtype="bf16", max_T=16, max_B=B)
+    try:
+        m.forward(torch.randn(T, B, 16, generator=g, device="cuda"))
+        m.check()
+        assert m.info()["launches_per_forward"] == launches
+    finally:
+        m.close()
+
+
+def test_small_shapes_of_stacks_nan_in_one_unit(oracle):
+    w, weights, x, h0, c0 = make((24, 300, 6, 13, 1.0), 3)
+    c0[0, 11, 66] = np.nan
+    ref = oracle.forward(weights, x, h0, c0, layers=2, bidir=False, hidden=300)
+    for name, got, want in zip(("y", "hT", "cT"), run_gpu(w, weights, x, h0, c0), ref):
+        assert np.array_equal(np.isnan(got), np.isnan(want)), name
+        ok = ~np.isnan(want)
+        assert np.abs(got - want)[ok].max() <= wl.TOLERANCE["bf16"], name
+
+
+@pytest.mark.parametrize("density", [1.0, 0.2])
+def test_stacks_recorded_timed_out_and_of_different_lengths(oracle, density):
+    """Calls of different lengths and rows on one handle, a recorded one replayed between them, and ones whose words are withheld:
+    every call meets cleared words and counts, whatever the calls before it wrote."""
+    import torch
+    import paper_1901_10997_b200 as pkg
+    w, weights, x, _, _ = make((40, 300, 19, 15, density), 5)
+    ws, mode = (weights, "dense") if density == 1 else (csr_weights(oracle, weights), "csr")
+    m = pkg.LSTM(ws, layers=2, in_dim=40, hidden=300, dtype="bf16", exec_mode=mode, max_T=19, max_B=15)
+    try:
+        xd = torch.from_numpy(x).cuda()
+        xs = [xd[:T, :B].contiguous() for T, B in ((19, 15), (4, 9), (2, 15), (19, 15), (7, 5), (19, 8))]
+        refs = [oracle.forward(weights, v.cpu().numpy(), layers=2, bidir=False, hidden=300) for v in xs]
+
+        def ordinary():
+            for v, ref in zip(xs, refs):
+                got = m.forward(v)
+                m.check()
+                assert_close([t.cpu().numpy() for t in got], ref, "bf16", "stack, mixed calls")
+
+        ordinary()
+        out = tuple(torch.empty_like(t) for t in m.forward(xs[4]))
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            m.forward(xs[4], out=out)
+        for _ in range(3):
+            for t in out:
+                t.zero_()
+            graph.replay()
+            m.check()
+            assert_close([t.cpu().numpy() for t in out], refs[4], "bf16", "stack, replayed")
+            ordinary()
+        for cta in (5, 60, 0):                      # of the lower and of the upper layer
+            m.selftest_timeout(cta, 2_000_000)
+            m.forward(xd)
+            assert m.status() == pkg.LSTM_ERR_TIMEOUT
+            m.selftest_timeout(-1)
+            ordinary()
+        del graph
+    finally:
+        m.close()
