@@ -22,6 +22,8 @@
 #include "common.cuh"
 #include "device_util.cuh"
 
+#include <algorithm>
+
 namespace lstm {
 namespace {
 
@@ -43,6 +45,10 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
     constexpr int RGS = MODE == 2 ? 2 : 1;
     constexpr int NF1 = (N1 * RGS + 3) / 4;            // r items per thread and sub-pass
     constexpr int KB = MODE == 2 || N1 * KT > 12 ? 6 : 12;             // pass 2: column tiles in flight
+    // pass 2: the weights of a batch of tiles out of shared memory ahead of its words, where row groups take turns beside large
+    // fragments (us per call, T = 35: 1500, Hh = 1500, 12 rows 620 -> 552; 1400, Hh = 1200, 16 rows 582 -> 533; elsewhere the registers
+    // are not there: MODE 0 298 -> 308, and spills with twelve tiles in flight)
+    constexpr bool kAhead = MODE == 1 && N1 * KT > 12;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int abort_s;
 
@@ -270,14 +276,17 @@ __global__ void __launch_bounds__(kThreads, 1) hlstm_tile_kernel(const HlstmTile
                 const uint4 *Aw = A2 + (size_t)warp * KT2 * 32 + lane;
 #pragma unroll 1
                 for (int k0 = 0; k0 < m_tiles; k0 += KB) {
-                    uint4 w[KB][RGS];
+                    uint4 w[KB][RGS], af[kAhead ? KB : 1];
+                    if (kAhead)
+#pragma unroll
+                        for (int i = 0; i < KB; ++i) af[kAhead ? i : 0] = k0 + i < m_tiles ? Aw[(size_t)(k0 + i) * 32] : make_uint4(0, 0, 0, 0);
                     fetch(w, src + (size_t)k0 * 256, rx, 2 * rslot, m_tiles - k0, rg0, r_phase, kRPhase);
 #pragma unroll
                     for (int i = 0; i < KB; ++i)
                         if (k0 + i < m_tiles) {
-                            const uint4 af = Aw[(size_t)(k0 + i) * 32];
+                            if (!kAhead) af[0] = Aw[(size_t)(k0 + i) * 32];
 #pragma unroll
-                            for (int rg = 0; rg < RGS; ++rg) multiply(acc[rg], af, w[i][rg], 0x7fff7fffu);
+                            for (int rg = 0; rg < RGS; ++rg) multiply(acc[rg], af[kAhead ? i : 0], w[i][rg], 0x7fff7fffu);
                         }
                 }
 #pragma unroll
@@ -330,8 +339,11 @@ KernelFn pick_mode(int n1, int kt)
         case 2 * 16 + 4: return hlstm_tile_kernel<2, 4, MODE>;
         case 3 * 16 + 4: return hlstm_tile_kernel<3, 4, MODE>;
         case 4 * 16 + 4: if constexpr (MODE != 2) return hlstm_tile_kernel<4, 4, MODE>; else return nullptr;     // (mode_of: n1 * kt <= 12)
+        case 1 * 16 + 5: return hlstm_tile_kernel<1, 5, MODE>;
         case 1 * 16 + 6: return hlstm_tile_kernel<1, 6, MODE>;
+        case 2 * 16 + 5: return hlstm_tile_kernel<2, 5, MODE>;
         case 2 * 16 + 6: return hlstm_tile_kernel<2, 6, MODE>;
+        case 3 * 16 + 5: if constexpr (MODE != 2) return hlstm_tile_kernel<3, 5, MODE>; else return nullptr;
         case 3 * 16 + 6: if constexpr (MODE != 2) return hlstm_tile_kernel<3, 6, MODE>; else return nullptr;
         default: return nullptr;
     }
@@ -358,7 +370,7 @@ bool hlstm_tile_plan(int H, int Hh, int max_cta, size_t max_smem, HlstmTilePlan 
     const int mt = 4 * ((Hh + 15) / 16), ut = (H + 15) / 16;
     p->H = H; p->Hh = Hh; p->max_smem = max_smem;
     p->n1 = (mt + max_cta - 1) / max_cta;
-    p->kt = (ut + 15) / 16 <= 4 ? 4 : 6;
+    p->kt = std::max(4, (ut + 15) / 16);
     p->ncta = (mt + p->n1 - 1) / p->n1;
     if (ut > p->ncta) p->ncta = ut;
     return ut <= max_cta && (ut + 15) / 16 <= 6 && pick(p->n1, p->kt, 0) && smem_bytes(Hh, p->n1, kHtRows, 1) <= max_smem;
