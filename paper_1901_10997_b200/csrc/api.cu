@@ -813,7 +813,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         if (h->use_mma) { h->seq_dirs = true; h->use_tcb = plan_tcb(h->ncta_dir, 1); }
         else { h->ncta_dir = nc; h->upc = up; h->threads = th; }
     }
-    if (h->use_tcb && D == 1 && layers == 2 && h->use_tc && !getenv("LSTM_B200_WAVE") && !getenv("LSTM_B200_RECUR")) {
+    if (h->use_tcb && h->tcb[0].pair && D == 1 && layers == 2 && h->use_tc && !getenv("LSTM_B200_WAVE") && !getenv("LSTM_B200_RECUR")) {
         const int smem = h->smem_optin - kTcStaticSmem;
         bool fits = false;
         h->use_stack = recur_stack_plan(H, h->sm_count, max_B, tc_terms, (size_t)smem, &h->stack) &&
@@ -946,11 +946,6 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                     rc = upload(h, (uint16_t **)&ly.wtc[i][d], p.data(), p.size() * 2, st, "recurrent weight rows");
                     if (rc == LSTM_OK) cudaStreamSynchronize(st);
                 }
-                if (rc == LSTM_OK && h->use_stack) {
-                    const std::vector<uint16_t> p = pack_tc_rows(m.data(), nullptr, H, h->stack);
-                    rc = upload(h, (uint16_t **)&ly.wst, p.data(), p.size() * 2, st, "recurrent weight rows");
-                    if (rc == LSTM_OK) cudaStreamSynchronize(st);
-                }
             } else {
                 HostCsr cx, ch;
                 snprintf(name, sizeof name, "wx[layer %d, dir %d]", l, d);
@@ -989,11 +984,6 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
                         rc = upload(h, (uint16_t **)&ly.wtc[i][d], p.data(), p.size() * 2, st, "recurrent weight rows");
                         if (rc == LSTM_OK) cudaStreamSynchronize(st);
                     }
-                    if (rc == LSTM_OK && h->use_stack) {
-                        const std::vector<uint16_t> p = pack_tc_rows(nullptr, &ch, H, h->stack);
-                        rc = upload(h, (uint16_t **)&ly.wst, p.data(), p.size() * 2, st, "recurrent weight rows");
-                        if (rc == LSTM_OK) cudaStreamSynchronize(st);
-                    }
                     if (rc) break;
                 }
                 if (h->use_csr_reg) {
@@ -1026,6 +1016,12 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
             }
         }
         if (rc) break;
+        if (h->use_stack) {
+            rc = dev_alloc(h, &ly.wst, (size_t)h->stack.ncta * h->stack.KH * 8 * h->stack.upc * 2, false, st, "recurrent weight rows");
+            if (rc == LSTM_OK && launch_repartition(ly.wtc[0][0], h->tcb[0], ly.wst, h->stack, H, st) != cudaSuccess)
+                rc = fail(h, LSTM_ERR_CUDA, "packing launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+            if (rc) break;
+        }
         rc = upload(h, &ly.bias, bias_p.data(), bias_p.size() * 4, st, "bias");
         if (rc == LSTM_OK && !csr)
             rc = bf16 ? upload(h, (uint16_t **)&ly.wx, wx16.data(), wx16.size() * 2, st, "input weights")
@@ -1094,7 +1090,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         const int upc = dtype == LSTM_F32 && !csr && D == 1 && !(env && strcmp(env, "0") == 0) ? recur_f32_wave_units(layers, H, in_dim, h->sm_count) : 0;
         if (rc == LSTM_OK && upc) {
             rc = alloc_phase_words(h, h->f32w_xch, (size_t)layers * std::min(max_T, kF32WaveMaxT) * H * 32, st);
-            if (rc == LSTM_OK && recur_f32_wave_prepare(in_dim, H, upc) != cudaSuccess)
+            if (rc == LSTM_OK && recur_f32_wave_prepare(in_dim, H, upc, max_B) != cudaSuccess)
                 rc = fail(h, LSTM_ERR_CUDA, "fp32 stack kernel set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
             h->f32w_upc = upc;
         }

@@ -242,7 +242,7 @@ struct RecurF32WaveArgs {
     int *status;
 };
 int recur_f32_wave_units(int L, int H, int in_dim, int max_cta);
-cudaError_t recur_f32_wave_prepare(int in_dim, int H, int upc);
+cudaError_t recur_f32_wave_prepare(int in_dim, int H, int upc, int max_B);
 cudaError_t launch_recur_f32_wave(const RecurF32WaveArgs &a, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------
@@ -377,6 +377,7 @@ struct RecurStackArgs {
 };
 struct StackProjMaps { alignas(64) unsigned char w[128], x[128], xlo[128]; };
 bool recur_stack_plan(int H, int sm_count, int rows_wanted, int terms, size_t max_smem, RecurTcPlan *p);
+cudaError_t launch_repartition(const uint4 *src, const RecurTcPlan &from, uint4 *dst, const RecurTcPlan &to, int H, cudaStream_t st);
 cudaError_t recur_stack_prepare(const RecurTcPlan &p, int sm_count, int max_smem, bool *fits);
 bool recur_stack_proj_plan(const RecurTcPlan &p, int H, int T, int B, int sm_count, size_t max_smem, StackProjArgs *a, int *chunk);
 bool stack_proj_maps(StackProjMaps *m, const __nv_bfloat16 *W, const __nv_bfloat16 *X, const __nv_bfloat16 *Xlo, const StackProjArgs &a, int K, int ldk, int ldx);

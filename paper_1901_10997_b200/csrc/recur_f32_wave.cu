@@ -309,9 +309,9 @@ int recur_f32_wave_units(int L, int H, int in_dim, int max_cta)
     return 0;
 }
 
-cudaError_t recur_f32_wave_prepare(int in_dim, int H, int upc)
+cudaError_t recur_f32_wave_prepare(int in_dim, int H, int upc, int max_B)
 {
-    for (int nt = 1; nt <= 4; ++nt) {
+    for (int nt = 1; nt <= 4 && 8 * (nt - 1) < max_B; ++nt) {
         const cudaError_t e = cudaFuncSetAttribute(pick(nt, (upc + 1) / 2), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(in_dim, H, nt, (upc + 1) / 2));
         if (e != cudaSuccess) return e;
     }

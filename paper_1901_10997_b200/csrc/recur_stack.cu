@@ -36,14 +36,24 @@ recur_stack_kernel(const __grid_constant__ RecurStackArgs a, const __grid_consta
     else stack_proj_role(smem_stack, &tmap_w, &tmap_x, &tmap_xlo, a.proj, b - 2 * n);
 }
 
+// Rows packed for one partition into pairs (recur_tc.cu's) as another one wants them; the K halves are the same.
+__global__ void repartition_kernel(const uint4 *src, int src_upc, uint4 *dst, int dst_upc, int H, int pieces, long long n)
+{
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const int rows = 8 * dst_upc, row = (int)(i % rows), piece = (int)(i / rows % pieces), cta = (int)(i / rows / pieces);
+        const int u = (cta >> 1) * 2 * dst_upc + (row >> 2), pair = u / (2 * src_upc);
+        dst[i] = u < H ? src[((long long)(2 * pair + (cta & 1)) * pieces + piece) * (8 * src_upc) + (u - pair * 2 * src_upc) * 4 + (row & 3)] : make_uint4(0, 0, 0, 0);
+    }
+}
+
 typedef void (*KernelFn)(const RecurStackArgs, const CUtensorMap, const CUtensorMap, const CUtensorMap);
-template <int TERMS, int MB> KernelFn pick_m(int rg)
+template <int TERMS, int MB> KernelFn pick_m(int rg, bool split)
 {
     switch (rg) {
-        case 1: return recur_stack_kernel<1, TERMS, MB>;
-        case 2: return recur_stack_kernel<2, TERMS, MB>;
-        case 3: if constexpr (TERMS == 2) return recur_stack_kernel<3, TERMS, MB>; else return nullptr;
-        case 4: if constexpr (TERMS == 2) return recur_stack_kernel<4, TERMS, MB>; else return nullptr;
+        case 1: return split ? recur_stack_kernel<1, TERMS, MB, true> : recur_stack_kernel<1, TERMS, MB, false>;
+        case 2: return split ? recur_stack_kernel<2, TERMS, MB, true> : recur_stack_kernel<2, TERMS, MB, false>;
+        case 3: if constexpr (TERMS == 2) return recur_stack_kernel<3, TERMS, MB, false>; else return nullptr;
+        case 4: if constexpr (TERMS == 2) return recur_stack_kernel<4, TERMS, MB, false>; else return nullptr;
         default: return nullptr;
     }
 }
@@ -95,6 +105,13 @@ bool recur_stack_plan(int H, int sm_count, int rows_wanted, int terms, size_t ma
         }
     }
     return false;
+}
+
+cudaError_t launch_repartition(const uint4 *src, const RecurTcPlan &from, uint4 *dst, const RecurTcPlan &to, int H, cudaStream_t st)
+{
+    const long long n = (long long)to.ncta * (to.KH / 8) * 8 * to.upc;
+    repartition_kernel<<<(int)std::min<long long>((n + 255) / 256, 4096), 256, 0, st>>>(src, from.upc, dst, to.upc, H, to.KH / 8, n);
+    return cudaGetLastError();
 }
 
 cudaError_t recur_stack_prepare(const RecurTcPlan &p, int sm_count, int max_smem, bool *fits)
