@@ -21,7 +21,7 @@
 namespace lstm {
 namespace {
 
-template <int RG, int TERMS, int MB>
+template <int RG, int TERMS, int MB, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 recur_stack_kernel(const __grid_constant__ RecurStackArgs a, const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                    const __grid_constant__ CUtensorMap tmap_xlo)
@@ -31,8 +31,8 @@ recur_stack_kernel(const __grid_constant__ RecurStackArgs a, const __grid_consta
     for (unsigned i = blockIdx.x * kThreads + threadIdx.x; i < a.clear_words / 4u; i += gridDim.x * kThreads)
         reinterpret_cast<uint4 *>(a.other_set)[i] = make_uint4(0, 0, 0, 0);
     const int n = a.layer[0].ncta_dir, b = blockIdx.x;
-    if (b < n) recur_tc_role<RG, true, TERMS, MB, kTcLower>(a.layer[0], b, TcLink{a.chunk, a.proj.stored_out, nullptr, 0});
-    else if (b < 2 * n) recur_tc_role<RG, true, TERMS, MB, kTcUpper>(a.layer[1], b - n, TcLink{a.chunk, nullptr, a.proj.ready, (unsigned)(gridDim.x - 2 * n)});
+    if (b < n) recur_tc_role<RG, true, TERMS, MB, kTcLower, SPLIT>(a.layer[0], b, TcLink{a.chunk, a.proj.stored_out, nullptr, 0});
+    else if (b < 2 * n) recur_tc_role<RG, true, TERMS, MB, kTcUpper, false>(a.layer[1], b - n, TcLink{a.chunk, nullptr, a.proj.ready, (unsigned)(gridDim.x - 2 * n)});
     else stack_proj_role(smem_stack, &tmap_w, &tmap_x, &tmap_xlo, a.proj, b - 2 * n);
 }
 
@@ -57,9 +57,9 @@ template <int TERMS, int MB> KernelFn pick_m(int rg, bool split)
         default: return nullptr;
     }
 }
-KernelFn pick(int rg, int terms, int mb)
+KernelFn pick(int rg, int terms, int mb, bool split)
 {
-    return terms == 3 ? (mb == 2 ? pick_m<3, 2>(rg) : pick_m<3, 1>(rg)) : (mb == 2 ? pick_m<2, 2>(rg) : pick_m<2, 1>(rg));
+    return terms == 3 ? (mb == 2 ? pick_m<3, 2>(rg, split) : pick_m<3, 1>(rg, split)) : (mb == 2 ? pick_m<2, 2>(rg, split) : pick_m<2, 1>(rg, split));
 }
 int groups_of(int rows) { return (rows + 7) / 8; }
 int blocks_of(int upc) { return 8 * upc > 128 ? 2 : 1; }
@@ -117,8 +117,8 @@ cudaError_t launch_repartition(const uint4 *src, const RecurTcPlan &from, uint4 
 cudaError_t recur_stack_prepare(const RecurTcPlan &p, int sm_count, int max_smem, bool *fits)
 {
     *fits = true;
-    for (int rg = 1; rg <= p.rows / 8; ++rg) {
-        KernelFn fn = pick(rg, p.terms, blocks_of(p.upc));
+    for (int v = 0; v < p.rows / 8 + std::min(2, p.rows / 8); ++v) {
+        KernelFn fn = v < p.rows / 8 ? pick(v + 1, p.terms, blocks_of(p.upc), false) : pick(v + 1 - p.rows / 8, p.terms, blocks_of(p.upc), true);
         const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
         if (e != cudaSuccess) return e;
         cudaLaunchAttribute attr[2];
@@ -131,8 +131,11 @@ cudaError_t recur_stack_prepare(const RecurTcPlan &p, int sm_count, int max_smem
     return cudaSuccess;
 }
 
-// Rows, blocks and chunk of the projecting CTAs of a call: the shortest chunk that keeps up with the recurrences, or the longest there is
-// room for; false when there is none.
+// Rows, blocks and chunk of the projecting CTAs of a call; false when there is no room for one timestep.  Four timesteps a chunk, as far as
+// tensor memory holds its accumulators: fewer cannot keep up with the recurrences at the wider layers, more make the lag longer.  us per
+// call at 2, 3, 4, 5, 6 timesteps: 2 x 1500, T = 35, 2 rows 249, 191, 187, 192, 189; 20 rows 320, 273, 259 (no room for five); 1000
+// with 24 rows 208, 185, 181, 181, 179; 517 with 8 126, 120, 118, 117, 118; 700, T = 20, 6 rows 89, 87, 85, 85, 87; 517, T = 23, 3
+// rows 93, 89, 89, 89, 90; 300 with 16 124, 122, 120, 122, 120; pruned 1500 with 16 300, 253, 251, 259, 257.
 bool recur_stack_proj_plan(const RecurTcPlan &p, int H, int T, int B, int sm_count, size_t max_smem, StackProjArgs *a, int *chunk)
 {
     const int nproj = sm_count / 2 * 2 - 2 * p.ncta;
@@ -141,16 +144,12 @@ bool recur_stack_proj_plan(const RecurTcPlan &p, int H, int T, int B, int sm_cou
     a->mb = (rows + 127) / 128;
     a->rb = ((rows + a->mb - 1) / a->mb + 7) / 8 * 8;
     a->nrp = 0;
-    const int step = blocks_of(p.upc) == 2 ? 7000 : 4500;           // clock ticks of a step of the recurrence, roughly
-    for (int c = 1; c <= T; ++c) {
+    for (int c = 1; c <= std::min(4, T); ++c) {
         const int nrp = (c * B + 7) / 8 * 8;
         if (nrp > 128 || a->mb * 2 * nrp > 512) break;
         a->nrp = nrp;
         a->chunk_rows = c * B;
         *chunk = c;
-        const int bytes = a->mb * a->rb * 128 + 2 * nrp * 128;
-        const int cost = a->kblocks * std::max(bytes / 48, a->mb * 4 * std::max(32, nrp)) + 4000;
-        if (cost * 10 < 9 * c * step) break;
     }
     if (a->nrp == 0) return false;
     a->nchunks = (T + *chunk - 1) / *chunk;
@@ -166,7 +165,7 @@ bool stack_proj_maps(StackProjMaps *m, const __nv_bfloat16 *W, const __nv_bfloat
 
 cudaError_t launch_recur_stack(const RecurStackArgs &a, const StackProjMaps &maps, const RecurTcPlan &p, int sm_count, cudaStream_t st)
 {
-    KernelFn fn = pick(groups_of(a.layer[0].B), p.terms, blocks_of(p.upc));
+    KernelFn fn = pick(groups_of(a.layer[0].B), p.terms, blocks_of(p.upc), a.layer[0].nsplit > 1);
     if (!fn) return cudaErrorInvalidValue;
     RecurStackArgs copy = a;
     StackProjMaps m = maps;

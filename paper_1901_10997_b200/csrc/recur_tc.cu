@@ -52,31 +52,31 @@
 namespace lstm {
 namespace {
 
-template <int RG, bool PAIR, int TERMS>
+template <int RG, bool PAIR, int TERMS, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1) recur_tc_kernel(const RecurTcArgs a)
 {
-    recur_tc_role<RG, PAIR, TERMS, 1, kTcAlone>(a, blockIdx.x, TcLink());
+    recur_tc_role<RG, PAIR, TERMS, 1, kTcAlone, SPLIT>(a, blockIdx.x, TcLink());
 }
 
 typedef void (*KernelFn)(const RecurTcArgs);
 template <bool PAIR, int TERMS>
-KernelFn pick_p(int rg)
+KernelFn pick_p(int rg, bool split)
 {
     switch (rg) {
-        case 1: return recur_tc_kernel<1, PAIR, TERMS>;
-        case 2: return recur_tc_kernel<2, PAIR, TERMS>;
-        case 3: return recur_tc_kernel<3, PAIR, TERMS>;
-        case 4: return recur_tc_kernel<4, PAIR, TERMS>;
-        case 5: return recur_tc_kernel<5, PAIR, TERMS>;
-        case 6: return recur_tc_kernel<6, PAIR, TERMS>;
-        case 7: return recur_tc_kernel<7, PAIR, TERMS>;
-        case 8: return recur_tc_kernel<8, PAIR, TERMS>;
+        case 1: return split ? recur_tc_kernel<1, PAIR, TERMS, true> : recur_tc_kernel<1, PAIR, TERMS, false>;
+        case 2: return split ? recur_tc_kernel<2, PAIR, TERMS, true> : recur_tc_kernel<2, PAIR, TERMS, false>;
+        case 3: return recur_tc_kernel<3, PAIR, TERMS, false>;
+        case 4: return recur_tc_kernel<4, PAIR, TERMS, false>;
+        case 5: return recur_tc_kernel<5, PAIR, TERMS, false>;
+        case 6: return recur_tc_kernel<6, PAIR, TERMS, false>;
+        case 7: return recur_tc_kernel<7, PAIR, TERMS, false>;
+        case 8: return recur_tc_kernel<8, PAIR, TERMS, false>;
         default: return nullptr;
     }
 }
-KernelFn pick(int rg, bool pair, int terms)
+KernelFn pick(int rg, bool pair, int terms, bool split)
 {
-    return terms == 3 ? (pair ? pick_p<true, 3>(rg) : pick_p<false, 3>(rg)) : (pair ? pick_p<true, 2>(rg) : pick_p<false, 2>(rg));
+    return terms == 3 ? (pair ? pick_p<true, 3>(rg, split) : pick_p<false, 3>(rg, split)) : (pair ? pick_p<true, 2>(rg, split) : pick_p<false, 2>(rg, split));
 }
 int groups_of(int rows) { return (rows + 7) / 8; }
 
@@ -128,8 +128,8 @@ bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, int terms, siz
 cudaError_t recur_tc_prepare(int terms, int max_smem)
 {
     for (int rg = 1; rg <= kTcMaxRows / 8; ++rg) {
-        for (int pair = 0; pair < 2; ++pair) {
-            const cudaError_t e = cudaFuncSetAttribute(pick(rg, pair != 0, terms), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+        for (int v = 0; v < (rg <= 2 ? 4 : 2); ++v) {
+            const cudaError_t e = cudaFuncSetAttribute(pick(rg, (v & 1) != 0, terms, v >= 2), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
             if (e != cudaSuccess) return e;
         }
     }
@@ -143,7 +143,7 @@ bool recur_tc_pair_supported(int grid, const RecurTcPlan &p)
     cudaLaunchConfig_t cfg = config(attr, grid, recur_tc_smem_bytes(p.KH, p.upc, p.rows, 1, p.terms), 1, nullptr);
     cfg.attrs = attr + 1; cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)pick(groups_of(p.rows), true, p.terms), &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)pick(groups_of(p.rows), true, p.terms, false), &cfg) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -152,7 +152,7 @@ bool recur_tc_pair_supported(int grid, const RecurTcPlan &p)
 
 cudaError_t launch_recur_tc(const RecurTcArgs &a, cudaStream_t st)
 {
-    KernelFn fn = pick(groups_of(a.B), a.pair != 0, a.terms);
+    KernelFn fn = pick(groups_of(a.B), a.pair != 0, a.terms, a.nsplit > 1);
     if (!fn) return cudaErrorInvalidValue;
     RecurTcArgs copy = a;
     void *params[] = {&copy};

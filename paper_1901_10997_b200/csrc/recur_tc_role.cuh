@@ -128,7 +128,8 @@ __device__ __forceinline__ void add_count(unsigned *count)
 // RG: groups of eight batch rows of a pass; TERMS: bf16 terms of h, two from words {hi | lo}, three from words that are h itself
 // MB: blocks of accumulator rows: 128 with their weights in tensor memory, and up to 64 with theirs in shared memory; LINK: place in a stack.
 // block: this CTA's place in the group of CTAs that run the layer.
-template <int RG, bool PAIR, int TERMS, int MB, int LINK>
+// SPLIT: the projection may come in several planes along K, and few rows: see g below.
+template <int RG, bool PAIR, int TERMS, int MB, int LINK, bool SPLIT>
 __device__ __forceinline__ void recur_tc_role(const RecurTcArgs &a, int block, const TcLink &link)
 {
     static_assert(MB == 1 || (PAIR && tc_columns(RG, TERMS) <= 64), "two blocks: an accumulator and an issuing warp each");
@@ -314,7 +315,17 @@ __device__ __forceinline__ void recur_tc_role(const RecurTcArgs &a, int block, c
     // Projection terms of this thread's row, requested between the last poll and the wait for the products, which hides the
     // trip to L2; the lines are requested from HBM two steps ahead.  Requested ahead of the polls, or a whole step ahead,
     // they delayed them: 2.63 -> 3.08 us per step (two directions of 800, 16 rows).
-    float g[MB][RS];
+    // SPLIT: the further planes of a projection split along K are added behind the products, which take less time than the loads (2 x 517,
+    // 3 rows: 1020 of 4600 clocks a step stood here).  A build of its own: with one plane the registers cost more (pruned 2 x
+    // 1500, 16 rows 243 -> 257 us), and with more rows the products hide the sum.
+    constexpr bool LATE = SPLIT && RS == 4 && LINK != kTcUpper;
+    float g[MB][RS], gx[MB][LATE ? 3 : 1][RS];
+#pragma unroll
+    for (int k = 0; k < MB; ++k)
+#pragma unroll
+        for (int p = 0; p < (LATE ? 3 : 1); ++p)
+#pragma unroll
+            for (int i = 0; i < RS; ++i) gx[k][p][i] = 0.0f;
     int chunk_end = 0;                          // kTcUpper: first step whose rows of G have not been waited for
     auto load_g = [&](int s) {
         if constexpr (LINK == kTcUpper) {
@@ -347,7 +358,10 @@ __device__ __forceinline__ void recur_tc_role(const RecurTcArgs &a, int block, c
                         w[i] = i0 + i < n3 ? ld_nc_early(p3 + (i0 + i) * gstep + 4 * k * dj) : 0.0f;
                     }
 #pragma unroll
-                    for (int i = 0; i < C; ++i) g[k][i0 + i] += (v[i] + u[i]) + w[i];
+                    for (int i = 0; i < C; ++i) {
+                        if constexpr (LATE) { gx[k][0][i0 + i] = v[i]; gx[k][1][i0 + i] = u[i]; gx[k][2][i0 + i] = w[i]; }
+                        else g[k][i0 + i] += (v[i] + u[i]) + w[i];
+                    }
                 }
             }
         }
@@ -583,7 +597,10 @@ __device__ __forceinline__ void recur_tc_role(const RecurTcArgs &a, int block, c
 #pragma unroll
                 for (int k = 0; k < MB; ++k) {
 #pragma unroll
-                    for (int i = 0; i < RS; ++i) z[k][i] = gate_fast(z[k][i] + g[k][i], act_k, act_sc, act_of);
+                    for (int i = 0; i < RS; ++i) {
+                        if constexpr (LATE) g[k][i] += (gx[k][0][i] + gx[k][1][i]) + gx[k][2][i];
+                        z[k][i] = gate_fast(z[k][i] + g[k][i], act_k, act_sc, act_of);
+                    }
                     unsigned *dst = (MB == 2 && k ? out1 : out0) + (size_t)(s & 1) * slot_words;
 #pragma unroll
                     for (int m = 0; m < RS / 4; ++m) {
