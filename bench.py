@@ -344,10 +344,14 @@ def trimmed_mean(ms, drop=0.1):
     return float(sum(keep) / len(keep))
 
 
-def kernel_of(pkg, info):
-    """The recurrent kernel of the last call and its source file."""
-    name = pkg.RECUR_KERNELS[info["kernel"]]
-    return name, name.removesuffix("_kernel") + ".cu"
+def kernel_of(pkg, info, layers=1):
+    """The recurrent kernel of the last call, its source file, and the layers that one launch of it ran."""
+    name, launches, at_once = pkg.RECUR_KERNELS[info["kernel"]], info["launches_per_forward"], 1
+    if layers == 2 and info["kernel"] == pkg.LSTM_RAN_BATCHED and launches == 3:          # staging, one projection, both layers
+        name, at_once = "recur_stack_kernel", 2
+    elif layers > 1 and info["kernel"] == pkg.LSTM_RAN_F32 and launches == 1:
+        name, at_once = "recur_f32_wave_kernel", layers
+    return name, name.removesuffix("_kernel") + ".cu", at_once
 
 
 class GpuCase:
@@ -433,10 +437,12 @@ class GpuCase:
         rec_avg_ms = rec_ms / max(rec_n, 1)
         achieved = alg_bytes / (rec_avg_ms * 1e-3) / 1e9 if rec_avg_ms > 0 else None
         info = self.model.info()
-        kernel_name, kernel_src = kernel_of(self.pkg, info)
+        kernel_name, kernel_src, at_once = kernel_of(self.pkg, info, w.layers)
+        alg_bytes *= at_once
+        achieved = alg_bytes / (rec_avg_ms * 1e-3) / 1e9 if rec_avg_ms > 0 else None
         traffic, source = measured_traffic(kernel_name, self.name, kernel_src)
         steps_per_launch = w.T * (2 if (w.dirs == 2 and info.get("ctas_per_dir") == info.get("sm_count")) else 1)
-        return {"bound": "hbm", "kernel": f"{kernel_name} (one launch = one layer, all T steps" + (", its input projection in the prologue)" if fused else ")"),
+        return {"bound": "hbm", "kernel": f"{kernel_name} (one launch = {'one layer' if at_once == 1 else f'{at_once} layers'}, all T steps" + (", its input projection in the prologue)" if fused else ")"),
                 "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": (achieved / peak if achieved else None), "peak_kind": f"of {peak_kind}",
                 "traffic": traffic, "traffic_source": source, "algorithmic_bytes_per_launch": alg_bytes,
