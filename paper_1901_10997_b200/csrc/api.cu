@@ -1090,7 +1090,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         const int upc = dtype == LSTM_F32 && !csr && D == 1 && !(env && strcmp(env, "0") == 0) ? recur_f32_wave_units(layers, H, in_dim, h->sm_count) : 0;
         if (rc == LSTM_OK && upc) {
             rc = alloc_phase_words(h, h->f32w_xch, (size_t)layers * std::min(max_T, kF32WaveMaxT) * H * 32, st);
-            if (rc == LSTM_OK && recur_f32_wave_prepare(in_dim, H, upc, max_B) != cudaSuccess)
+            if (rc == LSTM_OK && recur_f32_wave_prepare(upc, max_B, h->smem_optin) != cudaSuccess)
                 rc = fail(h, LSTM_ERR_CUDA, "fp32 stack kernel set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
             h->f32w_upc = upc;
         }

@@ -26,6 +26,7 @@ namespace lstm {
 namespace {
 
 constexpr int kThreads = kF32Threads, kWarps = kThreads / 32;
+constexpr int kStaticSmem = 256;               // static shared memory of the kernel, at most
 
 __host__ __device__ constexpr int f32_wave_red_doubles(int nt, int mt) { return kWarps * 8 * mt * (8 * nt + 4); }
 
@@ -309,10 +310,11 @@ int recur_f32_wave_units(int L, int H, int in_dim, int max_cta)
     return 0;
 }
 
-cudaError_t recur_f32_wave_prepare(int in_dim, int H, int upc, int max_B)
+// The limit is a property of the kernel, not of a handle: the most the device has, or a handle made later for less would lower it.
+cudaError_t recur_f32_wave_prepare(int upc, int max_B, int smem_optin)
 {
     for (int nt = 1; nt <= 4 && 8 * (nt - 1) < max_B; ++nt) {
-        const cudaError_t e = cudaFuncSetAttribute(pick(nt, (upc + 1) / 2), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(in_dim, H, nt, (upc + 1) / 2));
+        const cudaError_t e = cudaFuncSetAttribute(pick(nt, (upc + 1) / 2), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - kStaticSmem);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

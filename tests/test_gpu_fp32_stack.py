@@ -80,3 +80,22 @@ def test_fp32_narrow_stack_recorded_timed_out_and_shorter_calls(oracle):
         del graph
     finally:
         m.close()
+
+
+def test_fp32_narrow_stack_beside_a_smaller_one(oracle):
+    """A handle that needs less shared memory, made later, takes nothing from the one made before it."""
+    import torch
+    import paper_1901_10997_b200 as pkg
+    models = []
+    try:
+        for s in ((2, 256, 256, 3, 32), (2, 160, 160, 3, 32)):
+            w, weights, x, _, _ = make(s)
+            models.append((pkg.LSTM(weights, layers=2, in_dim=s[1], hidden=s[2], dtype="fp32", max_T=3, max_B=32), torch.from_numpy(x).cuda(),
+                           oracle.forward(weights, x, layers=2, bidir=False, hidden=s[2])))
+        for m, x, ref in models + models[:1]:
+            got = m.forward(x)
+            m.check()
+            assert_close([t.cpu().numpy() for t in got], ref, "fp32", "fp32 stack, two handles")
+    finally:
+        for m, _, _ in models:
+            m.close()
