@@ -124,6 +124,18 @@ __device__ __forceinline__ void cp_async_wait_all()
 
 // named barriers over n threads of the CTA
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+// ... and was the condition true for all of them?
+__device__ __forceinline__ bool bar_all(int id, int n, bool ok)
+{
+    int all;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.s32 p, %3, 0;\n\t"
+        "barrier.cta.red.and.pred q, %1, %2, p;\n\t"
+        "selp.s32 %0, 1, 0, q;\n\t}"
+        : "=r"(all) : "r"(id), "r"(n), "r"((int)ok) : "memory");
+    return all != 0;
+}
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 // D += A (8x4, row) * B (4x8, col) in double precision

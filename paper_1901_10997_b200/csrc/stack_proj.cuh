@@ -113,12 +113,11 @@ __device__ __forceinline__ void stack_proj_role(unsigned char *smem_raw, const C
         // columns (four warps alone take 7.5 us for 3 x 104 rows by 80, during which the products wait)
         const int lq = warp & 3, part = (warp >> 2) - 1, row = lq * 32 + lane;
         for (int chunk = 0; chunk < a.nchunks; ++chunk) {
-            const bool ok = mbar_wait(smem_u32(&accum_bar), (uint32_t)chunk & 1u, abort_v);
-            if (!__all_sync(0xffffffffu, ok)) break;
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&accum_bar), (uint32_t)chunk & 1u, abort_v));
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int m0 = chunk * a.chunk_rows, nr = min(a.chunk_rows, a.M - m0);
             int turn = part;
-            for (int b = 0; b < a.mb; ++b) {
+            for (int b = 0; b < a.mb && ok; ++b) {
                 const int n = r0 + b * a.rb + row;
                 const bool real = row < a.rb && n < a.N;
                 const float bv = real ? a.bias[n] : 0.0f;
@@ -149,7 +148,9 @@ __device__ __forceinline__ void stack_proj_role(unsigned char *smem_raw, const C
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&drained_bar));
-            bar_sync(kSpBar, 12 * 32);
+            // One answer for all twelve warps: a wait that gives up does so warp by warp, and one of them may see the flag just before
+            // the accumulators are complete and the others just behind; none may leave while others come to this barrier.
+            if (!bar_all(kSpBar, 12 * 32, ok)) break;
             if (tid == 128) add_count(a.ready + chunk);
         }
     }

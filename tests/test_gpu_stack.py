@@ -97,3 +97,25 @@ def test_stacks_recorded_timed_out_and_of_different_lengths(oracle, density):
         del graph
     finally:
         m.close()
+
+
+def test_stack_that_gives_up_while_the_projection_runs(oracle):
+    """The upper layer's wait ends long before the lower layer does: the CTAs that project find the status between two chunks, with
+    products of theirs under way, at another point of the chunk for every limit."""
+    import torch
+    import paper_1901_10997_b200 as pkg
+    w, weights, x, _, _ = make((40, 300, 256, 15, 1.0), 7)
+    ref = oracle.forward(weights, x, layers=2, bidir=False, hidden=300)
+    m = pkg.LSTM(weights, layers=2, in_dim=40, hidden=300, dtype="bf16", max_T=256, max_B=15)
+    try:
+        xd = torch.from_numpy(x).cuda()
+        for limit in range(200_000, 300_000, 5_000):         # about 0.1 ms; the call takes 0.6
+            m.selftest_timeout(60, limit)
+            m.forward(xd)
+            assert m.status() == pkg.LSTM_ERR_TIMEOUT
+        m.selftest_timeout(-1)
+        got = m.forward(xd)
+        m.check()
+        assert_close([t.cpu().numpy() for t in got], ref, "bf16", "stack, after the waits that gave up")
+    finally:
+        m.close()
