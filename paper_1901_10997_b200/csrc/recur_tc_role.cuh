@@ -319,6 +319,7 @@ __device__ __forceinline__ void recur_tc_role(const RecurTcArgs &a, int block, c
     // 3 rows: 1020 of 4600 clocks a step stood here).  A build of its own: with one plane the registers cost more (pruned 2 x
     // 1500, 16 rows 243 -> 257 us), and with more rows the products hide the sum.
     constexpr bool LATE = SPLIT && RS == 4 && LINK != kTcUpper;
+    constexpr bool PLANES = (SPLIT || RG > 2) && LINK != kTcUpper;          // up to two row groups there is a build for one plane and one for several
     float g[MB][RS], gx[MB][LATE ? 3 : 1][RS];
 #pragma unroll
     for (int k = 0; k < MB; ++k)
@@ -341,7 +342,7 @@ __device__ __forceinline__ void recur_tc_role(const RecurTcArgs &a, int block, c
             for (int i = 0; i < RS; ++i)
                 g[k][i] = i < nrow[k] ? (LINK == kTcUpper ? __uint_as_float(ld_relaxed_u32(reinterpret_cast<const unsigned *>(gp + i * gstep + 4 * k * dj)))
                                                           : ld_nc_early(gp + i * gstep + 4 * k * dj)) : 0.0f;
-        if (LINK != kTcUpper && a.nsplit > 1) {
+        if constexpr (PLANES) if (a.nsplit > 1) {
             // further planes of a projection split along K: all of them on their way together
             const float *p1 = gp + a.g_split_stride, *p2 = a.nsplit > 2 ? p1 + a.g_split_stride : p1, *p3 = a.nsplit > 3 ? p2 + a.g_split_stride : p1;
             constexpr int C = RS < 8 ? RS : 8;
