@@ -264,6 +264,7 @@ __device__ __forceinline__ void recur_tc_role(const RecurTcArgs &a, int block, c
     const float *gp = a.G + m0 * gstep + (long long)d * 4 * H + 4 * (long long)j + fq;
     const float *gpre = a.G + (m0 + 2 * dir * a.Bs + lane) * gstep + (long long)d * 4 * H + 4 * (long long)(j - (lane >> 2));
     const bool pre = LINK != kTcUpper && lane < RS && fb0 + lane < B && fin && j - (lane >> 2) < H;
+    const bool pre2 = MB == 2 && j - (lane >> 2) + dj < H;                  // (the second block's units of the last pair may not exist)
     float *yp = a.y ? a.y + (m0 + fq) * D * H + (long long)d * H + j : nullptr;
     __nv_bfloat16 *xp = a.xb_next ? a.xb_next + (m0 + fq) * a.xb_ld + (long long)d * H + j : nullptr;
     const long long gadv = dir * a.Bs * gstep, yadv = dir * a.Bs * D * H, xadv = dir * a.Bs * a.xb_ld;
@@ -367,8 +368,9 @@ __device__ __forceinline__ void recur_tc_role(const RecurTcArgs &a, int block, c
             }
         }
         if (pre && s + 2 < T) {
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(gpre));
-            if (MB == 2) asm volatile("prefetch.global.L2 [%0];" ::"l"(gpre + 4 * dj));
+            if (LSTM_CHECK_INDEX(gpre - a.G, (long long)T * a.Bs * gstep, a.status)) asm volatile("prefetch.global.L2 [%0];" ::"l"(gpre));
+            if (pre2 && LSTM_CHECK_INDEX(gpre + 4 * dj - a.G, (long long)T * a.Bs * gstep, a.status))
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(gpre + 4 * dj));
         }
         gp += gadv;
         gpre += gadv;
