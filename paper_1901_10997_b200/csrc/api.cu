@@ -1692,13 +1692,14 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         if (phase_sets(h->stack_xch, rec, st, &base, &set, &s.clear_words) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
         unsigned *counts = base + (size_t)set * h->stack_xch.set_words;
         s.other_set = base + (size_t)(set ^ 1) * h->stack_xch.set_words;
+        const int withhold = h->withhold_cta < 0 ? -1 : h->withhold_cta % (h->sm_count / 2 * 2);
         for (int l = 0; l < 2; ++l) {
             RecurTcArgs &m = s.layer[l];
             m.ndirs = 1; m.H = H; m.B = m.Bs = B; m.T = T; m.D = 1;
             m.ncta_dir = plan.ncta; m.upc = plan.upc; m.KH = plan.KH; m.pair = 1; m.terms = plan.terms;
             m.nsplit = l ? 1 : nsplit;
             m.spin_limit = h->spin_limit;
-            m.withhold_cta = h->withhold_cta < 0 ? -1 : h->withhold_cta % (2 * plan.ncta);
+            m.withhold_cta = withhold;
             m.wpack[0] = h->layers[l].wst;
             m.G = l ? h->stack_G : h->G;
             m.g_split_stride = (long long)M * 4 * H;
@@ -1713,6 +1714,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
             m.status = h->status_dev;
         }
         s.proj = h->stack_proj;
+        s.proj.withhold_cta = withhold - 2 * plan.ncta;
         s.proj.bias = up.bias; s.proj.G = h->stack_G;
         s.proj.stored = s.proj.stored_out = counts; s.proj.n_stored = (unsigned)plan.ncta;
         s.proj.ready = counts + kStackMaxChunks;

@@ -365,6 +365,7 @@ struct StackProjArgs {
     unsigned *stored_out;       //   (the same, for the lower layer)
     unsigned n_stored;
     unsigned *ready;            // [chunk] projecting CTAs that have stored their rows of G
+    int withhold_cta;           // self-test: this CTA (of the projecting ones) is never counted
     long long spin_limit;
     int *status;
 };

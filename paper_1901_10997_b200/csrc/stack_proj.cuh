@@ -151,7 +151,7 @@ __device__ __forceinline__ void stack_proj_role(unsigned char *smem_raw, const C
             // One answer for all twelve warps: a wait that gives up does so warp by warp, and one of them may see the flag just before
             // the accumulators are complete and the others just behind; none may leave while others come to this barrier.
             if (!bar_all(kSpBar, 12 * 32, ok)) break;
-            if (tid == 128) add_count(a.ready + chunk);
+            if (tid == 128 && cta != a.withhold_cta) add_count(a.ready + chunk);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

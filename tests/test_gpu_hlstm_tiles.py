@@ -8,7 +8,7 @@ from test_gpu_hlstm import run
 pytestmark = pytest.mark.gpu
 
 # (layers, bidir, in_dim, H, Hh, T, B, scale): four, eight, nine, sixteen rows and more than one launch; several hidden tiles
-# per CTA with six column tiles per warp (row groups in turn), exact and ragged tiles, a step count of one
+# per CTA with five and six column tiles per warp (row groups in turn), exact and ragged tiles, a step count of one
 SHAPES = [
     (1, False, 20, 64, 48, 3, 4, 0.3),
     (2, True, 24, 130, 100, 4, 9, 0.2),
@@ -31,3 +31,18 @@ def test_tile_kernel_and_row_kernel_match_the_oracle(oracle, shape, kernel, monk
     h0, c0 = wl.make_states(w)
     ref = oracle.forward_hlstm(weights, x, h0, c0, layers=L, bidir=bidir, hidden=H, gate_hidden=Hh)
     assert_close(run(w, Hh, weights, x, h0, c0), ref, "bf16", f"hlstm tiles/{kernel or 'default'}")
+
+
+# (layers, bidir, in_dim, H, Hh, T, scale): five column tiles per warp, one to three hidden tiles per CTA, ragged tiles on both sides
+FIVE = [(1, False, 24, 1200, 320, 5, 0.03), (1, False, 16, 1025, 600, 5, 0.03), (1, False, 16, 1271, 1300, 5, 0.03), (2, True, 16, 1100, 610, 5, 0.03)]
+
+
+@pytest.mark.parametrize("B", [3, 8, 16])
+@pytest.mark.parametrize("shape", FIVE, ids=lambda s: f"L{s[0]}D{1 + s[1]}_H{s[3]}_Hh{s[4]}")
+def test_tile_kernel_with_five_column_tiles(oracle, shape, B):
+    L, bidir, in_dim, H, Hh, T, scale = shape
+    w = wl.Workload("hlstm_tiles", L, bidir, in_dim, H, T, B, "bf16", scale, seed=H + Hh + B)
+    weights, x = wl.make_hlstm(w, Hh)
+    h0, c0 = wl.make_states(w)
+    ref = oracle.forward_hlstm(weights, x, h0, c0, layers=L, bidir=bidir, hidden=H, gate_hidden=Hh)
+    assert_close(run(w, Hh, weights, x, h0, c0), ref, "bf16", "hlstm, five column tiles")

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import lstm_workloads as wl
-from gpu_util import assert_close, csr_weights, run_gpu
+from gpu_util import GUARD, assert_close, csr_weights, run_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -117,5 +117,65 @@ def test_stack_that_gives_up_while_the_projection_runs(oracle):
         got = m.forward(xd)
         m.check()
         assert_close([t.cpu().numpy() for t in got], ref, "bf16", "stack, after the waits that gave up")
+    finally:
+        m.close()
+
+
+# (in_dim, H, B, density): the lower layer's projection in several planes for calls of up to 128 rows, in one beyond them
+@pytest.mark.parametrize("in_dim,H,B,density", [(517, 300, 8, 1.0), (301, 517, 3, 1.0), (1500, 1300, 8, 1.0), (700, 600, 20, 1.0), (600, 400, 16, 0.2)])
+def test_stack_behind_a_projection_in_several_planes(oracle, in_dim, H, B, density):
+    import torch
+    import paper_1901_10997_b200 as pkg
+    T = 128 // B
+    w, weights, x, _, _ = make((in_dim, H, T + 1, B, density), 9)
+    ws, mode = (weights, "dense") if density == 1 else (csr_weights(oracle, weights), "csr")
+    ref = oracle.forward(weights, x, layers=2, bidir=False, hidden=H)
+    m = pkg.LSTM(ws, layers=2, in_dim=in_dim, hidden=H, dtype="bf16", exec_mode=mode, max_T=T + 1, max_B=B)
+    try:
+        xd, got = torch.from_numpy(x).cuda(), {}
+        for t in (T, T + 1):
+            y, hT, cT = m.forward(xd[:t].contiguous())
+            m.check()
+            info = m.info()
+            assert info["launches_per_forward"] == 3
+            got[info["proj_splits"] > 1] = y.cpu().numpy()
+            if t > T:
+                assert_close([v.cpu().numpy() for v in (y, hT, cT)], ref, "bf16", "stack behind one plane")
+        assert set(got) == {True, False}
+        # the same products in another order: each side within the guard of the oracle, so within twice that of the other
+        assert np.abs(got[True] - got[False][:T]).max() <= 2 * GUARD["bf16"] * np.abs(ref[0]).max()
+        assert_close([got[True]], [ref[0][:T]], "bf16", "stack behind several planes")
+    finally:
+        m.close()
+
+
+def test_small_shapes_of_stacks_nan_in_one_unit_of_the_second_block(oracle):
+    """Two blocks of accumulator rows (1300 units): a NaN in one unit of either block reaches what it has to and nothing else."""
+    for unit in (3, 36, 1299):                  # of the first pair's first and second block, and of the last pair
+        w, weights, x, h0, c0 = make((24, 1300, 16, 5, 1.0), 3)
+        c0[0, 2, unit] = np.nan
+        ref = oracle.forward(weights, x, h0, c0, layers=2, bidir=False, hidden=1300)
+        for name, got, want in zip(("y", "hT", "cT"), run_gpu(w, weights, x, h0, c0), ref):
+            assert np.array_equal(np.isnan(got), np.isnan(want)), (name, unit)
+            ok = ~np.isnan(want)
+            assert np.abs(got - want)[ok].max() <= wl.TOLERANCE["bf16"], (name, unit)
+
+
+def test_stack_with_two_blocks_whose_words_or_projection_are_withheld(oracle):
+    import torch
+    import paper_1901_10997_b200 as pkg
+    w, weights, x, _, _ = make((24, 1300, 16, 5, 1.0), 4)
+    ref = oracle.forward(weights, x, layers=2, bidir=False, hidden=1300)
+    m = pkg.LSTM(weights, layers=2, in_dim=24, hidden=1300, dtype="bf16", max_T=16, max_B=5)
+    try:
+        xd = torch.from_numpy(x).cuda()
+        for cta in (1, 66, 132, 147):           # of the lower layer, of the upper one (33 pairs each), two that project
+            m.selftest_timeout(cta, 2_000_000)
+            m.forward(xd)
+            assert m.status() == pkg.LSTM_ERR_TIMEOUT
+            m.selftest_timeout(-1)
+            got = m.forward(xd)
+            m.check()
+            assert_close([t.cpu().numpy() for t in got], ref, "bf16", "stack, after a withheld CTA")
     finally:
         m.close()
