@@ -117,7 +117,8 @@ typedef struct {
  *   LSTM_B200_PROJ_TILE = 128  the 128-row-tile projection kernel (two CTAs per SM) also where the persistent
  *                           256-row-tile kernel would run (several activation tiles)
  *   LSTM_B200_PROJ_SMEM_KB = 48..200  shared-memory budget of the 128-row-tile projection kernel (ring depth)
- *   LSTM_B200_CTAS  = <n>   at most n CTAs per direction in the recurrent kernels (measurement)
+ *   LSTM_B200_CTAS  = <n>   at most n CTAs per direction in the recurrent kernels, for all layers together where batched or fp32
+ *                           layers run in one launch; the layer-wavefront kernel takes all SMs (measurement)
  *   LSTM_B200_COMPACT = 0   keep row/column-pruned units as explicit zeros, = 1 always run on the surviving units
  *                           (unset: handles with max_B >= 5 compact, smaller ones keep the zeros; see below)
  * Row/column-pruned stacks (Section 4.2, Algorithm 1: whole rows and columns of the gate matrices are zero).

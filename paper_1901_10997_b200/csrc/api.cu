@@ -67,6 +67,7 @@ struct PhaseWords {
 struct lstm_handle {
     int L = 0, D = 1, in_dim = 0, H = 0, dtype = 0, exec_mode = 0, max_T = 0, max_B = 0;
     int device = 0, sm_count = 0, smem_optin = 0;
+    int cta_limit = 0;                 // most CTAs of a launch that runs the layers of a stack side by side
     int Hp8 = 0, Hs = 0;
     int ncta_dir = 0, upc = 0, threads = 0;
     bool use_tc = false;
@@ -97,7 +98,7 @@ struct lstm_handle {
     bool use_stack = false;
     RecurTcPlan stack = {0, 0, 0, 0, 0, 0};
     PhaseWords stack_xch;
-    float *stack_G = nullptr; int stack_M = 0;
+    float *stack_G = nullptr; int stack_M = 0, stack_ctas = 0;
     StackProjArgs stack_proj; StackProjMaps stack_maps; int stack_chunk = 0, stack_T = 0, stack_B = 0;
     PhaseWords f32_xch;                // fp32 dense, at most two units per CTA
     int f32w_upc = 0;                  // fp32 stacks, all layers in one launch: units per CTA (0: not served) and exchange words
@@ -583,7 +584,7 @@ bool stack_serves(const lstm_handle *h, int T, int B)
 {
     if (!h->use_stack || h->probe || B < kStackMinRows || B > h->stack.rows || (long long)T * B > h->stack_M || T > kStackMaxChunks || lists_serve(h, T, B)) return false;
     if (8 * h->stack.upc <= 128) return T >= 4;
-    const int blocks = (4 * h->H + 128 * (h->sm_count / 2 * 2 - 2 * h->stack.ncta) - 1) / (128 * (h->sm_count / 2 * 2 - 2 * h->stack.ncta));
+    const int blocks = (4 * h->H + 128 * (h->stack_ctas - 2 * h->stack.ncta) - 1) / (128 * (h->stack_ctas - 2 * h->stack.ncta));
     return T >= 16 && (blocks < 3 || B <= 24);
 }
 
@@ -741,9 +742,11 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     h->Hp8 = round_up(H, 8);
     h->Hs = round_up(H, 256);
     h->ncta_dir = std::max(1, std::min(h->sm_count / D, H));
+    h->cta_limit = h->sm_count;
     if (const char *e = getenv("LSTM_B200_CTAS")) {     // measurement: fewer CTAs per direction than SMs
         const int want = atoi(e);
         if (want >= 1 && want <= h->ncta_dir) h->ncta_dir = want;
+        if (want >= 1 && want <= h->cta_limit) h->cta_limit = want;
     }
     h->upc = (H + h->ncta_dir - 1) / h->ncta_dir;
     // fp32 storage: no more CTAs than full slices (H = 200: 100 CTAs of two units, not 52 of two and 96 of one).
@@ -816,8 +819,8 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     if (h->use_tcb && h->tcb[0].pair && D == 1 && layers == 2 && h->use_tc && !getenv("LSTM_B200_WAVE") && !getenv("LSTM_B200_RECUR")) {
         const int smem = h->smem_optin - kTcStaticSmem;
         bool fits = false;
-        h->use_stack = recur_stack_plan(H, h->sm_count, max_B, tc_terms, (size_t)smem, &h->stack) &&
-                       recur_stack_prepare(h->stack, h->sm_count, smem, &fits) == cudaSuccess && fits;
+        h->use_stack = recur_stack_plan(H, h->cta_limit, max_B, tc_terms, (size_t)smem, &h->stack, &h->stack_ctas) &&
+                       recur_stack_prepare(h->stack, h->stack_ctas, smem, &fits) == cudaSuccess && fits;
         if (!h->use_stack) cudaGetLastError();
         h->stack_M = std::min(max_T * std::min(max_B, h->stack.rows), kStackMaxRows);
     }
@@ -1087,7 +1090,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         rc = alloc_phase_words(h, h->f32_xch, (size_t)D * 2 * H * 32, st);
     {
         const char *env = getenv("LSTM_B200_WAVE");
-        const int upc = dtype == LSTM_F32 && !csr && D == 1 && !(env && strcmp(env, "0") == 0) ? recur_f32_wave_units(layers, H, in_dim, h->sm_count) : 0;
+        const int upc = dtype == LSTM_F32 && !csr && D == 1 && !(env && strcmp(env, "0") == 0) ? recur_f32_wave_units(layers, H, in_dim, h->cta_limit) : 0;
         if (rc == LSTM_OK && upc) {
             rc = alloc_phase_words(h, h->f32w_xch, (size_t)layers * std::min(max_T, kF32WaveMaxT) * H * 32, st);
             if (rc == LSTM_OK && recur_f32_wave_prepare(upc, max_B, h->smem_optin) != cudaSuccess)
@@ -1678,7 +1681,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         if (h->stack_T != T || h->stack_B != B) {
             memset(&h->stack_proj, 0, sizeof h->stack_proj);
             h->stack_T = 0;
-            if (!recur_stack_proj_plan(plan, H, T, B, h->sm_count, (size_t)h->smem_optin - kTcStaticSmem, &h->stack_proj, &h->stack_chunk) ||
+            if (!recur_stack_proj_plan(plan, H, T, B, h->stack_ctas, (size_t)h->smem_optin - kTcStaticSmem, &h->stack_proj, &h->stack_chunk) ||
                 !stack_proj_maps(&h->stack_maps, (const __nv_bfloat16 *)up.wx, h->xbn[0], h->xbn[0] + plane, h->stack_proj, H, up.ldk, h->ldn))
                 return fail(h, LSTM_ERR_CUDA, "stack projection plan failed");
             h->stack_T = T; h->stack_B = B;
@@ -1692,7 +1695,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         if (phase_sets(h->stack_xch, rec, st, &base, &set, &s.clear_words) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
         unsigned *counts = base + (size_t)set * h->stack_xch.set_words;
         s.other_set = base + (size_t)(set ^ 1) * h->stack_xch.set_words;
-        const int withhold = h->withhold_cta < 0 ? -1 : h->withhold_cta % (h->sm_count / 2 * 2);
+        const int withhold = h->withhold_cta < 0 ? -1 : h->withhold_cta % h->stack_ctas;
         for (int l = 0; l < 2; ++l) {
             RecurTcArgs &m = s.layer[l];
             m.ndirs = 1; m.H = H; m.B = m.Bs = B; m.T = T; m.D = 1;
@@ -1721,9 +1724,9 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         s.proj.spin_limit = h->spin_limit; s.proj.status = h->status_dev;
         s.chunk = h->stack_chunk;
         if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
-        e = launch_recur_stack(s, h->stack_maps, plan, h->sm_count, st);
+        e = launch_recur_stack(s, h->stack_maps, plan, h->stack_ctas, st);
         if (e == cudaSuccess) phase_launched(h->stack_xch, rec, (unsigned)(2 * kStackMaxChunks + 2 * recur_tc_xch_words(H, B, 1)));
-        ran(h, LSTM_RAN_BATCHED, h->sm_count / 2 * 2, kTcThreads, recur_stack_smem_bytes(plan, B, s.proj));
+        ran(h, LSTM_RAN_BATCHED, h->stack_ctas, kTcThreads, recur_stack_smem_bytes(plan, B, s.proj));
         ++h->last_launches;
         if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "stack launch failed: %s", cudaGetErrorString(e));

@@ -377,13 +377,13 @@ struct RecurStackArgs {
     unsigned clear_words;
 };
 struct StackProjMaps { alignas(64) unsigned char w[128], x[128], xlo[128]; };
-bool recur_stack_plan(int H, int sm_count, int rows_wanted, int terms, size_t max_smem, RecurTcPlan *p);
+bool recur_stack_plan(int H, int max_cta, int rows_wanted, int terms, size_t max_smem, RecurTcPlan *p, int *ctas);
 cudaError_t launch_repartition(const uint4 *src, const RecurTcPlan &from, uint4 *dst, const RecurTcPlan &to, int H, cudaStream_t st);
-cudaError_t recur_stack_prepare(const RecurTcPlan &p, int sm_count, int max_smem, bool *fits);
-bool recur_stack_proj_plan(const RecurTcPlan &p, int H, int T, int B, int sm_count, size_t max_smem, StackProjArgs *a, int *chunk);
+cudaError_t recur_stack_prepare(const RecurTcPlan &p, int ctas, int max_smem, bool *fits);
+bool recur_stack_proj_plan(const RecurTcPlan &p, int H, int T, int B, int ctas, size_t max_smem, StackProjArgs *a, int *chunk);
 bool stack_proj_maps(StackProjMaps *m, const __nv_bfloat16 *W, const __nv_bfloat16 *X, const __nv_bfloat16 *Xlo, const StackProjArgs &a, int K, int ldk, int ldx);
 size_t recur_stack_smem_bytes(const RecurTcPlan &p, int rows, const StackProjArgs &a);
-cudaError_t launch_recur_stack(const RecurStackArgs &a, const StackProjMaps &maps, const RecurTcPlan &p, int sm_count, cudaStream_t st);
+cudaError_t launch_recur_stack(const RecurStackArgs &a, const StackProjMaps &maps, const RecurTcPlan &p, int ctas, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------
 // H-LSTM recurrent kernel (one ReLU hidden layer of width Hh inside each gate; bf16 weights, dense).

@@ -89,18 +89,19 @@ cudaLaunchConfig_t config(cudaLaunchAttribute (&attr)[2], int grid, size_t smem,
 
 size_t recur_stack_smem_bytes(const RecurTcPlan &p, int rows, const StackProjArgs &a) { return std::max(role_smem(p.KH, p.upc, rows, p.terms), proj_smem(a)); }
 
-// Partition of a stack whose calls have up to rows_wanted rows: CTA pairs of each layer, the others project.
-bool recur_stack_plan(int H, int sm_count, int rows_wanted, int terms, size_t max_smem, RecurTcPlan *p)
+// Partition of a stack whose calls have up to rows_wanted rows: CTA pairs of each layer, the others project; *ctas: all of them.
+bool recur_stack_plan(int H, int max_cta, int rows_wanted, int terms, size_t max_smem, RecurTcPlan *p, int *ctas)
 {
     if (H <= 64) return false;
     const int KH = ((H + 1) / 2 + 15) / 16 * 16;
     for (int upc = 4; upc <= 24; upc += 4) {
         const int n = (H + 2 * upc - 1) / (2 * upc) * 2, mb = blocks_of(upc);
-        if (2 * n + kStackMinProj > sm_count) continue;
+        if (2 * n + kStackMinProj > max_cta / 2 * 2) continue;
         for (int rg = std::min(terms == 3 ? 2 : 4, groups_of(rows_wanted)); rg >= 1; --rg) {
             const int acc = mb == 2 ? 2 * tc_columns(rg, terms) : tc_acc_columns(rg, terms);
             if (KH / 2 + acc > 512 || KH > 16 * kPollers * kMaxGroups || role_smem(KH, upc, 8 * rg, terms) > max_smem) continue;
             p->upc = upc; p->ncta = n; p->KH = KH; p->pair = 1; p->rows = 8 * rg; p->terms = terms;
+            *ctas = max_cta / 2 * 2;
             return true;
         }
     }
@@ -114,7 +115,7 @@ cudaError_t launch_repartition(const uint4 *src, const RecurTcPlan &from, uint4 
     return cudaGetLastError();
 }
 
-cudaError_t recur_stack_prepare(const RecurTcPlan &p, int sm_count, int max_smem, bool *fits)
+cudaError_t recur_stack_prepare(const RecurTcPlan &p, int ctas, int max_smem, bool *fits)
 {
     *fits = true;
     for (int v = 0; v < p.rows / 8 + std::min(2, p.rows / 8); ++v) {
@@ -122,11 +123,11 @@ cudaError_t recur_stack_prepare(const RecurTcPlan &p, int sm_count, int max_smem
         const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
         if (e != cudaSuccess) return e;
         cudaLaunchAttribute attr[2];
-        cudaLaunchConfig_t cfg = config(attr, sm_count / 2 * 2, max_smem, nullptr);
+        cudaLaunchConfig_t cfg = config(attr, ctas, max_smem, nullptr);
         cfg.numAttrs = 1;
         int clusters = 0;
         if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)fn, &cfg) != cudaSuccess) { cudaGetLastError(); clusters = 0; }
-        if (clusters < sm_count / 2) *fits = false;
+        if (clusters < ctas / 2) *fits = false;
     }
     return cudaSuccess;
 }
@@ -136,9 +137,9 @@ cudaError_t recur_stack_prepare(const RecurTcPlan &p, int sm_count, int max_smem
 // call at 2, 3, 4, 5, 6 timesteps: 2 x 1500, T = 35, 2 rows 249, 191, 187, 192, 189; 20 rows 320, 273, 259 (no room for five); 1000
 // with 24 rows 208, 185, 181, 181, 179; 517 with 8 126, 120, 118, 117, 118; 700, T = 20, 6 rows 89, 87, 85, 85, 87; 517, T = 23, 3
 // rows 93, 89, 89, 89, 90; 300 with 16 124, 122, 120, 122, 120; pruned 1500 with 16 300, 253, 251, 259, 257.
-bool recur_stack_proj_plan(const RecurTcPlan &p, int H, int T, int B, int sm_count, size_t max_smem, StackProjArgs *a, int *chunk)
+bool recur_stack_proj_plan(const RecurTcPlan &p, int H, int T, int B, int ctas, size_t max_smem, StackProjArgs *a, int *chunk)
 {
-    const int nproj = sm_count / 2 * 2 - 2 * p.ncta;
+    const int nproj = ctas - 2 * p.ncta;
     a->M = T * B; a->N = 4 * H; a->kblocks = (H + 63) / 64;
     const int rows = (a->N + nproj - 1) / nproj;
     a->mb = (rows + 127) / 128;
@@ -163,7 +164,7 @@ bool stack_proj_maps(StackProjMaps *m, const __nv_bfloat16 *W, const __nv_bfloat
            encode_tmap_bf16_2d(m->xlo, Xlo, a.M, K, ldx, a.nrp);
 }
 
-cudaError_t launch_recur_stack(const RecurStackArgs &a, const StackProjMaps &maps, const RecurTcPlan &p, int sm_count, cudaStream_t st)
+cudaError_t launch_recur_stack(const RecurStackArgs &a, const StackProjMaps &maps, const RecurTcPlan &p, int ctas, cudaStream_t st)
 {
     KernelFn fn = pick(groups_of(a.layer[0].B), p.terms, blocks_of(p.upc), a.layer[0].nsplit > 1);
     if (!fn) return cudaErrorInvalidValue;
@@ -171,7 +172,7 @@ cudaError_t launch_recur_stack(const RecurStackArgs &a, const StackProjMaps &map
     StackProjMaps m = maps;
     void *params[] = {&copy, m.w, m.x, m.xlo};
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = config(attr, sm_count / 2 * 2, recur_stack_smem_bytes(p, a.layer[0].B, a.proj), st);
+    const cudaLaunchConfig_t cfg = config(attr, ctas, recur_stack_smem_bytes(p, a.layer[0].B, a.proj), st);
     return cudaLaunchKernelExC(&cfg, (const void *)fn, params);
 }
 

@@ -80,3 +80,24 @@ def test_kernel_of_a_call(case, kernel, threads):
     assert pkg.RECUR_KERNELS[info["kernel"]] == pkg.RECUR_KERNELS[getattr(pkg, "LSTM_RAN_" + kernel)]
     assert info["kernel_ctas"] >= 1 and (threads is None or info["kernel_threads"] == threads)
     assert info["kernel_smem_bytes"] <= 227 * 1024
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("ctas", [20, 61, 100])
+def test_stacks_on_fewer_ctas(oracle, dtype, ctas, monkeypatch):
+    """The limit on the CTAs of a direction holds for the kernels that run the layers of a stack side by side too."""
+    import torch
+    import lstm_workloads as wl
+    import paper_1901_10997_b200 as pkg
+    from gpu_util import assert_close
+    monkeypatch.setenv("LSTM_B200_CTAS", str(ctas))
+    w = wl.Workload("ctas", 2, False, 40, 200, 9, 10, dtype, 0.1, seed=ctas)
+    weights, x = wl.make(w)
+    m = pkg.LSTM(weights, layers=2, in_dim=40, hidden=200, dtype=dtype, max_T=9, max_B=10)
+    try:
+        got = m.forward(torch.from_numpy(x).cuda())
+        m.check()
+        assert 1 <= m.info()["kernel_ctas"] <= ctas
+        assert_close([t.cpu().numpy() for t in got], oracle.forward(weights, x, layers=2, bidir=False, hidden=200), dtype, "fewer CTAs")
+    finally:
+        m.close()
