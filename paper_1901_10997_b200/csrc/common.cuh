@@ -352,6 +352,7 @@ cudaError_t launch_recur_tc(const RecurTcArgs &a, cudaStream_t st);
 // ---------------------------------------------------------------------------------------------------
 constexpr int kStackMaxChunks = 256;
 constexpr int kStackMinProj = 16;     // projecting CTAs, at least
+constexpr int kStackNarrow = 296;     // units of layers whose launch leaves SMs to others, at most
 constexpr int kStackMinRows = 2;
 constexpr int kStackMaxRows = 8192;   // rows (timesteps x sequences) of a call, at most
 struct StackProjArgs {

@@ -90,18 +90,26 @@ cudaLaunchConfig_t config(cudaLaunchAttribute (&attr)[2], int grid, size_t smem,
 size_t recur_stack_smem_bytes(const RecurTcPlan &p, int rows, const StackProjArgs &a) { return std::max(role_smem(p.KH, p.upc, rows, p.terms), proj_smem(a)); }
 
 // Partition of a stack whose calls have up to rows_wanted rows: CTA pairs of each layer, the others project; *ctas: all of them.
+// Narrow layers take no more CTAs than they gain from: up to 296 units the launches of two handles and more fit the chip at once when
+// the layers run one after the other, and so they do here: pairs of 24 units, about 72 rows of G on a projecting CTA.  us per call with 1, 2,
+// 3, 6 handles on streams of their own, T = 35, one layer after the other; side by side on all SMs; on these CTAs: H = 128 with 8 rows 131, 67, 46,
+// 32; 96, 82, 82, 81; 93, 49, 33, 19 (32 CTAs); 200 with 20 181, 91, 73, 73; 120, 107, 103, 103; 122, 61, 43, 36 (48); 296 with 32 207, 105, 98, 95;
+// 134, 120, 119, 118; 132, 67, 59, 60 (70).  One handle against all SMs: 65 to 296 units, 5 to 32 rows, T = 4 to 70 0.92 - 1.02.  Eight projecting
+// CTAs at 296: up to 1.10 at T = 4; pairs of 32 units 1.03 with 32 rows; 400 units with pairs of 24 1.06 with 8 rows.
 bool recur_stack_plan(int H, int max_cta, int rows_wanted, int terms, size_t max_smem, RecurTcPlan *p, int *ctas)
 {
     if (H <= 64) return false;
+    const bool narrow = H <= kStackNarrow;
+    const int min_proj = narrow ? std::max(8, (4 * H + 143) / 144 * 2) : kStackMinProj;
     const int KH = ((H + 1) / 2 + 15) / 16 * 16;
-    for (int upc = 4; upc <= 24; upc += 4) {
+    for (int upc = narrow ? 12 : 4; upc <= 24; upc += 4) {
         const int n = (H + 2 * upc - 1) / (2 * upc) * 2, mb = blocks_of(upc);
-        if (2 * n + kStackMinProj > max_cta / 2 * 2) continue;
+        if (2 * n + min_proj > max_cta / 2 * 2) continue;
         for (int rg = std::min(terms == 3 ? 2 : 4, groups_of(rows_wanted)); rg >= 1; --rg) {
             const int acc = mb == 2 ? 2 * tc_columns(rg, terms) : tc_acc_columns(rg, terms);
             if (KH / 2 + acc > 512 || KH > 16 * kPollers * kMaxGroups || role_smem(KH, upc, 8 * rg, terms) > max_smem) continue;
             p->upc = upc; p->ncta = n; p->KH = KH; p->pair = 1; p->rows = 8 * rg; p->terms = terms;
-            *ctas = max_cta / 2 * 2;
+            *ctas = narrow ? 2 * n + min_proj : max_cta / 2 * 2;
             return true;
         }
     }

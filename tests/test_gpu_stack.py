@@ -179,3 +179,33 @@ def test_stack_with_two_blocks_whose_words_or_projection_are_withheld(oracle):
             assert_close([t.cpu().numpy() for t in got], ref, "bf16", "stack, after a withheld CTA")
     finally:
         m.close()
+
+
+# narrow layers: (in_dim, H, T, B, density) at the edges of pairs of 24 units and of the projecting CTAs' blocks of rows
+@pytest.mark.parametrize("s", [(30, 65, 9, 17, 1.0), (24, 96, 5, 32, 1.0), (300, 97, 8, 8, 1.0), (20, 256, 7, 25, 1.0), (200, 295, 6, 20, 1.0), (40, 296, 13, 9, 1.0), (33, 296, 9, 16, 0.2)],
+                         ids=lambda s: "in{}_H{}_T{}_B{}_p{}".format(*s))
+def test_small_shapes_of_stacks_that_leave_sms_to_others(oracle, s):
+    """Two layers of up to 296 units take less than half of the SMs, so that the calls of two handles run at once."""
+    import torch
+    import paper_1901_10997_b200 as pkg
+    w, weights, x, h0, c0 = make(s)
+    ref = oracle.forward(weights, x, h0, c0, layers=2, bidir=False, hidden=w.hidden)
+    mode, ws = ("dense", weights) if w.density == 1 else ("csr", csr_weights(oracle, weights))
+    xd, hd, cd = (torch.from_numpy(v).cuda() for v in (x, h0, c0))
+    models, streams = [], [torch.cuda.Stream() for _ in range(3)]
+    try:
+        for _ in streams:
+            models.append(pkg.LSTM(ws, layers=2, in_dim=w.in_dim, hidden=w.hidden, dtype="bf16", exec_mode=mode, max_T=w.T, max_B=w.B))
+        outs = [(torch.empty(w.T, w.B, w.hidden, device="cuda"), torch.empty(2, w.B, w.hidden, device="cuda"), torch.empty(2, w.B, w.hidden, device="cuda")) for _ in streams]
+        torch.cuda.synchronize()
+        for _ in range(20):
+            for m, st, out in zip(models, streams, outs):
+                m.forward(xd, hd, cd, out=out, stream=st.cuda_stream)
+        for m, out in zip(models, outs):
+            m.check()
+            assert_close([t.cpu().numpy() for t in out], ref, "bf16", "narrow stack")
+            info = m.info()
+            assert info["launches_per_forward"] == 3 and 2 * info["kernel_ctas"] <= info["sm_count"]
+    finally:
+        for m in models:
+            m.close()
