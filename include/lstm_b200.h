@@ -108,9 +108,10 @@ typedef struct {
  *                   = tc1   batched tensor-core recurrence without cluster pairs
  *   LSTM_B200_FUSE  = 0     never compute the input projection inside the recurrent kernel (single sequences of up
  *                           to 40 steps on the register-resident kernel do so by default)
- *   LSTM_B200_WAVE  = 0     one launch per layer even where a kernel that runs the layers of a stack side by side would serve it
+ *   LSTM_B200_WAVE  = 0     one launch per layer, bf16 and fp32, even where a kernel that runs the layers of a stack side by side
+ *                           would serve it
  *                   = 1     the layer-wavefront kernel for every call of up to four sequences, single timesteps
- *                           included, where it serves the stack
+ *                           included, where it serves the stack; all other calls one launch per layer
  *   LSTM_B200_PROJ  = simt  CUDA-core input projection instead of the tensor-core one
  *                   = csr   CSR handles walk the lists of Wx in the projection too (by default bf16 CSR handles keep a
  *                           dense copy of Wx and project on the tensor cores; the recurrence stays sparse)

@@ -573,6 +573,13 @@ bool wave_serves(const lstm_handle *h, int T, int B)
 // 1.00 - 1.09; six steps with 2 rows 0.95 - 1.07; one step with 5 rows 1.00 - 1.08.
 bool lists_serve(const lstm_handle *h, int T, int B) { return h->use_csr_reg && (B == 1 || !h->use_tcb || (B <= 4 && T * B <= 8)); }
 
+// LSTM_B200_WAVE=0 and =1 both say which kernel a stack's calls run on: what =1 does not give to the layer-wavefront kernel runs layer by layer.
+bool side_by_side_wanted()
+{
+    const char *env = getenv("LSTM_B200_WAVE");
+    return !(env && (strcmp(env, "0") == 0 || strcmp(env, "1") == 0));
+}
+
 // Do two layers of a batch run side by side?  The lag of the upper layer, one chunk and its projection, has to be earned back.  Time per
 // call, side by side / one after the other, T = 4, 8, 16, 35, 70: H = 200 with 8, 32 rows 0.86, 0.82, 0.79, 0.75, 0.74 and 0.78,
 // 0.75, 0.72, 0.68, 0.67; 517 with 3, 20 rows 0.80, 0.76, 0.68, 0.70, 0.70 and 0.86, 0.75, 0.72, 0.67, 0.64; 1000 with 2, 32 rows
@@ -816,7 +823,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         if (h->use_mma) { h->seq_dirs = true; h->use_tcb = plan_tcb(h->ncta_dir, 1); }
         else { h->ncta_dir = nc; h->upc = up; h->threads = th; }
     }
-    if (h->use_tcb && h->tcb[0].pair && D == 1 && layers == 2 && h->use_tc && !getenv("LSTM_B200_WAVE") && !getenv("LSTM_B200_RECUR")) {
+    if (h->use_tcb && h->tcb[0].pair && D == 1 && layers == 2 && h->use_tc && side_by_side_wanted()) {
         const int smem = h->smem_optin - kTcStaticSmem;
         bool fits = false;
         h->use_stack = recur_stack_plan(H, h->cta_limit, max_B, tc_terms, (size_t)smem, &h->stack, &h->stack_ctas) &&
@@ -1089,8 +1096,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     if (rc == LSTM_OK && dtype == LSTM_F32 && !csr && h->upc <= 2 && H <= kF32MaxUnits)
         rc = alloc_phase_words(h, h->f32_xch, (size_t)D * 2 * H * 32, st);
     {
-        const char *env = getenv("LSTM_B200_WAVE");
-        const int upc = dtype == LSTM_F32 && !csr && D == 1 && !(env && strcmp(env, "0") == 0) ? recur_f32_wave_units(layers, H, in_dim, h->cta_limit) : 0;
+        const int upc = dtype == LSTM_F32 && !csr && D == 1 && side_by_side_wanted() ? recur_f32_wave_units(layers, H, in_dim, h->cta_limit) : 0;
         if (rc == LSTM_OK && upc) {
             rc = alloc_phase_words(h, h->f32w_xch, (size_t)layers * std::min(max_T, kF32WaveMaxT) * H * 32, st);
             if (rc == LSTM_OK && recur_f32_wave_prepare(upc, max_B, h->smem_optin) != cudaSuccess)

@@ -101,3 +101,15 @@ def test_stacks_on_fewer_ctas(oracle, dtype, ctas, monkeypatch):
         assert_close([t.cpu().numpy() for t in got], oracle.forward(weights, x, layers=2, bidir=False, hidden=200), dtype, "fewer CTAs")
     finally:
         m.close()
+
+
+@pytest.mark.parametrize("value,side_by_side", [(None, True), ("", True), ("0", False), ("1", False)])
+@pytest.mark.parametrize("dtype,launches", [("bf16", (3, 5)), ("fp32", (1, 4))])
+def test_switch_that_keeps_the_layers_of_a_stack_apart(dtype, launches, value, side_by_side, monkeypatch):
+    if value is None:
+        monkeypatch.delenv("LSTM_B200_WAVE", raising=False)
+    else:
+        monkeypatch.setenv("LSTM_B200_WAVE", value)
+    monkeypatch.setenv("LSTM_B200_RECUR", "")              # an empty switch is an unset one
+    info = forward("lstm", dtype, False, 2, 200, 6, 9)
+    assert info["launches_per_forward"] == launches[0 if side_by_side else 1]
