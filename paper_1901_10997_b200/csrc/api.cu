@@ -585,14 +585,17 @@ bool side_by_side_wanted()
 // 0.75, 0.72, 0.68, 0.67; 517 with 3, 20 rows 0.80, 0.76, 0.68, 0.70, 0.70 and 0.86, 0.75, 0.72, 0.67, 0.64; 1000 with 2, 32 rows
 // 0.96, 0.84, 0.75, 0.67, 0.64 and 1.00, 0.84, 0.77, 0.71, 0.66.  Wider layers, whose pairs have a second block of rows: 1250 with 2,
 // 20 rows 1.06, 0.97, 0.88, 0.84, 0.81 and 1.14, 1.04, 0.96, 0.91, 0.84; 1500 with 4, 20, 24, 32 rows 1.12, 1.05, 0.95, 0.82, 0.75;
-// 1.20, 0.98, 0.93, 0.88, 0.82; 1.15, 1.00, 0.99, 0.92, 0.91; 1.12, 1.04, 1.07, 1.06, 1.06 (three blocks of rows on each projecting CTA,
-// which no longer keep up).  Pruned layers the same: 800 with 2, 16 rows, T = 8 0.80, 0.72; 1500 with 16 rows, T = 35 0.84.
+// 1.20, 0.98, 0.93, 0.88, 0.82; 1.15, 1.00, 0.99, 0.92, 0.91; 1.12, 1.04, 1.07, 1.06, 1.06: with many rows of G on each projecting CTA
+// these no longer keep up.  T = 16, 35, 70, 330 rows of G: 1320 with 16, 20, 24 rows 0.96, 0.93, 0.87; 0.96, 0.91, 0.85; 1.00, 1.02, 0.98; 396:
+// 1584 with 9, 12, 16, 20, 24 0.99, 0.94, 0.91; 1.01, 0.98, 0.92; 1.04, 1.06, 1.00; 1.10, 1.02, 1.05; 1.23, 1.25, 1.27.  With one block of
+// rows in a pair there is no such line: 1056 (264 rows of G) with 24, 32 rows, T = 4, 8, 16, 35, 70 1.00, 0.90, 0.84, 0.82, 0.79; 0.95, 0.91,
+// 0.95, 0.93, 0.93.  Pruned layers the same: 800 with 2, 16 rows, T = 8 0.80, 0.72; 1500 with 16 rows, T = 35 0.84.
 bool stack_serves(const lstm_handle *h, int T, int B)
 {
     if (!h->use_stack || h->probe || B < kStackMinRows || B > h->stack.rows || (long long)T * B > h->stack_M || T > kStackMaxChunks || lists_serve(h, T, B)) return false;
     if (8 * h->stack.upc <= 128) return T >= 4;
-    const int blocks = (4 * h->H + 128 * (h->stack_ctas - 2 * h->stack.ncta) - 1) / (128 * (h->stack_ctas - 2 * h->stack.ncta));
-    return T >= 16 && (blocks < 3 || B <= 24);
+    const int nproj = h->stack_ctas - 2 * h->stack.ncta, rows = (4 * h->H + nproj - 1) / nproj;
+    return T >= 16 && B <= (rows <= 256 ? h->stack.rows : rows <= 312 ? 24 : rows <= 384 ? 20 : 12);
 }
 
 // Rows of a [4H x H] recurrent matrix (row q*H + j, dense or as lists) as the batched tensor-core kernel wants them: per CTA [8-column

@@ -31,7 +31,8 @@ def test_small_shapes_of_stacks(oracle, s):
 
 
 # H, T, B -> launches: beside each other three, one after the other five
-@pytest.mark.parametrize("H,T,B,launches", [(300, 4, 9, 3), (300, 3, 9, 5), (300, 4, 32, 3), (300, 4, 33, 5), (1200, 16, 9, 3), (1200, 15, 9, 5), (1500, 16, 24, 3), (1500, 16, 25, 5)])
+@pytest.mark.parametrize("H,T,B,launches", [(300, 4, 9, 3), (300, 3, 9, 5), (300, 4, 32, 3), (300, 4, 33, 5), (1200, 16, 9, 3), (1200, 15, 9, 5), (1500, 16, 24, 3), (1500, 16, 25, 5),
+                                              (1320, 16, 20, 3), (1320, 16, 21, 5), (1584, 16, 12, 3), (1584, 16, 13, 5), (1056, 4, 32, 3)])
 def test_calls_that_run_two_layers_at_once(H, T, B, launches):
     import torch
     import paper_1901_10997_b200 as pkg
