@@ -99,7 +99,7 @@ struct lstm_handle {
     RecurTcPlan stack = {0, 0, 0, 0, 0, 0};
     PhaseWords stack_xch;
     float *stack_G = nullptr; int stack_M = 0, stack_ctas = 0;
-    StackProjArgs stack_proj; StackProjMaps stack_maps; int stack_chunk = 0, stack_T = 0, stack_B = 0;
+    StackProjArgs stack_proj; StackProjMaps stack_maps; int stack_chunk = 0, stack_T = 0, stack_B = 0; bool stack_planned = false;
     PhaseWords f32_xch;                // fp32 dense, at most two units per CTA
     int f32w_upc = 0;                  // fp32 stacks, all layers in one launch: units per CTA (0: not served) and exchange words
     PhaseWords f32w_xch;
@@ -596,6 +596,20 @@ bool stack_serves(const lstm_handle *h, int T, int B)
     if (8 * h->stack.upc <= 128) return T >= 4;
     const int nproj = h->stack_ctas - 2 * h->stack.ncta, rows = (4 * h->H + nproj - 1) / nproj;
     return T >= 16 && B <= (rows <= 256 ? h->stack.rows : rows <= 312 ? 24 : rows <= 384 ? 20 : 12);
+}
+
+// The projecting CTAs' work for calls of T x B, kept until the sizes change; false when there is no such plan (the layers then run one
+// after the other).
+bool stack_plan_call(lstm_handle *h, int T, int B)
+{
+    if (h->stack_T == T && h->stack_B == B) return h->stack_planned;
+    const Layer &up = h->layers[1];
+    memset(&h->stack_proj, 0, sizeof h->stack_proj);
+    h->stack_T = T; h->stack_B = B;
+    h->stack_planned = recur_stack_proj_plan(h->stack, h->H, T, B, h->stack_ctas, (size_t)h->smem_optin - kTcStaticSmem, &h->stack_proj, &h->stack_chunk) &&
+                       stack_proj_maps(&h->stack_maps, (const __nv_bfloat16 *)up.wx, h->xbn[0], h->xbn[0] + (long long)h->max_T * h->max_B * h->ldn,
+                                       h->stack_proj, h->H, up.ldk, h->ldn);
+    return h->stack_planned;
 }
 
 // Rows of a [4H x H] recurrent matrix (row q*H + j, dense or as lists) as the batched tensor-core kernel wants them: per CTA [8-column
@@ -1682,19 +1696,11 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         return LSTM_OK;
     }
 
-    if (stack_serves(h, T, B)) {
+    if (stack_serves(h, T, B) && stack_plan_call(h, T, B)) {
         // two layers of a batch: the lower one's projection, then both recurrences and the upper one's projection in one launch
         const Layer &up = h->layers[1];
         const RecurTcPlan &plan = h->stack;
         const long long plane = (long long)h->max_T * h->max_B * h->ldn;
-        if (h->stack_T != T || h->stack_B != B) {
-            memset(&h->stack_proj, 0, sizeof h->stack_proj);
-            h->stack_T = 0;
-            if (!recur_stack_proj_plan(plan, H, T, B, h->stack_ctas, (size_t)h->smem_optin - kTcStaticSmem, &h->stack_proj, &h->stack_chunk) ||
-                !stack_proj_maps(&h->stack_maps, (const __nv_bfloat16 *)up.wx, h->xbn[0], h->xbn[0] + plane, h->stack_proj, H, up.ldk, h->ldn))
-                return fail(h, LSTM_ERR_CUDA, "stack projection plan failed");
-            h->stack_T = T; h->stack_B = B;
-        }
         int nsplit = 1;
         { const int prc = run_projection(h, 0, x, x, M, 4 * H, &nsplit, st); if (prc != LSTM_OK) return prc; }
         RecurStackArgs s;
