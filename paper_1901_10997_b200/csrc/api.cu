@@ -590,12 +590,14 @@ bool side_by_side_wanted()
 // 1584 with 9, 12, 16, 20, 24 0.99, 0.94, 0.91; 1.01, 0.98, 0.92; 1.04, 1.06, 1.00; 1.10, 1.02, 1.05; 1.23, 1.25, 1.27.  With one block of
 // rows in a pair there is no such line: 1056 (264 rows of G) with 24, 32 rows, T = 4, 8, 16, 35, 70 1.00, 0.90, 0.84, 0.82, 0.79; 0.95, 0.91,
 // 0.95, 0.93, 0.93.  Pruned layers the same: 800 with 2, 16 rows, T = 8 0.80, 0.72; 1500 with 16 rows, T = 35 0.84.
+int stack_min_steps(const RecurTcPlan &p) { return 8 * p.upc <= 128 ? 4 : 16; }
 bool stack_serves(const lstm_handle *h, int T, int B)
 {
     if (!h->use_stack || h->probe || B < kStackMinRows || B > h->stack.rows || (long long)T * B > h->stack_M || T > kStackMaxChunks || lists_serve(h, T, B)) return false;
-    if (8 * h->stack.upc <= 128) return T >= 4;
+    if (T < stack_min_steps(h->stack)) return false;
+    if (8 * h->stack.upc <= 128) return true;
     const int nproj = h->stack_ctas - 2 * h->stack.ncta, rows = (4 * h->H + nproj - 1) / nproj;
-    return T >= 16 && B <= (rows <= 256 ? h->stack.rows : rows <= 312 ? 24 : rows <= 384 ? 20 : 12);
+    return B <= (rows <= 256 ? h->stack.rows : rows <= 312 ? 24 : rows <= 384 ? 20 : 12);
 }
 
 // The projecting CTAs' work for calls of T x B, kept until the sizes change; false when there is no such plan (the layers then run one
@@ -818,7 +820,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         const char *env = getenv("LSTM_B200_RECUR");
         if (!bf16 || (csr && !h->csr_dense_proj) || max_B < kTcMinRows || (env && (strcmp(env, "mma") == 0 || strcmp(env, "simt") == 0))) return false;
         const size_t smem = (size_t)h->smem_optin - kTcStaticSmem;
-        if (recur_tc_prepare(tc_terms, (int)smem) != cudaSuccess) { cudaGetLastError(); return false; }
+        if (recur_tc_prepare(tc_terms, max_B, (int)smem) != cudaSuccess) { cudaGetLastError(); return false; }
         if (!(env && strcmp(env, "tc1") == 0) && recur_tc_plan(H, ncta, max_B, 1, tc_terms, smem, &h->tcb[0]) &&
             recur_tc_pair_supported(h->tcb[0].ncta * dirs_side_by_side, h->tcb[0])) {
             const int rows = std::min(max_B, tc_single_rows(H, D, tc_terms));
@@ -844,7 +846,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         const int smem = h->smem_optin - kTcStaticSmem;
         bool fits = false;
         h->use_stack = recur_stack_plan(H, h->cta_limit, max_B, tc_terms, (size_t)smem, &h->stack, &h->stack_ctas) &&
-                       recur_stack_prepare(h->stack, h->stack_ctas, smem, &fits) == cudaSuccess && fits;
+                       max_T >= stack_min_steps(h->stack) && recur_stack_prepare(h->stack, h->stack_ctas, smem, &fits) == cudaSuccess && fits;
         if (!h->use_stack) cudaGetLastError();
         h->stack_M = std::min(max_T * std::min(max_B, h->stack.rows), kStackMaxRows);
     }

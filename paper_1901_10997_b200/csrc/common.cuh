@@ -343,7 +343,7 @@ size_t recur_tc_smem_bytes(int KH, int upc, int rows, int pair, int terms);
 size_t recur_tc_xch_words(int H, int rows, int dirs);    // exchange words of one launch with `rows` batch rows
 bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, int terms, size_t max_smem, RecurTcPlan *p);
 bool recur_tc_pair_supported(int grid, const RecurTcPlan &p);
-cudaError_t recur_tc_prepare(int terms, int max_smem);
+cudaError_t recur_tc_prepare(int terms, int rows, int max_smem);
 cudaError_t launch_recur_tc(const RecurTcArgs &a, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------

@@ -125,17 +125,19 @@ cudaError_t launch_repartition(const uint4 *src, const RecurTcPlan &from, uint4 
 
 cudaError_t recur_stack_prepare(const RecurTcPlan &p, int ctas, int max_smem, bool *fits)
 {
-    *fits = true;
+    *fits = false;
     for (int v = 0; v < p.rows / 8 + std::min(2, p.rows / 8); ++v) {
         KernelFn fn = v < p.rows / 8 ? pick(v + 1, p.terms, blocks_of(p.upc), false) : pick(v + 1 - p.rows / 8, p.terms, blocks_of(p.upc), true);
         const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
         if (e != cudaSuccess) return e;
+        // (each build takes all of an SM's registers and, here, of its shared memory: one answer for all of them)
+        if (v > 0) continue;
         cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg = config(attr, ctas, max_smem, nullptr);
         cfg.numAttrs = 1;
         int clusters = 0;
         if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)fn, &cfg) != cudaSuccess) { cudaGetLastError(); clusters = 0; }
-        if (clusters < ctas / 2) *fits = false;
+        *fits = clusters >= ctas / 2;
     }
     return cudaSuccess;
 }

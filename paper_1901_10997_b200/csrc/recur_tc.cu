@@ -125,9 +125,10 @@ bool recur_tc_plan(int H, int max_cta, int rows_wanted, int pair, int terms, siz
     return false;
 }
 
-cudaError_t recur_tc_prepare(int terms, int max_smem)
+// (the builds that calls of up to `rows` sequences can reach)
+cudaError_t recur_tc_prepare(int terms, int rows, int max_smem)
 {
-    for (int rg = 1; rg <= kTcMaxRows / 8; ++rg) {
+    for (int rg = 1; rg <= groups_of(rows < kTcMaxRows ? rows : kTcMaxRows); ++rg) {
         for (int v = 0; v < (rg <= 2 ? 4 : 2); ++v) {
             const cudaError_t e = cudaFuncSetAttribute(pick(rg, (v & 1) != 0, terms, v >= 2), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
             if (e != cudaSuccess) return e;

@@ -210,3 +210,25 @@ def test_small_shapes_of_stacks_that_leave_sms_to_others(oracle, s):
     finally:
         for m in models:
             m.close()
+
+
+@pytest.mark.parametrize("H,max_T,holds_more", [(1500, 15, False), (1500, 16, True), (1050, 3, False), (1050, 4, True)])
+def test_memory_of_handles_whose_calls_are_too_short(H, max_T, holds_more, monkeypatch):
+    """Rows, words and the second G for two layers side by side only where a call of the handle can use them."""
+    import torch
+    import paper_1901_10997_b200 as pkg
+    g = torch.Generator(device="cuda").manual_seed(H)
+    ws = [{"wx": torch.randn(4 * H, n, generator=g, device="cuda"), "wh": torch.randn(4 * H, H, generator=g, device="cuda")} for n in (16, H)]
+
+    def held():
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        m = pkg.LSTM(ws, layers=2, in_dim=16, hidden=H, dtype="bf16", max_T=max_T, max_B=20)
+        used = free - torch.cuda.mem_get_info()[0]
+        m.close()
+        return used
+
+    held()                                          # (what the first handle of a process sets up)
+    both = held()
+    monkeypatch.setenv("LSTM_B200_WAVE", "0")
+    assert (both - held() >= 2 * 4 * H * H * 2) == holds_more      # the rows of both layers' recurrent matrices, at least
