@@ -1117,7 +1117,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     {
         const int upc = dtype == LSTM_F32 && !csr && D == 1 && side_by_side_wanted() ? recur_f32_wave_units(layers, H, in_dim, h->cta_limit) : 0;
         if (rc == LSTM_OK && upc) {
-            rc = alloc_phase_words(h, h->f32w_xch, (size_t)layers * std::min(max_T, kF32WaveMaxT) * recur_f32_wave_slot_words(H, max_B), st);
+            rc = alloc_phase_words(h, h->f32w_xch, (size_t)layers * std::min(max_T, kF32WaveMaxT) * H * 32, st);
             if (rc == LSTM_OK && recur_f32_wave_prepare(upc, max_B, h->smem_optin) != cudaSuccess)
                 rc = fail(h, LSTM_ERR_CUDA, "fp32 stack kernel set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
             h->f32w_upc = upc;
@@ -1684,7 +1684,6 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         }
         m.h0 = h0; m.c0 = c0; m.hT = hT; m.cT = cT; m.y = y;
         m.slots = std::min(h->max_T, kF32WaveMaxT);
-        m.slot_words = recur_f32_wave_slot_words(H, h->max_B);
         unsigned clear_T = 0;
         if (phase_sets(h->f32w_xch, rec, st, &m.xch, &m.set, &clear_T) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "exchange reset failed");
         m.clear_T = (int)clear_T;

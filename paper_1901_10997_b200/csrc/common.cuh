@@ -236,12 +236,11 @@ struct RecurF32WaveArgs {
     const float *h0, *c0;               // [L][B][H] or nullptr
     float *hT, *cT;
     float *y;                           // [T][B][H]: the top layer's h
-    unsigned *xch;                      // exchange words [2 sets][L][slots][slot_words]
-    int slots, slot_words;              // timesteps there is room for; words of one
+    unsigned *xch;                      // exchange words [2 sets][L][slots][H][32 batch rows]
+    int slots;                          // timesteps there is room for
     int set, clear_T;                   // the set this launch uses; it clears the other one as far as clear_T timesteps
     int *status;
 };
-int recur_f32_wave_slot_words(int H, int rows);
 int recur_f32_wave_units(int L, int H, int in_dim, int max_cta);
 cudaError_t recur_f32_wave_prepare(int upc, int max_B, int smem_optin);
 cudaError_t launch_recur_f32_wave(const RecurF32WaveArgs &a, cudaStream_t st);

@@ -22,8 +22,6 @@
 #include "common.cuh"
 #include "device_util.cuh"
 
-#include <algorithm>
-
 namespace lstm {
 namespace {
 
@@ -66,8 +64,8 @@ __global__ void __launch_bounds__(kThreads, 1) recur_f32_wave_kernel(const Recur
     const int XP = f32_wave_x_pitch(Kx);
     LSTM_CHECK_SMEM_END(reinterpret_cast<unsigned char *>(xs + (l ? 0 : 2 * B * XP)) - reinterpret_cast<unsigned char *>(smem), a.status);
 
-    // exchange words [set][layer][timestep (room for the handle's rows)][unit][8 rows][V tiles]
-    const unsigned slot_words = (unsigned)a.slot_words;
+    // exchange words [set][layer][timestep (room for 32 rows)][unit][8 rows][V tiles]
+    const unsigned slot_words = (unsigned)H * 32u;
     const size_t layer_words = (size_t)a.slots * slot_words, set_words = a.L * layer_words;
     unsigned *own = a.xch + (size_t)a.set * set_words + l * layer_words;
     const unsigned *below = own - (l ? layer_words : 0);
@@ -322,16 +320,9 @@ cudaError_t recur_f32_wave_prepare(int upc, int max_B, int smem_optin)
     return cudaSuccess;
 }
 
-// words of a timestep of one layer for up to `rows` sequences: a unit has eight rows of whole vector loads, one, two or four words
-int recur_f32_wave_slot_words(int H, int rows)
-{
-    const int nt = (std::min(rows, kF32MaxRows) + 7) / 8;
-    return H * 8 * (nt == 3 ? 4 : nt);
-}
-
 cudaError_t launch_recur_f32_wave(const RecurF32WaveArgs &a, cudaStream_t st)
 {
-    if (a.B < 1 || a.B > kF32MaxRows || a.T > a.slots || recur_f32_wave_slot_words(a.H, a.B) > a.slot_words) return cudaErrorInvalidValue;
+    if (a.B < 1 || a.B > kF32MaxRows || a.T > a.slots) return cudaErrorInvalidValue;
     const int nt = (a.B + 7) / 8, mt = (a.upc + 1) / 2;
     RecurF32WaveArgs copy = a;
     void *params[] = {&copy};

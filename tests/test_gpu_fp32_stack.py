@@ -99,23 +99,3 @@ def test_fp32_narrow_stack_beside_a_smaller_one(oracle):
     finally:
         for m, _, _ in models:
             m.close()
-
-
-@pytest.mark.parametrize("max_B,rows", [(1, (1,)), (8, (8, 3)), (9, (9, 8, 1)), (17, (17, 8, 16)), (33, (32, 5, 24))])
-def test_fp32_narrow_stack_words_for_the_rows_of_the_handle(oracle, max_B, rows):
-    """A handle has exchange words for the rows that its calls can have; calls of fewer rows, whose words lie otherwise, come between."""
-    import torch
-    import paper_1901_10997_b200 as pkg
-    w, weights, x, _, _ = make((2, 40, 150, 7, max(rows)), 6)
-    m = pkg.LSTM(weights, layers=2, in_dim=40, hidden=150, dtype="fp32", max_T=7, max_B=max_B)
-    try:
-        xd = torch.from_numpy(x).cuda()
-        for T, B in [(t, b) for b in rows for t in (7, 2)] * 2:
-            v = xd[:T, :B].contiguous()
-            got = m.forward(v)
-            m.check()
-            assert m.info()["launches_per_forward"] == 1
-            ref = oracle.forward(weights, v.cpu().numpy(), layers=2, bidir=False, hidden=150)
-            assert_close([t.cpu().numpy() for t in got], ref, "fp32", "fp32 stack, rows")
-    finally:
-        m.close()
