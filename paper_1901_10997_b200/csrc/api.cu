@@ -301,13 +301,48 @@ int alloc_phase_words(lstm_handle *h, PhaseWords &x, size_t set_words, cudaStrea
     x.set_words = set_words;
     return dev_alloc(h, &x.words, 2 * set_words * sizeof(unsigned), true, st, "exchange words");
 }
-// (last of a handle's allocations: what a step touches stays close together)
+// (behind a handle's other allocations: what a step touches stays close together)
 int alloc_recorded_words(lstm_handle *h, cudaStream_t st)
 {
     int rc = LSTM_OK;
-    for (PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->stack_xch, &h->f32_xch, &h->f32w_xch, &h->ht_hx, &h->ht_rx})
+    for (PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->f32_xch, &h->ht_hx, &h->ht_rx})
         if (rc == LSTM_OK && x->words) rc = dev_alloc(h, &x->recorded, 2 * x->set_words * sizeof(unsigned), true, st, "exchange words");
     return rc;
+}
+
+// What only calls need whose layers run side by side: rows for the pairs, words, the upper layer's G.  All other calls do without, and on
+// a handle that finds no room for it these run layer by layer too.  Last of all, so that nothing else goes short for it.
+void free_side_by_side(lstm_handle *h)
+{
+    for (Layer &ly : h->layers) { cudaFree(ly.wst); ly.wst = nullptr; }
+    for (PhaseWords *x : {&h->stack_xch, &h->f32w_xch}) { cudaFree(x->words); cudaFree(x->recorded); *x = PhaseWords(); }
+    cudaFree(h->stack_G);
+    h->stack_G = nullptr;
+}
+int alloc_side_by_side(lstm_handle *h, cudaStream_t st)
+{
+    int rc = LSTM_OK;
+    auto words = [&](PhaseWords &x, size_t set_words) {
+        if (rc == LSTM_OK) rc = alloc_phase_words(h, x, set_words, st);
+        if (rc == LSTM_OK) rc = dev_alloc(h, &x.recorded, 2 * set_words * sizeof(unsigned), true, st, "exchange words");
+    };
+    if (h->use_stack) {
+        words(h->stack_xch, 2 * kStackMaxChunks + 2 * recur_tc_xch_words(h->H, h->stack.rows, 1));
+        if (rc == LSTM_OK) rc = dev_alloc(h, &h->stack_G, (size_t)h->stack_M * 4 * h->H * 4, false, st, "upper layer's projection");
+        for (Layer &ly : h->layers) {
+            if (rc == LSTM_OK) rc = dev_alloc(h, &ly.wst, (size_t)h->stack.ncta * h->stack.KH * 8 * h->stack.upc * 2, false, st, "recurrent weight rows");
+            if (rc == LSTM_OK && launch_repartition(ly.wtc[0][0], h->tcb[0], ly.wst, h->stack, h->H, st) != cudaSuccess)
+                rc = fail(h, LSTM_ERR_CUDA, "packing launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+        }
+    }
+    if (h->f32w_upc) words(h->f32w_xch, (size_t)h->L * std::min(h->max_T, kF32WaveMaxT) * h->H * 32);
+    if (rc != LSTM_ERR_NOMEM) return rc;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "workspace set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
+    free_side_by_side(h);
+    h->use_stack = false;
+    h->f32w_upc = 0;
+    h->err.clear();
+    return LSTM_OK;
 }
 
 bool recording(cudaStream_t st)
@@ -681,11 +716,11 @@ void free_all(lstm_handle *h)
         for (int d = 0; d < 2; ++d) { cudaFree(ly.wh[d]); cudaFree(ly.wh_ptr[d]); cudaFree(ly.wh_ent[d]); cudaFree(ly.wfrag[d]); cudaFree(ly.ofrag[d]); cudaFree(ly.oxfrag[d]); cudaFree(ly.xfrag[d]); cudaFree(ly.frag2[d]); cudaFree(ly.tfrag[d]); cudaFree(ly.tfrag2[d]); cudaFree(ly.csr_reg_ent[d]); cudaFree(ly.csr_reg_rows[d]); }
         cudaFree(ly.bias_out);
         for (int i = 0; i < 4; ++i) cudaFree(ly.wtc[i >> 1][i & 1]);
-        cudaFree(ly.wst);
     }
-    cudaFree(h->G); cudaFree(h->stack_G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
+    free_side_by_side(h);
+    cudaFree(h->G); cudaFree(h->xb0); cudaFree(h->xbn[0]); cudaFree(h->xbn[1]);
     cudaFree(h->ybuf[0]); cudaFree(h->ybuf[1]); cudaFree(h->xch); cudaFree(h->rxch); 
-    for (const PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->stack_xch, &h->f32_xch, &h->f32w_xch, &h->ht_hx, &h->ht_rx}) { cudaFree(x->words); cudaFree(x->recorded); }
+    for (const PhaseWords *x : {&h->one_xch, &h->tcb_xch[0], &h->tcb_xch[1], &h->f32_xch, &h->ht_hx, &h->ht_rx}) { cudaFree(x->words); cudaFree(x->recorded); }
     cudaFree(h->status_dev);
     for (int l = 0; l < kMaxWaveLayers; ++l) cudaFree(h->wave_frag[l]);
     cudaFree(h->wave_xch);
@@ -1045,12 +1080,6 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
             }
         }
         if (rc) break;
-        if (h->use_stack) {
-            rc = dev_alloc(h, &ly.wst, (size_t)h->stack.ncta * h->stack.KH * 8 * h->stack.upc * 2, false, st, "recurrent weight rows");
-            if (rc == LSTM_OK && launch_repartition(ly.wtc[0][0], h->tcb[0], ly.wst, h->stack, H, st) != cudaSuccess)
-                rc = fail(h, LSTM_ERR_CUDA, "packing launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-            if (rc) break;
-        }
         rc = upload(h, &ly.bias, bias_p.data(), bias_p.size() * 4, st, "bias");
         if (rc == LSTM_OK && !csr)
             rc = bf16 ? upload(h, (uint16_t **)&ly.wx, wx16.data(), wx16.size() * 2, st, "input weights")
@@ -1117,18 +1146,13 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
     {
         const int upc = dtype == LSTM_F32 && !csr && D == 1 && side_by_side_wanted() ? recur_f32_wave_units(layers, H, in_dim, h->cta_limit) : 0;
         if (rc == LSTM_OK && upc) {
-            rc = alloc_phase_words(h, h->f32w_xch, (size_t)layers * std::min(max_T, kF32WaveMaxT) * H * 32, st);
-            if (rc == LSTM_OK && recur_f32_wave_prepare(upc, max_B, h->smem_optin) != cudaSuccess)
+            if (recur_f32_wave_prepare(upc, max_B, h->smem_optin) != cudaSuccess)
                 rc = fail(h, LSTM_ERR_CUDA, "fp32 stack kernel set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
             h->f32w_upc = upc;
         }
     }
     for (int i = 0; i < 2 && rc == LSTM_OK; ++i)
         if (i ? h->use_tc1 : h->use_tcb) rc = alloc_phase_words(h, h->tcb_xch[i], recur_tc_xch_words(H, h->tcb[i].rows, D), st);
-    if (rc == LSTM_OK && h->use_stack) {
-        rc = alloc_phase_words(h, h->stack_xch, 2 * kStackMaxChunks + 2 * recur_tc_xch_words(H, h->stack.rows, 1), st);
-        if (rc == LSTM_OK) rc = dev_alloc(h, &h->stack_G, (size_t)h->stack_M * 4 * H * 4, false, st, "upper layer's projection");
-    }
     if (rc == LSTM_OK) rc = dev_alloc(h, &h->status_dev, sizeof(int), true, st, "status word");
     if (rc == LSTM_OK && h->use_wave) {
         h->wave_xch_words = (size_t)layers * max_T * std::min(max_B, 4) * H;
@@ -1146,6 +1170,7 @@ static int create_impl(lstm_handle **out, int layers, int in_dim, int hidden, in
         if (e != cudaSuccess) rc = fail(h, LSTM_ERR_CUDA, "kernel set-up failed: %s", cudaGetErrorString(e));
     }
     if (rc == LSTM_OK) rc = alloc_recorded_words(h, st);
+    if (rc == LSTM_OK) rc = alloc_side_by_side(h, st);
     if (rc == LSTM_OK && cudaStreamSynchronize(st) != cudaSuccess)
         rc = fail(h, LSTM_ERR_CUDA, "workspace set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
     if (rc) return bail(rc);

@@ -232,3 +232,41 @@ def test_memory_of_handles_whose_calls_are_too_short(H, max_T, holds_more, monke
     both = held()
     monkeypatch.setenv("LSTM_B200_WAVE", "0")
     assert (both - held() >= 2 * 4 * H * H * 2) == holds_more      # the rows of both layers' recurrent matrices, at least
+
+
+def test_handle_without_room_for_two_layers_side_by_side(oracle):
+    """Memory for everything but the second copy of the rows and the second G: the layers run one after the other."""
+    import torch
+    import paper_1901_10997_b200 as pkg
+    w, weights, x, _, _ = make((16, 1200, 16, 5, 1.0), 8)
+    ref = oracle.forward(weights, x, layers=2, bidir=False, hidden=1200)
+    shape = dict(layers=2, in_dim=16, hidden=1200, dtype="bf16", max_T=409, max_B=20)      # a second G of 157 MB
+    xd = torch.from_numpy(x).cuda()
+
+    def run(m):
+        got = m.forward(xd)
+        m.check()
+        assert_close([t.cpu().numpy() for t in got], ref, "bf16", "stack, little memory")
+        return m.info()["launches_per_forward"]
+
+    pkg.LSTM(weights, **shape).close()              # (what the first handle of a process sets up)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    m = pkg.LSTM(weights, **shape)
+    needs = before - torch.cuda.mem_get_info()[0]
+    try:
+        assert run(m) == 3
+    finally:
+        m.close()
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - needs + (100 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        m = pkg.LSTM(weights, **shape)
+        try:
+            assert run(m) == 5
+        finally:
+            m.close()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
