@@ -96,7 +96,8 @@ def measured_peaks():
 def measured_traffic(kernel: str, workload: str, source: str):
     """(DRAM bytes per launch, where they come from) of the dominant kernel from the committed ncu summary
     profiles/<kernel>_<workload>.md; (None, reason) when there is none or the kernel's source has changed
-    since the counters were taken (the summary records the sha256 of the source file it profiled)."""
+    since the counters were taken (the summary records the sha256 of the source file it profiled, followed by the headers
+    that hold parts of its kernel)."""
     import hashlib
     import re
     f = ROOT / "profiles" / f"{kernel}_{workload}.md"
@@ -108,7 +109,9 @@ def measured_traffic(kernel: str, workload: str, source: str):
     m_tr = re.search(r"traffic_bytes_per_launch:\s*([0-9]+)", text)
     if not (m_sha and m_tr):
         return None, f"profiles/{f.name} carries no counters"
-    if hashlib.sha256(src.read_bytes()).hexdigest() != m_sha.group(1):
+    code = src.read_bytes()
+    parts = [h.decode() for h in re.findall(rb'#include "(\w+\.cuh)"', code) if h not in (b"common.cuh", b"device_util.cuh")]
+    if hashlib.sha256(b"".join([code, *((src.parent / h).read_bytes() for h in parts)])).hexdigest() != m_sha.group(1):
         return None, f"profiles/{f.name} was taken from an earlier revision of {source}"
     return int(m_tr.group(1)), f"profiles/{f.name} (one ncu capture, dram__bytes_read.sum + dram__bytes_write.sum; not measured in this run)"
 
@@ -344,13 +347,11 @@ def trimmed_mean(ms, drop=0.1):
     return float(sum(keep) / len(keep))
 
 
-def kernel_of(pkg, info, layers=1):
+def kernel_of(pkg, info):
     """The recurrent kernel of the last call, its source file, and the layers that one launch of it ran."""
-    name, launches, at_once = pkg.RECUR_KERNELS[info["kernel"]], info["launches_per_forward"], 1
-    if layers == 2 and info["kernel"] == pkg.LSTM_RAN_BATCHED and launches == 3:          # staging, one projection, both layers
-        name, at_once = "recur_stack_kernel", 2
-    elif layers > 1 and info["kernel"] == pkg.LSTM_RAN_F32 and launches == 1:
-        name, at_once = "recur_f32_wave_kernel", layers
+    name, at_once = pkg.RECUR_KERNELS[info["kernel"]], info["kernel_layers"]
+    if at_once > 1:
+        name = {pkg.LSTM_RAN_BATCHED: "recur_stack_kernel", pkg.LSTM_RAN_F32: "recur_f32_wave_kernel"}.get(info["kernel"], name)
     return name, name.removesuffix("_kernel") + ".cu", at_once
 
 
@@ -429,16 +430,20 @@ class GpuCase:
     def roofline(self, rec_ms, rec_n, peak, peak_kind, fused=False):
         w = self.w
         alg_bytes = recurrence_bytes_per_launch(w, "hlstm" if self.mode == "hlstm" else self.nnz())
-        if fused:
+        info = self.model.info()
+        kernel_name, kernel_src, at_once = kernel_of(self.pkg, info)
+        wbytes = 2 if w.dtype == "bf16" else 4
+        if at_once > 1:
+            # all layers in one launch, with the projections of the upper ones (the fp32 stack: of the lowest one too): their input
+            # matrices and activations once, and no rows of a projection launch for them
+            first = 0 if kernel_name == "recur_f32_wave_kernel" else 1
+            widths = [w.in_dim if layer == 0 else w.hidden for layer in range(first, at_once)]
+            alg_bytes = at_once * alg_bytes + sum(4.0 * w.hidden * (n * wbytes - w.T * w.B * 4.0) + w.T * w.B * n * 4.0 for n in widths)
+        elif fused:
             # the launch also computes its layer's input projection: the input matrix and the activations once
-            wbytes = 2 if w.dtype == "bf16" else 4
             in_avg = (w.in_dim + (w.layers - 1) * w.dirs * w.hidden) / w.layers
             alg_bytes += w.dirs * 4.0 * w.hidden * in_avg * wbytes + w.T * w.B * in_avg * 4.0
         rec_avg_ms = rec_ms / max(rec_n, 1)
-        achieved = alg_bytes / (rec_avg_ms * 1e-3) / 1e9 if rec_avg_ms > 0 else None
-        info = self.model.info()
-        kernel_name, kernel_src, at_once = kernel_of(self.pkg, info, w.layers)
-        alg_bytes *= at_once
         achieved = alg_bytes / (rec_avg_ms * 1e-3) / 1e9 if rec_avg_ms > 0 else None
         traffic, source = measured_traffic(kernel_name, self.name, kernel_src)
         steps_per_launch = w.T * (2 if (w.dirs == 2 and info.get("ctas_per_dir") == info.get("sm_count")) else 1)

@@ -269,7 +269,7 @@ enum {
 /*
  * Read-only facts about how the handle runs (for reports): writes up to n values into out and
  * returns the number available.  [1]..[5] and [9]..[11] describe the per-layer kernel that serves whatever no
- * other kernel of the handle does; [19]..[22] describe what the last lstm_forward launched.
+ * other kernel of the handle does; [19]..[23] describe what the last lstm_forward launched.
  * Order: [0] SM count, [1] CTAs of the per-layer kernel per direction,
  * [2] threads per CTA, [3] dynamic shared memory bytes per CTA at max_B, [4] recurrent-matrix rows
  * resident in shared memory per CTA (max over CTAs), [5] rows streamed from L2 per CTA (max),
@@ -290,7 +290,8 @@ enum {
  * the layers: all layers in one launch, layer l on timestep t beside layer l-1 on t+1) for one sequence and, where it is
  * faster than the batched kernel, for up to four,
  * [19] the recurrent kernel the last lstm_forward launched (LSTM_RAN_*), [20] CTAs of that launch (the last one of the
- * call), [21] its threads per CTA, [22] its dynamic shared memory per CTA in bytes.
+ * call), [21] its threads per CTA, [22] its dynamic shared memory per CTA in bytes, [23] the layers that this one launch ran
+ * (LSTM_RAN_BATCHED: 2 is recur_stack_kernel; LSTM_RAN_F32: more than one is recur_f32_wave_kernel).
  */
 LSTM_API int lstm_info(const lstm_handle *h, int64_t *out, int n);
 

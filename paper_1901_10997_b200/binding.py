@@ -172,7 +172,7 @@ def lstm_info(handle):
             "col_tiles_in_registers", "col_tiles_in_smem", "recur_batched_tensor_core",
             "recur_csr_register_resident", "csr_slots_per_lane", "csr_bank_conflict_wavefronts",
             "compact_hidden", "units_removed", "layer_wavefront",
-            "kernel", "kernel_ctas", "kernel_threads", "kernel_smem_bytes"]
+            "kernel", "kernel_ctas", "kernel_threads", "kernel_smem_bytes", "kernel_layers"]
     return {k: int(out[i]) for i, k in enumerate(keys[:n])}
 
 

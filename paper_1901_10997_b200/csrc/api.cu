@@ -132,7 +132,7 @@ struct lstm_handle {
     std::vector<int> ev_kind;
     int ev_used = 0;
     int last_launches = 0;
-    int ran_kernel = LSTM_RAN_NONE, ran_ctas = 0, ran_threads = 0;     // recurrent kernel of the last forward call, as last launched
+    int ran_kernel = LSTM_RAN_NONE, ran_ctas = 0, ran_threads = 0, ran_layers = 0;     // recurrent kernel of the last forward call, as last launched
     size_t ran_smem = 0;
     // layer-wavefront kernel (unidirectional stacks, up to four sequences): CTAs per layer, units per CTA, tiling
     bool use_wave = false, wave_all = false;    // wave_all: LSTM_B200_WAVE=1, whatever else could serve the call
@@ -1497,9 +1497,9 @@ int hlstm_create(lstm_handle **out, int layers, int in_dim, int hidden, int gate
     return LSTM_OK;
 }
 
-static void ran(lstm_handle *h, int kernel, int ctas, int threads, size_t smem)
+static void ran(lstm_handle *h, int kernel, int ctas, int threads, size_t smem, int layers = 1)
 {
-    h->ran_kernel = kernel; h->ran_ctas = ctas; h->ran_threads = threads; h->ran_smem = smem;
+    h->ran_kernel = kernel; h->ran_ctas = ctas; h->ran_threads = threads; h->ran_smem = smem; h->ran_layers = layers;
 }
 
 static int record(lstm_handle *h, int kind, cudaStream_t st)
@@ -1687,7 +1687,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         const size_t smem = recur_wave_smem_bytes(h->wave_mt, h->wave_nkr, h->wave_nkw_max, h->wave_upc, B);
         if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         e = launch_recur_wave(m, h->wave_mt, h->wave_nkr, smem, st);
-        ran(h, LSTM_RAN_WAVE, m.ncta_layer * L, 16 * 32, smem);
+        ran(h, LSTM_RAN_WAVE, m.ncta_layer * L, 16 * 32, smem, L);
         ++h->last_launches;
         if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "wavefront launch failed: %s", cudaGetErrorString(e));
@@ -1716,7 +1716,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         e = launch_recur_f32_wave(m, st);
         if (e == cudaSuccess) phase_launched(h->f32w_xch, rec, (unsigned)T);
-        ran(h, LSTM_RAN_F32, m.ncta * L, kF32Threads, 0);
+        ran(h, LSTM_RAN_F32, m.ncta * L, kF32Threads, recur_f32_wave_smem_bytes(m), L);
         ++h->last_launches;
         if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "stack launch failed: %s", cudaGetErrorString(e));
@@ -1768,7 +1768,7 @@ int lstm_forward(lstm_handle *h, const float *x, int T, int B, const float *h0, 
         if (record(h, LSTM_K_RECUR, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         e = launch_recur_stack(s, h->stack_maps, plan, h->stack_ctas, st);
         if (e == cudaSuccess) phase_launched(h->stack_xch, rec, (unsigned)(2 * kStackMaxChunks + 2 * recur_tc_xch_words(H, B, 1)));
-        ran(h, LSTM_RAN_BATCHED, h->stack_ctas, kTcThreads, recur_stack_smem_bytes(plan, B, s.proj));
+        ran(h, LSTM_RAN_BATCHED, h->stack_ctas, kTcThreads, recur_stack_smem_bytes(plan, B, s.proj), 2);
         ++h->last_launches;
         if (record(h, -1, st)) return fail(h, LSTM_ERR_CUDA, "event record failed");
         if (e != cudaSuccess) return fail(h, LSTM_ERR_CUDA, "stack launch failed: %s", cudaGetErrorString(e));
@@ -2222,13 +2222,13 @@ int lstm_info(const lstm_handle *h, int64_t *out, int n)
     const int launches = h->last_launches > 0 ? h->last_launches : h->L * 2 + (h->use_tc ? 1 : 0);
     const int tcb_at_max = h->use_tcb ? (h->tcb[0].pair ? 2 : 1) : 0;
     if (h->use_csr_reg) shp.smem = recur_csr_reg_smem_bytes(h->csr_nw, h->csr_kspan, h->csr_mt, h->upc, h->max_B);
-    const int64_t vals[23] = {h->sm_count, h->ncta_dir, h->use_mma ? h->mma_nw * 32 : h->use_csr_reg ? h->csr_nw * 32 : h->threads, (int64_t)shp.smem,
+    const int64_t vals[24] = {h->sm_count, h->ncta_dir, h->use_mma ? h->mma_nw * 32 : h->use_csr_reg ? h->csr_nw * 32 : h->threads, (int64_t)shp.smem,
                               rows_res, rows_str, (l0.plan_M >= 0) ? l0.plan.nsplit : 1, h->use_tc ? 1 : 0, launches,
                               h->use_mma ? 1 : 0, h->use_mma ? h->mma_nkr : 0, h->use_mma ? h->mma_nks : 0, tcb_at_max,
                               h->use_csr_reg ? 1 : 0, h->use_csr_reg ? h->csr_slots : 0, h->use_csr_reg ? h->csr_conflicts : 0, 0, 0, h->use_wave ? 1 : 0,
-                              h->ran_kernel, h->ran_ctas, h->ran_threads, (int64_t)h->ran_smem};
-    for (int i = 0; i < n && i < 23; ++i) out[i] = vals[i];
-    return 23;
+                              h->ran_kernel, h->ran_ctas, h->ran_threads, (int64_t)h->ran_smem, h->ran_layers};
+    for (int i = 0; i < n && i < 24; ++i) out[i] = vals[i];
+    return 24;
 }
 
 }  // extern "C"

@@ -243,6 +243,7 @@ struct RecurF32WaveArgs {
 };
 int recur_f32_wave_units(int L, int H, int in_dim, int max_cta);
 cudaError_t recur_f32_wave_prepare(int upc, int max_B, int smem_optin);
+size_t recur_f32_wave_smem_bytes(const RecurF32WaveArgs &a);
 cudaError_t launch_recur_f32_wave(const RecurF32WaveArgs &a, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------------

@@ -320,13 +320,15 @@ cudaError_t recur_f32_wave_prepare(int upc, int max_B, int smem_optin)
     return cudaSuccess;
 }
 
+size_t recur_f32_wave_smem_bytes(const RecurF32WaveArgs &a) { return smem_bytes(a.in_dim, a.H, (a.B + 7) / 8, (a.upc + 1) / 2); }
+
 cudaError_t launch_recur_f32_wave(const RecurF32WaveArgs &a, cudaStream_t st)
 {
     if (a.B < 1 || a.B > kF32MaxRows || a.T > a.slots) return cudaErrorInvalidValue;
     const int nt = (a.B + 7) / 8, mt = (a.upc + 1) / 2;
     RecurF32WaveArgs copy = a;
     void *params[] = {&copy};
-    return cudaLaunchCooperativeKernel((const void *)pick(nt, mt), dim3(a.L * a.ncta), dim3(kThreads), params, smem_bytes(a.in_dim, a.H, nt, mt), st);
+    return cudaLaunchCooperativeKernel((const void *)pick(nt, mt), dim3(a.L * a.ncta), dim3(kThreads), params, recur_f32_wave_smem_bytes(a), st);
 }
 
 }  // namespace lstm

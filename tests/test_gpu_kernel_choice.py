@@ -113,3 +113,12 @@ def test_switch_that_keeps_the_layers_of_a_stack_apart(dtype, launches, value, s
     monkeypatch.setenv("LSTM_B200_RECUR", "")              # an empty switch is an unset one
     info = forward("lstm", dtype, False, 2, 200, 6, 9)
     assert info["launches_per_forward"] == launches[0 if side_by_side else 1]
+
+
+# (dtype, layers, H, T, B) -> kernel, layers of its last launch
+@pytest.mark.parametrize("dtype,L,H,T,B,kernel,layers", [("bf16", 2, 200, 6, 9, "BATCHED", 2), ("bf16", 3, 200, 6, 9, "BATCHED", 1), ("bf16", 3, 200, 6, 1, "WAVE", 3),
+                                                         ("fp32", 3, 100, 6, 9, "F32", 3), ("fp32", 1, 100, 6, 9, "F32", 1), ("bf16", 2, 200, 1, 3, "STEP", 1)])
+def test_layers_of_a_launch(dtype, L, H, T, B, kernel, layers):
+    import paper_1901_10997_b200 as pkg
+    info = forward("lstm", dtype, False, L, H, T, B)
+    assert (info["kernel"], info["kernel_layers"]) == (getattr(pkg, "LSTM_RAN_" + kernel), layers)
