@@ -300,7 +300,7 @@ cudaError_t launch_recur_csr_reg(const RecurCsrArgs &a, int slots, int nw, size_
 // ---------------------------------------------------------------------------------------------------
 constexpr int kTcMaxRows = 64;        // batch rows of one pass; larger calls run several passes
 constexpr int kTcThreads = 512;
-constexpr int kTcStaticSmem = 1024;   // bytes kept free for the kernel's static shared memory (barriers, flags: under 100)
+constexpr int kTcStaticSmem = 1024;   // bytes kept free for the kernel's static shared memory (barriers, flags: under 300)
 // h enters the products as `terms` bf16 terms: two (16 bits of h) for dense handles, three (all 24) for pruned ones, whose
 // lists multiply h as it is.  Columns of the operand with rg groups of eight batch rows (a multiple of 16):
 __host__ __device__ constexpr int tc_columns(int rg, int terms) { return (8 * rg * terms + 15) / 16 * 16; }

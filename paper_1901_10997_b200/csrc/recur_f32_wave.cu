@@ -15,9 +15,10 @@
 // conflict-free 8-byte load, two cycles of shared memory beside four of the tensor instruction.
 // A layer may run any number of steps ahead of the one above: its words have a slot for every timestep, which also makes the
 // phase bit (device_util.cuh) a plain "written" mark; the other set is cleared for the next launch.
-// Measured (us per call, T = 35, layer by layer on recur_f32.cu -> here): 2 x 200 with 20 rows 210 -> 145, 2 x 256 with 32 rows, T = 70
+// Measured (us per call, T = 35, layer by layer on recur_f32.cu -> here): 2 x 200 with 20 rows 210 -> 135, 2 x 256 with 32 rows, T = 70
 // 568 -> 387, 2 x 149 with 9 rows, T = 17 101 -> 60, 2 x 64 with one row, T = 4 34 -> 16, three layers of 150 with 16 rows, T = 12
-// 114 -> 47.  A step of 2 x 200 with 20 rows is 3.7 us: 1400 cycles of each half's products, 900 for the fetch of h, 1500 for sums and gates.
+// 114 -> 47.  A step of 2 x 200 with 20 rows is 3.7 us, 7100 cycles: 1400 for each half's products, 900 for the fetch of h, 1500 for sums and
+// gates; the rest was not told apart.
 // Every wait is bounded; on expiry the CTA records a timeout status, stops waiting and runs to the end.
 #include "common.cuh"
 #include "device_util.cuh"
@@ -301,7 +302,7 @@ size_t smem_bytes(int in_dim, int H, int nt, int mt)
 }  // namespace
 
 // Units per CTA so that all layers' CTAs fit the device at once, or 0: whole tiles of two units, four units at most (2 x 200, 20 rows:
-// 161 us with three units on 67 CTAs a layer, 162 with four on 50, which leaves the words with fewer readers).
+// 161 us with three units on 67 CTAs a layer and 162 with four on 50 in the first form of this kernel; four leave the words with fewer readers).
 int recur_f32_wave_units(int L, int H, int in_dim, int max_cta)
 {
     if (L < 2 || L > kMaxWaveLayers || H > kF32MaxUnits || in_dim > kF32MaxUnits) return 0;

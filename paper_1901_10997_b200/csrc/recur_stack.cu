@@ -6,8 +6,8 @@
 // resident (up to 192 accumulator rows a pair: the first 128 from tensor memory, the others from shared memory), and
 // between them the CTAs of stack_proj.cuh, which turn a chunk of timesteps of the lower layer's h into rows of the upper layer's G.
 // All three of the matrices do not fit the chip at 1500 x 1500; the one without a recurrence is streamed once per chunk.
-// Measured (us per call, one after the other -> here): 2 x 517, 3 rows, T = 23 137 -> 93; 2 x 1000, 8 rows, T = 35 206 -> 134; 2 x 1500, 20
-// rows, T = 35 296 -> 259; pruned, 16 rows 294 -> 244.  At 1500 and 20 rows a step takes 5.1 us (products 2650 clocks: 47 of 128 and
+// Measured (us per call, one after the other -> here): 2 x 517, 3 rows, T = 23 128 -> 81; 2 x 1000, 8 rows, T = 35 206 -> 134; 2 x 1500, 20
+// rows, T = 35 289 -> 254; pruned, 16 rows 286 -> 233.  At 1500 and 20 rows a step takes 5.1 us (products 2650 clocks: 47 of 128 and
 // 47 of 64 rows at N = 48) and a chunk of four steps 22 us of the projecting CTAs, whose products are bound by shared memory:
 // 167 KB a K block, weights once in and once out, activations once in and three times out.
 // The groups meet through counts in global memory, one per chunk: "planes of X stored" and "rows of G stored".
@@ -96,6 +96,9 @@ size_t recur_stack_smem_bytes(const RecurTcPlan &p, int rows, const StackProjArg
 // 32; 96, 82, 82, 81; 93, 49, 33, 19 (32 CTAs); 200 with 20 181, 91, 73, 73; 120, 107, 103, 103; 122, 61, 43, 36 (48); 296 with 32 207, 105, 98, 95;
 // 134, 120, 119, 118; 132, 67, 59, 60 (70).  One handle against all SMs: 65 to 296 units, 5 to 32 rows, T = 4 to 70 0.92 - 1.02.  Eight projecting
 // CTAs at 296: up to 1.10 at T = 4; pairs of 32 units 1.03 with 32 rows; 400 units with pairs of 24 1.06 with 8 rows.
+// Wider ones take the fewest units per CTA that leave 16 CTAs to project, and all SMs: 592 units with 8, 20, 32 rows on 16 units and 108 CTAs 118, 146, 157,
+// on 8 and all 116, 144, 153; 517 on 16 units and 92 CTAs 116, 144, 153, on 8 and all 116, 146, 155.  Without the 16: 1000 on 136 CTAs 204, 298,
+// 413, on 148 134, 179, 200.
 bool recur_stack_plan(int H, int max_cta, int rows_wanted, int terms, size_t max_smem, RecurTcPlan *p, int *ctas)
 {
     if (H <= 64) return false;
